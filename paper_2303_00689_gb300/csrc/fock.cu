@@ -218,16 +218,22 @@ __global__ void __launch_bounds__(128) fock_pair_kernel(MolDev m, PairDev pd, El
   for (int k = 0; k < 10; ++k) { cA[k] = ca[k]; cB[k] = cb[k]; }
 }
 
-// one-centre part of G on one atom, product p = (mu nu), from the packed density
-// block pa: sum_{la,si} P_la,si [2 (mu nu|la si) - (mu la|nu si)] with the five
-// one-centre integrals written out
-__device__ __forceinline__ double onec_fock(const Elem& e, int p, const double* __restrict__ pa) {
-  if (e.norb == 1) return p == 0 ? pa[0] * e.G_ss : 0.0;
+// g plus the one-centre part of G_mu,nu on one atom, from the packed density block
+// pa: sum_{la,si} P_la,si [2 (mu nu|la si) - (mu la|nu si)].  The five one-centre
+// integrals leave four terms of the sixteen (mu = nu) or two; they are added in the
+// order of la, si, so that an element is rounded the same way whoever sums it.
+__device__ __forceinline__ double add_onec(double g, const Elem& e, int mu, int nu, const double* __restrict__ pa) {
+  if (mu != nu) {
+    const bool s = mu == 0 || nu == 0;
+    const double H = s ? e.H_sp : e.H_pp, c = 2.0 * H - (s ? e.G_sp : e.G_p2), p = pa[c_pidx[mu][nu]];
+    return fma(p, mu < nu ? H : c, fma(p, mu < nu ? c : H, g));
+  }
   const double sp = 2.0 * e.G_sp - e.H_sp, pp = 2.0 * e.G_p2 - e.H_pp;
-  if (p == 0) return pa[0] * e.G_ss + (pa[4] + pa[5] + pa[6]) * sp;
-  if (p < 4) return pa[p] * (3.0 * e.H_sp - e.G_sp);
-  if (p < 7) return pa[0] * sp + pa[p] * e.G_pp + (pa[4] + pa[5] + pa[6] - pa[p]) * pp;
-  return pa[p] * (3.0 * e.H_pp - e.G_p2);
+  g = fma(pa[0], mu == 0 ? e.G_ss : sp, g);
+  if (e.norb > 1)
+#pragma unroll
+    for (int la = 1; la < 4; ++la) g = fma(pa[3 + la], mu == 0 ? sp : (la == mu ? e.G_pp : pp), g);
+  return g;
 }
 
 // one warp per atom: Coulomb sums over partners (lanes over partners, fixed
@@ -262,7 +268,7 @@ __global__ void fock_atom_kernel(MolDev m, PairDev pd, ElemTable tab, const doub
 #pragma unroll
   for (int k = 0; k < 10; ++k)
     if (k == p) g = acc[k];
-  g = 2.0 * g + onec_fock(e, p, Pd + (size_t)A * 10);
+  g = add_onec(2.0 * g, e, mu, nu, Pd + (size_t)A * 10);
   const size_t ix = (size_t)(o + mu) * m.n + o + nu;
   out[ix] = (h ? h[ix] : 0.0) + g;
 }
