@@ -117,6 +117,7 @@ struct sim_handle {
   long long ph_n[PH_COUNT] = {};
   int cur_phase = -1;
   cudaEvent_t cur_start = nullptr;
+  bool shared = false;   // its eigensolver grid runs beside those of other handles (batches, serving)
   // CUDA graphs of one step, one per phase of the 8-slot X ring
   bool graphs = false;
   cudaGraphExec_t gexec[8] = {};
@@ -301,7 +302,7 @@ static bool concurrent(const sim_handle* h) { return h->side && !h->prof; }
 // eigenvectors are formed, and the caller joins before the density
 static int eig(sim_handle* h, bool fermi_side = false) {
   phase_begin(h, PH_TRIDIAG);
-  int st = eig_tridiagonalize(h->stream, h->n, h->Fock, h->ew, &h->sc->status, h->sms, mixed(h));
+  int st = eig_tridiagonalize(h->stream, h->n, h->Fock, h->ew, &h->sc->status, h->sms, mixed(h), h->shared);
   phase_end(h);
   if (st != 0) return fail(SIM_EINTERNAL, "tridiagonalisation launch failed (code " + std::to_string(st) + ")");
   phase_begin(h, PH_BISECT);
@@ -784,8 +785,9 @@ static int scf(sim_handle* h, int* iters, bool from_current = false) {
   return fail(SIM_ENOCONV, msg);
 }
 
-int sim_create(const sim_config* cfg, const sim_param_table* table, int natoms, const int* Z,
-               const double* R, const double* V, int charge, const double* P0, sim_handle** out) {
+static int create_handle(const sim_config* cfg, const sim_param_table* table, int natoms, const int* Z,
+                         const double* R, const double* V, int charge, const double* P0, bool shared,
+                         sim_handle** out) {
   if (!cfg || !table || !Z || !R || !out || natoms < 1) return fail(SIM_EINVAL, "null argument or natoms < 1");
   *out = nullptr;
   if (!(cfg->Te > 0.0) || !(cfg->dt > 0.0) || cfg->m_max < 1 || cfg->m_max > 16 || cfg->m_min < 1 ||
@@ -803,6 +805,7 @@ int sim_create(const sim_config* cfg, const sim_param_table* table, int natoms, 
   h->table_raw = *table;
   h->Z_h.assign(Z, Z + natoms);
   h->charge = charge;
+  h->shared = shared;
   for (int e = 0; e < 4; ++e)
     if (build_elem(table->v[e], h->tab.e[e]) != 0) {
       delete h;
@@ -942,6 +945,11 @@ int sim_create(const sim_config* cfg, const sim_param_table* table, int natoms, 
   }
   *out = h;
   return SIM_OK;
+}
+
+int sim_create(const sim_config* cfg, const sim_param_table* table, int natoms, const int* Z, const double* R,
+               const double* V, int charge, const double* P0, sim_handle** out) {
+  return create_handle(cfg, table, natoms, Z, R, V, charge, P0, false, out);
 }
 
 int sim_step_async(sim_handle* h, int nsteps) {
@@ -1098,7 +1106,12 @@ static int batch_capture(sim_batch* b, int p) {
     if (cudaEventRecord(b->fork, b->master) != cudaSuccess) rc = SIM_EINTERNAL;
     for (int i = g0; i < g1 && rc == SIM_OK; ++i)
       if (cudaStreamWaitEvent(b->hs[i]->stream, b->fork, 0) != cudaSuccess) rc = SIM_EINTERNAL;
-    for (int i = g0; i < g1 && rc == SIM_OK; ++i) rc = one_step(b->hs[i]);
+    for (int i = g0; i < g1 && rc == SIM_OK; ++i) {
+      const bool shared = b->hs[i]->shared;
+      b->hs[i]->shared = true;             // (same results, a smaller eigensolver grid)
+      rc = one_step(b->hs[i]);
+      b->hs[i]->shared = shared;
+    }
     for (int i = g0; i < g1 && rc == SIM_OK; ++i)
       if (cudaEventRecord(b->join[i], b->hs[i]->stream) != cudaSuccess ||
           cudaStreamWaitEvent(b->master, b->join[i], 0) != cudaSuccess)
@@ -1147,7 +1160,7 @@ int sim_batch_create(sim_handle* const* hs, int count, sim_batch** out) {
   const long long cap = 1000LL * hs[0]->sms;
   long long load = 0;
   for (int i = 0; i < count; ++i) {
-    long long w = eig_tridiag_weight(hs[i]->n, hs[i]->sms);
+    long long w = eig_tridiag_weight(hs[i]->n, hs[i]->sms, mixed(hs[i]), true);
     if (i > 0 && load + w > cap) {
       b->group_end.push_back(i);
       load = 0;
@@ -1215,12 +1228,14 @@ int sim_batch_step(sim_handle* const* hs, int count, int nsteps) {
   int first = SIM_OK;
   // groups of consecutive handles whose persistent eigensolver grids fit on
   // the device at the same time (their grid barriers need every block resident)
+  // several handles: small grids, except in step graphs, which are captured already
+  auto few = [count](const sim_handle* h) { return h->shared || (count > 1 && !(h->graphs && !h->prof)); };
   for (int g0 = 0; g0 < count;) {
     const long long cap = 1000LL * hs[g0]->sms;
     long long load = 0;
     int g1 = g0;
     while (g1 < count) {
-      long long w = eig_tridiag_weight(hs[g1]->n, hs[g1]->sms);
+      long long w = eig_tridiag_weight(hs[g1]->n, hs[g1]->sms, mixed(hs[g1]), few(hs[g1]));
       if (g1 > g0 && load + w > cap) break;
       load += w;
       ++g1;
@@ -1230,7 +1245,10 @@ int sim_batch_step(sim_handle* const* hs, int count, int nsteps) {
     for (int k = 0; k < nsteps; ++k)
       for (int i = g0; i < g1; ++i) {
         if (k == 0) reset_records(hs[i]);
+        const bool shared = hs[i]->shared;
+        hs[i]->shared = few(hs[i]);
         int rc = launch_step(hs[i]);
+        hs[i]->shared = shared;
         if (rc) return rc;
       }
     for (int i = g0; i < g1; ++i) {
@@ -1512,3 +1530,8 @@ void sim_destroy(sim_handle* h) {
 }
 
 }  // extern "C"
+
+int kx::create_shared(const sim_config* cfg, const sim_param_table* table, int natoms, const int* Z, const double* R,
+                      const double* V, int charge, sim_handle** out) {
+  return create_handle(cfg, table, natoms, Z, R, V, charge, nullptr, true, out);
+}

@@ -1,19 +1,7 @@
 // FP64 symmetric eigensolver for F = Q diag(eps) Q^T (eq. 19 needs the
 // eigenpairs; eq. 36 needs them again for the DMPT response).
 //
-//  1. Householder tridiagonalisation in ONE persistent kernel: the rank-2
-//     update of column k is applied lazily, fused with the symmetric
-//     matrix-vector product of column k + 1, so every column costs one read
-//     and one write of the trailing matrix and one grid-wide barrier.  All
-//     blocks compute the reflector redundantly (same data, same reduction
-//     order, bitwise identical), so no broadcast is needed.  The barrier is a
-//     counter/generation pair with a bounded spin: on expiry the kernel sets
-//     kStatusTimeout and returns.
-//     The mixed-precision path runs the same algorithm in double-float
-//     arithmetic (df.cuh): the trailing matrix is held as FP32 (hi, lo)
-//     pairs and the O(n^2)-per-column update and matrix-vector product run on
-//     the FP32 pipe, 64 times GB300's FP64 rate, at about 48 significant bits;
-//     the reflector scalars (beta, tau) stay FP64.
+//  1. Householder tridiagonalisation (tridiag.cu).
 //  2. Eigenvalues of the tridiagonal matrix by bisection on Sturm counts,
 //     one thread per eigenvalue (ascending order by construction): a coarse
 //     FP32 phase, an FP64 bracket check, then FP64 bisection.
@@ -34,533 +22,14 @@
 
 namespace kx {
 
-constexpr int kTriThreads = 512;
 constexpr int kBtBlock = 64;          // reflectors per back-transform block (FP64 path)
 constexpr int kBtBlockTc = 128;       // reflectors per back-transform block (tensor-core path)
 constexpr double kEps = 2.220446049250313e-16;
 
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Grid-wide barrier of the persistent tridiagonalisation.  The wait is bounded
-// in wall time (kBarrierNs) and by an iteration cap; a block that gives up, or
-// that finds another block's timeout flag set, records kStatusTimeout and the
-// kernel returns.  Correct operation needs every block resident at once
-// (cooperative launch; callers that run several such grids concurrently keep
-// their total within what the device holds at one time, eig_tridiag_weight).
-constexpr unsigned long long kBarrierNs = 2000000000ull;   // 2 s
-// the wall-time limit the barriers use (per device; tests set it through
-// eig_set_barrier_limit; 0 makes every wait expire at once, even one that
-// would be satisfied, so a test can force the expiry path of a real step)
-__device__ unsigned long long g_barrier_ns = kBarrierNs;
-
-__device__ bool grid_barrier(unsigned* bar, unsigned nblocks, int* status) {
-  __shared__ int s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    volatile unsigned* vgen = bar + 1;
-    unsigned g = *vgen;
-    __threadfence();
-    unsigned arrived = atomicAdd(bar, 1u);
-    if (g_barrier_ns == 0) {
-      atomicOr(status, (int)kStatusTimeout);
-    } else if (arrived == nblocks - 1) {
-      atomicExch(bar, 0u);
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
-    } else {
-      const unsigned long long t0 = global_ns();
-      long long it = 0;
-      while (*vgen == g) {
-        ++it;
-        if ((it & 63) == 0 &&
-            (global_ns() - t0 > g_barrier_ns || it > (1LL << 27) ||
-             ((*(volatile int*)status) & kStatusTimeout))) {
-          atomicOr(status, (int)kStatusTimeout);
-          break;
-        }
-        __nanosleep(32);
-      }
-    }
-    __threadfence();
-    s_ok = ((*(volatile int*)status) & kStatusTimeout) ? 0 : 1;
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
-
-// Split-phase grid barrier on a monotonically increasing arrival counter
-// (reset to 0 before the launch): the e-th barrier of a block is passed once
-// the counter reaches e * nblocks.  grid_arrive makes the block's earlier
-// writes visible (CTA barrier, then a release reduction by thread 0), so
-// independent work can run before grid_wait (an acquire load, bounded in wall
-// time like grid_barrier; on expiry kStatusTimeout is set and false returned).
-__device__ __forceinline__ void grid_arrive(unsigned* cnt) {
-  __syncthreads();
-  if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
-}
-__device__ bool grid_wait(const unsigned* cnt, unsigned target, int* status) {
-  __shared__ int s_ok;
-  if (threadIdx.x == 0) {
-    const unsigned long long t0 = global_ns();
-    long long it = 0;
-    if (g_barrier_ns == 0) atomicOr(status, (int)kStatusTimeout);
-    for (; g_barrier_ns != 0;) {
-      unsigned v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
-      if ((int)(v - target) >= 0) break;
-      ++it;
-      if ((it & 63) == 0 && (global_ns() - t0 > g_barrier_ns || it > (1LL << 27) ||
-                             ((*(volatile int*)status) & kStatusTimeout))) {
-        atomicOr(status, (int)kStatusTimeout);
-        break;
-      }
-      __nanosleep(16);
-    }
-    s_ok = ((*(volatile int*)status) & kStatusTimeout) ? 0 : 1;
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
-
-__global__ void __launch_bounds__(kTriThreads) tridiag_kernel(int n, double* __restrict__ A,
-                                                              double* __restrict__ Vst,
-                                                              double* __restrict__ d,
-                                                              double* __restrict__ e,
-                                                              double* __restrict__ tau,
-                                                              double* __restrict__ pbuf,
-                                                              unsigned* bar, int* status) {
-  extern __shared__ double sm[];
-  double* vp = sm;           // previous reflector (valid for indices >= k)
-  double* wp = sm + n;       // previous w
-  double* vc = sm + 2 * n;   // current reflector
-  double* red = sm + 3 * n;  // 32 doubles of reduction scratch
-  __shared__ double s_par[4];  // beta, tau, scale, d_k
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int wpb = blockDim.x >> 5;
-  // row r of the trailing matrix goes to block r % G, warp (r / G) % wpb: every
-  // block keeps an equal share of rows as the trailing matrix shrinks
-  const int gw = blockIdx.x + gridDim.x * (tid >> 5);
-  const int totw = gridDim.x * wpb;
-  bool prev = false;
-
-  for (int k = 0; k < n - 2; ++k) {
-    // 1. row k of the lazily updated matrix
-    double loc = 0.0;
-    for (int j = k + 2 + tid; j < n; j += blockDim.x) {
-      double x = A[(size_t)k * n + j];
-      if (prev) x -= vp[k] * wp[j] + wp[k] * vp[j];
-      vc[j] = x;
-      loc += x * x;
-    }
-    double sigma = block_sum(loc, red);
-    if (tid == 0) {
-      double xk = A[(size_t)k * n + k];
-      double x1 = A[(size_t)k * n + k + 1];
-      if (prev) {
-        xk -= 2.0 * vp[k] * wp[k];
-        x1 -= vp[k] * wp[k + 1] + wp[k] * vp[k + 1];
-      }
-      double beta, t, scale;
-      if (sigma == 0.0) {
-        beta = x1; t = 0.0; scale = 0.0;
-      } else {
-        double nrm = ::sqrt(x1 * x1 + sigma);
-        beta = (x1 >= 0.0) ? -nrm : nrm;
-        t = (beta - x1) / beta;
-        scale = 1.0 / (x1 - beta);
-      }
-      s_par[0] = beta; s_par[1] = t; s_par[2] = scale; s_par[3] = xk;
-    }
-    __syncthreads();
-    const double t = s_par[1], scale = s_par[2];
-    for (int j = k + 2 + tid; j < n; j += blockDim.x) vc[j] *= scale;
-    if (tid == 0) vc[k + 1] = 1.0;
-    __syncthreads();
-    if (blockIdx.x == 0) {
-      if (tid == 0) { d[k] = s_par[3]; e[k] = s_par[0]; tau[k] = t; }
-      for (int j = tid; j < n; j += blockDim.x) Vst[(size_t)k * n + j] = (j > k) ? vc[j] : 0.0;
-    }
-    // 2. fused: apply the previous rank-2 update to rows/cols >= k+1 and
-    //    form p = tau A v for the current reflector
-    double* pb = pbuf + (size_t)(k & 1) * n;
-    for (int i = k + 1 + gw; i < n; i += totw) {
-      double* row = A + (size_t)i * n;
-      double acc = 0.0, acc2 = 0.0, acc3 = 0.0, acc4 = 0.0;   // four chains hide the FP64 latency
-      if (prev) {
-        const double vi = vp[i], wi = wp[i];
-        int j = k + 1 + lane;
-        for (; j + 96 < n; j += 128) {
-          double a = fma(-vi, wp[j], fma(-wi, vp[j], row[j]));
-          double b = fma(-vi, wp[j + 32], fma(-wi, vp[j + 32], row[j + 32]));
-          double c = fma(-vi, wp[j + 64], fma(-wi, vp[j + 64], row[j + 64]));
-          double e = fma(-vi, wp[j + 96], fma(-wi, vp[j + 96], row[j + 96]));
-          row[j] = a;
-          row[j + 32] = b;
-          row[j + 64] = c;
-          row[j + 96] = e;
-          acc = fma(a, vc[j], acc);
-          acc2 = fma(b, vc[j + 32], acc2);
-          acc3 = fma(c, vc[j + 64], acc3);
-          acc4 = fma(e, vc[j + 96], acc4);
-        }
-        for (; j < n; j += 32) {
-          double a = fma(-vi, wp[j], fma(-wi, vp[j], row[j]));
-          row[j] = a;
-          acc = fma(a, vc[j], acc);
-        }
-      } else {
-        int j = k + 1 + lane;
-        for (; j + 32 < n; j += 64) {
-          acc = fma(row[j], vc[j], acc);
-          acc2 = fma(row[j + 32], vc[j + 32], acc2);
-        }
-        for (; j < n; j += 32) acc = fma(row[j], vc[j], acc);
-      }
-      acc = warp_sum((acc + acc2) + (acc3 + acc4));
-      if (lane == 0) pb[i] = t * acc;
-    }
-    if (!grid_barrier(bar, gridDim.x, status)) return;
-    // 3. w = p - (tau/2)(p.v) v
-    loc = 0.0;
-    for (int j = k + 1 + tid; j < n; j += blockDim.x) loc += pb[j] * vc[j];
-    double pv = block_sum(loc, red);
-    for (int j = k + 1 + tid; j < n; j += blockDim.x) {
-      wp[j] = pb[j] - 0.5 * t * pv * vc[j];
-      vp[j] = vc[j];
-    }
-    prev = true;
-    __syncthreads();
-  }
-  if (blockIdx.x == 0 && tid == 0) {
-    if (n == 1) {
-      d[0] = A[0];
-    } else {
-      int a = n - 2, b = n - 1;
-      double a00 = A[(size_t)a * n + a], a10 = A[(size_t)b * n + a], a11 = A[(size_t)b * n + b];
-      if (prev) {
-        a00 -= 2.0 * vp[a] * wp[a];
-        a10 -= vp[b] * wp[a] + wp[b] * vp[a];
-        a11 -= 2.0 * vp[b] * wp[b];
-      }
-      d[a] = a00; d[b] = a11; e[a] = a10;
-    }
-  }
-}
-
-// ---- double-float tridiagonalisation (mixed path) -------------------------
-// block-wide double-float sum in a fixed order; every thread gets the total.
-// `scratch` holds >= 32 dfl of shared memory.
-__device__ __forceinline__ dfl df_block_sum(dfl v, dfl* scratch) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
-  v = df_warp_sum(df_norm(v));
-  __syncthreads();
-  if (lane == 0) scratch[wid] = v;
-  __syncthreads();
-  dfl t = (threadIdx.x < nw) ? scratch[threadIdx.x] : dfl{0.0f, 0.0f};
-  if (wid == 0) t = df_warp_sum(t);
-  if (threadIdx.x == 0) scratch[0] = t;
-  __syncthreads();
-  dfl r = scratch[0];
-  __syncthreads();
-  return r;
-}
-
-__global__ void to_df_kernel(size_t len, const double* __restrict__ x, dfl* __restrict__ y) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < len) y[i] = df_from_double_bits(x[i]);
-}
-
-// Same reduction as tridiag_kernel (lazy rank-2 update fused with the
-// matrix-vector product, one grid barrier per column), with the per-column
-// critical path shortened for a kernel that is latency- rather than FP64-bound:
-//  * after the barrier every block reads p_{k-1} and row k in one pass, forms
-//    w_{k-1} = p - (tau/2)(p.v)v and the updated row k (x = row k of A_k);
-//  * the matrix-vector product uses the unscaled x (x_{k+1} = x_1) and
-//    keeps a_{i,k+1}, so it need not wait for beta, tau and the scale, which
-//    thread 0 forms meanwhile:
-//    p_i = tau scale (sum_j a_ij x_j - beta a_{i,k+1}) since v = scale (x - beta e_{k+1});
-//  * a block's rows (i = k+1+b+rG) are cut into segments of 512 columns (256
-//    and 128 once the trailing matrix is narrower than 500 and 200 columns)
-//    and the (row, segment) items dealt over the warps, so the warps stay
-//    balanced while the trailing matrix shrinks; warp 0, which forms the
-//    reflector scalars first, takes the last item of each round, so it never
-//    holds more items than another warp; each lane issues the loads of its
-//    item before the arithmetic;
-//  * block reductions take one CTA barrier each.
-// Shared memory: PW[j] = (v_{k-1}, w_{k-1}) as one 16-byte pair (during the
-// first passes it holds row k and p_{k-1}), VC[j] = x_k, then v_k, plus
-// reduction scratch and the (row, segment) partial sums.
-constexpr int kTriThreadsDf = 512;    // threads per block of the double-float kernel
-constexpr int kDfRed = 32;
-constexpr int kDfSeg = 512;           // columns per (row, segment) work item: 16 per lane
-constexpr int kDfNarrow1 = 500;       // trailing width at and below which items are 256 columns
-constexpr int kDfNarrow2 = 200;       // ... and 128 columns
-static_assert(kTriThreadsDf / 32 <= kDfRed, "one reduction slot per warp");
-// rows per block at the first column, for a grid of G blocks
-static int tridiag_df_rmax(int n, int G) { return (n - 1 + G - 1) / G; }
-static size_t tridiag_smem_df(int n, int G) {
-  // at most 2 segments per row while the narrow items are in use
-  const size_t rmax = (size_t)tridiag_df_rmax(n, G),
-               smax = std::max<size_t>((size_t)(n - 1 + kDfSeg - 1) / kDfSeg, 2);
-  return (3 * (size_t)n + 2 * kDfRed + rmax + rmax * smax) * sizeof(dfl);
-}
-
-// Loads of data other blocks wrote since the last grid barrier (and of rows
-// this block does not own in every column) go past L1 to L2.
-__device__ __forceinline__ dfl ldcg_df(const dfl* p) {
-  const float2 v = __ldcg((const float2*)p);
-  return dfl{v.x, v.y};
-}
 // read-only data of this launch (written by an earlier one): cached loads
 __device__ __forceinline__ dfl ldg_df(const dfl* p) {
   const float2 v = __ldg((const float2*)p);
   return dfl{v.x, v.y};
-}
-
-// every thread gets the sum of the kTriThreadsDf / 32 warp partials (written to
-// scratch[warp] by lane 0 before a CTA barrier), added as a pairwise tree
-__device__ __forceinline__ dfl df_sum_partials(const dfl* scratch) {
-  constexpr int NW = kTriThreadsDf / 32;
-  dfl t[NW];
-#pragma unroll
-  for (int w = 0; w < NW; ++w) t[w] = scratch[w];
-#pragma unroll
-  for (int st = 1; st < NW; st <<= 1)
-#pragma unroll
-    for (int w = 0; w + st < NW; w += 2 * st) t[w] = df_add(t[w], t[w + st]);
-  return t[0];
-}
-
-__device__ __forceinline__ dfl lo2(float4 a) { return dfl{a.x, a.y}; }
-__device__ __forceinline__ dfl hi2(float4 a) { return dfl{a.z, a.w}; }
-__device__ __forceinline__ float4 pack4(dfl a, dfl b) { return make_float4(a.hi, a.lo, b.hi, b.lo); }
-
-// The fused items of column k for one block: the pending rank-2 update
-// (v_{k-1}, w_{k-1}) of rows/cols >= k+1, stored back, and sum_j a_ij x_j of
-// each (row, SEG-column segment) item into part[r * S + sg] (a_{i,k+1} of the
-// block's rows into ak1s).  Warp w starts at item w - 1, warp 0 at NW - 1.
-template <int SEG>
-__device__ __forceinline__ void df_items(dfl* __restrict__ A, int n, int k, int G, int R, int wid, int lane,
-                                         bool prev, const float4* PW, const dfl* VC, dfl* part, dfl* ak1s) {
-  constexpr int PER = SEG / 32, NW = kTriThreadsDf / 32;
-  const int S = (n - (k + 1) + SEG - 1) / SEG;
-  const int Q = R * S;
-  for (int q = (wid == 0) ? NW - 1 : wid - 1; q < Q; q += NW) {
-    const int r = q / S, sg = q - r * S;
-    const int i = k + 1 + (int)blockIdx.x + r * G;
-    float2* row = (float2*)(A + (size_t)i * n);
-    const int jb = k + 1 + sg * SEG + lane;
-    const bool full = (k + 1 + (sg + 1) * SEG) <= n;
-    dfl a0 = {0.0f, 0.0f}, a1 = {0.0f, 0.0f}, first = {0.0f, 0.0f};
-    if (full) {
-      float2 xr[PER];
-#pragma unroll
-      for (int u = 0; u < PER; ++u) xr[u] = __ldcg(row + jb + 32 * u);
-      if (prev) {
-        const float4 pwi = PW[i];
-        const dfl vi = lo2(pwi), wi = hi2(pwi);
-#pragma unroll
-        for (int u = 0; u < PER; ++u) {
-          const int j = jb + 32 * u;
-          const float4 pw = PW[j];
-          const dfl x = df_rank2(dfl{xr[u].x, xr[u].y}, vi, hi2(pw), wi, lo2(pw));
-          row[j] = make_float2(x.hi, x.lo);
-          if (u == 0) first = x;
-          if (u & 1) df_acc_mul(a1, x, VC[j]); else df_acc_mul(a0, x, VC[j]);
-        }
-      } else {
-#pragma unroll
-        for (int u = 0; u < PER; ++u) {
-          const int j = jb + 32 * u;
-          const dfl x = dfl{xr[u].x, xr[u].y};
-          if (u == 0) first = x;
-          if (u & 1) df_acc_mul(a1, x, VC[j]); else df_acc_mul(a0, x, VC[j]);
-        }
-      }
-    } else {
-      float2 xr[PER];
-#pragma unroll
-      for (int u = 0; u < PER; ++u) {
-        const int j = jb + 32 * u;
-        xr[u] = (j < n) ? __ldcg(row + j) : make_float2(0.0f, 0.0f);
-      }
-      const float4 pwi = prev ? PW[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      const dfl vi = lo2(pwi), wi = hi2(pwi);
-#pragma unroll
-      for (int u = 0; u < PER; ++u) {
-        const int j = jb + 32 * u;
-        if (j < n) {
-          dfl x = dfl{xr[u].x, xr[u].y};
-          if (prev) {
-            const float4 pw = PW[j];
-            x = df_rank2(x, vi, hi2(pw), wi, lo2(pw));
-            row[j] = make_float2(x.hi, x.lo);
-          }
-          if (u == 0) first = x;
-          if (u & 1) df_acc_mul(a1, x, VC[j]); else df_acc_mul(a0, x, VC[j]);
-        }
-      }
-    }
-    const dfl acc = df_warp_sum(df_add(df_norm(a0), df_norm(a1)));
-    if (lane == 0) {
-      part[r * S + sg] = acc;
-      if (sg == 0) ak1s[r] = first;        // lane 0, u = 0 is column k+1
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kTriThreadsDf) tridiag_df_kernel(int n, dfl* __restrict__ A,
-                                                                 double* __restrict__ Vst,
-                                                                 double* __restrict__ d,
-                                                                 double* __restrict__ e,
-                                                                 double* __restrict__ tau,
-                                                                 dfl* __restrict__ pbuf,
-                                                                 unsigned* bar, int* status, int rmax) {
-  extern __shared__ float4 sm4[];
-  float4* PW = sm4;                          // n pairs
-  dfl* VC = (dfl*)(sm4 + n);                 // n
-  dfl* redA = VC + n;                        // partials of p.v
-  dfl* redB = redA + kDfRed;                 // partials of sigma
-  dfl* ak1s = redB + kDfRed;                 // a_{i,k+1} of the block's rows (rmax)
-  dfl* part = ak1s + rmax;                   // (row, segment) partial sums (rmax x smax)
-  __shared__ dfl s_df[4];                    // beta, tau * scale, tau, scale
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  constexpr int T = kTriThreadsDf, NW = kTriThreadsDf / 32;
-  const int G = gridDim.x;
-  dfl tau_prev = {0.0f, 0.0f};               // tau_{k-1}
-  if (n == 1) {
-    if (blockIdx.x == 0 && tid == 0) d[0] = df_to_double(A[0]);
-    return;
-  }
-  for (int k = 0;; ++k) {
-    const bool prev = k > 0;
-    const bool last = (k == n - 2);
-    const dfl* pbp = pbuf + (size_t)((k + 1) & 1) * n;   // p_{k-1}
-    // pass 1: row k and p_{k-1} in one sweep of loads (kept in PW); partial p.v
-    dfl loc = {0.0f, 0.0f};
-#pragma unroll 4
-    for (int j = k + tid; j < n; j += T) {
-      const dfl a = ldcg_df(A + (size_t)k * n + j);
-      dfl p = {0.0f, 0.0f};
-      if (prev) {
-        p = ldcg_df(pbp + j);
-        df_acc_mul(loc, p, VC[j]);           // VC = v_{k-1}
-      }
-      PW[j] = pack4(a, p);
-    }
-    dfl wk = {0.0f, 0.0f}, vk = {0.0f, 0.0f}, coef = {0.0f, 0.0f};
-    if (prev) {
-      loc = df_warp_sum(df_norm(loc));
-      if (lane == 0) redA[wid] = loc;
-      __syncthreads();
-      const dfl pv = df_sum_partials(redA);
-      coef = df_mul(df_mul(dfl{0.5f, 0.0f}, tau_prev), pv);
-      vk = VC[k];
-      wk = df_sub(hi2(PW[k]), df_mul(coef, vk));   // PW[k] is not overwritten below
-    }
-    // pass 2: w_{k-1} and the updated row k; sigma = sum_{j >= k+2} x_j^2
-    dfl sig = {0.0f, 0.0f};
-    dfl dk = {0.0f, 0.0f};
-    for (int j = k + tid; j < n; j += T) {
-      const float4 ap = PW[j];
-      dfl x = lo2(ap);
-      if (prev) {
-        const dfl vj = VC[j];
-        const dfl wj = (j == k) ? wk : df_sub(hi2(ap), df_mul(coef, vj));
-        x = df_rank2(x, vk, wj, wk, vj);
-        if (j > k) PW[j] = pack4(vj, wj);
-      }
-      if (j == k) {
-        dk = x;
-      } else {
-        VC[j] = x;
-        if (j >= k + 2) df_acc_mul(sig, x, x);
-      }
-    }
-    if (last) {
-      __syncthreads();
-      if (blockIdx.x == 0 && tid == 0) {
-        const int b = n - 1;
-        dfl abb = ldcg_df(A + (size_t)b * n + b);
-        if (prev) abb = df_rank2(abb, lo2(PW[b]), hi2(PW[b]), hi2(PW[b]), lo2(PW[b]));
-        d[n - 2] = df_to_double(dk);
-        e[n - 2] = df_to_double(VC[b]);
-        d[b] = df_to_double(abb);
-      }
-      return;
-    }
-    sig = df_warp_sum(df_norm(sig));
-    if (lane == 0) redB[wid] = sig;
-    __syncthreads();
-    // thread 0: reflector scalars (double-float: GB300's FP64 divide and square
-    // root are long dependent chains) while the other warps start the product
-    if (tid == 0) {
-      const dfl sigma = df_sum_partials(redB);
-      const dfl x1 = VC[k + 1];
-      dfl beta, t, scale;
-      if (sigma.hi == 0.0f) {
-        beta = x1; t = dfl{0.0f, 0.0f}; scale = dfl{0.0f, 0.0f};
-      } else {
-        const dfl nrm = df_sqrt(df_add(df_mul(x1, x1), sigma));
-        beta = (x1.hi >= 0.0f) ? df_neg(nrm) : nrm;
-        t = df_mul(df_sub(beta, x1), df_recip(beta));
-        scale = df_recip(df_sub(x1, beta));
-      }
-      s_df[0] = beta;
-      s_df[1] = df_mul(t, scale);
-      s_df[2] = t;
-      s_df[3] = scale;
-      if (blockIdx.x == 0) { d[k] = df_to_double(dk); e[k] = df_to_double(beta); tau[k] = df_to_double(t); }
-    }
-    // fused: pending rank-2 update (v_{k-1}, w_{k-1}) of rows/cols >= k+1 and
-    // sum_j a_ij x_j over (row, segment) items
-    const int R = (n - (k + 1) - (int)blockIdx.x + G - 1) / G;
-    const int m1 = n - (k + 1);
-    const int segw = (m1 > kDfNarrow1) ? kDfSeg : ((m1 > kDfNarrow2) ? 256 : 128);
-    const int S = (m1 + segw - 1) / segw;
-    if (segw == kDfSeg) df_items<kDfSeg>(A, n, k, G, R, wid, lane, prev, PW, VC, part, ak1s);
-    else if (segw == 256) df_items<256>(A, n, k, G, R, wid, lane, prev, PW, VC, part, ak1s);
-    else df_items<128>(A, n, k, G, R, wid, lane, prev, PW, VC, part, ak1s);
-    __syncthreads();
-    const dfl beta_df = s_df[0], ts_df = s_df[1], scale_df = s_df[3];
-    tau_prev = s_df[2];
-    // p_i = tau scale (sum_j a_ij x_j - beta a_{i,k+1}), segments summed as a
-    // fixed tree (one warp per row while a row has at most 32 segments)
-    dfl* pb = pbuf + (size_t)(k & 1) * n;
-    if (S <= 32) {
-      int lpr = 1;                                  // lanes per row: power of two >= S
-      while (lpr < S) lpr <<= 1;
-      const int rpw = 32 / lpr;                     // rows per warp
-      const int sub = lane / lpr, sl = lane - sub * lpr;
-      for (int r0 = wid * rpw; r0 < R; r0 += NW * rpw) {
-        const int r = r0 + sub;
-        dfl v = (r < R && sl < S) ? part[r * S + sl] : dfl{0.0f, 0.0f};
-        for (int o = lpr >> 1; o > 0; o >>= 1) v = df_add(v, df_shfl_xor(v, o));
-        if (r < R && sl == 0) pb[k + 1 + (int)blockIdx.x + r * G] = df_mul(ts_df, df_sub(v, df_mul(beta_df, ak1s[r])));
-      }
-    } else {
-      for (int r = tid; r < R; r += T) {
-        dfl* pr = part + r * S;
-        for (int st = 1; st < S; st <<= 1)
-          for (int sg = 0; sg + st < S; sg += 2 * st) pr[sg] = df_add(pr[sg], pr[sg + st]);
-        pb[k + 1 + (int)blockIdx.x + r * G] = df_mul(ts_df, df_sub(pr[0], df_mul(beta_df, ak1s[r])));
-      }
-    }
-    grid_arrive(bar);
-    // while the other blocks finish: v_k = scale x (v_{k+1} = 1) and the
-    // reflector store row k, spread over blocks
-    for (int j = k + 1 + tid; j < n; j += T) {
-      const dfl v = (j == k + 1) ? dfl{1.0f, 0.0f} : df_mul(VC[j], scale_df);
-      VC[j] = v;
-      if (j % G == (int)blockIdx.x) Vst[(size_t)k * n + j] = df_to_double_fast(v);
-    }
-    if (!grid_wait(bar, (unsigned)(k + 1) * (unsigned)G, status)) return;
-  }
 }
 
 // Gershgorin interval, squared off-diagonals, pivmin; one block
@@ -1309,100 +778,6 @@ size_t eig_work_bytes(int n) { return eig_layout(n, nullptr, nullptr); }
 // base must be 256-byte aligned (arena allocations are)
 void eig_work_bind(EigWork& w, void* base, int n) { eig_layout(n, base, &w); }
 
-// About 64K (FP64 kernel) or 32K (double-float kernel, whose columns cost
-// less arithmetic and more latency) elements of the initial matrix per block,
-// at most one block per SM; small systems keep small grids, so that many of
-// them fit on the device at once (molecule batches, serving).
-static int tridiag_blocks(int n, int sm_count, bool df) {
-  const int sh = df ? 15 : 16;
-  long long work = ((long long)n * n + (1LL << sh) - 1) >> sh;
-  int blocks = (int)work;
-  if (blocks < 1) blocks = 1;
-  if (blocks > sm_count) blocks = sm_count;           // one block per SM (two were slower)
-  return blocks;
-}
-
-static size_t tridiag_smem(int n) { return (3 * (size_t)n + 32) * sizeof(double); }
-
-// raise the kernel's opt-in dynamic shared memory monotonically, per device
-// (the attribute belongs to the device that is current; thread-safe)
-static bool tridiag_smem_attribute(size_t smem, bool df) {
-  if (smem <= 48 * 1024) return true;
-  static std::mutex mu;
-  static size_t smem_set[2][kMaxDevices] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
-  std::lock_guard<std::mutex> lk(mu);
-  if (smem > smem_set[df][dev]) {
-    const void* fn = df ? (const void*)tridiag_df_kernel : (const void*)tridiag_kernel;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    smem_set[df][dev] = smem;
-  }
-  return true;
-}
-
-// (the larger share of the FP64 and the double-float kernel)
-int eig_set_barrier_limit(unsigned long long ns) {
-  return cudaMemcpyToSymbol(g_barrier_ns, &ns, sizeof(ns)) == cudaSuccess ? 0 : -1;
-}
-
-int eig_tridiag_weight(int n, int sm_count) {
-  if (n <= 0) return 0;
-  int weight = 0;
-  for (int df = 0; df < 2; ++df) {
-    int p = 0;
-    const long long b = tridiag_blocks(n, sm_count, df != 0);
-    const size_t smem = df ? tridiag_smem_df(n, (int)b) : tridiag_smem(n);
-    const void* fn = df ? (const void*)tridiag_df_kernel : (const void*)tridiag_kernel;
-    if (!tridiag_smem_attribute(smem, df != 0) ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, fn, df ? kTriThreadsDf : kTriThreads, smem) !=
-            cudaSuccess ||
-        p < 1) {
-      cudaGetLastError();
-      p = 1;
-    }
-    const int wgt = (int)((1000LL * b + p - 1) / p);
-    weight = (wgt > weight) ? wgt : weight;
-  }
-  return weight;
-}
-
-int eig_tridiagonalize(cudaStream_t s, int n, const double* F, EigWork& w, int* status, int sm_count, bool df) {
-  if (n <= 0) return 0;
-  const size_t nn2 = (size_t)n * n;
-  if (df) {
-    // the workspace holds n x n (hi, lo) pairs: the same bytes as n x n doubles
-    to_df_kernel<<<(unsigned)((nn2 + 255) / 256), 256, 0, s>>>(nn2, F, (dfl*)w.A);
-    count_launch();
-  } else {
-    cudaMemcpyAsync(w.A, F, nn2 * sizeof(double), cudaMemcpyDeviceToDevice, s);
-  }
-  cudaMemsetAsync(w.bar, 0, 2 * sizeof(unsigned), s);
-  cudaMemsetAsync(w.e, 0, (size_t)n * sizeof(double), s);
-  // 1. tridiagonalisation
-  int blocks = tridiag_blocks(n, sm_count, df);
-  size_t smem = df ? tridiag_smem_df(n, blocks) : tridiag_smem(n);
-  if (!tridiag_smem_attribute(smem, df)) return -1;
-  if (df) cudaMemsetAsync(w.Vst, 0, nn2 * sizeof(double), s);   // entries left of the reflectors
-  int nn = n;
-  double *A = w.A, *V = w.Vst, *d = w.d, *e = w.e, *t = w.tau, *pb = w.pbuf;
-  unsigned* bar = w.bar;
-  int* st = status;
-  int rmax = tridiag_df_rmax(n, blocks);
-  void* args_fp64[] = {&nn, &A, &V, &d, &e, &t, &pb, &bar, &st};
-  void* args_df[] = {&nn, &A, &V, &d, &e, &t, &pb, &bar, &st, &rmax};
-  void** args = df ? args_df : args_fp64;
-  const void* fn = df ? (const void*)tridiag_df_kernel : (const void*)tridiag_kernel;
-  if (cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(df ? kTriThreadsDf : kTriThreads), args, smem, s) !=
-      cudaSuccess)
-    return -2;
-  count_launch();
-  return 0;
-}
-
 void eig_bisect(cudaStream_t s, int n, double* eps, EigWork& w, double rel_tol, bool df_path) {
   if (n <= 0) return;
   // 2. eigenvalues
@@ -1651,7 +1026,7 @@ int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork
 
 int symmetric_eig(cudaStream_t s, int n, const double* F, double* eps, double* Q, EigWork& w,
                   int* status, int sm_count) {
-  int rc = eig_tridiagonalize(s, n, F, w, status, sm_count, false);
+  int rc = eig_tridiagonalize(s, n, F, w, status, sm_count, false, false);
   if (rc) return rc;
   eig_bisect(s, n, eps, w, 1e-12, false);
   eig_vectors(s, n, eps, Q, w, false);

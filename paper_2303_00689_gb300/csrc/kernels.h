@@ -3,7 +3,15 @@
 #include <cuda_runtime.h>
 #include "common.cuh"
 
+struct sim_handle;
+struct sim_config;
+struct sim_param_table;
 namespace kx {
+
+// ---- api.cu -----------------------------------------------------------------
+// sim_create for a handle whose eigensolver grids run beside those of others (server)
+int create_shared(const sim_config* cfg, const sim_param_table* table, int natoms, const int* Z, const double* R,
+                  const double* V, int charge, sim_handle** out);
 
 // ---- pairs.cu ---------------------------------------------------------------
 bool upload_overlap_tables();
@@ -68,12 +76,13 @@ void eig_work_bind(EigWork& w, void* base, int n);
 // F (n x n symmetric, row-major) -> eps ascending, Q (eigenvectors as columns),
 // in three stages (tridiagonalise; tridiagonal eigenpairs into Q; back-transform Q)
 // df: double-float arithmetic on the FP32 pipe (mixed path), else FP64
+// shared: the grid runs beside those of other handles, whose total is kept within the device
 int eig_tridiagonalize(cudaStream_t s, int n, const double* F, EigWork& w, int* status, int sm_count,
-                       bool df);
+                       bool df, bool shared);
 // Share of the device, in thousandths of an SM, that the cooperative
 // tridiagonalisation grid of size n occupies while resident (blocks divided by
 // blocks per SM).  Grids that run concurrently must sum to <= 1000 x SMs.
-int eig_tridiag_weight(int n, int sm_count);
+int eig_tridiag_weight(int n, int sm_count, bool df, bool shared);
 // wall-time limit of the eigensolver's grid barriers on the current device (default 2 s)
 int eig_set_barrier_limit(unsigned long long ns);
 // rel_tol: eigenvalues to rel_tol x max(1, ||T||) (1e-12 FP64 path, 1e-9 mixed path)

@@ -152,8 +152,8 @@ void admission_loop(sim_server* s, int slot) {
     c.device = s->cfg.device;
     c.stream = nullptr;
     mark(s, slot, A_CREATE, j->ticket);
-    int rc = sim_create(&c, &j->req.table, j->req.natoms, j->Z.data(), j->R.data(),
-                        j->has_V ? j->V.data() : nullptr, j->req.charge, nullptr, &j->h);
+    int rc = kx::create_shared(&c, &j->req.table, j->req.natoms, j->Z.data(), j->R.data(),
+                               j->has_V ? j->V.data() : nullptr, j->req.charge, &j->h);
     mark(s, slot, A_GRAPHS, j->ticket);
     // Born-Oppenheimer steps read the SCF residual on the host: they run without graphs
     if (rc == SIM_OK && s->cfg.use_graphs && c.kernel != SIM_KERNEL_BOMD) rc = sim_enable_graphs(j->h, 1);
@@ -337,7 +337,7 @@ int sim_submit(sim_server* s, const sim_request* req, unsigned long long* ticket
     for (int A = 0; A < req->natoms; ++A) n += (req->Z[A] == 1) ? 1 : 4;
     cudaGetDevice(&prev);
     cudaSetDevice(s->cfg.device);
-    j->weight = kx::eig_tridiag_weight(n, s->sms);
+    j->weight = kx::eig_tridiag_weight(n, s->sms, j->req.cfg.precision == SIM_PREC_MIXED, true);
     cudaSetDevice(prev);
   }
   j->t_submit = Clock::now();
