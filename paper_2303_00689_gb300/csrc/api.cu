@@ -104,6 +104,7 @@ struct sim_handle {
   long long rec_count = 0;          // host: records written since the last reset
   EigWork ew;
   TcWork tw;
+  Tc64Work t64;
   int xhead = 0;
   int scf_iters = 0;   // SCF iterations used by sim_create (0 when P0 was given)
   double scf_residual = 0.0;
@@ -232,6 +233,13 @@ static double* xslot(sim_handle* h, int k) { return h->X[(h->xhead + k) % 8]; }
 
 static bool mixed(const sim_handle* h) { return h->cfg.precision == SIM_PREC_MIXED; }
 
+// C = A B^T of cut n x n operands (the size's tensor map was encoded at creation)
+static void tc64_mul(sim_handle* h, const Tc64Op& A, const Tc64Op& B, double* C, int sym, const int* gate = nullptr) {
+  const int n = h->n;
+  if (tc64_gemm(h->stream, n, n, 0, n, A, 0, B, 0, 0, 1.0, 0, C, n, sym, 0, h->t64.err, gate) != 0)
+    cudaMemsetAsync(h->t64.err, 1, sizeof(int), h->stream);
+}
+
 // D0 = Q diag(f) Q^T = (Q f^1/2)(Q f^1/2)^T, exactly symmetric
 static void density(sim_handle* h) {
   cudaStream_t s = h->stream;
@@ -242,13 +250,22 @@ static void density(sim_handle* h) {
     // all slices of a k-tile staged together (tc_gemm_grouped4)
     tc_split(s, h->tw, kSlotQs, h->Qs, 4, 0);
     tc_gemm_grouped4(s, h->tw, kSlotQs, kSlotQs, 1.0, h->D, 1);
+  } else if (h->t64.base) {
+    const Tc64Op q = tc64_slot(h->t64, 2, n, n);
+    tc64_cut_rows(s, q, 0, n, h->Qs, n);
+    tc64_mul(h, q, q, h->D, 1);
   } else {
     dgemm(s, 0, 1, n, n, n, 1.0, h->Qs, n, h->Qs, n, 0.0, h->D, n, 1);
   }
 }
 
-// BF16 pieces of Q and Q^T for the DMPT products (once per evaluation)
+// slices of Q and Q^T for the DMPT products (once per evaluation)
 static void dmpt_prepare(sim_handle* h) {
+  if (h->t64.base) {
+    const int n = h->n;
+    tc64_cut_rows(h->stream, tc64_slot(h->t64, 0, n, n), 0, n, h->Q, n);
+    tc64_cut_cols(h->stream, tc64_slot(h->t64, 1, n, n), n, h->Q, n);
+  }
   if (!mixed(h)) return;
   tc_split(h->stream, h->tw, kSlotQ, h->Q, 3, 0);
   tc_split(h->stream, h->tw, kSlotQt, h->Q, 3, 1);
@@ -274,6 +291,20 @@ static void dmpt(sim_handle* h, const double* F1, double* D1) {
     tc_gemm_grouped(s, h->tw, kSlotQ, kSlotT0, 1.0, h->T1, 0, g);       // T1 = Q Y
     tc_split(s, h->tw, kSlotT1, h->T1, 3, 0, g);
     tc_gemm_grouped(s, h->tw, kSlotT1, kSlotQ, 1.0, D1, 1, g);          // D1 = (Q Y) Q^T
+    return;
+  }
+  if (h->t64.base) {
+    const Tc64Op q = tc64_slot(h->t64, 0, n, n), qt = tc64_slot(h->t64, 1, n, n), x = tc64_slot(h->t64, 2, n, n);
+    tc64_cut_rows(s, x, 0, n, F1, n, g);
+    tc64_mul(h, qt, x, h->T1, 0, g);                     // T1 = Q^T F1
+    tc64_cut_rows(s, x, 0, n, h->T1, n, g);
+    tc64_mul(h, x, qt, h->T2, 1, g);                     // T2 = (Q^T F1) Q
+    launch_dmu(s, n, h->T2, h->eps, h->f, h->beta, h->sc);
+    launch_dmpt_y(s, n, h->T2, h->K, h->sc, h->Y);
+    tc64_cut_rows(s, x, 0, n, h->Y, n, g);
+    tc64_mul(h, q, x, h->T1, 0, g);                      // T1 = Q Y
+    tc64_cut_rows(s, x, 0, n, h->T1, n, g);
+    tc64_mul(h, x, q, D1, 1, g);                         // D1 = (Q Y) Q^T
     return;
   }
   dgemm(s, 0, 0, n, n, n, 1.0, F1, n, h->Q, n, 0.0, h->T1, n, 0, g);         // T1 = F1 Q
@@ -316,7 +347,8 @@ static int eig(sim_handle* h, bool fermi_side = false) {
   eig_vectors(h->stream, h->n, h->eps, h->Q, h->ew, mixed(h));
   phase_end(h);
   phase_begin(h, PH_BACKTR);
-  const int bt = eig_backtransform(h->stream, h->n, h->Q, h->ew, mixed(h) ? &h->tw : nullptr);
+  const int bt = eig_backtransform(h->stream, h->n, h->Q, h->ew, mixed(h) ? &h->tw : nullptr,
+                                   h->t64.base ? &h->t64 : nullptr);
   phase_end(h);
   if (bt != 0) return fail(SIM_EINTERNAL, "back-transformation: tensor map encoding failed");
   return SIM_OK;
@@ -585,13 +617,14 @@ static int launch_step(sim_handle* h) {
 static int check_status(sim_handle* h) {
   int st = 0, tce = 0;
   CUDA_TRY(cudaMemcpyAsync(&st, &h->sc->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  if (mixed(h)) CUDA_TRY(cudaMemcpyAsync(&tce, tc_error_flag(h->tw), sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  int* tc_err = mixed(h) ? tc_error_flag(h->tw) : h->t64.err;
+  if (tc_err) CUDA_TRY(cudaMemcpyAsync(&tce, tc_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));
   CUDA_TRY(cudaGetLastError());
   if (st || tce) {
     // an error is reported once: the device words are cleared for the next call
     CUDA_TRY(cudaMemsetAsync(&h->sc->status, 0, sizeof(int), h->stream));
-    if (mixed(h)) CUDA_TRY(cudaMemsetAsync(tc_error_flag(h->tw), 0, sizeof(int), h->stream));
+    if (tc_err) CUDA_TRY(cudaMemsetAsync(tc_err, 0, sizeof(int), h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
   }
   if (tce) return fail(SIM_ETIMEOUT, "a bounded tensor-core pipeline wait expired");
@@ -667,6 +700,10 @@ static void layout(sim_handle* h, Arena& a) {
   if (h->cfg.precision == SIM_PREC_MIXED) {
     void* twb = a.take<char>(tc_work_bytes(h->n));
     if (a.base) tc_work_bind(h->tw, twb, h->n);
+  } else if (tc_available()) {
+    // (without tensor maps the products run on the FP64 pipe, gemm64.cu)
+    void* t64 = a.take<char>(tc64_work_bytes(h->n));
+    if (a.base && !tc64_work_bind(h->t64, t64, h->n)) h->t64 = Tc64Work{};
   }
 }
 

@@ -91,9 +91,10 @@ void eig_bisect(cudaStream_t s, int n, double* eps, EigWork& w, double rel_tol, 
 // tridiagonal eigenvectors by inverse iteration; df_path: double-float arithmetic (mixed path)
 void eig_vectors(cudaStream_t s, int n, const double* eps, double* Q, EigWork& w, bool df_path);
 struct TcWork;
+struct Tc64Work;
 // tw != nullptr: the large products run on the tensor cores (mixed path)
 // returns nonzero when the tensor-core path could not encode its tensor maps
-int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork* tw);
+int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork* tw, const Tc64Work* t64);
 int symmetric_eig(cudaStream_t s, int n, const double* F, double* eps, double* Q, EigWork& w,
                   int* status, int sm_count);
 

@@ -79,6 +79,37 @@ void tc_reduce_split_rows(cudaStream_t s, int rows, int cols, const double* P, i
                           __nv_bfloat16* base, int ld, size_t stride);
 // test of the pipeline's bounded mbarrier wait: sets *err when `limit` tries expire
 void tc_mbar_expiry(cudaStream_t s, int* err, long long limit);
+bool tc_encode_map_box(CUtensorMap* m, void* ptr, int rows, int cols, int ld, int bk, int box_rows);
+
+// FP64 products (tc_gemm64.cu): an operand's rows cut into eight digits each
+constexpr int kTc64Slices = 8;
+struct Tc64Op {
+  __nv_bfloat16* p = nullptr;   // digit a of row r at p + (a rows + r) ld
+  int* ex = nullptr;            // row exponents
+  int rows = 0, ld = 0;
+};
+size_t tc64_op_bytes(int rows, int cols);              // a multiple of 256
+Tc64Op tc64_op(void* base, int rows, int cols);        // base 256-byte aligned
+// the device buffers of an FP64 handle: three operands of n x n and an error word
+struct Tc64Work {
+  char* base = nullptr;
+  int* err = nullptr;
+  int n = 0;
+};
+size_t tc64_work_bytes(int n);
+bool tc64_work_bind(Tc64Work& w, void* base, int n);   // false: no tensor map of this size
+Tc64Op tc64_slot(const Tc64Work& w, int slot, int rows, int cols);
+// columns [c0, cols) of the rows of X (c0 a multiple of 32); the rows of X^T, X of `cols` rows
+void tc64_cut_rows(cudaStream_t s, const Tc64Op& op, int c0, int cols, const double* X, size_t ldx,
+                   const int* gate = nullptr);
+void tc64_cut_cols(cudaStream_t s, const Tc64Op& op, int cols, const double* X, size_t ldx, const int* gate = nullptr);
+// C (M x N) = alpha A B^T (+ C if beta) over the columns k0 (a multiple of 32) to k1 of
+// rows a0 .. of A and b0 .. of B (there bx, a multiple of 32, columns on), zeros in both from k1 to the next multiple of 32;
+// diag (a multiple of 128): the diagonal blocks of that size only, one after the
+// other at C (ldc = diag); < 0 on a tensor-map error
+int tc64_gemm(cudaStream_t s, int M, int N, int k0, int k1, const Tc64Op& A, int a0, const Tc64Op& B, int b0, int bx,
+              double alpha, int beta, double* C, int ldc, int sym, int diag, int* err, const int* gate = nullptr);
+
 // raw access to a slot's slice buffers (for the back-transformation)
 __nv_bfloat16* tc_slot_base(const TcWork& w, int slot);
 size_t tc_slot_stride(const TcWork& w);
