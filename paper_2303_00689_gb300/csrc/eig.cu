@@ -1,0 +1,1137 @@
+// FP64 symmetric eigensolver for F = Q diag(eps) Q^T (eq. 19 needs the
+// eigenpairs; eq. 36 needs them again for the DMPT response).
+//
+//  1. Householder tridiagonalisation (tridiag.cu).
+//  2. Eigenvalues of the tridiagonal matrix by bisection on Sturm counts,
+//     one thread per eigenvalue (ascending order by construction): a coarse
+//     FP32 phase, an FP64 bracket check, then FP64 bisection.
+//  3. Eigenvectors by inverse iteration (two steps) with a partially pivoted
+//     tridiagonal LU, one thread per cluster of close eigenvalues; members of
+//     a cluster are re-orthogonalised (modified Gram-Schmidt) in order.
+//  4. Back-transformation Q = H_0 ... H_{n-3} Z with blocks of reflectors in
+//     compact WY form (I - V T V^T): FP64 GEMMs (64 per block) on the FP64
+//     path; on the mixed path (128 per block) the two large products
+//     V^T Z and V (T W) run on the tensor cores with 4 fixed-point BF16
+//     slices, while the T factor and T W stay in FP64.
+#include <algorithm>
+#include <mutex>
+
+#include "common.cuh"
+#include "df.cuh"
+#include "kernels.h"
+#include "tc_gemm.h"
+
+namespace kx {
+
+constexpr int kBtBlock = 64;          // reflectors per back-transform block (FP64 path)
+constexpr int kBtBlockTc = 128;       // reflectors per back-transform block (tensor-core path)
+constexpr double kEps = 2.220446049250313e-16;
+
+// read-only data of this launch (written by an earlier one): cached loads
+__device__ __forceinline__ dfl ldg_df(const dfl* p) {
+  const float2 v = __ldg((const float2*)p);
+  return dfl{v.x, v.y};
+}
+
+// Gershgorin interval, squared off-diagonals, pivmin; one block
+__global__ void gersh_kernel(int n, const double* __restrict__ d, const double* __restrict__ e,
+                             double* __restrict__ e2, double* __restrict__ scal, float* __restrict__ df,
+                             float* __restrict__ e2f, dfl* __restrict__ d_dfl, dfl* __restrict__ e2_dfl,
+                             dfl* __restrict__ e_dfl) {
+  double lo = 1e300, hi = -1e300, em = 0.0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    double r = 0.0;
+    df[i] = (float)d[i];                 // FP32 copies for the coarse phase (no per-step conversions)
+    e2f[i] = 0.0f;
+    d_dfl[i] = df_from_double(d[i]);     // double-float copies for the multisection and the
+    e2_dfl[i] = dfl{0.0f, 0.0f};         // inverse iteration (mixed path)
+    e_dfl[i] = (i < n - 1) ? df_from_double(e[i]) : dfl{0.0f, 0.0f};
+    if (i > 0) r += fabs(e[i - 1]);
+    if (i < n - 1) {
+      r += fabs(e[i]);
+      e2[i] = e[i] * e[i];
+      e2f[i] = (float)e2[i];
+      e2_dfl[i] = df_from_double(e2[i]);
+      em = fmax(em, e[i] * e[i]);
+    }
+    lo = fmin(lo, d[i] - r);
+    hi = fmax(hi, d[i] + r);
+  }
+  // min/max reductions through negation-free warp shuffles
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    em = fmax(em, __shfl_xor_sync(0xffffffffu, em, o));
+  }
+  __shared__ double slo[32], shi[32], sem[32];
+  int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) { slo[w] = lo; shi[w] = hi; sem[w] = em; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int nw = (blockDim.x + 31) >> 5;
+    for (int i = 1; i < nw; ++i) { lo = fmin(lo, slo[i]); hi = fmax(hi, shi[i]); em = fmax(em, sem[i]); }
+    double tn = fmax(fabs(lo), fabs(hi));
+    double pivmin = 1e-290 * fmax(1.0, em);
+    lo -= 4.0 * kEps * tn + 2.0 * pivmin;
+    hi += 4.0 * kEps * tn + 2.0 * pivmin;
+    scal[0] = lo; scal[1] = hi; scal[2] = tn; scal[3] = pivmin;
+  }
+}
+
+// Number of eigenvalues of T below x: sign changes of the leading principal
+// minors p_j = (d_j - x) p_{j-1} - e_{j-1}^2 p_{j-2} (Sturm sequence), kept in
+// range by exact power-of-two rescaling, so each step is two FMAs and no
+// division.  An exact zero minor counts as negative (the pivmin convention).
+__device__ __forceinline__ int sturm_count(int n, const double* __restrict__ d,
+                                           const double* __restrict__ e2, double x, double) {
+  // FP64 work per step is one multiply and one FMA; signs, zero tests and the
+  // rescaling test read the bit pattern with integer instructions.
+  double pm = 1.0;                    // p_{j-1}
+  double p = d[0] - x;                // p_0
+  long long b = __double_as_longlong(p);
+  int sp = (b < 0 || (b & 0x7FFFFFFFFFFFFFFFLL) == 0) ? 1 : 0;   // 1: negative (zero counts as negative)
+  int c = sp;
+  for (int j = 1; j < n; ++j) {
+    double pn = fma(d[j] - x, p, -e2[j - 1] * pm);
+    pm = p;
+    p = pn;
+    b = __double_as_longlong(pn);
+    int zero = (b & 0x7FFFFFFFFFFFFFFFLL) == 0;
+    int sn = zero ? (sp ^ 1) : (int)((unsigned long long)b >> 63);
+    c += sn ^ sp;
+    sp = sn;
+    int ex = (int)((b >> 52) & 0x7FF);             // biased exponent of p_j
+    if (ex > 1023 + 400) {
+      p *= 0x1p-400; pm *= 0x1p-400;
+    } else if (ex < 1023 - 400 && (int)((__double_as_longlong(pm) >> 52) & 0x7FF) < 1023 - 400) {
+      p *= 0x1p400; pm *= 0x1p400;
+    }
+  }
+  return c;
+}
+
+// FP32 Sturm count (ratio form with a pivot floor) for the coarse phase
+__device__ __forceinline__ int sturm_count_f32(int n, const float* __restrict__ d,
+                                               const float* __restrict__ e2, float x, float pivmin) {
+  float q = d[0] - x;
+  if (fabsf(q) <= pivmin) q = -pivmin;
+  int c = (q < 0.0f);
+  for (int j = 1; j < n; ++j) {
+    q = (d[j] - x) - e2[j - 1] / q;
+    if (fabsf(q) <= pivmin) q = -pivmin;
+    c += (q < 0.0f);
+  }
+  return c;
+}
+
+// FP64 path: eigenvalue i of T by multisection, M lanes a group: FP32 counts down to
+// ~2^-22 of the Gershgorin interval, a round of FP64 counts that takes both ends in
+// (and widens the bracket where the FP32 counts erred), then FP64 rounds to the
+// tolerance.  A count is a chain of n FP64 steps on a pipe that takes ~62 cycles a warp
+// instruction however many lanes are live, so lanes that count at other points of
+// the same interval are free until there are more warps than FP64 pipes (kFp64Pipes);
+// M = 32, 16, 8 up to 1, 1 and 2 warps a pipe.  n = 26, 240, 574,
+// 1680: 53, 290, 670, 3020 us; 165, 1370, 3160, 9220 with one lane an eigenvalue.
+constexpr int kFp64Pipes = 4 * 152;
+template <int M>
+__global__ void __launch_bounds__(32) bisect_kernel(int n, const double* __restrict__ d, const double* __restrict__ e2,
+                                                  const double* __restrict__ scal, const float* __restrict__ df,
+                                                  const float* __restrict__ e2f, double rel_tol,
+                                                  double* __restrict__ ev) {
+  const int t = blockIdx.x * 32 + threadIdx.x;
+  const int i = t / M, m = t % M;             // eigenvalue of this group, point of the lane
+  const int gbase = threadIdx.x & ~(M - 1);
+  const unsigned gmask = (M == 32) ? 0xffffffffu : (1u << M) - 1u;
+  const bool live = i < n;                    // whole groups are live or not
+  const double glo = scal[0], ghi = scal[1], pivmin = scal[3];
+  const double width = ghi - glo;
+  // points of the group with a count above i, as bits
+  auto above = [&](bool a) { return (__ballot_sync(0xffffffffu, a) >> gbase) & gmask; };
+  float lo32 = (float)glo, hi32 = (float)ghi;
+  const float piv32 = fmaxf((float)(1e-30 * fmax(1.0, width)), 1e-30f);
+  for (float left = 0x1p22f; left > 1.0f; left /= (float)(M + 1)) {
+    const float h = (hi32 - lo32) / (float)(M + 1);
+    const unsigned g = above(live && sturm_count_f32(n, df, e2f, lo32 + (float)(m + 1) * h, piv32) > i);
+    const int f = g ? __ffs(g) - 1 : M;       // first point above, M: none
+    const float nlo = (f == 0) ? lo32 : lo32 + (float)f * h;
+    hi32 = (f == M) ? hi32 : lo32 + (float)(f + 1) * h;
+    lo32 = nlo;
+  }
+  double w = fmax((double)hi32 - (double)lo32, 1e-12 * width);
+  double lo = (double)lo32 - w, hi = (double)hi32 + w;
+  // rel_tol (1e-12) of the spectral range is far below what the occupations and
+  // the DMPT weights resolve, and inverse iteration converges from such a shift
+  // in two steps.  A looser shift costs orthogonality: after two steps the
+  // component along a neighbour at distance g is ~(shift error / g)^2, which at
+  // 1e-9 of the range left Q^T Q - I at 5e-7 for n = 3360.
+  const double tol = fmax(2.0 * kEps * fmax(fabs(glo), fabs(ghi)), rel_tol * fmax(1.0, scal[2])) + pivmin;
+  bool done = !live, ends = true;             // ends: the points of the round are 0 .. M - 1, both ends among them
+  for (int it = 0, widened = 0; it < 260 && __any_sync(0xffffffffu, !done); ++it) {
+    const double h = (hi - lo) / (double)(ends ? M - 1 : M + 1);
+    const double x = (ends && m == M - 1) ? hi : lo + (double)(ends ? m : m + 1) * h;
+    const unsigned g = above(!done && sturm_count(n, d, e2, x, pivmin) > i);
+    if (done) continue;
+    int f = g ? __ffs(g) - 1 : M;             // first point above, M: none
+    if (ends) {
+      const bool low = f == 0 && lo > glo, high = f == M && hi < ghi;
+      if ((low || high) && widened < 60) {
+        w *= 4.0;
+        ++widened;
+        if (low) lo = fmax(glo, lo - w);
+        if (high) hi = fmin(ghi, hi + w);
+        continue;
+      }
+      f = min(max(f, 1), M - 1) - 1;          // as a point 1 .. M - 2 between the ends
+      const double nlo = lo + (double)f * h;
+      hi = (f == M - 2) ? hi : lo + (double)(f + 1) * h;
+      lo = nlo;
+      ends = false;
+    } else {
+      const double nlo = (f == 0) ? lo : lo + (double)f * h;
+      hi = (f == M) ? hi : lo + (double)(f + 1) * h;
+      lo = nlo;
+    }
+    const double mid = 0.5 * (lo + hi);
+    done = hi - lo <= tol || mid <= lo || mid >= hi;
+  }
+  if (live && m == 0) ev[i] = 0.5 * (lo + hi);
+}
+
+// Mixed path: eigenvalue i by multisection in double-float arithmetic.  A
+// group of kMsLanes lanes evaluates the Sturm count at kMsLanes interior
+// points of the current interval, which shrinks (kMsLanes + 1)-fold per round;
+// every group starts from the Gershgorin interval, so all groups take the same
+// number of rounds.  The count is the product form of sturm_count on the FP32
+// pipe (about 48-bit arithmetic), kept in range by exact power-of-two scaling.
+constexpr int kMsLanes = 8;
+
+__device__ __forceinline__ int sturm_count_df(int n, const dfl* __restrict__ d, const dfl* __restrict__ e2,
+                                              dfl x) {
+  dfl pm = {1.0f, 0.0f};
+  dfl p = df_sub(ldg_df(d), x);
+  int sp = (p.hi < 0.0f || p.hi == 0.0f) ? 1 : 0;        // zero counts as negative
+  int c = sp;
+#pragma unroll 4
+  for (int j = 1; j < n; ++j) {
+    const dfl dj = ldg_df(d + j), ej = ldg_df(e2 + j - 1);
+    const dfl pn = df_sub(df_mul(df_sub(dj, x), p), df_mul(ej, pm));
+    const int sn = (pn.hi == 0.0f) ? (sp ^ 1) : (int)(__float_as_uint(pn.hi) >> 31);
+    c += sn ^ sp;
+    sp = sn;
+    // keep |p| within [2^-32, 2^32] (both p and pm scale by the same power of two)
+    const int ex = (int)((__float_as_uint(pn.hi) >> 23) & 0xFF);
+    const float sc = (ex > 127 + 32) ? 0x1p-64f : ((ex < 127 - 32) ? 0x1p+64f : 1.0f);
+    pm = dfl{KX_FMUL(p.hi, sc), KX_FMUL(p.lo, sc)};
+    p = dfl{KX_FMUL(pn.hi, sc), KX_FMUL(pn.lo, sc)};
+  }
+  return c;
+}
+
+__global__ void bisect_df_kernel(int n, const dfl* __restrict__ d, const dfl* __restrict__ e2,
+                                 const double* __restrict__ scal, double rel_tol, double* __restrict__ ev) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = t / kMsLanes;                 // eigenvalue of this group
+  const int m = t % kMsLanes;                 // point m + 1 of the group
+  const int gbase = (threadIdx.x & 31) & ~(kMsLanes - 1);
+  const bool live = i < n;                    // whole groups are live or not (n * kMsLanes threads)
+  const double glo = scal[0], ghi = scal[1], pivmin = scal[3];
+  double lo = glo, hi = ghi;
+  const double tol = fmax(2.0 * kEps * fmax(fabs(glo), fabs(ghi)), rel_tol * fmax(1.0, scal[2])) + pivmin;
+  int rounds = 0;
+  for (double w = ghi - glo; w > tol && rounds < 64; w /= (double)(kMsLanes + 1)) ++rounds;
+  for (int r = 0; r < rounds; ++r) {
+    const double h = (hi - lo) / (double)(kMsLanes + 1);
+    const double x = lo + (double)(m + 1) * h;
+    const bool above = live && sturm_count_df(n, d, e2, df_from_double(x)) > i;
+    const unsigned bal = __ballot_sync(0xffffffffu, above);
+    const unsigned g = (bal >> gbase) & ((1u << kMsLanes) - 1u);
+    // counts grow with x: the first point with count > i is the new upper end
+    const int f = g ? (__ffs(g) - 1) : kMsLanes;      // 0-based point index, kMsLanes: none
+    const double nlo = (f == 0) ? lo : lo + (double)f * h;
+    const double nhi = (f == kMsLanes) ? hi : lo + (double)(f + 1) * h;
+    lo = nlo;
+    hi = nhi;
+  }
+  if (live && m == 0) ev[i] = 0.5 * (lo + hi);
+}
+
+__global__ void cluster_kernel(int n, const double* __restrict__ ev, const double* __restrict__ scal,
+                               int* __restrict__ clus) {
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double ctol = 1e-7 * fmax(1.0, scal[2]);
+  // a NaN gap starts a new cluster: non-finite input must not merge the whole
+  // spectrum into one cluster (one thread would then orthogonalise n vectors)
+  clus[i] = (i == 0 || !(ev[i] - ev[i - 1] <= ctol)) ? 1 : 0;
+}
+
+__device__ __forceinline__ unsigned start_hash(int row, int col) {
+  unsigned h = (unsigned)row * 0x9E3779B1u ^ ((unsigned)col * 0x85EBCA77u + 0x165667B1u);
+  h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; h ^= h >> 15;
+  return h;
+}
+__device__ __forceinline__ double start_value(int row, int col) {
+  return ((double)(start_hash(row, col) & 0xFFFFF) / 524288.0) - 1.0 + 1e-3;
+}
+// the same pseudo-random start entry in FP32 arithmetic (a start vector only
+// needs a component along the eigenvector, not FP64 values)
+__device__ __forceinline__ float start_value_f(int row, int col) {
+  return __fadd_rn(__fmul_rn((float)(start_hash(row, col) & 0xFFFFF), 0x1p-19f), -0.999f);
+}
+
+// inverse iteration; one thread per cluster leader; lu: 5 x n x n workspace.
+// The recurrences carry their running values in registers, and the loads of
+// each sweep are issued kIvB rows at a time ahead of the dependent arithmetic
+// (one thread walks n rows of a column: a load-use chain per row would put
+// the memory latency on the critical path n times); the arithmetic and its
+// order are those of the textbook pivoted tridiagonal LU and its
+// forward/backward substitutions.
+constexpr int kIvB = 8;
+
+__global__ void invit_kernel(int n, const double* __restrict__ d, const double* __restrict__ e,
+                             const double* __restrict__ ev, const double* __restrict__ scal,
+                             const int* __restrict__ clus, double* __restrict__ lu,
+                             double* __restrict__ Z) {
+  int L = blockIdx.x * blockDim.x + threadIdx.x;
+  if (L >= n || !clus[L]) return;
+  int end = L + 1;
+  while (end < n && !clus[end]) ++end;
+  const double tn = fmax(scal[2], 1e-300);
+  const double tiny = kEps * tn;
+  const size_t nn = (size_t)n * n;
+  double* __restrict__ dl = lu + 0 * nn;
+  double* __restrict__ rdd = lu + 1 * nn;   // reciprocal pivots
+  double* __restrict__ du = lu + 2 * nn;
+  double* __restrict__ du2 = lu + 3 * nn;
+  double* __restrict__ pv = lu + 4 * nn;
+#define LU(a, r) a[(size_t)(r) * n + L]
+#define ZC(r, c) Z[(size_t)(r) * n + (c)]
+  double prevlam = 0.0;
+  for (int j = L; j < end; ++j) {
+    double lam = ev[j];
+    if (j > L && lam - prevlam < 10.0 * tiny) lam = prevlam + 10.0 * tiny;
+    prevlam = lam;
+    if (n == 1) { ZC(0, j) = 1.0; continue; }
+    // LU of T - lam I with partial pivoting; a, u: pivot-row diagonal and superdiagonal
+    double a = d[0] - lam, u = e[0];
+    for (int r = 0; r < n - 1; ++r) {
+      const double b = e[r];
+      const double dn = d[r + 1] - lam;
+      const double un = (r < n - 2) ? e[r + 1] : 0.0;
+      if (fabs(a) >= fabs(b)) {
+        LU(pv, r) = 0.0;
+        if (fabs(a) < tiny) a = (a >= 0.0) ? tiny : -tiny;
+        const double ra = 1.0 / a;          // one division per row (the FP64 divide is slow)
+        const double f = b * ra;
+        LU(dl, r) = f;
+        LU(rdd, r) = ra;
+        LU(du, r) = u;
+        LU(du2, r) = 0.0;
+        a = dn - f * u;
+        u = un;
+      } else {
+        LU(pv, r) = 1.0;
+        const double rb = 1.0 / b;
+        const double f = a * rb;
+        LU(rdd, r) = rb;
+        LU(dl, r) = f;
+        LU(du, r) = dn;
+        const double na = u - f * dn;
+        if (r < n - 2) {
+          LU(du2, r) = un;
+          u = -f * un;
+        } else {
+          LU(du2, r) = 0.0;
+        }
+        a = na;
+      }
+    }
+    if (fabs(a) < tiny) a = (a >= 0.0) ? tiny : -tiny;
+    LU(rdd, n - 1) = 1.0 / a;
+    for (int r = 0; r < n; ++r) ZC(r, j) = start_value(r, j);
+    for (int it = 0; it < 2; ++it) {
+      // forward (L with pivots); cur = current row r of the right-hand side
+      double cur = ZC(0, j);
+      for (int r0 = 0; r0 < n - 1; r0 += kIvB) {
+        double nx[kIvB], fv[kIvB], pf[kIvB];
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 + q;
+          if (r < n - 1) { nx[q] = ZC(r + 1, j); fv[q] = LU(dl, r); pf[q] = LU(pv, r); }
+        }
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 + q;
+          if (r < n - 1) {
+            if (pf[q] == 0.0) {
+              ZC(r, j) = cur;
+              cur = nx[q] - fv[q] * cur;
+            } else {
+              ZC(r, j) = nx[q];
+              cur = cur - fv[q] * nx[q];
+            }
+          }
+        }
+      }
+      // backward (U, three diagonals, reciprocal pivots); z1 = x[r+1], z2 = x[r+2]
+      double z2 = cur * LU(rdd, n - 1);
+      ZC(n - 1, j) = z2;
+      double z1 = z2;
+      if (n > 1) {
+        z1 = (ZC(n - 2, j) - LU(du, n - 2) * z2) * LU(rdd, n - 2);
+        ZC(n - 2, j) = z1;
+      }
+      for (int r0 = n - 3; r0 >= 0; r0 -= kIvB) {
+        double zv[kIvB], uv[kIvB], u2[kIvB], rv[kIvB];
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 - q;
+          if (r >= 0) { zv[q] = ZC(r, j); uv[q] = LU(du, r); u2[q] = LU(du2, r); rv[q] = LU(rdd, r); }
+        }
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 - q;
+          if (r >= 0) {
+            const double x = (zv[q] - uv[q] * z1 - u2[q] * z2) * rv[q];
+            ZC(r, j) = x;
+            z2 = z1;
+            z1 = x;
+          }
+        }
+      }
+      // scale, re-orthogonalise within the cluster, normalise
+      double mx = 0.0;
+#pragma unroll 8
+      for (int r = 0; r < n; ++r) mx = fmax(mx, fabs(ZC(r, j)));
+      double s = (mx > 0.0) ? 1.0 / mx : 1.0;
+#pragma unroll 8
+      for (int r = 0; r < n; ++r) ZC(r, j) *= s;
+      for (int c = L; c < j; ++c) {
+        double dot = 0.0;
+#pragma unroll 8
+        for (int r = 0; r < n; ++r) dot += ZC(r, c) * ZC(r, j);
+#pragma unroll 8
+        for (int r = 0; r < n; ++r) ZC(r, j) -= dot * ZC(r, c);
+      }
+      double nrm = 0.0;
+#pragma unroll 8
+      for (int r = 0; r < n; ++r) nrm += ZC(r, j) * ZC(r, j);
+      nrm = ::sqrt(nrm);
+      s = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+#pragma unroll 8
+      for (int r = 0; r < n; ++r) ZC(r, j) *= s;
+    }
+  }
+#undef LU
+#undef ZC
+}
+
+// Mixed path: the same inverse iteration in double-float arithmetic.  The LU
+// factors and the iterates are held as (hi, lo) pairs in the same workspace
+// (the iterates in Q, converted to FP64 at the end); one reciprocal per row
+// from the FP32 estimate and one Newton step; the pivot floor and the shift
+// separation use the double-float unit 2^-46 |T| instead of the FP64 epsilon.
+__device__ __forceinline__ float df_abs_hi(dfl a) { return fabsf(a.hi); }
+
+// Each cluster leader runs its recurrences alone, so the kernel is bound by
+// their latency: kIvLanes active lanes per 32-thread block spread the n
+// chains over n / kIvLanes warps (about 5 per SM at n = 3360 instead of
+// one), so each SM interleaves several independent chains; four lanes keep
+// every access a whole 32-byte sector and limit divergence at the pivots.
+constexpr int kIvLanes = 4;
+__global__ void __launch_bounds__(32) invit_df_kernel(int n, const dfl* __restrict__ d, const double* __restrict__ e,
+                                                    const dfl* __restrict__ edf,
+                                                    const double* __restrict__ ev, const double* __restrict__ scal,
+                                                    const int* __restrict__ clus, dfl* __restrict__ lu,
+                                                    double* __restrict__ Zout) {
+  if (threadIdx.x >= kIvLanes) return;
+  int L = blockIdx.x * kIvLanes + threadIdx.x;
+  if (L >= n || !clus[L]) return;
+  int end = L + 1;
+  while (end < n && !clus[end]) ++end;
+  const double tn = fmax(scal[2], 1e-300);
+  const double tiny_d = 0x1p-46 * tn;
+  const dfl tiny = df_from_double(tiny_d);
+  const size_t nn = (size_t)n * n;
+  dfl* __restrict__ dl = lu + 0 * nn;
+  dfl* __restrict__ rdd = lu + 1 * nn;   // reciprocal pivots
+  dfl* __restrict__ du = lu + 2 * nn;
+  dfl* __restrict__ du2 = lu + 3 * nn;
+  int* __restrict__ pv = (int*)(lu + 4 * nn);
+  dfl* __restrict__ Z = (dfl*)Zout;      // iterates in place of the FP64 output
+#define LU(a, r) a[(size_t)(r) * n + L]
+#define ZC(r, c) Z[(size_t)(r) * n + (c)]
+  if (end == L + 1 && n > 1) {
+    // An eigenvalue alone in its cluster (the common case): the same two
+    // inverse-iteration steps with the passes fused.  Step 1 solves from the
+    // start vector without storing it, its backward sweep tracks max|x|;
+    // step 2 reads x scaled by 1/max (inverse iteration is linear, the scale
+    // only keeps the values in range), its backward sweep accumulates ||x||^2;
+    // one last pass writes x / ||x|| in FP64.  Six sweeps of n instead of 15.
+    // no FP64 instruction per row: GB300 issues one FP64 warp instruction per
+    // ~76 cycles per scheduler, which would put the FP64 pipe on the chain
+    const dfl lam = df_from_double(ev[L]);
+    dfl a = df_sub(ldg_df(d), lam), u = ldg_df(edf);
+    for (int r = 0; r < n - 1; ++r) {
+      const dfl b = ldg_df(edf + r);
+      const dfl dn = df_sub(ldg_df(d + r + 1), lam);
+      const dfl un = (r < n - 2) ? ldg_df(edf + r + 1) : dfl{0.0f, 0.0f};
+      if (df_abs_hi(a) >= df_abs_hi(b)) {
+        LU(pv, r) = 0;
+        if (df_abs_hi(a) < tiny.hi) a = (a.hi >= 0.0f) ? tiny : df_neg(tiny);
+        const dfl ra = df_recip(a);
+        const dfl f = df_mul(b, ra);
+        LU(dl, r) = f;
+        LU(rdd, r) = ra;
+        LU(du, r) = u;
+        LU(du2, r) = dfl{0.0f, 0.0f};
+        a = df_sub(dn, df_mul(f, u));
+        u = un;
+      } else {
+        LU(pv, r) = 1;
+        const dfl rb = df_recip(b);
+        const dfl f = df_mul(a, rb);
+        LU(rdd, r) = rb;
+        LU(dl, r) = f;
+        LU(du, r) = dn;
+        const dfl na = df_sub(u, df_mul(f, dn));
+        if (r < n - 2) {
+          LU(du2, r) = un;
+          u = df_neg(df_mul(f, un));
+        } else {
+          LU(du2, r) = dfl{0.0f, 0.0f};
+        }
+        a = na;
+      }
+    }
+    if (df_abs_hi(a) < tiny.hi) a = (a.hi >= 0.0f) ? tiny : df_neg(tiny);
+    LU(rdd, n - 1) = df_recip(a);
+    dfl scl = {1.0f, 0.0f};
+    dfl nrm = {0.0f, 0.0f};
+    for (int it = 0; it < 2; ++it) {
+      // forward (L with pivots); step 1 takes the start vector, step 2 the scaled x
+      dfl cur = (it == 0) ? dfl{start_value_f(0, L), 0.0f} : df_mul(ZC(0, L), scl);
+      for (int r0 = 0; r0 < n - 1; r0 += kIvB) {
+        dfl nx[kIvB], fv[kIvB];
+        int pf[kIvB];
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 + q;
+          if (r < n - 1) {
+            nx[q] = (it == 0) ? dfl{start_value_f(r + 1, L), 0.0f} : df_mul(ZC(r + 1, L), scl);
+            fv[q] = LU(dl, r);
+            pf[q] = LU(pv, r);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 + q;
+          if (r < n - 1) {
+            if (pf[q] == 0) {
+              ZC(r, L) = cur;
+              cur = df_sub(nx[q], df_mul(fv[q], cur));
+            } else {
+              ZC(r, L) = nx[q];
+              cur = df_sub(cur, df_mul(fv[q], nx[q]));
+            }
+          }
+        }
+      }
+      // backward (U, three diagonals, reciprocal pivots), with max|x| or ||x||^2
+      float mx = 0.0f;
+      dfl z2 = df_mul(cur, LU(rdd, n - 1));
+      ZC(n - 1, L) = z2;
+      mx = fmaxf(mx, df_abs_hi(z2));
+      if (it == 1) df_acc_mul(nrm, z2, z2);
+      dfl z1 = z2;
+      if (n > 1) {
+        z1 = df_mul(df_sub(ZC(n - 2, L), df_mul(LU(du, n - 2), z2)), LU(rdd, n - 2));
+        ZC(n - 2, L) = z1;
+        mx = fmaxf(mx, df_abs_hi(z1));
+        if (it == 1) df_acc_mul(nrm, z1, z1);
+      }
+      for (int r0 = n - 3; r0 >= 0; r0 -= kIvB) {
+        dfl zv[kIvB], uv[kIvB], u2[kIvB], rv[kIvB];
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 - q;
+          if (r >= 0) { zv[q] = ZC(r, L); uv[q] = LU(du, r); u2[q] = LU(du2, r); rv[q] = LU(rdd, r); }
+        }
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 - q;
+          if (r >= 0) {
+            const dfl x = df_mul(df_sub(df_sub(zv[q], df_mul(uv[q], z1)), df_mul(u2[q], z2)), rv[q]);
+            ZC(r, L) = x;
+            mx = fmaxf(mx, df_abs_hi(x));
+            if (it == 1) df_acc_mul(nrm, x, x);
+            z2 = z1;
+            z1 = x;
+          }
+        }
+      }
+      if (it == 0) scl = (mx > 0.0f) ? df_recip(dfl{mx, 0.0f}) : dfl{1.0f, 0.0f};
+    }
+    const double nd = ::sqrt(df_to_double(df_norm(nrm)));
+    const dfl sc = (nd > 0.0) ? df_from_double(1.0 / nd) : dfl{0.0f, 0.0f};
+#pragma unroll 8
+    for (int r = 0; r < n; ++r) {
+      const dfl z = df_mul(ZC(r, L), sc);
+      Zout[(size_t)r * n + L] = df_to_double_fast(z);
+    }
+    return;
+  }
+  double prevlam = 0.0;
+  for (int j = L; j < end; ++j) {
+    double lamd = ev[j];
+    if (j > L && lamd - prevlam < 10.0 * tiny_d) lamd = prevlam + 10.0 * tiny_d;
+    prevlam = lamd;
+    if (n == 1) { ZC(0, j) = dfl{1.0f, 0.0f}; continue; }
+    const dfl lam = df_from_double(lamd);
+    // LU of T - lam I with partial pivoting; a, u: pivot-row diagonal and superdiagonal
+    dfl a = df_sub(ldg_df(d), lam), u = df_from_double(e[0]);
+    for (int r = 0; r < n - 1; ++r) {
+      const dfl b = df_from_double(e[r]);
+      const dfl dn = df_sub(ldg_df(d + r + 1), lam);
+      const dfl un = (r < n - 2) ? df_from_double(e[r + 1]) : dfl{0.0f, 0.0f};
+      if (df_abs_hi(a) >= df_abs_hi(b)) {
+        LU(pv, r) = 0;
+        if (df_abs_hi(a) < tiny.hi) a = (a.hi >= 0.0f) ? tiny : df_neg(tiny);
+        const dfl ra = df_recip(a);
+        const dfl f = df_mul(b, ra);
+        LU(dl, r) = f;
+        LU(rdd, r) = ra;
+        LU(du, r) = u;
+        LU(du2, r) = dfl{0.0f, 0.0f};
+        a = df_sub(dn, df_mul(f, u));
+        u = un;
+      } else {
+        LU(pv, r) = 1;
+        const dfl rb = df_recip(b);
+        const dfl f = df_mul(a, rb);
+        LU(rdd, r) = rb;
+        LU(dl, r) = f;
+        LU(du, r) = dn;
+        const dfl na = df_sub(u, df_mul(f, dn));
+        if (r < n - 2) {
+          LU(du2, r) = un;
+          u = df_neg(df_mul(f, un));
+        } else {
+          LU(du2, r) = dfl{0.0f, 0.0f};
+        }
+        a = na;
+      }
+    }
+    if (df_abs_hi(a) < tiny.hi) a = (a.hi >= 0.0f) ? tiny : df_neg(tiny);
+    LU(rdd, n - 1) = df_recip(a);
+    for (int r = 0; r < n; ++r) ZC(r, j) = df_from_double(start_value(r, j));
+    for (int it = 0; it < 2; ++it) {
+      // forward (L with pivots)
+      dfl cur = ZC(0, j);
+      for (int r0 = 0; r0 < n - 1; r0 += kIvB) {
+        dfl nx[kIvB], fv[kIvB];
+        int pf[kIvB];
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 + q;
+          if (r < n - 1) { nx[q] = ZC(r + 1, j); fv[q] = LU(dl, r); pf[q] = LU(pv, r); }
+        }
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 + q;
+          if (r < n - 1) {
+            if (pf[q] == 0) {
+              ZC(r, j) = cur;
+              cur = df_sub(nx[q], df_mul(fv[q], cur));
+            } else {
+              ZC(r, j) = nx[q];
+              cur = df_sub(cur, df_mul(fv[q], nx[q]));
+            }
+          }
+        }
+      }
+      // backward (U, three diagonals, reciprocal pivots)
+      dfl z2 = df_mul(cur, LU(rdd, n - 1));
+      ZC(n - 1, j) = z2;
+      dfl z1 = z2;
+      if (n > 1) {
+        z1 = df_mul(df_sub(ZC(n - 2, j), df_mul(LU(du, n - 2), z2)), LU(rdd, n - 2));
+        ZC(n - 2, j) = z1;
+      }
+      for (int r0 = n - 3; r0 >= 0; r0 -= kIvB) {
+        dfl zv[kIvB], uv[kIvB], u2[kIvB], rv[kIvB];
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 - q;
+          if (r >= 0) { zv[q] = ZC(r, j); uv[q] = LU(du, r); u2[q] = LU(du2, r); rv[q] = LU(rdd, r); }
+        }
+#pragma unroll
+        for (int q = 0; q < kIvB; ++q) {
+          const int r = r0 - q;
+          if (r >= 0) {
+            const dfl x = df_mul(df_sub(df_sub(zv[q], df_mul(uv[q], z1)), df_mul(u2[q], z2)), rv[q]);
+            ZC(r, j) = x;
+            z2 = z1;
+            z1 = x;
+          }
+        }
+      }
+      // scale, re-orthogonalise within the cluster, normalise
+      float mx = 0.0f;
+#pragma unroll 8
+      for (int r = 0; r < n; ++r) mx = fmaxf(mx, df_abs_hi(ZC(r, j)));
+      dfl sc = (mx > 0.0f) ? df_recip(dfl{mx, 0.0f}) : dfl{1.0f, 0.0f};
+#pragma unroll 8
+      for (int r = 0; r < n; ++r) ZC(r, j) = df_mul(ZC(r, j), sc);
+      for (int c = L; c < j; ++c) {
+        dfl dot = {0.0f, 0.0f};
+#pragma unroll 8
+        for (int r = 0; r < n; ++r) df_acc_mul(dot, ZC(r, c), ZC(r, j));
+        dot = df_norm(dot);
+#pragma unroll 8
+        for (int r = 0; r < n; ++r) ZC(r, j) = df_sub(ZC(r, j), df_mul(dot, ZC(r, c)));
+      }
+      dfl nrm = {0.0f, 0.0f};
+#pragma unroll 8
+      for (int r = 0; r < n; ++r) df_acc_mul(nrm, ZC(r, j), ZC(r, j));
+      const double nd = ::sqrt(df_to_double(df_norm(nrm)));
+      sc = (nd > 0.0) ? df_from_double(1.0 / nd) : dfl{0.0f, 0.0f};
+#pragma unroll 8
+      for (int r = 0; r < n; ++r) ZC(r, j) = df_mul(ZC(r, j), sc);
+    }
+  }
+  // FP64 output (same slots, same thread)
+  for (int j = L; j < end; ++j)
+    for (int r = 0; r < n; ++r) {
+      const dfl z = ZC(r, j);
+      Zout[(size_t)r * n + j] = df_to_double_fast(z);
+    }
+#undef LU
+#undef ZC
+}
+
+// T factor of a block of kb reflectors (forward, columnwise): one block,
+// T held in shared memory, each entry a dot product split over 4 partial sums
+__device__ void tfactor_body(int kb, const double* __restrict__ tau, const double* __restrict__ G, int ldg,
+                             double* __restrict__ T, int ldt) {
+  extern __shared__ double ts[];          // kb x kb
+  __shared__ double gcol[kBtBlockTc];
+  const int i = threadIdx.x;
+  for (int e = i; e < kb * kb; e += blockDim.x) ts[e] = 0.0;
+  __syncthreads();
+  for (int j = 0; j < kb; ++j) {
+    if (i < j) gcol[i] = G[i * ldg + j];
+    __syncthreads();
+    if (i < j) {
+      double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+      int l = i;
+      for (; l + 3 < j; l += 4) {
+        a0 = fma(ts[i * kb + l], gcol[l], a0);
+        a1 = fma(ts[i * kb + l + 1], gcol[l + 1], a1);
+        a2 = fma(ts[i * kb + l + 2], gcol[l + 2], a2);
+        a3 = fma(ts[i * kb + l + 3], gcol[l + 3], a3);
+      }
+      for (; l < j; ++l) a0 = fma(ts[i * kb + l], gcol[l], a0);
+      ts[i * kb + j] = -tau[j] * ((a0 + a1) + (a2 + a3));
+    }
+    if (i == j) ts[j * kb + j] = tau[j];
+    __syncthreads();
+  }
+  for (int e = i; e < kb * kb; e += blockDim.x) T[(e / kb) * ldt + e % kb] = ts[e];
+}
+
+__global__ void tfactor_kernel(int kb, const double* __restrict__ tau, const double* __restrict__ G,
+                               int ldg, double* __restrict__ T, int ldt) {
+  tfactor_body(kb, tau, G, ldg, T, ldt);
+}
+
+// T factors of every block of kblk reflectors at once (block b: reflectors
+// b*kblk .. ; they depend on the reflectors only, not on the vectors updated)
+__global__ void tfactor_all_kernel(int nref, int kblk, const double* __restrict__ tau,
+                                   const double* __restrict__ Gall, double* __restrict__ Tall) {
+  const int b = blockIdx.x;
+  const int k0 = b * kblk;
+  const int kb = (k0 + kblk < nref) ? kblk : nref - k0;
+  const size_t off = (size_t)b * kblk * kblk;
+  tfactor_body(kb, tau + k0, Gall + off, kblk, Tall + off, kblk);
+}
+
+// number of blocks of kBtBlockTc reflectors (n - 2 reflectors)
+static int tc_blocks(int n) { return n > 2 ? (n - 2 + kBtBlockTc - 1) / kBtBlockTc : 1; }
+
+struct BtScratch;
+static size_t bt_scratch_layout(int n, void* base, BtScratch* out);
+struct Bt64Scratch;
+static size_t bt64_scratch(int n, void* base, Bt64Scratch* out);
+// the inverse-iteration workspace (5 n^2) also serves as back-transformation scratch
+static size_t lu_doubles(int n) {
+  const size_t a = 5 * (size_t)n * n;
+  const size_t b = (bt_scratch_layout(n, nullptr, nullptr) + 7) / 8;
+  return std::max({a, b, bt64_scratch(n, nullptr, nullptr) / 8});
+}
+
+// One layout for sizing and binding.  Every buffer starts on a 256-byte
+// boundary: the back-transformation cuts BF16 slices into the lu region and
+// hands them to TMA, whose tensor maps need 16-byte aligned bases (with odd n
+// an unpadded layout would leave the region 8 bytes off).
+static size_t eig_layout(int n, void* base, EigWork* w) {
+  const size_t nn = (size_t)n * n;
+  size_t off = 0;
+  auto take = [&](size_t doubles) {
+    double* q = base ? (double*)base + off : nullptr;
+    off += (doubles + 31) & ~(size_t)31;
+    return q;
+  };
+  double* A = take(nn);
+  double* Vst = take(nn);
+  double* d = take(n);
+  double* e = take(n);
+  double* e2 = take(n);
+  double* tau = take(n);
+  double* pbuf = take(4 * (size_t)n);
+  double* lu = take(lu_doubles(n));
+  double* Tm = take((size_t)tc_blocks(n) * kBtBlockTc * kBtBlockTc);   // T and Gram of every reflector block
+  double* Gm = take((size_t)tc_blocks(n) * kBtBlockTc * kBtBlockTc);
+  double* Wt = take((size_t)kBtBlockTc * n);
+  double* Wt2 = take((size_t)kBtBlockTc * n);
+  double* scal = take(16);
+  double* bar = take(8);
+  double* clus = take(((size_t)n * sizeof(int) + 7) / 8);
+  if (w) {
+    w->A = A; w->Vst = Vst; w->d = d; w->e = e; w->e2 = e2; w->tau = tau; w->pbuf = pbuf; w->lu = lu;
+    w->Tm = Tm; w->Gm = Gm; w->Wt = Wt; w->Wt2 = Wt2; w->scal = scal;
+    w->bar = (unsigned*)bar;
+    w->clus = (int*)clus;
+  }
+  return off * sizeof(double) + 256;
+}
+
+size_t eig_work_bytes(int n) { return eig_layout(n, nullptr, nullptr); }
+
+// base must be 256-byte aligned (arena allocations are)
+void eig_work_bind(EigWork& w, void* base, int n) { eig_layout(n, base, &w); }
+
+void eig_bisect(cudaStream_t s, int n, double* eps, EigWork& w, double rel_tol, bool df_path) {
+  if (n <= 0) return;
+  // 2. eigenvalues
+  // pbuf (4n doubles, free after the tridiagonalisation) holds the FP32 and double-float copies
+  float* df = (float*)w.pbuf;
+  float* e2f = df + n;
+  dfl* d_dfl = (dfl*)(w.pbuf + n);
+  dfl* e2_dfl = d_dfl + n;
+  dfl* e_dfl = e2_dfl + n;
+  gersh_kernel<<<1, 1024, 0, s>>>(n, w.d, w.e, w.e2, w.scal, df, e2f, d_dfl, e2_dfl, e_dfl);
+  count_launch();
+  if (df_path) {
+    const long long thr = (long long)n * kMsLanes;
+    // one warp (4 eigenvalues) per block, so the n / 4 blocks spread over all SMs
+    bisect_df_kernel<<<(unsigned)((thr + 31) / 32), 32, 0, s>>>(n, d_dfl, e2_dfl, w.scal, rel_tol, eps);
+  } else {
+    auto run = [&](auto kernel, int m) {
+      kernel<<<(unsigned)(((long long)n * m + 31) / 32), 32, 0, s>>>(n, w.d, w.e2, w.scal, df, e2f, rel_tol, eps);
+    };
+    if (n <= kFp64Pipes)
+      run(bisect_kernel<32>, 32);
+    else if (n <= 2 * kFp64Pipes)
+      run(bisect_kernel<16>, 16);
+    else if (n <= 8 * kFp64Pipes)
+      run(bisect_kernel<8>, 8);
+    else
+      run(bisect_kernel<4>, 4);
+  }
+  count_launch();
+}
+
+void eig_vectors(cudaStream_t s, int n, const double* eps, double* Q, EigWork& w, bool df_path) {
+  if (n <= 0) return;
+  // 3. eigenvectors of the tridiagonal matrix
+  cluster_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, eps, w.scal, w.clus);
+  count_launch();
+  if (df_path) {
+    const dfl* d_dfl = (const dfl*)(w.pbuf + n);     // written by eig_bisect
+    const dfl* e_dfl = d_dfl + 2 * (size_t)n;
+    invit_df_kernel<<<(n + kIvLanes - 1) / kIvLanes, 32, 0, s>>>(n, d_dfl, w.e, e_dfl, eps, w.scal, w.clus,
+                                                                (dfl*)w.lu, Q);
+  } else {
+    invit_kernel<<<(n + 31) / 32, 32, 0, s>>>(n, w.d, w.e, eps, w.scal, w.clus, w.lu, Q);
+  }
+  count_launch();
+}
+
+// tensor-core back-transformation (mixed path), carried out on Z^T so that
+// every large operand is K-major: Z^T <- Z^T (I - V T V^T)^T block by block,
+//   U   = Z^T_sub V_b^T     (n x kb)      tensor cores, 4 slices, split over K
+//   Z^T_sub -= U Y_b        (n x m_b)     tensor cores, 4 slices
+// with Y_b = T_b^T V_b formed for all blocks before the loop (it does not
+// depend on Z).  The Gram matrices V_b V_b^T (for the T factors) and Y_b are
+// double-float products on the FP32 pipe, one launch each for all blocks; the
+// slices of V_b and Y_b^T are cut once, in two launches.
+__global__ void transpose_sq_kernel(int n, const double* __restrict__ A, double* __restrict__ At) {
+  __shared__ double tile[32][33];
+  int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
+  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+    int i = i0 + r, j = j0 + threadIdx.x;
+    tile[r][threadIdx.x] = (i < n && j < n) ? A[(size_t)i * n + j] : 0.0;
+  }
+  __syncthreads();
+  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+    int j = j0 + r, i = i0 + threadIdx.x;
+    if (i < n && j < n) At[(size_t)j * n + i] = tile[threadIdx.x][r];
+  }
+}
+
+static void transpose_sq(cudaStream_t s, int n, const double* A, double* At) {
+  int t = (n + 31) / 32;
+  transpose_sq_kernel<<<dim3(t, t), dim3(32, 8), 0, s>>>(n, A, At);
+  count_launch();
+}
+
+// G_b = V_b V_b^T (upper 32 x 32 tiles) for every block b of kBtBlockTc
+// reflectors; V_b = rows k0.. of the reflector store, columns c0 = k0 + 1 ..
+__global__ void __launch_bounds__(256) gram_df_kernel(int n, int nref, const double* __restrict__ Vst,
+                                                      double* __restrict__ Gall) {
+  constexpr int KB = kBtBlockTc, TL = 32, CH = 64;
+  const int b = blockIdx.y;
+  const int k0 = b * KB, kb = min(KB, nref - k0), c0 = k0 + 1, m = n - c0;
+  const int ti = blockIdx.x / (KB / TL), tj = blockIdx.x % (KB / TL);
+  if (ti > tj || ti * TL >= kb || tj * TL >= kb) return;
+  __shared__ dfl sa[TL][CH + 1], sb[TL][CH + 1];
+  const int t = threadIdx.x, ii = t >> 3, jj = (t & 7) * 4;
+  dfl acc[4] = {};
+  for (int l0 = 0; l0 < m; l0 += CH) {
+    for (int e = t; e < TL * CH; e += blockDim.x) {
+      const int r = e / CH, c = e % CH;
+      const int l = l0 + c;
+      const int ra = ti * TL + r, rb = tj * TL + r;
+      sa[r][c] = (ra < kb && l < m) ? df_from_double(Vst[(size_t)(k0 + ra) * n + c0 + l]) : dfl{0.0f, 0.0f};
+      sb[r][c] = (rb < kb && l < m) ? df_from_double(Vst[(size_t)(k0 + rb) * n + c0 + l]) : dfl{0.0f, 0.0f};
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int c = 0; c < CH; ++c) {
+      const dfl a = sa[ii][c];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) df_acc_mul(acc[q], a, sb[jj + q][c]);
+    }
+    __syncthreads();
+  }
+  const int i = ti * TL + ii;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int j = tj * TL + jj + q;
+    if (i < kb && j < kb) Gall[(size_t)b * KB * KB + (size_t)i * KB + j] = df_to_double_fast(df_norm(acc[q]));
+  }
+}
+
+// Y_b^T = V_b^T T_b (m_b x kb, row length KB) for every block b; T_b upper
+// triangular (kb x kb, ld KB); 64 rows of Y_b^T per CTA, T_b and the V_b
+// columns in shared memory as double-float
+constexpr int kYRows = 64;
+constexpr size_t kYSmem = (size_t)(kBtBlockTc * kBtBlockTc + kBtBlockTc * kYRows) * sizeof(dfl);
+__global__ void __launch_bounds__(256) y_df_kernel(int n, int nref, const double* __restrict__ Vst,
+                                                   const double* __restrict__ Tall, double* __restrict__ YT) {
+  constexpr int KB = kBtBlockTc;
+  extern __shared__ dfl ysm[];
+  dfl* sT = ysm;                   // KB x KB
+  dfl* sV = ysm + KB * KB;         // KB (reflector) x kYRows (column)
+  const int b = blockIdx.y;
+  const int k0 = b * KB, kb = min(KB, nref - k0), c0 = k0 + 1, m = n - c0;
+  const int l0 = blockIdx.x * kYRows;
+  if (l0 >= m) return;
+  const double* Tb = Tall + (size_t)b * KB * KB;
+  for (int e = threadIdx.x; e < KB * KB; e += blockDim.x) {
+    const int i = e / KB, j = e % KB;
+    sT[e] = (i < kb && j < kb && i <= j) ? df_from_double(Tb[(size_t)i * KB + j]) : dfl{0.0f, 0.0f};
+  }
+  for (int e = threadIdx.x; e < KB * kYRows; e += blockDim.x) {
+    const int i = e / kYRows, c = e % kYRows;
+    const int l = l0 + c;
+    sV[e] = (i < kb && l < m) ? df_from_double(Vst[(size_t)(k0 + i) * n + c0 + l]) : dfl{0.0f, 0.0f};
+  }
+  __syncthreads();
+  // thread t: row c = t / 4 of the tile, columns j = (t % 4) * 32 .. + 31
+  const int c = threadIdx.x >> 2, jb = (threadIdx.x & 3) * 32;
+  dfl acc[32];
+#pragma unroll
+  for (int q = 0; q < 32; ++q) acc[q] = dfl{0.0f, 0.0f};
+  for (int i = 0; i < kb; ++i) {
+    const dfl v = sV[i * kYRows + c];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) df_acc_mul(acc[q], v, sT[i * KB + jb + q]);
+  }
+  const int l = l0 + c;
+  if (l < m) {
+    double* out = YT + (size_t)b * n * KB + (size_t)l * KB;
+#pragma unroll
+    for (int q = 0; q < 32; ++q) out[jb + q] = (jb + q < kb) ? df_to_double_fast(df_norm(acc[q])) : 0.0;
+  }
+}
+
+// back-transformation scratch (in the inverse-iteration workspace, free by then)
+static int bt_blocks(int n) { return n > 2 ? (n - 2 + kBtBlockTc - 1) / kBtBlockTc : 0; }
+constexpr int kBtSplitK = 6;
+struct BtScratch {
+  __nv_bfloat16* vs;   size_t vs_blk, vs_slice;   // V_b slices
+  double* yt;                                     // Y_b^T, FP64
+  __nv_bfloat16* ys;   size_t ys_blk, ys_slice;   // Y_b^T slices
+  double* part;                                   // split-K partial products of U
+};
+static size_t bt_scratch_layout(int n, void* base, BtScratch* out) {
+  const size_t nblk = (size_t)bt_blocks(n), KB = kBtBlockTc;
+  const size_t ldn = (size_t)tc_ld(n > 1 ? n : 1);
+  size_t off = 0;
+  auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~(size_t)255; return o; };
+  const size_t vs_slice = KB * ldn, vs_blk = (size_t)kTcMaxSlices * vs_slice;
+  const size_t o_vs = take(nblk * vs_blk * 2);
+  const size_t o_yt = take(nblk * (size_t)n * KB * 8);
+  const size_t ys_slice = (size_t)n * KB, ys_blk = (size_t)kTcMaxSlices * ys_slice;
+  const size_t o_ys = take(nblk * ys_blk * 2);
+  const size_t o_part = take((size_t)(kBtSplitK + 1) * n * KB * 8);
+  if (out) {
+    char* c = (char*)base;
+    out->vs = (__nv_bfloat16*)(c + o_vs); out->vs_blk = vs_blk; out->vs_slice = vs_slice;
+    out->yt = (double*)(c + o_yt);
+    out->ys = (__nv_bfloat16*)(c + o_ys); out->ys_blk = ys_blk; out->ys_slice = ys_slice;
+    out->part = (double*)(c + o_part);
+  }
+  return off;
+}
+
+static void bt_attributes() {
+  static PerDeviceOnce attr;
+  once_per_device(attr, [] {
+    return cudaFuncSetAttribute(tfactor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kBtBlockTc * kBtBlockTc * (int)sizeof(double)) == cudaSuccess &&
+           cudaFuncSetAttribute(tfactor_all_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kBtBlockTc * kBtBlockTc * (int)sizeof(double)) == cudaSuccess &&
+           cudaFuncSetAttribute(y_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kYSmem) ==
+               cudaSuccess;
+  });
+}
+
+static int eig_backtransform_tc(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork& tw) {
+  bt_attributes();
+  const int nref = n - 2;
+  const int nblk = bt_blocks(n);
+  const size_t stride = tc_slot_stride(tw);
+  int* err = tc_error_flag(tw);
+  BtScratch sc;
+  bt_scratch_layout(n, w.lu, &sc);
+  double* Zt = w.A;                      // tridiagonalisation workspace is free now
+  transpose_sq(s, n, Q, Zt);
+  // Gram matrices and T factors of all blocks, then Y_b^T = V_b^T T_b, then slices
+  gram_df_kernel<<<dim3((kBtBlockTc / 32) * (kBtBlockTc / 32), nblk), 256, 0, s>>>(n, nref, w.Vst, w.Gm);
+  count_launch();
+  tfactor_all_kernel<<<nblk, kBtBlockTc, kBtBlockTc * kBtBlockTc * sizeof(double), s>>>(nref, kBtBlockTc, w.tau,
+                                                                                      w.Gm, w.Tm);
+  count_launch();
+  y_df_kernel<<<dim3((n + kYRows - 1) / kYRows, nblk), 256, kYSmem, s>>>(n, nref, w.Vst, w.Tm, sc.yt);
+  count_launch();
+  tc_split_blocks(s, 0, n, nref, kBtBlockTc, w.Vst, sc.vs, sc.vs_blk, sc.vs_slice, 4);
+  tc_split_blocks(s, 1, n, nref, kBtBlockTc, sc.yt, sc.ys, sc.ys_blk, sc.ys_slice, 4);
+  __nv_bfloat16* sZ = tc_slot_base(tw, kSlotT0);
+  __nv_bfloat16* sU = tc_slot_base(tw, kSlotT1);
+  for (int b = nblk - 1; b >= 0; --b) {
+    const int k0 = b * kBtBlockTc, kb = (k0 + kBtBlockTc < nref) ? kBtBlockTc : nref - k0;
+    const int c0 = k0 + 1, m = n - c0;
+    const int ldm = tc_ld(m);
+    double* Zs = Zt + c0;                                // n x m, ld n
+    tc_split_rows(s, n, m, Zs, n, 4, sZ, ldm, stride);
+    const int parts = tc_gemm_grouped_rc_splitk(s, n, kb, m, sZ, ldm, stride, sc.vs + (size_t)b * sc.vs_blk, ldm,
+                                                sc.vs_slice, 1.0, sc.part, kBtBlockTc, kBtSplitK, err);   // U parts
+    if (parts <= 0) return -1;
+    const int ldk = tc_ld(kb);                           // U slices fit the slot: kb <= n
+    tc_reduce_split_rows(s, n, kb, sc.part, parts, kBtBlockTc, 4, sU, ldk, stride);
+    if (tc_gemm_grouped_rc(s, n, m, kb, sU, ldk, stride, sc.ys + (size_t)b * sc.ys_blk, kBtBlockTc, sc.ys_slice,
+                           -1.0, Zs, n, 1, err) != 0)                                        // Zs -= U Y_b
+      return -1;
+  }
+  transpose_sq(s, n, Zt, Q);
+  return 0;
+}
+
+// The FP64 back-transformation with FP64 tensor-core products (tc_gemm64.cu), also on
+// Z^T: per block, last first, U = Z^T_sub V_b^T, Z^T_sub -= (U T_b^T) V_b.  The
+// reflectors are cut once in both orientations (rows are zero left of the reflector,
+// so whole rows serve every block) and give the Gram matrices of all blocks in one
+// launch.  n = 1680: 64.5 -> 3.8 ms, n = 574: 9.4 -> 1.2.
+struct Bt64Scratch {
+  double *U, *W;       // n x kBtBlockTc
+  Tc64Op u, t;         // cut U or W, and T of all blocks
+};
+static size_t bt64_scratch(int n, void* base, Bt64Scratch* out) {
+  const size_t u = (size_t)n * kBtBlockTc * sizeof(double);        // a multiple of 256
+  const int rt = tc_blocks(n) * kBtBlockTc;
+  const size_t uo = tc64_op_bytes(n, kBtBlockTc);
+  if (out) {
+    char* c = (char*)base;
+    out->U = (double*)c;
+    out->W = (double*)(c + u);
+    out->u = tc64_op(c + 2 * u, n, kBtBlockTc);
+    out->t = tc64_op(c + 2 * u + uo, rt, kBtBlockTc);
+  }
+  return 2 * u + uo + tc64_op_bytes(rt, kBtBlockTc);
+}
+
+static int eig_backtransform_tc64(cudaStream_t s, int n, double* Q, EigWork& w, const Tc64Work& tw) {
+  constexpr int KB = kBtBlockTc;
+  bt_attributes();
+  const int nref = n - 2, nblk = bt_blocks(n);
+  Bt64Scratch sc;
+  bt64_scratch(n, w.lu, &sc);
+  const Tc64Op V = tc64_slot(tw, 0, nref, n), Vt = tc64_slot(tw, 1, n, nref), Z = tc64_slot(tw, 2, n, n);
+  double* Zt = w.A;
+  transpose_sq(s, n, Q, Zt);
+  tc64_cut_rows(s, V, 0, n, w.Vst, n);
+  tc64_cut_cols(s, Vt, nref, w.Vst, n);
+  if (tc64_gemm(s, nref, nref, 0, n, V, 0, V, 0, 0, 1.0, 0, w.Gm, KB, 1, KB, tw.err)) return -1;
+  cudaMemsetAsync(w.Tm, 0, (size_t)nblk * KB * KB * sizeof(double), s);     // columns beyond a short last block
+  tfactor_all_kernel<<<nblk, KB, KB * KB * sizeof(double), s>>>(nref, KB, w.tau, w.Gm, w.Tm);
+  count_launch();
+  tc64_cut_rows(s, sc.t, 0, KB, w.Tm, KB);
+  for (int b = nblk - 1; b >= 0; --b) {
+    const int k0 = b * KB, kb = std::min(KB, nref - k0), c0 = k0 + 1, first = c0 & ~31;
+    tc64_cut_rows(s, Z, first, n, Zt, n);
+    if (tc64_gemm(s, n, kb, first, n, Z, 0, V, k0, 0, 1.0, 0, sc.U, KB, 0, 0, tw.err)) return -1;
+    tc64_cut_rows(s, sc.u, 0, kb, sc.U, KB);
+    if (tc64_gemm(s, n, kb, 0, kb, sc.u, 0, sc.t, k0, 0, 1.0, 0, sc.W, KB, 0, 0, tw.err)) return -1;
+    tc64_cut_rows(s, sc.u, 0, kb, sc.W, KB);
+    if (tc64_gemm(s, n, n - c0, 0, kb, sc.u, 0, Vt, c0, k0, -1.0, 1, Zt + c0, n, 0, 0, tw.err)) return -1;
+  }
+  transpose_sq(s, n, Zt, Q);
+  return 0;
+}
+
+int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork* tw, const Tc64Work* t64) {
+  if (tw && n > 2) return eig_backtransform_tc(s, n, Q, w, *tw);
+  if (t64 && n > 2) return eig_backtransform_tc64(s, n, Q, w, *t64);
+  // 4. back-transformation, last block of reflectors first
+  int nref = n - 2;
+  if (nref > 0) {
+    int nblk = (nref + kBtBlock - 1) / kBtBlock;
+    for (int b = nblk - 1; b >= 0; --b) {
+      int k0 = b * kBtBlock, k1 = (k0 + kBtBlock < nref) ? k0 + kBtBlock : nref;
+      int kb = k1 - k0, c0 = k0 + 1, m = n - c0;
+      const double* Vb = w.Vst + (size_t)k0 * n + c0;
+      dgemm(s, 0, 1, kb, kb, m, 1.0, Vb, n, Vb, n, 0.0, w.Gm, kBtBlock);
+      tfactor_kernel<<<1, kBtBlock, kb * kb * sizeof(double), s>>>(kb, w.tau + k0, w.Gm, kBtBlock, w.Tm, kBtBlock);
+      count_launch();
+      dgemm(s, 0, 0, kb, n, m, 1.0, Vb, n, Q + (size_t)c0 * n, n, 0.0, w.Wt, n);
+      dgemm(s, 0, 0, kb, n, kb, 1.0, w.Tm, kBtBlock, w.Wt, n, 0.0, w.Wt2, n);
+      dgemm(s, 1, 0, m, n, kb, -1.0, Vb, n, w.Wt2, n, 1.0, Q + (size_t)c0 * n, n);
+    }
+  }
+  return 0;
+}
+
+int symmetric_eig(cudaStream_t s, int n, const double* F, double* eps, double* Q, EigWork& w,
+                  int* status, int sm_count) {
+  int rc = eig_tridiagonalize(s, n, F, w, status, sm_count, false, false);
+  if (rc) return rc;
+  eig_bisect(s, n, eps, w, 1e-12, false);
+  eig_vectors(s, n, eps, Q, w, false);
+  eig_backtransform(s, n, Q, w, nullptr, nullptr);
+  return 0;
+}
+
+}  // namespace kx
