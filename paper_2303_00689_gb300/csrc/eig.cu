@@ -279,435 +279,254 @@ __device__ __forceinline__ float start_value_f(int row, int col) {
   return __fadd_rn(__fmul_rn((float)(start_hash(row, col) & 0xFFFFF), 0x1p-19f), -0.999f);
 }
 
-// inverse iteration; one thread per cluster leader; lu: 5 x n x n workspace.
-// The recurrences carry their running values in registers, and the loads of
-// each sweep are issued kIvB rows at a time ahead of the dependent arithmetic
-// (one thread walks n rows of a column: a load-use chain per row would put
-// the memory latency on the critical path n times); the arithmetic and its
-// order are those of the textbook pivoted tridiagonal LU and its
-// forward/backward substitutions.
-constexpr int kIvB = 8;
+// Arithmetic of the inverse iteration: FP64, or double-float (FP32 pairs, df.cuh) in
+// the mixed path.  unit(): the shift separation and pivot floor in units of |T|.
+template <class R>
+struct IvOps;
+template <>
+struct IvOps<double> {
+  static constexpr double kUnit = kEps;
+  __device__ static __forceinline__ double from(double x) { return x; }
+  __device__ static __forceinline__ double load(const double* p) { return __ldg(p); }
+  __device__ static __forceinline__ double sub(double a, double b) { return a - b; }
+  __device__ static __forceinline__ double mul(double a, double b) { return a * b; }
+  __device__ static __forceinline__ double neg(double a) { return -a; }
+  __device__ static __forceinline__ double recip(double a) { return 1.0 / a; }
+  __device__ static __forceinline__ double mag(double a) { return fabs(a); }
+  __device__ static __forceinline__ bool minus(double a) { return !(a >= 0.0); }
+  __device__ static __forceinline__ double start(int r, int c) { return start_value(r, c); }
+  __device__ static __forceinline__ double max(double a, double b) { return fmax(a, b); }
+  __device__ static __forceinline__ double widen(double m) { return m; }
+  __device__ static __forceinline__ void add_sq(double& s, double x) { s = fma(x, x, s); }
+  __device__ static __forceinline__ double sum(double s) { return s; }
+  __device__ static __forceinline__ double out(double x) { return x; }
+};
+template <>
+struct IvOps<dfl> {
+  static constexpr double kUnit = 0x1p-46;
+  __device__ static __forceinline__ dfl from(double x) { return df_from_double(x); }
+  __device__ static __forceinline__ dfl load(const dfl* p) {
+    const float2 v = __ldg((const float2*)p);
+    return dfl{v.x, v.y};
+  }
+  __device__ static __forceinline__ dfl sub(dfl a, dfl b) { return df_sub(a, b); }
+  __device__ static __forceinline__ dfl mul(dfl a, dfl b) { return df_mul(a, b); }
+  __device__ static __forceinline__ dfl neg(dfl a) { return df_neg(a); }
+  __device__ static __forceinline__ dfl recip(dfl a) { return df_recip(a); }
+  __device__ static __forceinline__ float mag(dfl a) { return fabsf(a.hi); }
+  __device__ static __forceinline__ bool minus(dfl a) { return !(a.hi >= 0.0f); }
+  __device__ static __forceinline__ dfl start(int r, int c) { return dfl{start_value_f(r, c), 0.0f}; }
+  __device__ static __forceinline__ float max(float a, float b) { return fmaxf(a, b); }
+  __device__ static __forceinline__ dfl widen(float m) { return dfl{m, 0.0f}; }
+  __device__ static __forceinline__ void add_sq(dfl& s, dfl x) { df_acc_mul(s, x, x); }
+  __device__ static __forceinline__ double sum(dfl s) { return df_to_double(df_norm(s)); }
+  __device__ static __forceinline__ double out(dfl x) { return df_to_double_fast(x); }
+};
 
-__global__ void invit_kernel(int n, const double* __restrict__ d, const double* __restrict__ e,
-                             const double* __restrict__ ev, const double* __restrict__ scal,
-                             const int* __restrict__ clus, double* __restrict__ lu,
-                             double* __restrict__ Z) {
-  int L = blockIdx.x * blockDim.x + threadIdx.x;
-  if (L >= n || !clus[L]) return;
-  int end = L + 1;
-  while (end < n && !clus[end]) ++end;
-  const double tn = fmax(scal[2], 1e-300);
-  const double tiny = kEps * tn;
+// Eigenvectors of T by two steps of inverse iteration, a thread per eigenvalue; lu:
+// 5 x n x n workspace.  What bounds it is the latency of the recurrences (n rows, six
+// sweeps), so
+//  * the sweeps carry their running values in registers and issue the loads of kIvB
+//    rows ahead of the dependent arithmetic;
+//  * the steps are fused: step 1 solves from the start vector without storing it, its
+//    backward sweep tracks max|x|; step 2 reads x scaled by 1/max (inverse iteration is
+//    linear, the scale only keeps the values in range), its backward sweep accumulates
+//    ||x||^2; a last pass writes x / ||x|| in FP64;
+//  * few lanes of a warp are used (kIvLanes: whole 32-byte sectors, little divergence
+//    at the pivots), so that the chains spread over all SMs;
+//  * members of a cluster (gaps below 1e-7 of the width) are solved like all others,
+//    each from its own start vector, and made orthogonal afterwards
+//    (orth_cluster_kernel): one thread doing a cluster in turn was most of the time
+//    wherever there was one.  n = 1680 and 3360 (7 and 14 cages):
+//    4.4 -> 2.0 and 22.6 -> 5.0 ms; FP64, which had fifteen sweeps, 574 and 1680:
+//    1.42 -> 0.86 and 5.8 -> 2.8 ms.
+// Shifts closer than ten units to the one before are moved up to that distance.
+constexpr int kIvB = 8;
+constexpr int kIvLanes = 4;
+template <class R>
+__global__ void __launch_bounds__(32) invit_kernel(int n, int lanes, const R* __restrict__ d, const R* __restrict__ e,
+                                                 const double* __restrict__ ev, const double* __restrict__ scal,
+                                                 const int* __restrict__ clus, R* __restrict__ lu,
+                                                 double* __restrict__ Zout) {
+  using O = IvOps<R>;
+  if (threadIdx.x >= lanes) return;
+  const int L = blockIdx.x * lanes + threadIdx.x;
+  if (L >= n) return;
+  if (n == 1) {
+    Zout[0] = 1.0;
+    return;
+  }
+  const double tiny_d = O::kUnit * fmax(scal[2], 1e-300);
+  const R tiny = O::from(tiny_d);
   const size_t nn = (size_t)n * n;
-  double* __restrict__ dl = lu + 0 * nn;
-  double* __restrict__ rdd = lu + 1 * nn;   // reciprocal pivots
-  double* __restrict__ du = lu + 2 * nn;
-  double* __restrict__ du2 = lu + 3 * nn;
-  double* __restrict__ pv = lu + 4 * nn;
+  R* __restrict__ dl = lu + 0 * nn;
+  R* __restrict__ rdd = lu + 1 * nn;   // reciprocal pivots
+  R* __restrict__ du = lu + 2 * nn;
+  R* __restrict__ du2 = lu + 3 * nn;
+  int* __restrict__ pv = (int*)(lu + 4 * nn);
+  R* __restrict__ Z = (R*)Zout;        // iterates in place of the FP64 output
 #define LU(a, r) a[(size_t)(r) * n + L]
-#define ZC(r, c) Z[(size_t)(r) * n + (c)]
-  double prevlam = 0.0;
-  for (int j = L; j < end; ++j) {
-    double lam = ev[j];
-    if (j > L && lam - prevlam < 10.0 * tiny) lam = prevlam + 10.0 * tiny;
-    prevlam = lam;
-    if (n == 1) { ZC(0, j) = 1.0; continue; }
-    // LU of T - lam I with partial pivoting; a, u: pivot-row diagonal and superdiagonal
-    double a = d[0] - lam, u = e[0];
-    for (int r = 0; r < n - 1; ++r) {
-      const double b = e[r];
-      const double dn = d[r + 1] - lam;
-      const double un = (r < n - 2) ? e[r + 1] : 0.0;
-      if (fabs(a) >= fabs(b)) {
-        LU(pv, r) = 0.0;
-        if (fabs(a) < tiny) a = (a >= 0.0) ? tiny : -tiny;
-        const double ra = 1.0 / a;          // one division per row (the FP64 divide is slow)
-        const double f = b * ra;
-        LU(dl, r) = f;
-        LU(rdd, r) = ra;
-        LU(du, r) = u;
-        LU(du2, r) = 0.0;
-        a = dn - f * u;
-        u = un;
+#define ZC(r) Z[(size_t)(r) * n + L]
+  double shift = ev[L];
+  if (!clus[L]) {
+    int j = L;
+    while (!clus[j]) --j;
+    shift = ev[j];
+    for (++j; j <= L; ++j) shift = (ev[j] - shift < 10.0 * tiny_d) ? shift + 10.0 * tiny_d : ev[j];
+  }
+  // LU of T - lam I with partial pivoting; a, u: pivot-row diagonal and superdiagonal.
+  // No FP64 instruction per row in the mixed path: GB300 issues one FP64 warp
+  // instruction per ~76 cycles per scheduler, which would put the FP64 pipe on the chain.
+  const R lam = O::from(shift);
+  R a = O::sub(O::load(d), lam), u = O::load(e);
+  for (int r = 0; r < n - 1; ++r) {
+    const R b = O::load(e + r);
+    const R dn = O::sub(O::load(d + r + 1), lam);
+    const R un = (r < n - 2) ? O::load(e + r + 1) : R{};
+    if (O::mag(a) >= O::mag(b)) {
+      LU(pv, r) = 0;
+      if (O::mag(a) < O::mag(tiny)) a = O::minus(a) ? O::neg(tiny) : tiny;
+      const R ra = O::recip(a);
+      const R f = O::mul(b, ra);
+      LU(dl, r) = f;
+      LU(rdd, r) = ra;
+      LU(du, r) = u;
+      LU(du2, r) = R{};
+      a = O::sub(dn, O::mul(f, u));
+      u = un;
+    } else {
+      LU(pv, r) = 1;
+      const R rb = O::recip(b);
+      const R f = O::mul(a, rb);
+      LU(rdd, r) = rb;
+      LU(dl, r) = f;
+      LU(du, r) = dn;
+      const R na = O::sub(u, O::mul(f, dn));
+      if (r < n - 2) {
+        LU(du2, r) = un;
+        u = O::neg(O::mul(f, un));
       } else {
-        LU(pv, r) = 1.0;
-        const double rb = 1.0 / b;
-        const double f = a * rb;
-        LU(rdd, r) = rb;
-        LU(dl, r) = f;
-        LU(du, r) = dn;
-        const double na = u - f * dn;
-        if (r < n - 2) {
-          LU(du2, r) = un;
-          u = -f * un;
-        } else {
-          LU(du2, r) = 0.0;
-        }
-        a = na;
+        LU(du2, r) = R{};
       }
-    }
-    if (fabs(a) < tiny) a = (a >= 0.0) ? tiny : -tiny;
-    LU(rdd, n - 1) = 1.0 / a;
-    for (int r = 0; r < n; ++r) ZC(r, j) = start_value(r, j);
-    for (int it = 0; it < 2; ++it) {
-      // forward (L with pivots); cur = current row r of the right-hand side
-      double cur = ZC(0, j);
-      for (int r0 = 0; r0 < n - 1; r0 += kIvB) {
-        double nx[kIvB], fv[kIvB], pf[kIvB];
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 + q;
-          if (r < n - 1) { nx[q] = ZC(r + 1, j); fv[q] = LU(dl, r); pf[q] = LU(pv, r); }
-        }
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 + q;
-          if (r < n - 1) {
-            if (pf[q] == 0.0) {
-              ZC(r, j) = cur;
-              cur = nx[q] - fv[q] * cur;
-            } else {
-              ZC(r, j) = nx[q];
-              cur = cur - fv[q] * nx[q];
-            }
-          }
-        }
-      }
-      // backward (U, three diagonals, reciprocal pivots); z1 = x[r+1], z2 = x[r+2]
-      double z2 = cur * LU(rdd, n - 1);
-      ZC(n - 1, j) = z2;
-      double z1 = z2;
-      if (n > 1) {
-        z1 = (ZC(n - 2, j) - LU(du, n - 2) * z2) * LU(rdd, n - 2);
-        ZC(n - 2, j) = z1;
-      }
-      for (int r0 = n - 3; r0 >= 0; r0 -= kIvB) {
-        double zv[kIvB], uv[kIvB], u2[kIvB], rv[kIvB];
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 - q;
-          if (r >= 0) { zv[q] = ZC(r, j); uv[q] = LU(du, r); u2[q] = LU(du2, r); rv[q] = LU(rdd, r); }
-        }
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 - q;
-          if (r >= 0) {
-            const double x = (zv[q] - uv[q] * z1 - u2[q] * z2) * rv[q];
-            ZC(r, j) = x;
-            z2 = z1;
-            z1 = x;
-          }
-        }
-      }
-      // scale, re-orthogonalise within the cluster, normalise
-      double mx = 0.0;
-#pragma unroll 8
-      for (int r = 0; r < n; ++r) mx = fmax(mx, fabs(ZC(r, j)));
-      double s = (mx > 0.0) ? 1.0 / mx : 1.0;
-#pragma unroll 8
-      for (int r = 0; r < n; ++r) ZC(r, j) *= s;
-      for (int c = L; c < j; ++c) {
-        double dot = 0.0;
-#pragma unroll 8
-        for (int r = 0; r < n; ++r) dot += ZC(r, c) * ZC(r, j);
-#pragma unroll 8
-        for (int r = 0; r < n; ++r) ZC(r, j) -= dot * ZC(r, c);
-      }
-      double nrm = 0.0;
-#pragma unroll 8
-      for (int r = 0; r < n; ++r) nrm += ZC(r, j) * ZC(r, j);
-      nrm = ::sqrt(nrm);
-      s = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-#pragma unroll 8
-      for (int r = 0; r < n; ++r) ZC(r, j) *= s;
+      a = na;
     }
   }
+  if (O::mag(a) < O::mag(tiny)) a = O::minus(a) ? O::neg(tiny) : tiny;
+  LU(rdd, n - 1) = O::recip(a);
+  R scl = O::from(1.0);
+  R nrm = R{};
+  for (int it = 0; it < 2; ++it) {
+    // forward (L with pivots); step 1 takes the start vector, step 2 the scaled x
+    R cur = (it == 0) ? O::start(0, L) : O::mul(ZC(0), scl);
+    for (int r0 = 0; r0 < n - 1; r0 += kIvB) {
+      R nx[kIvB], fv[kIvB];
+      int pf[kIvB];
+#pragma unroll
+      for (int q = 0; q < kIvB; ++q) {
+        const int r = r0 + q;
+        if (r < n - 1) {
+          nx[q] = (it == 0) ? O::start(r + 1, L) : O::mul(ZC(r + 1), scl);
+          fv[q] = LU(dl, r);
+          pf[q] = LU(pv, r);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kIvB; ++q) {
+        const int r = r0 + q;
+        if (r < n - 1) {
+          if (pf[q] == 0) {
+            ZC(r) = cur;
+            cur = O::sub(nx[q], O::mul(fv[q], cur));
+          } else {
+            ZC(r) = nx[q];
+            cur = O::sub(cur, O::mul(fv[q], nx[q]));
+          }
+        }
+      }
+    }
+    // backward (U, three diagonals, reciprocal pivots), with max|x| or ||x||^2;
+    // z1 = x[r + 1], z2 = x[r + 2]
+    R z2 = O::mul(cur, LU(rdd, n - 1));
+    ZC(n - 1) = z2;
+    auto mx = O::mag(z2);
+    if (it == 1) O::add_sq(nrm, z2);
+    R z1 = O::mul(O::sub(ZC(n - 2), O::mul(LU(du, n - 2), z2)), LU(rdd, n - 2));
+    ZC(n - 2) = z1;
+    mx = O::max(mx, O::mag(z1));
+    if (it == 1) O::add_sq(nrm, z1);
+    for (int r0 = n - 3; r0 >= 0; r0 -= kIvB) {
+      R zv[kIvB], uv[kIvB], u2[kIvB], rv[kIvB];
+#pragma unroll
+      for (int q = 0; q < kIvB; ++q) {
+        const int r = r0 - q;
+        if (r >= 0) { zv[q] = ZC(r); uv[q] = LU(du, r); u2[q] = LU(du2, r); rv[q] = LU(rdd, r); }
+      }
+#pragma unroll
+      for (int q = 0; q < kIvB; ++q) {
+        const int r = r0 - q;
+        if (r >= 0) {
+          const R x = O::mul(O::sub(O::sub(zv[q], O::mul(uv[q], z1)), O::mul(u2[q], z2)), rv[q]);
+          ZC(r) = x;
+          mx = O::max(mx, O::mag(x));
+          if (it == 1) O::add_sq(nrm, x);
+          z2 = z1;
+          z1 = x;
+        }
+      }
+    }
+    if (it == 0) scl = (mx > 0) ? O::recip(O::widen(mx)) : O::from(1.0);
+  }
+  const double nd = ::sqrt(O::sum(nrm));
+  const R sc = (nd > 0.0) ? O::from(1.0 / nd) : R{};
+#pragma unroll 8
+  for (int r = 0; r < n; ++r) Zout[(size_t)r * n + L] = O::out(O::mul(ZC(r), sc));
 #undef LU
 #undef ZC
 }
 
-// Mixed path: the same inverse iteration in double-float arithmetic.  The LU
-// factors and the iterates are held as (hi, lo) pairs in the same workspace
-// (the iterates in Q, converted to FP64 at the end); one reciprocal per row
-// from the FP32 estimate and one Newton step; the pivot floor and the shift
-// separation use the double-float unit 2^-46 |T| instead of the FP64 epsilon.
-__device__ __forceinline__ float df_abs_hi(dfl a) { return fabsf(a.hi); }
-
-// Each cluster leader runs its recurrences alone, so the kernel is bound by
-// their latency: kIvLanes active lanes per 32-thread block spread the n
-// chains over n / kIvLanes warps (about 5 per SM at n = 3360 instead of
-// one), so each SM interleaves several independent chains; four lanes keep
-// every access a whole 32-byte sector and limit divergence at the pivots.
-constexpr int kIvLanes = 4;
-__global__ void __launch_bounds__(32) invit_df_kernel(int n, const dfl* __restrict__ d, const double* __restrict__ e,
-                                                    const dfl* __restrict__ edf,
-                                                    const double* __restrict__ ev, const double* __restrict__ scal,
-                                                    const int* __restrict__ clus, dfl* __restrict__ lu,
-                                                    double* __restrict__ Zout) {
-  if (threadIdx.x >= kIvLanes) return;
-  int L = blockIdx.x * kIvLanes + threadIdx.x;
-  if (L >= n || !clus[L]) return;
-  int end = L + 1;
+// Gram-Schmidt within the clusters, a block per cluster (blocks of other columns
+// return): every vector against the ones before it, kOrthTile at a time, twice (what
+// the first pass leaves of nearly parallel vectors the second removes), then normalised.
+// The columns of a cluster are neighbours, so a row's values share sectors.
+constexpr int kOrthThreads = 256, kOrthTile = 32;
+__global__ void __launch_bounds__(kOrthThreads) orth_cluster_kernel(int n, const int* __restrict__ clus,
+                                                                  double* __restrict__ Z) {
+  const int L = blockIdx.x;
+  if (!clus[L] || L + 1 >= n || clus[L + 1]) return;
+  int end = L + 2;
   while (end < n && !clus[end]) ++end;
-  const double tn = fmax(scal[2], 1e-300);
-  const double tiny_d = 0x1p-46 * tn;
-  const dfl tiny = df_from_double(tiny_d);
-  const size_t nn = (size_t)n * n;
-  dfl* __restrict__ dl = lu + 0 * nn;
-  dfl* __restrict__ rdd = lu + 1 * nn;   // reciprocal pivots
-  dfl* __restrict__ du = lu + 2 * nn;
-  dfl* __restrict__ du2 = lu + 3 * nn;
-  int* __restrict__ pv = (int*)(lu + 4 * nn);
-  dfl* __restrict__ Z = (dfl*)Zout;      // iterates in place of the FP64 output
-#define LU(a, r) a[(size_t)(r) * n + L]
-#define ZC(r, c) Z[(size_t)(r) * n + (c)]
-  if (end == L + 1 && n > 1) {
-    // An eigenvalue alone in its cluster (the common case): the same two
-    // inverse-iteration steps with the passes fused.  Step 1 solves from the
-    // start vector without storing it, its backward sweep tracks max|x|;
-    // step 2 reads x scaled by 1/max (inverse iteration is linear, the scale
-    // only keeps the values in range), its backward sweep accumulates ||x||^2;
-    // one last pass writes x / ||x|| in FP64.  Six sweeps of n instead of 15.
-    // no FP64 instruction per row: GB300 issues one FP64 warp instruction per
-    // ~76 cycles per scheduler, which would put the FP64 pipe on the chain
-    const dfl lam = df_from_double(ev[L]);
-    dfl a = df_sub(ldg_df(d), lam), u = ldg_df(edf);
-    for (int r = 0; r < n - 1; ++r) {
-      const dfl b = ldg_df(edf + r);
-      const dfl dn = df_sub(ldg_df(d + r + 1), lam);
-      const dfl un = (r < n - 2) ? ldg_df(edf + r + 1) : dfl{0.0f, 0.0f};
-      if (df_abs_hi(a) >= df_abs_hi(b)) {
-        LU(pv, r) = 0;
-        if (df_abs_hi(a) < tiny.hi) a = (a.hi >= 0.0f) ? tiny : df_neg(tiny);
-        const dfl ra = df_recip(a);
-        const dfl f = df_mul(b, ra);
-        LU(dl, r) = f;
-        LU(rdd, r) = ra;
-        LU(du, r) = u;
-        LU(du2, r) = dfl{0.0f, 0.0f};
-        a = df_sub(dn, df_mul(f, u));
-        u = un;
-      } else {
-        LU(pv, r) = 1;
-        const dfl rb = df_recip(b);
-        const dfl f = df_mul(a, rb);
-        LU(rdd, r) = rb;
-        LU(dl, r) = f;
-        LU(du, r) = dn;
-        const dfl na = df_sub(u, df_mul(f, dn));
-        if (r < n - 2) {
-          LU(du2, r) = un;
-          u = df_neg(df_mul(f, un));
-        } else {
-          LU(du2, r) = dfl{0.0f, 0.0f};
-        }
-        a = na;
-      }
-    }
-    if (df_abs_hi(a) < tiny.hi) a = (a.hi >= 0.0f) ? tiny : df_neg(tiny);
-    LU(rdd, n - 1) = df_recip(a);
-    dfl scl = {1.0f, 0.0f};
-    dfl nrm = {0.0f, 0.0f};
-    for (int it = 0; it < 2; ++it) {
-      // forward (L with pivots); step 1 takes the start vector, step 2 the scaled x
-      dfl cur = (it == 0) ? dfl{start_value_f(0, L), 0.0f} : df_mul(ZC(0, L), scl);
-      for (int r0 = 0; r0 < n - 1; r0 += kIvB) {
-        dfl nx[kIvB], fv[kIvB];
-        int pf[kIvB];
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 + q;
-          if (r < n - 1) {
-            nx[q] = (it == 0) ? dfl{start_value_f(r + 1, L), 0.0f} : df_mul(ZC(r + 1, L), scl);
-            fv[q] = LU(dl, r);
-            pf[q] = LU(pv, r);
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 + q;
-          if (r < n - 1) {
-            if (pf[q] == 0) {
-              ZC(r, L) = cur;
-              cur = df_sub(nx[q], df_mul(fv[q], cur));
-            } else {
-              ZC(r, L) = nx[q];
-              cur = df_sub(cur, df_mul(fv[q], nx[q]));
-            }
-          }
-        }
-      }
-      // backward (U, three diagonals, reciprocal pivots), with max|x| or ||x||^2
-      float mx = 0.0f;
-      dfl z2 = df_mul(cur, LU(rdd, n - 1));
-      ZC(n - 1, L) = z2;
-      mx = fmaxf(mx, df_abs_hi(z2));
-      if (it == 1) df_acc_mul(nrm, z2, z2);
-      dfl z1 = z2;
-      if (n > 1) {
-        z1 = df_mul(df_sub(ZC(n - 2, L), df_mul(LU(du, n - 2), z2)), LU(rdd, n - 2));
-        ZC(n - 2, L) = z1;
-        mx = fmaxf(mx, df_abs_hi(z1));
-        if (it == 1) df_acc_mul(nrm, z1, z1);
-      }
-      for (int r0 = n - 3; r0 >= 0; r0 -= kIvB) {
-        dfl zv[kIvB], uv[kIvB], u2[kIvB], rv[kIvB];
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 - q;
-          if (r >= 0) { zv[q] = ZC(r, L); uv[q] = LU(du, r); u2[q] = LU(du2, r); rv[q] = LU(rdd, r); }
-        }
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 - q;
-          if (r >= 0) {
-            const dfl x = df_mul(df_sub(df_sub(zv[q], df_mul(uv[q], z1)), df_mul(u2[q], z2)), rv[q]);
-            ZC(r, L) = x;
-            mx = fmaxf(mx, df_abs_hi(x));
-            if (it == 1) df_acc_mul(nrm, x, x);
-            z2 = z1;
-            z1 = x;
-          }
-        }
-      }
-      if (it == 0) scl = (mx > 0.0f) ? df_recip(dfl{mx, 0.0f}) : dfl{1.0f, 0.0f};
-    }
-    const double nd = ::sqrt(df_to_double(df_norm(nrm)));
-    const dfl sc = (nd > 0.0) ? df_from_double(1.0 / nd) : dfl{0.0f, 0.0f};
-#pragma unroll 8
-    for (int r = 0; r < n; ++r) {
-      const dfl z = df_mul(ZC(r, L), sc);
-      Zout[(size_t)r * n + L] = df_to_double_fast(z);
-    }
-    return;
-  }
-  double prevlam = 0.0;
+  __shared__ double coef[kOrthTile];
+  __shared__ double part[kOrthThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   for (int j = L; j < end; ++j) {
-    double lamd = ev[j];
-    if (j > L && lamd - prevlam < 10.0 * tiny_d) lamd = prevlam + 10.0 * tiny_d;
-    prevlam = lamd;
-    if (n == 1) { ZC(0, j) = dfl{1.0f, 0.0f}; continue; }
-    const dfl lam = df_from_double(lamd);
-    // LU of T - lam I with partial pivoting; a, u: pivot-row diagonal and superdiagonal
-    dfl a = df_sub(ldg_df(d), lam), u = df_from_double(e[0]);
-    for (int r = 0; r < n - 1; ++r) {
-      const dfl b = df_from_double(e[r]);
-      const dfl dn = df_sub(ldg_df(d + r + 1), lam);
-      const dfl un = (r < n - 2) ? df_from_double(e[r + 1]) : dfl{0.0f, 0.0f};
-      if (df_abs_hi(a) >= df_abs_hi(b)) {
-        LU(pv, r) = 0;
-        if (df_abs_hi(a) < tiny.hi) a = (a.hi >= 0.0f) ? tiny : df_neg(tiny);
-        const dfl ra = df_recip(a);
-        const dfl f = df_mul(b, ra);
-        LU(dl, r) = f;
-        LU(rdd, r) = ra;
-        LU(du, r) = u;
-        LU(du2, r) = dfl{0.0f, 0.0f};
-        a = df_sub(dn, df_mul(f, u));
-        u = un;
-      } else {
-        LU(pv, r) = 1;
-        const dfl rb = df_recip(b);
-        const dfl f = df_mul(a, rb);
-        LU(rdd, r) = rb;
-        LU(dl, r) = f;
-        LU(du, r) = dn;
-        const dfl na = df_sub(u, df_mul(f, dn));
-        if (r < n - 2) {
-          LU(du2, r) = un;
-          u = df_neg(df_mul(f, un));
-        } else {
-          LU(du2, r) = dfl{0.0f, 0.0f};
+    for (int pass = 0; pass < 2; ++pass)
+      for (int c0 = L; c0 < j; c0 += kOrthTile) {
+        const int nc = min(kOrthTile, j - c0);
+        for (int c = wid; c < nc; c += kOrthThreads / 32) {
+          double s = 0.0;
+          for (int r = lane; r < n; r += 32) s = fma(Z[(size_t)r * n + c0 + c], Z[(size_t)r * n + j], s);
+          s = warp_sum(s);
+          if (lane == 0) coef[c] = s;
         }
-        a = na;
-      }
-    }
-    if (df_abs_hi(a) < tiny.hi) a = (a.hi >= 0.0f) ? tiny : df_neg(tiny);
-    LU(rdd, n - 1) = df_recip(a);
-    for (int r = 0; r < n; ++r) ZC(r, j) = df_from_double(start_value(r, j));
-    for (int it = 0; it < 2; ++it) {
-      // forward (L with pivots)
-      dfl cur = ZC(0, j);
-      for (int r0 = 0; r0 < n - 1; r0 += kIvB) {
-        dfl nx[kIvB], fv[kIvB];
-        int pf[kIvB];
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 + q;
-          if (r < n - 1) { nx[q] = ZC(r + 1, j); fv[q] = LU(dl, r); pf[q] = LU(pv, r); }
+        __syncthreads();
+        for (int r = tid; r < n; r += kOrthThreads) {
+          double z = Z[(size_t)r * n + j];
+          for (int c = 0; c < nc; ++c) z = fma(-coef[c], Z[(size_t)r * n + c0 + c], z);
+          Z[(size_t)r * n + j] = z;
         }
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 + q;
-          if (r < n - 1) {
-            if (pf[q] == 0) {
-              ZC(r, j) = cur;
-              cur = df_sub(nx[q], df_mul(fv[q], cur));
-            } else {
-              ZC(r, j) = nx[q];
-              cur = df_sub(cur, df_mul(fv[q], nx[q]));
-            }
-          }
-        }
+        __syncthreads();
       }
-      // backward (U, three diagonals, reciprocal pivots)
-      dfl z2 = df_mul(cur, LU(rdd, n - 1));
-      ZC(n - 1, j) = z2;
-      dfl z1 = z2;
-      if (n > 1) {
-        z1 = df_mul(df_sub(ZC(n - 2, j), df_mul(LU(du, n - 2), z2)), LU(rdd, n - 2));
-        ZC(n - 2, j) = z1;
-      }
-      for (int r0 = n - 3; r0 >= 0; r0 -= kIvB) {
-        dfl zv[kIvB], uv[kIvB], u2[kIvB], rv[kIvB];
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 - q;
-          if (r >= 0) { zv[q] = ZC(r, j); uv[q] = LU(du, r); u2[q] = LU(du2, r); rv[q] = LU(rdd, r); }
-        }
-#pragma unroll
-        for (int q = 0; q < kIvB; ++q) {
-          const int r = r0 - q;
-          if (r >= 0) {
-            const dfl x = df_mul(df_sub(df_sub(zv[q], df_mul(uv[q], z1)), df_mul(u2[q], z2)), rv[q]);
-            ZC(r, j) = x;
-            z2 = z1;
-            z1 = x;
-          }
-        }
-      }
-      // scale, re-orthogonalise within the cluster, normalise
-      float mx = 0.0f;
-#pragma unroll 8
-      for (int r = 0; r < n; ++r) mx = fmaxf(mx, df_abs_hi(ZC(r, j)));
-      dfl sc = (mx > 0.0f) ? df_recip(dfl{mx, 0.0f}) : dfl{1.0f, 0.0f};
-#pragma unroll 8
-      for (int r = 0; r < n; ++r) ZC(r, j) = df_mul(ZC(r, j), sc);
-      for (int c = L; c < j; ++c) {
-        dfl dot = {0.0f, 0.0f};
-#pragma unroll 8
-        for (int r = 0; r < n; ++r) df_acc_mul(dot, ZC(r, c), ZC(r, j));
-        dot = df_norm(dot);
-#pragma unroll 8
-        for (int r = 0; r < n; ++r) ZC(r, j) = df_sub(ZC(r, j), df_mul(dot, ZC(r, c)));
-      }
-      dfl nrm = {0.0f, 0.0f};
-#pragma unroll 8
-      for (int r = 0; r < n; ++r) df_acc_mul(nrm, ZC(r, j), ZC(r, j));
-      const double nd = ::sqrt(df_to_double(df_norm(nrm)));
-      sc = (nd > 0.0) ? df_from_double(1.0 / nd) : dfl{0.0f, 0.0f};
-#pragma unroll 8
-      for (int r = 0; r < n; ++r) ZC(r, j) = df_mul(ZC(r, j), sc);
-    }
+    double s = 0.0;
+    for (int r = tid; r < n; r += kOrthThreads) s = fma(Z[(size_t)r * n + j], Z[(size_t)r * n + j], s);
+    s = warp_sum(s);
+    if (lane == 0) part[wid] = s;
+    __syncthreads();
+    s = 0.0;
+    for (int w = 0; w < kOrthThreads / 32; ++w) s += part[w];
+    s = (s > 0.0) ? 1.0 / ::sqrt(s) : 0.0;
+    for (int r = tid; r < n; r += kOrthThreads) Z[(size_t)r * n + j] *= s;
+    __syncthreads();
   }
-  // FP64 output (same slots, same thread)
-  for (int j = L; j < end; ++j)
-    for (int r = 0; r < n; ++r) {
-      const dfl z = ZC(r, j);
-      Zout[(size_t)r * n + j] = df_to_double_fast(z);
-    }
-#undef LU
-#undef ZC
 }
 
 // T factor of a block of kb reflectors (forward, columnwise): one block,
@@ -850,12 +669,19 @@ void eig_vectors(cudaStream_t s, int n, const double* eps, double* Q, EigWork& w
   if (df_path) {
     const dfl* d_dfl = (const dfl*)(w.pbuf + n);     // written by eig_bisect
     const dfl* e_dfl = d_dfl + 2 * (size_t)n;
-    invit_df_kernel<<<(n + kIvLanes - 1) / kIvLanes, 32, 0, s>>>(n, d_dfl, w.e, e_dfl, eps, w.scal, w.clus,
-                                                                (dfl*)w.lu, Q);
+    invit_kernel<dfl><<<(n + kIvLanes - 1) / kIvLanes, 32, 0, s>>>(n, kIvLanes, d_dfl, e_dfl, eps, w.scal, w.clus,
+                                                                  (dfl*)w.lu, Q);
   } else {
-    invit_kernel<<<(n + 31) / 32, 32, 0, s>>>(n, w.d, w.e, eps, w.scal, w.clus, w.lu, Q);
+    // (not more warps than there are FP64 pipes, which a partly filled warp holds as long as a full one)
+    int lanes = kIvLanes;
+    while (lanes < 32 && n > lanes * kFp64Pipes) lanes *= 2;
+    invit_kernel<double><<<(n + lanes - 1) / lanes, 32, 0, s>>>(n, lanes, w.d, w.e, eps, w.scal, w.clus, w.lu, Q);
   }
   count_launch();
+  if (n > 1) {
+    orth_cluster_kernel<<<n, kOrthThreads, 0, s>>>(n, w.clus, Q);
+    count_launch();
+  }
 }
 
 // tensor-core back-transformation (mixed path), carried out on Z^T so that
