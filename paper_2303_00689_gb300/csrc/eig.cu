@@ -564,15 +564,53 @@ __global__ void tfactor_kernel(int kb, const double* __restrict__ tau, const dou
   tfactor_body(kb, tau, G, ldg, T, ldt);
 }
 
-// T factors of every block of kblk reflectors at once (block b: reflectors
-// b*kblk .. ; they depend on the reflectors only, not on the vectors updated)
-__global__ void tfactor_all_kernel(int nref, int kblk, const double* __restrict__ tau,
-                                   const double* __restrict__ Gall, double* __restrict__ Tall) {
-  const int b = blockIdx.x;
-  const int k0 = b * kblk;
-  const int kb = (k0 + kblk < nref) ? kblk : nref - k0;
-  const size_t off = (size_t)b * kblk * kblk;
-  tfactor_body(kb, tau + k0, Gall + off, kblk, Tall + off, kblk);
+// T factors of every block of kBtBlockTc reflectors at once (block b: reflectors
+// b kBtBlockTc ..; they depend on the reflectors only, not on the vectors updated).
+// Row i of T is a recurrence of its own, T_ij = -tau_j sum_l T_il G_lj, a chain of FP64
+// operations: four lanes a row take one of tfactor_body's four partial sums each (the
+// same sums in the same order), and kTfRows rows a CTA spread the rows over the SMs,
+// one warp per FP64 pipe.  Blocks of 128: 520 us with one thread
+// a row on one SM, 185 now.
+constexpr int kTfRows = 32;
+constexpr int kTfLd = kBtBlockTc + 3;     // rows of T: the eight of a warp in different banks
+constexpr int kTfSmem = (kBtBlockTc * (kBtBlockTc + 1) + kTfRows * kTfLd + kBtBlockTc) * (int)sizeof(double);
+__global__ void __launch_bounds__(4 * kTfRows) tfactor_all_kernel(int nref, const double* __restrict__ tau,
+                                                                const double* __restrict__ Gall,
+                                                                double* __restrict__ Tall) {
+  constexpr int KB = kBtBlockTc;
+  extern __shared__ double ts[];
+  double* gt = ts;                        // column j of G at gt + j (KB + 1)
+  double* trow = gt + KB * (KB + 1);
+  double* tj = trow + kTfRows * kTfLd;
+  const int k0 = blockIdx.y * KB, kb = min(KB, nref - k0), i0 = blockIdx.x * kTfRows;
+  if (i0 >= kb) return;
+  const double* G = Gall + (size_t)blockIdx.y * KB * KB;
+  for (int e = threadIdx.x; e < KB * KB; e += blockDim.x) {
+    const int l = e / KB, j = e % KB;
+    if (l < j && j < kb) gt[j * (KB + 1) + l] = G[e];
+  }
+  for (int j = threadIdx.x; j < kb; j += blockDim.x) tj[j] = tau[k0 + j];
+  __syncthreads();
+  const int i = i0 + (threadIdx.x >> 2), q = threadIdx.x & 3;
+  double* t = trow + (threadIdx.x >> 2) * kTfLd;
+  for (int j = i0; j < kb; ++j) {
+    const double* g = gt + j * (KB + 1);
+    double a = 0.0;
+    int l = i;
+    for (; l + 3 < j; l += 4) a = fma(t[l + q], g[l + q], a);
+    if (q == 0)
+      for (; l < j; ++l) a = fma(t[l], g[l], a);
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    a += __shfl_xor_sync(0xffffffffu, a, 2);
+    if (q == 0) t[j] = (j > i) ? -tj[j] * a : (j == i ? tj[j] : 0.0);
+    __syncwarp();
+  }
+  __syncthreads();
+  double* T = Tall + (size_t)blockIdx.y * KB * KB;
+  for (int e = threadIdx.x; e < kTfRows * kb; e += blockDim.x) {
+    const int r = e / kb, j = e % kb;
+    if (i0 + r < kb) T[(size_t)(i0 + r) * KB + j] = (j < i0) ? 0.0 : trow[r * kTfLd + j];
+  }
 }
 
 // number of blocks of kBtBlockTc reflectors (n - 2 reflectors)
@@ -828,8 +866,8 @@ static void bt_attributes() {
   once_per_device(attr, [] {
     return cudaFuncSetAttribute(tfactor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 kBtBlockTc * kBtBlockTc * (int)sizeof(double)) == cudaSuccess &&
-           cudaFuncSetAttribute(tfactor_all_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                kBtBlockTc * kBtBlockTc * (int)sizeof(double)) == cudaSuccess &&
+           cudaFuncSetAttribute(tfactor_all_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTfSmem) ==
+               cudaSuccess &&
            cudaFuncSetAttribute(y_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kYSmem) ==
                cudaSuccess;
   });
@@ -848,8 +886,7 @@ static int eig_backtransform_tc(cudaStream_t s, int n, double* Q, EigWork& w, co
   // Gram matrices and T factors of all blocks, then Y_b^T = V_b^T T_b, then slices
   gram_df_kernel<<<dim3((kBtBlockTc / 32) * (kBtBlockTc / 32), nblk), 256, 0, s>>>(n, nref, w.Vst, w.Gm);
   count_launch();
-  tfactor_all_kernel<<<nblk, kBtBlockTc, kBtBlockTc * kBtBlockTc * sizeof(double), s>>>(nref, kBtBlockTc, w.tau,
-                                                                                      w.Gm, w.Tm);
+  tfactor_all_kernel<<<dim3(kBtBlockTc / kTfRows, nblk), 4 * kTfRows, kTfSmem, s>>>(nref, w.tau, w.Gm, w.Tm);
   count_launch();
   y_df_kernel<<<dim3((n + kYRows - 1) / kYRows, nblk), 256, kYSmem, s>>>(n, nref, w.Vst, w.Tm, sc.yt);
   count_launch();
@@ -912,7 +949,7 @@ static int eig_backtransform_tc64(cudaStream_t s, int n, double* Q, EigWork& w, 
   tc64_cut_cols(s, Vt, nref, w.Vst, n);
   if (tc64_gemm(s, nref, nref, 0, n, V, 0, V, 0, 0, 1.0, 0, w.Gm, KB, 1, KB, tw.err)) return -1;
   cudaMemsetAsync(w.Tm, 0, (size_t)nblk * KB * KB * sizeof(double), s);     // columns beyond a short last block
-  tfactor_all_kernel<<<nblk, KB, KB * KB * sizeof(double), s>>>(nref, KB, w.tau, w.Gm, w.Tm);
+  tfactor_all_kernel<<<dim3(KB / kTfRows, nblk), 4 * kTfRows, kTfSmem, s>>>(nref, w.tau, w.Gm, w.Tm);
   count_launch();
   tc64_cut_rows(s, sc.t, 0, KB, w.Tm, KB);
   for (int b = nblk - 1; b >= 0; --b) {
