@@ -202,6 +202,26 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// sums over the warp of N = 2 ... 32 values at once: lane l gets the total of
+// value l / (32 / N), N - 1 + log2(32 / N) additions instead of 5 N (each in the order of
+// warp_sum, so with its bits)
+template <int N>
+__device__ __forceinline__ double warp_totals(double (&v)[N], int lane) {
+#pragma unroll
+  for (int half = N / 2, o = 16; half > 0; half >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int u = 0; u < half; ++u) {
+      const double keep = up ? v[u + half] : v[u], send = up ? v[u] : v[u + half];
+      v[u] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  double t = v[0];
+#pragma unroll
+  for (int o = 16 / N; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
 // Block-wide sum in a fixed order (deterministic); every thread gets the total.
 // `scratch` holds >= 32 doubles of shared memory.
 __device__ __forceinline__ double block_sum(double v, double* scratch) {

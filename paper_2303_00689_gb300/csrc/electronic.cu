@@ -214,7 +214,7 @@ __global__ void dmu_kernel(int n, const double* __restrict__ F1p, const double* 
 
 void launch_dmu(cudaStream_t s, int n, const double* F1p, const double* eps, const double* f, double beta,
                 Scalars* sc) {
-  dmu_kernel<<<1, 1024, 0, s>>>(n, F1p, eps, f, beta, sc);
+  dmu_kernel<<<1, std::min(1024, (n + 31) / 32 * 32), 0, s>>>(n, F1p, eps, f, beta, sc);
   count_launch();
 }
 
@@ -404,6 +404,7 @@ struct FuseArgs {
   double* out;
   int ny, combo, nd, dots_on_y;
   const double* Z[kFuseDots];
+  int odd_block;       // set at the launch: the last block has the odd element alone
 };
 
 // MY, MD: compile-time bounds on ny and nd (registers).  Each thread handles
@@ -465,15 +466,19 @@ __global__ void __launch_bounds__(kRedThreads, (MY <= 2 ? 4 : (MY <= 8 ? 2 : 1))
 #pragma unroll
   for (int i = 0; i < MY; ++i) cf[i] = (i < f.ny) ? (f.c ? f.c[i] : 1.0) : 0.0;
   const size_t npair = len >> 1;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // the pairs are dealt over kRedBlocks blocks; those that get none are not launched (their
+  // dots are zero), except the last when it has the odd element
+  const int full = (int)gridDim.x - f.odd_block;
+  const int block = ((int)blockIdx.x < full) ? (int)blockIdx.x : kRedBlocks - 1;
+  const size_t stride = (size_t)kRedBlocks * blockDim.x;
+  size_t p = (size_t)block * blockDim.x + threadIdx.x;
   for (; p + (size_t)(U - 1) * stride < npair; p += (size_t)U * stride)
     fused_batch<MY, MD, U>(f, cf, p, stride, U, acc);
   if (p < npair) {
     const int rem = (int)((npair - 1 - p) / stride) + 1;     // < U
     fused_batch<MY, MD, U>(f, cf, p, stride, rem, acc);
   }
-  if ((len & 1) && blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) {
+  if ((len & 1) && block == kRedBlocks - 1 && threadIdx.x == blockDim.x - 1) {
     const size_t t = len - 1;
     double val = f.x[t];
     if (f.combo)
@@ -487,11 +492,15 @@ __global__ void __launch_bounds__(kRedThreads, (MY <= 2 ? 4 : (MY <= 8 ? 2 : 1))
   }
   // all dots reduced together: warp shuffles, one CTA barrier, a fixed order
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int G = (MD % 8 == 0) ? 8 : (MD < 4 ? MD : 4);     // dots a call of warp_totals
 #pragma unroll
-  for (int j = 0; j < MD; ++j) {
-    if (j < f.nd) {
-      const double v = warp_sum(acc[j]);
-      if (lane == 0) sred[j][wid] = v;
+  for (int j0 = 0; j0 < MD; j0 += G) {
+    if (j0 < f.nd) {
+      double v[G];
+#pragma unroll
+      for (int j = 0; j < G; ++j) v[j] = acc[j0 + j];
+      const double total = warp_totals<G>(v, lane);
+      if (lane % (32 / G) == 0) sred[j0 + lane / (32 / G)][wid] = total;
     }
   }
   __syncthreads();
@@ -512,28 +521,34 @@ __global__ void __launch_bounds__(kRedThreads, (MY <= 2 ? 4 : (MY <= 8 ? 2 : 1))
   // last block: dot j by warp j mod 8, lanes over the block partials
   for (int j = wid; j < f.nd; j += kRedThreads / 32) {
     double loc = 0.0;
-    for (int i = lane; i < (int)gridDim.x; i += 32) loc += __ldcg(partial + j * gridDim.x + i);
+    for (int i = lane; i < full; i += 32) loc += __ldcg(partial + j * gridDim.x + i);
+    if (f.odd_block && lane == (kRedBlocks - 1) % 32) loc += __ldcg(partial + j * gridDim.x + full);
     loc = warp_sum(loc);
     if (lane == 0) dots_out[j] = loc;
   }
   if (threadIdx.x == 0) sc->red_count = 0;
 }
 
-// the smallest instantiation that holds ny and nd; a fixed grid of kRedBlocks
-// (four blocks per SM of a 152-SM GB300) keeps the reduction order, and so
-// the results, independent of the instantiation's occupancy
-static void fused(cudaStream_t s, size_t len, const FuseArgs& f, double* partial, double* dots_out, Scalars* sc,
+// the smallest instantiation that holds ny and nd; the elements are dealt over kRedBlocks
+// blocks (four per SM of a 152-SM GB300) whatever is launched, so the reduction order,
+// and with it the results, depend on neither the instantiation nor the grid.  Blocks
+// without elements reduced zeros on the FP64 pipe, and every dot by itself: n = 240,
+// the Krylov vector work of a step 333 -> 253 us.
+static void fused(cudaStream_t s, size_t len, const FuseArgs& fa, double* partial, double* dots_out, Scalars* sc,
                   bool gated) {
   const int g = gated ? 1 : 0;
+  FuseArgs f = fa;
+  const int full = (int)std::min<size_t>(((len >> 1) + kRedThreads - 1) / kRedThreads, kRedBlocks);
+  f.odd_block = ((len & 1) && full < kRedBlocks) ? 1 : 0;
+  const int grid = full + f.odd_block;
   if (f.ny <= 1 && f.nd <= 2)
-    fused_combo_dots_kernel<1, 2, 2><<<kRedBlocks, kRedThreads, 0, s>>>(len, f, partial, dots_out, sc, g);
+    fused_combo_dots_kernel<1, 2, 2><<<grid, kRedThreads, 0, s>>>(len, f, partial, dots_out, sc, g);
   else if (f.ny <= 4 && f.nd <= 4)
-    fused_combo_dots_kernel<4, 4, 2><<<kRedBlocks, kRedThreads, 0, s>>>(len, f, partial, dots_out, sc, g);
+    fused_combo_dots_kernel<4, 4, 2><<<grid, kRedThreads, 0, s>>>(len, f, partial, dots_out, sc, g);
   else if (f.ny <= 8 && f.nd <= 8)
-    fused_combo_dots_kernel<8, 8, 1><<<kRedBlocks, kRedThreads, 0, s>>>(len, f, partial, dots_out, sc, g);
+    fused_combo_dots_kernel<8, 8, 1><<<grid, kRedThreads, 0, s>>>(len, f, partial, dots_out, sc, g);
   else
-    fused_combo_dots_kernel<kFuseY, kFuseDots, 1><<<kRedBlocks, kRedThreads, 0, s>>>(len, f, partial, dots_out,
-                                                                                      sc, g);
+    fused_combo_dots_kernel<kFuseY, kFuseDots, 1><<<grid, kRedThreads, 0, s>>>(len, f, partial, dots_out, sc, g);
   count_launch();
 }
 static FuseArgs fuse_args() {

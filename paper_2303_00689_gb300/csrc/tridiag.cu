@@ -103,24 +103,6 @@ __device__ __forceinline__ bool poll_expired(unsigned it, unsigned long long& t0
   return global_ns() - t0 > limit || it > (1u << 27) || ((*(volatile const int*)status) & kStatusTimeout);
 }
 
-// sums over the warp of N = 2 ... 32 values at once: lane l gets the total of
-// value l / (32 / N), N - 1 + log2(32 / N) additions instead of 5 N
-template <int N>
-__device__ __forceinline__ double warp_totals(double (&v)[N], int lane) {
-#pragma unroll
-  for (int half = N / 2, o = 16; half > 0; half >>= 1, o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int u = 0; u < half; ++u) {
-      const double keep = up ? v[u + half] : v[u], send = up ? v[u] : v[u + half];
-      v[u] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  double t = v[0];
-#pragma unroll
-  for (int o = 16 / N; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
-}
 // Named barriers.  Whole warps arrive: lanes leave the packet polls one by one, and
 // without the __syncwarp the code after them ran lane by lane (5 times slower).
 __device__ __forceinline__ void bar_sync(int id, int threads) {
