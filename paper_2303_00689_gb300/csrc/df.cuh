@@ -94,6 +94,23 @@ __device__ __forceinline__ dfl df_from_double_bits(double x) {
   const float s = __fadd_rn(hi, lo);
   return dfl{s, __fsub_rn(lo, __fsub_rn(s, hi))};
 }
+// df_from_double (the same bits) without FP64 instructions: x = q 2^k + r 2^(k - 29) with
+// q of 24 bits, q rounded to nearest even as the conversion does, what is left signed.
+// Exponents for which a scale would leave the normal FP32 range take the plain form.
+__device__ __forceinline__ dfl df_from_double_exact(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned hw = (unsigned)(b >> 32), lw = (unsigned)b;
+  const int ex = (int)((hw >> 20) & 0x7FFu);
+  if (b << 1 == 0) return dfl{__uint_as_float(hw), 0.0f};
+  if (ex < 960 || ex > 1140) return df_from_double(x);
+  unsigned q = ((hw & 0xFFFFFu) | 0x100000u) << 3 | lw >> 29;
+  const unsigned r = lw & 0x1FFFFFFFu;
+  const unsigned up = (r > 0x10000000u || (r == 0x10000000u && (q & 1u))) ? 1u : 0u;
+  const float hi = __fmul_rn(__uint2float_rn(q + up), __uint_as_float((unsigned)(ex - 1075 + 29 + 127) << 23));
+  const float lo = __fmul_rn(__int2float_rn((int)(r - (up << 29))), __uint_as_float((unsigned)(ex - 1075 + 127) << 23));
+  const unsigned sign = hw & 0x80000000u;
+  return dfl{__uint_as_float(__float_as_uint(hi) ^ sign), lo == 0.0f ? 0.0f : __uint_as_float(__float_as_uint(lo) ^ sign)};
+}
 // hi + lo as a double with one FP64 addition (the two conversions by integer operations)
 __device__ __forceinline__ double df_to_double_fast(dfl a) { return f2d_int(a.hi) + f2d_int(a.lo); }
 __host__ __device__ __forceinline__ dfl df_neg(dfl a) { return dfl{-a.hi, -a.lo}; }

@@ -767,8 +767,8 @@ __global__ void __launch_bounds__(256) gram_df_kernel(int n, int nref, const dou
       const int r = e / CH, c = e % CH;
       const int l = l0 + c;
       const int ra = ti * TL + r, rb = tj * TL + r;
-      sa[r][c] = (ra < kb && l < m) ? df_from_double(Vst[(size_t)(k0 + ra) * n + c0 + l]) : dfl{0.0f, 0.0f};
-      sb[r][c] = (rb < kb && l < m) ? df_from_double(Vst[(size_t)(k0 + rb) * n + c0 + l]) : dfl{0.0f, 0.0f};
+      sa[r][c] = (ra < kb && l < m) ? df_from_double_exact(Vst[(size_t)(k0 + ra) * n + c0 + l]) : dfl{0.0f, 0.0f};
+      sb[r][c] = (rb < kb && l < m) ? df_from_double_exact(Vst[(size_t)(k0 + rb) * n + c0 + l]) : dfl{0.0f, 0.0f};
     }
     __syncthreads();
 #pragma unroll 4
@@ -788,46 +788,48 @@ __global__ void __launch_bounds__(256) gram_df_kernel(int n, int nref, const dou
 }
 
 // Y_b^T = V_b^T T_b (m_b x kb, row length KB) for every block b; T_b upper
-// triangular (kb x kb, ld KB); 64 rows of Y_b^T per CTA, T_b and the V_b
-// columns in shared memory as double-float
-constexpr int kYRows = 64;
-constexpr size_t kYSmem = (size_t)(kBtBlockTc * kBtBlockTc + kBtBlockTc * kYRows) * sizeof(dfl);
+// triangular (kb x kb, ld KB); ROWS rows of Y_b^T per CTA, T_b and the V_b
+// columns in shared memory as double-float.  64 rows read T_b least often; 16 where
+// that would leave SMs idle (n = 240: 8 CTAs, 167 us).
+constexpr size_t y_smem(int rows) { return (size_t)(kBtBlockTc * kBtBlockTc + kBtBlockTc * rows) * sizeof(dfl); }
+template <int ROWS>
 __global__ void __launch_bounds__(256) y_df_kernel(int n, int nref, const double* __restrict__ Vst,
                                                    const double* __restrict__ Tall, double* __restrict__ YT) {
   constexpr int KB = kBtBlockTc;
   extern __shared__ dfl ysm[];
   dfl* sT = ysm;                   // KB x KB
-  dfl* sV = ysm + KB * KB;         // KB (reflector) x kYRows (column)
+  dfl* sV = ysm + KB * KB;         // KB (reflector) x ROWS (column)
   const int b = blockIdx.y;
   const int k0 = b * KB, kb = min(KB, nref - k0), c0 = k0 + 1, m = n - c0;
-  const int l0 = blockIdx.x * kYRows;
+  const int l0 = blockIdx.x * ROWS;
   if (l0 >= m) return;
   const double* Tb = Tall + (size_t)b * KB * KB;
   for (int e = threadIdx.x; e < KB * KB; e += blockDim.x) {
     const int i = e / KB, j = e % KB;
-    sT[e] = (i < kb && j < kb && i <= j) ? df_from_double(Tb[(size_t)i * KB + j]) : dfl{0.0f, 0.0f};
+    sT[e] = (i < kb && j < kb && i <= j) ? df_from_double_exact(Tb[(size_t)i * KB + j]) : dfl{0.0f, 0.0f};
   }
-  for (int e = threadIdx.x; e < KB * kYRows; e += blockDim.x) {
-    const int i = e / kYRows, c = e % kYRows;
+  for (int e = threadIdx.x; e < KB * ROWS; e += blockDim.x) {
+    const int i = e / ROWS, c = e % ROWS;
     const int l = l0 + c;
-    sV[e] = (i < kb && l < m) ? df_from_double(Vst[(size_t)(k0 + i) * n + c0 + l]) : dfl{0.0f, 0.0f};
+    sV[e] = (i < kb && l < m) ? df_from_double_exact(Vst[(size_t)(k0 + i) * n + c0 + l]) : dfl{0.0f, 0.0f};
   }
   __syncthreads();
-  // thread t: row c = t / 4 of the tile, columns j = (t % 4) * 32 .. + 31
-  const int c = threadIdx.x >> 2, jb = (threadIdx.x & 3) * 32;
-  dfl acc[32];
+  // thread t: row c of the tile, COLS consecutive columns
+  constexpr int COLS = KB * ROWS / 256;
+  const int c = threadIdx.x / (KB / COLS), jb = threadIdx.x % (KB / COLS) * COLS;
+  dfl acc[COLS];
 #pragma unroll
-  for (int q = 0; q < 32; ++q) acc[q] = dfl{0.0f, 0.0f};
+  for (int q = 0; q < COLS; ++q) acc[q] = dfl{0.0f, 0.0f};
   for (int i = 0; i < kb; ++i) {
-    const dfl v = sV[i * kYRows + c];
+    const dfl v = sV[i * ROWS + c];
 #pragma unroll
-    for (int q = 0; q < 32; ++q) df_acc_mul(acc[q], v, sT[i * KB + jb + q]);
+    for (int q = 0; q < COLS; ++q) df_acc_mul(acc[q], v, sT[i * KB + jb + q]);
   }
   const int l = l0 + c;
   if (l < m) {
     double* out = YT + (size_t)b * n * KB + (size_t)l * KB;
 #pragma unroll
-    for (int q = 0; q < 32; ++q) out[jb + q] = (jb + q < kb) ? df_to_double_fast(df_norm(acc[q])) : 0.0;
+    for (int q = 0; q < COLS; ++q) out[jb + q] = (jb + q < kb) ? df_to_double_fast(df_norm(acc[q])) : 0.0;
   }
 }
 
@@ -868,7 +870,9 @@ static void bt_attributes() {
                                 kBtBlockTc * kBtBlockTc * (int)sizeof(double)) == cudaSuccess &&
            cudaFuncSetAttribute(tfactor_all_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTfSmem) ==
                cudaSuccess &&
-           cudaFuncSetAttribute(y_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kYSmem) ==
+           cudaFuncSetAttribute(y_df_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)y_smem(64)) ==
+               cudaSuccess &&
+           cudaFuncSetAttribute(y_df_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)y_smem(16)) ==
                cudaSuccess;
   });
 }
@@ -888,7 +892,10 @@ static int eig_backtransform_tc(cudaStream_t s, int n, double* Q, EigWork& w, co
   count_launch();
   tfactor_all_kernel<<<dim3(kBtBlockTc / kTfRows, nblk), 4 * kTfRows, kTfSmem, s>>>(nref, w.tau, w.Gm, w.Tm);
   count_launch();
-  y_df_kernel<<<dim3((n + kYRows - 1) / kYRows, nblk), 256, kYSmem, s>>>(n, nref, w.Vst, w.Tm, sc.yt);
+  if ((n + 63) / 64 * nblk >= 152)
+    y_df_kernel<64><<<dim3((n + 63) / 64, nblk), 256, y_smem(64), s>>>(n, nref, w.Vst, w.Tm, sc.yt);
+  else
+    y_df_kernel<16><<<dim3((n + 15) / 16, nblk), 256, y_smem(16), s>>>(n, nref, w.Vst, w.Tm, sc.yt);
   count_launch();
   tc_split_blocks(s, 0, n, nref, kBtBlockTc, w.Vst, sc.vs, sc.vs_blk, sc.vs_slice, 4);
   tc_split_blocks(s, 1, n, nref, kBtBlockTc, sc.yt, sc.ys, sc.ys_blk, sc.ys_slice, 4);

@@ -39,6 +39,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "df.cuh"
 #include "kernels.h"
 #include "tc_gemm.h"
 #include "tc_ptx.cuh"
@@ -71,6 +72,15 @@ __device__ __forceinline__ void twosum_acc(float& hi, float& lo, float b) {
   float err = (hi - (s - bb)) + (b - bb);
   hi = s;
   lo += err;
+}
+
+// alpha (hi + lo) in FP64 with one instruction on the FP64 pipe, two unless alpha = +-1:
+// GB300 takes 62 cycles for each, and the conversions, the sum and the product of a
+// 128 x 128 tile were 17 us of it (n = 240, 3 and 4 slices: 31 and 37 us -> 26 and 32).
+// Not in tc_gemm_kernel, which writes straight from registers and was slower with it.
+__device__ __forceinline__ double scaled_sum(double alpha, float hi, float lo) {
+  const double v = df_to_double_fast(dfl{hi, lo});
+  return alpha == 1.0 ? v : (alpha == -1.0 ? -v : alpha * v);
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -425,7 +435,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (ok) {
       const int rl = quarter * 32 + lane;
 #pragma unroll
-      for (int j = 0; j < 32; ++j) tile[rl * kLdT + cg * 32 + j] = alpha * ((double)hi[j] + (double)lo[j]);
+      for (int j = 0; j < 32; ++j) tile[rl * kLdT + cg * 32 + j] = scaled_sum(alpha, hi[j], lo[j]);
     }
     asm volatile("bar.sync 1, %0;" ::"r"(kEpiWarps * 32) : "memory");
     if (ktiles > 0 && *(volatile int*)err == 0) {
