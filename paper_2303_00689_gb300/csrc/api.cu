@@ -233,6 +233,14 @@ static double* xslot(sim_handle* h, int k) { return h->X[(h->xhead + k) % 8]; }
 
 static bool mixed(const sim_handle* h) { return h->cfg.precision == SIM_PREC_MIXED; }
 
+// Where FP64 products run.  The DMPT's: on the tensor cores above the size where cutting
+// and multiplying an operand (tc_gemm64.cu; 19 us at least) beats n^3 FMAs on the FP64 pipe
+// (gemm64.cu): n = 26, 131, 240, 288, 574: 21, 37, 45, 51, 82 us and 6, 13, 37, 62, 344 us.
+// The back-transformation: on the FP64 pipe while one block of reflectors is all there
+// is (n = 26, 59, 131, 240: 59, 169, 410, 756 us and 128, 181, 397, 460 us).
+constexpr int kTc64Above = 256, kBt64Above = 66;
+static bool dmpt64(const sim_handle* h) { return h->t64.base && h->n > kTc64Above; }
+
 // C = A B^T of cut n x n operands (the size's tensor map was encoded at creation)
 static void tc64_mul(sim_handle* h, const Tc64Op& A, const Tc64Op& B, double* C, int sym, const int* gate = nullptr) {
   const int n = h->n;
@@ -261,7 +269,7 @@ static void density(sim_handle* h) {
 
 // slices of Q and Q^T for the DMPT products (once per evaluation)
 static void dmpt_prepare(sim_handle* h) {
-  if (h->t64.base) {
+  if (dmpt64(h)) {
     const int n = h->n;
     tc64_cut_rows(h->stream, tc64_slot(h->t64, 0, n, n), 0, n, h->Q, n);
     tc64_cut_cols(h->stream, tc64_slot(h->t64, 1, n, n), n, h->Q, n);
@@ -293,7 +301,7 @@ static void dmpt(sim_handle* h, const double* F1, double* D1) {
     tc_gemm_grouped(s, h->tw, kSlotT1, kSlotQ, 1.0, D1, 1, g);          // D1 = (Q Y) Q^T
     return;
   }
-  if (h->t64.base) {
+  if (dmpt64(h)) {
     const Tc64Op q = tc64_slot(h->t64, 0, n, n), qt = tc64_slot(h->t64, 1, n, n), x = tc64_slot(h->t64, 2, n, n);
     tc64_cut_rows(s, x, 0, n, F1, n, g);
     tc64_mul(h, qt, x, h->T1, 0, g);                     // T1 = Q^T F1
@@ -344,11 +352,11 @@ static int eig(sim_handle* h, bool fermi_side = false) {
     launch_fermi(h->side, h->n, h->eps, (double)h->nocc, h->beta, h->f, h->sc);
   }
   phase_begin(h, PH_TRIEIG);
-  eig_vectors(h->stream, h->n, h->eps, h->Q, h->ew, mixed(h));
+  eig_vectors(h->stream, h->n, h->eps, h->Q, h->ew, mixed(h), h->shared);
   phase_end(h);
   phase_begin(h, PH_BACKTR);
   const int bt = eig_backtransform(h->stream, h->n, h->Q, h->ew, mixed(h) ? &h->tw : nullptr,
-                                   h->t64.base ? &h->t64 : nullptr);
+                                   h->t64.base && h->n > kBt64Above ? &h->t64 : nullptr);
   phase_end(h);
   if (bt != 0) return fail(SIM_EINTERNAL, "back-transformation: tensor map encoding failed");
   return SIM_OK;
