@@ -411,7 +411,7 @@ static int evaluate(sim_handle* h, bool krylov = true, bool pairs_ready = false)
   if (!pairs_ready) {
     phase_begin(h, PH_PAIRS);
     launch_pair_derivs(s, h->npair, h->pA, h->pB, h->elem, h->R, h->tab, h->W, h->S, h->E, h->dW, h->dS,
-                       h->dE, mixed(h));
+                       h->dE, mixed(h), h->shared);
     phase_end(h);
   }
   phase_begin(h, PH_FOCK);
@@ -516,7 +516,7 @@ static int bomd_step(sim_handle* h) {
   phase_end(h);
   phase_begin(h, PH_PAIRS);
   launch_pair_derivs(s, h->npair, h->pA, h->pB, h->elem, h->R, h->tab, h->W, h->S, h->E, h->dW, h->dS, h->dE,
-                     mixed(h));
+                     mixed(h), h->shared);
   launch_build_h(s, mol(h), pairs(h), h->tab, h->h);
   phase_end(h);
   int it = 0;
@@ -960,7 +960,7 @@ static int create_handle(const sim_config* cfg, const sim_param_table* table, in
     launch_fill(s, (size_t)h->n * h->n, h->K, 0.0);
     // pair blocks and h at R0
     launch_pair_derivs(s, h->npair, h->pA, h->pB, h->elem, h->R, h->tab, h->W, h->S, h->E, h->dW, h->dS, h->dE,
-                     mixed(h));
+                     mixed(h), h->shared);
     launch_build_h(s, mol(h), pairs(h), h->tab, h->h);
     size_t nn = (size_t)h->n * h->n;
     if (P0) {

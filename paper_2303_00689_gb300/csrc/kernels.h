@@ -21,7 +21,7 @@ void launch_pair_values(cudaStream_t s, int npair, const int* pA, const int* pB,
 // double-float on the FP32 pipe (mixed path) instead of FP64
 void launch_pair_derivs(cudaStream_t s, int npair, const int* pA, const int* pB, const int* elem,
                         const double* R, const ElemTable& tab, double* W, double* S, double* E,
-                        double* dW, double* dS, double* dE, bool df_rotation);
+                        double* dW, double* dS, double* dE, bool df_rotation, bool shared);
 
 // ---- fock.cu ----------------------------------------------------------------
 struct MolDev {          // read-only molecule description on the device

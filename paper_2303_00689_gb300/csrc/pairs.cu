@@ -351,7 +351,7 @@ __device__ __forceinline__ int grp_hi(int g) { return g == 0 ? 1 : (g == 1 ? 4 :
 // C is kept block by block (at most 6 products per row) and X one product
 // group at a time, which keeps the per-thread arrays small.
 __device__ void rotate_blocks_df(const G1 (&Ir)[10][10], const D3 (&Tf)[4][4], const double* uv, int pa, int pb,
-                                 double* __restrict__ W, double* __restrict__ dW, size_t np, int t) {
+                                 int q0, int q1, double* __restrict__ W, double* __restrict__ dW, size_t np, int t) {
   G3 Tg[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
@@ -381,7 +381,7 @@ __device__ void rotate_blocks_df(const G1 (&Ir)[10][10], const D3 (&Tf)[4][4], c
     const int lo = grp_lo(g), hi = grp_hi(g);
     G3 Xg[6][10];                       // X[pp][q] for pp in group g
     for (int pp = lo; pp < hi; ++pp)
-      for (int q = 0; q < pb; ++q) {
+      for (int q = q0; q < min(q1, pb); ++q) {
         G3 acc = g3_zero();
         dfl sd = {0.0f, 0.0f};
         const int gq = grp_of(q), qlo = grp_lo(gq);
@@ -401,7 +401,7 @@ __device__ void rotate_blocks_df(const G1 (&Ir)[10][10], const D3 (&Tf)[4][4], c
         Xg[pp - lo][q] = x;
       }
     for (int p = lo; p < hi; ++p)
-      for (int q = 0; q < 10; ++q) {
+      for (int q = q0; q < q1; ++q) {
         G3 acc = g3_zero();
         if (q < pb)
           for (int pp = lo; pp < hi; ++pp) g3_acc_mul(acc, Cb[p][pp - lo], Xg[pp - lo][q]);
@@ -415,7 +415,7 @@ __device__ void rotate_blocks_df(const G1 (&Ir)[10][10], const D3 (&Tf)[4][4], c
   }
   // products the partner's group structure leaves out (hydrogen on A: p >= 1)
   for (int p = (ngrp == 1 ? 1 : 10); p < 10; ++p)
-    for (int q = 0; q < 10; ++q) {
+    for (int q = q0; q < q1; ++q) {
       const size_t ix = (size_t)(p * 10 + q) * np + t;
       W[ix] = 0.0;
       dW[ix] = 0.0;
@@ -424,10 +424,32 @@ __device__ void rotate_blocks_df(const G1 (&Ir)[10][10], const D3 (&Tf)[4][4], c
     }
 }
 
+// What one thread does of a pair: columns [q0, q1) of W, the overlaps with an s orbital,
+// the p-p overlaps, the core repulsion.  All of it where pairs fill the device; with
+// fewer pairs than FP64 pipes (a warp each) a pair is shared by kPairParts threads of
+// different warps, since one thread's chain of FP64 operations is then the kernel's
+// time (kPairShareMax).
+struct PairPart {
+  int q0, q1;
+  bool s_sp, s_pp, core;
+};
+constexpr int kPairParts = 6;
+__device__ __forceinline__ PairPart pair_part(int part) {
+  switch (part) {
+    case 0: return PairPart{0, 4, false, false, false};
+    case 1: return PairPart{4, 7, false, false, false};
+    case 2: return PairPart{7, 10, false, false, false};
+    case 3: return PairPart{0, 0, true, false, false};
+    case 4: return PairPart{0, 0, false, true, false};
+    case 5: return PairPart{0, 0, false, false, true};
+    default: return PairPart{0, 10, true, true, true};
+  }
+}
+
 // DFROT (dual numbers only): W and dW go straight to Wg / dWg (column t of
 // stride np) and Wout is not used
 template <bool DFROT, typename T>
-__device__ void pair_block(const double* dvec, const Elem& ea, const Elem& eb, T* Wout /*100*/,
+__device__ void pair_block(const PairPart& part, const double* dvec, const Elem& ea, const Elem& eb, T* Wout /*100*/,
                            T* Sout /*16*/, T* Eout, double* Wg = nullptr, double* dWg = nullptr, size_t np = 0,
                            int t = 0) {
   typedef typename Radial<T>::type Tr;
@@ -438,6 +460,7 @@ __device__ void pair_block(const double* dvec, const Elem& ea, const Elem& eb, T
   T u[3] = {d[0] * iR, d[1] * iR, d[2] * iR};
   const double uv[3] = {val(u[0]), val(u[1]), val(u[2])};
   const Tr Rr = Radial<T>::seed(val(R));
+  if (part.q0 < part.q1) {
   // reference axis least aligned with u
   int ref = 0;
   double best = fabs(val(u[0]));
@@ -463,6 +486,8 @@ __device__ void pair_block(const double* dvec, const Elem& ea, const Elem& eb, T
 
   const int pa = (ea.norb == 4) ? 10 : 1;
   const int pb = (eb.norb == 4) ? 10 : 1;
+  // the columns of W's product groups
+  const int c0 = c_grp_lo[part.q0], c1 = min((int)c_grp_hi[part.q1 - 1], pb);
 
   // local integrals: the distinct ones (rows ss, sz, xx, zz of the sigma/
   // delta class, sx and xz of the pi class) from the charge sets, the rest by
@@ -476,35 +501,35 @@ __device__ void pair_block(const double* dvec, const Elem& ea, const Elem& eb, T
       for (int q = 0; q < 10; ++q) Ig[p][q] = g1_zero();
     for (int p = 0; p < pa; ++p) {
       if (p == 2 || p == 5 || p == 7 || p == 9) continue;        // mirrored or derived below
-      for (int q = 0; q < pb; ++q) {
+      for (int q = c0; q < c1; ++q) {
         if (c_prod_cls[p] != c_prod_cls[q]) continue;
         if (c_prod_cls[p] == 1 && (q == 2 || q == 9)) continue;
         Ig[p][q] = local_integral_df(p, q, ca, cb, Rd, e2);
       }
     }
     if (pa == 10) {
-      for (int q = 0; q < pb; ++q) {
+      for (int q = c0; q < c1; ++q) {
         const int mq = mirror_xy(q);
         if (c_prod_cls[q] == 0) Ig[5][q] = Ig[4][mq];
         if (c_prod_cls[q] == 2) { Ig[2][q] = Ig[1][mq]; Ig[9][q] = Ig[8][mq]; }
       }
       if (pb == 10) Ig[7][7] = g1_half(g1_sub(Ig[4][4], Ig[4][5]));
     }
-    rotate_blocks_df(Ig, Tf, uv, pa, pb, Wg, dWg, np, t);
+    rotate_blocks_df(Ig, Tf, uv, pa, pb, part.q0, part.q1, Wg, dWg, np, t);
   } else {
   Tr Ir[10][10];
   for (int p = 0; p < 10; ++p)
     for (int q = 0; q < 10; ++q) Ir[p][q] = cst<Tr>(0.0);
   for (int p = 0; p < pa; ++p) {
     if (p == 2 || p == 5 || p == 7 || p == 9) continue;        // mirrored or derived below
-    for (int q = 0; q < pb; ++q) {
+    for (int q = c0; q < c1; ++q) {
       if (c_prod_cls[p] != c_prod_cls[q]) continue;
       if (c_prod_cls[p] == 1 && (q == 2 || q == 9)) continue;
       Ir[p][q] = local_integral<Tr>(p, q, ea, eb, Rr);
     }
   }
   if (pa == 10) {
-    for (int q = 0; q < pb; ++q) {
+    for (int q = c0; q < c1; ++q) {
       const int mq = mirror_xy(q);
       if (c_prod_cls[q] == 0) Ir[5][q] = Ir[4][mq];
       if (c_prod_cls[q] == 2) { Ir[2][q] = Ir[1][mq]; Ir[9][q] = Ir[8][mq]; }
@@ -531,19 +556,20 @@ __device__ void pair_block(const double* dvec, const Elem& ea, const Elem& eb, T
   // X[p'][q] = sum_{q'} I[p'][q'] C[q][q'];  W[p][q] = sum_{p'} C[p][p'] X[p'][q]
   T X[10][10];
   for (int pp = 0; pp < pa; ++pp)
-    for (int q = 0; q < pb; ++q) {
+    for (int q = part.q0; q < min(part.q1, pb); ++q) {
       T acc = cst<T>(0.0);
       for (int qq = c_grp_lo[q]; qq < c_grp_hi[q]; ++qq)
         if (c_prod_cls[qq] == c_prod_cls[pp]) acc += I[pp][qq] * C[q][qq];   // other classes: I = 0
       X[pp][q] = acc;
     }
   for (int p = 0; p < 10; ++p)
-    for (int q = 0; q < 10; ++q) {
+    for (int q = part.q0; q < part.q1; ++q) {
       T acc = cst<T>(0.0);
       if (p < pa && q < pb)
         for (int pp = c_grp_lo[p]; pp < c_grp_hi[p]; ++pp) acc += C[p][pp] * X[pp][q];
       Wout[p * 10 + q] = acc;
     }
+  }
   }
 
   // overlaps in the local frame (functions of R), then in the molecular frame.
@@ -554,19 +580,19 @@ __device__ void pair_block(const double* dvec, const Elem& ea, const Elem& eb, T
   // the molecular-frame overlaps depend on u alone (no x', y').
   const T zero = cst<T>(0.0);
   for (int k = 0; k < 16; ++k) Sout[k] = zero;
-  Sout[0] = Radial<T>::promote(
+  if (part.s_sp) Sout[0] = Radial<T>::promote(
       sto_overlap<Tr>(Rr, ea.nprin, ea.zeta[0], ea.sto_nrm[0], 0, eb.nprin, eb.zeta[0], eb.sto_nrm[0], 0), uv);
-  if (ea.norb == 4) {
+  if (part.s_sp && ea.norb == 4) {
     const T szs = Radial<T>::promote(
         sto_overlap<Tr>(Rr, ea.nprin, ea.zeta[1], ea.sto_nrm[1], 1, eb.nprin, eb.zeta[0], eb.sto_nrm[0], 0), uv);
     for (int a = 1; a < 4; ++a) Sout[a * 4] = szs * u[a - 1];
   }
-  if (eb.norb == 4) {
+  if (part.s_sp && eb.norb == 4) {
     const T ssz = Radial<T>::promote(
         sto_overlap<Tr>(Rr, ea.nprin, ea.zeta[0], ea.sto_nrm[0], 0, eb.nprin, eb.zeta[1], eb.sto_nrm[1], 1), uv);
     for (int b = 1; b < 4; ++b) Sout[b] = ssz * u[b - 1];
   }
-  if (ea.norb == 4 && eb.norb == 4) {
+  if (part.s_pp && ea.norb == 4 && eb.norb == 4) {
     const T szz = Radial<T>::promote(
         sto_overlap<Tr>(Rr, ea.nprin, ea.zeta[1], ea.sto_nrm[1], 1, eb.nprin, eb.zeta[1], eb.sto_nrm[1], 1), uv);
     const T spp = Radial<T>::promote(
@@ -579,6 +605,7 @@ __device__ void pair_block(const double* dvec, const Elem& ea, const Elem& eb, T
   }
 
   // core-core repulsion (a function of R)
+  if (!part.core) return;
   const Tr gss = local_integral<Tr>(0, 0, ea, eb, Rr);
   const double zz = ea.zcore * eb.zcore;
   Tr en = zz * gss * (1.0 + ex(-ea.alpha * Rr) + ex(-eb.alpha * Rr));
@@ -602,13 +629,13 @@ __global__ void pair_values_kernel(int npair, const int* __restrict__ pA, const 
   const Elem& ea = tab.e[elem[A]];
   const Elem& eb = tab.e[elem[B]];
   double w[100], s[16], e;
-  pair_block<false, double>(d, ea, eb, w, s, &e);
+  pair_block<false, double>(pair_part(-1), d, ea, eb, w, s, &e);
   for (int k = 0; k < 100; ++k) W[(size_t)k * npair + t] = w[k];
   for (int k = 0; k < 16; ++k) S[(size_t)k * npair + t] = s[k];
   E[t] = e;
 }
 
-template <bool DFROT>
+template <bool DFROT, bool SHARED>
 __global__ void pair_derivs_kernel(int npair, const int* __restrict__ pA, const int* __restrict__ pB,
                                    const int* __restrict__ elem, const double* __restrict__ R,
                                    ElemTable tab, double* __restrict__ W, double* __restrict__ S,
@@ -622,24 +649,29 @@ __global__ void pair_derivs_kernel(int npair, const int* __restrict__ pA, const 
   const Elem& eb = tab.e[elem[B]];
   size_t np = (size_t)npair;
   D3 s[16], e;
+  const PairPart part = pair_part(SHARED ? (int)blockIdx.y : -1);
   if constexpr (DFROT) {
-    pair_block<true, D3>(d, ea, eb, nullptr, s, &e, W, dW, np, t);
+    pair_block<true, D3>(part, d, ea, eb, nullptr, s, &e, W, dW, np, t);
   } else {
     D3 w[100];
-    pair_block<false, D3>(d, ea, eb, w, s, &e);
-    for (int k = 0; k < 100; ++k) {
-      W[k * np + t] = w[k].v;
-      dW[(0 * 100 + k) * np + t] = w[k].d0;
-      dW[(1 * 100 + k) * np + t] = w[k].d1;
-      dW[(2 * 100 + k) * np + t] = w[k].d2;
-    }
+    pair_block<false, D3>(part, d, ea, eb, w, s, &e);
+    for (int p = 0; p < 10; ++p)
+      for (int q = part.q0; q < part.q1; ++q) {
+        const int k = p * 10 + q;
+        W[k * np + t] = w[k].v;
+        dW[(0 * 100 + k) * np + t] = w[k].d0;
+        dW[(1 * 100 + k) * np + t] = w[k].d1;
+        dW[(2 * 100 + k) * np + t] = w[k].d2;
+      }
   }
   for (int k = 0; k < 16; ++k) {
+    if (!((k < 4 || k % 4 == 0) ? part.s_sp : part.s_pp)) continue;
     S[k * np + t] = s[k].v;
     dS[(0 * 16 + k) * np + t] = s[k].d0;
     dS[(1 * 16 + k) * np + t] = s[k].d1;
     dS[(2 * 16 + k) * np + t] = s[k].d2;
   }
+  if (!part.core) return;
   E[t] = e.v;
   dE[0 * np + t] = e.d0;
   dE[1 * np + t] = e.d1;
@@ -723,14 +755,24 @@ void launch_pair_values(cudaStream_t s, int npair, const int* pA, const int* pB,
   count_launch();
 }
 
+// half as many pairs as FP64 pipes (4 an SM, a warp of 32 each): mixed 1770, 7140, 16110
+// pairs 313 -> 117, 361 -> 189, 369 -> 332 us, FP64 720 -> 320, 743 -> 471, 752 -> 847 us.
+// Not beside other handles (shared), where the frames and integrals formed more than
+// once take time from them.
+constexpr int kPairShareMax = 4 * 152 * 32 / 2;
+
 void launch_pair_derivs(cudaStream_t s, int npair, const int* pA, const int* pB, const int* elem,
                         const double* R, const ElemTable& tab, double* W, double* S, double* E,
-                        double* dW, double* dS, double* dE, bool df_rotation) {
+                        double* dW, double* dS, double* dE, bool df_rotation, bool shared) {
   if (npair <= 0) return;
-  if (df_rotation)
-    pair_derivs_kernel<true><<<(npair + 127) / 128, 128, 0, s>>>(npair, pA, pB, elem, R, tab, W, S, E, dW, dS, dE);
+  auto run = [&](auto kernel, dim3 grid, int threads) {
+    kernel<<<grid, threads, 0, s>>>(npair, pA, pB, elem, R, tab, W, S, E, dW, dS, dE);
+  };
+  const dim3 whole((npair + 127) / 128), parts((npair + 31) / 32, kPairParts);
+  if (npair <= kPairShareMax && !shared)
+    df_rotation ? run(pair_derivs_kernel<true, true>, parts, 32) : run(pair_derivs_kernel<false, true>, parts, 32);
   else
-    pair_derivs_kernel<false><<<(npair + 127) / 128, 128, 0, s>>>(npair, pA, pB, elem, R, tab, W, S, E, dW, dS, dE);
+    df_rotation ? run(pair_derivs_kernel<true, false>, whole, 128) : run(pair_derivs_kernel<false, false>, whole, 128);
   count_launch();
 }
 
