@@ -345,7 +345,7 @@ static int eig(sim_handle* h, bool fermi_side = false) {
   phase_end(h);
   if (st != 0) return fail(SIM_EINTERNAL, "tridiagonalisation launch failed (code " + std::to_string(st) + ")");
   phase_begin(h, PH_BISECT);
-  eig_bisect(h->stream, h->n, h->eps, h->ew, 1e-12, mixed(h));
+  eig_bisect(h->stream, h->n, h->eps, h->ew, 1e-12, mixed(h), h->shared);
   phase_end(h);
   if (fermi_side) {
     fork_side(h, 0);

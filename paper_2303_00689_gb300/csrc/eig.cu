@@ -130,7 +130,7 @@ __device__ __forceinline__ int sturm_count_f32(int n, const float* __restrict__ 
 // tolerance.  A count is a chain of n FP64 steps on a pipe that takes ~62 cycles a warp
 // instruction however many lanes are live, so lanes that count at other points of
 // the same interval are free until there are more warps than FP64 pipes (kFp64Pipes);
-// M = 32, 16, 8 up to 1, 1 and 2 warps a pipe.  n = 26, 240, 574,
+// M = 32, 16, 8 up to 1, 1 and 2 warps a pipe, 8 beside other handles.  n = 26, 240, 574,
 // 1680: 53, 290, 670, 3020 us; 165, 1370, 3160, 9220 with one lane an eigenvalue.
 constexpr int kFp64Pipes = 4 * 152;
 template <int M>
@@ -227,11 +227,28 @@ __device__ __forceinline__ int sturm_count_df(int n, const dfl* __restrict__ d, 
   return c;
 }
 
-__global__ void bisect_df_kernel(int n, const dfl* __restrict__ d, const dfl* __restrict__ e2,
-                                 const double* __restrict__ scal, double rel_tol, double* __restrict__ ev) {
+// Interval f of [lo, hi] cut by the kMsLanes points lo + (m + 1) h
+__device__ __forceinline__ void ms_interval(double& lo, double& hi, double h, int f) {
+  const double nlo = (f == 0) ? lo : lo + (double)f * h;
+  hi = (f == kMsLanes) ? hi : lo + (double)(f + 1) * h;
+  lo = nlo;
+}
+
+// WIDE: a block of kMsWide lanes per eigenvalue takes two rounds at once, lanes 0 .. 7 the
+// first round's points and eight lanes for each of its nine intervals the second's: the
+// same points and results, half the chains of n steps, two and a half times the work: n =
+// 131, 240, 480, 720: 156 -> 107, 258 -> 185, 490 -> 405, 718 -> 729 us.
+constexpr int kMsWideMax = 512;
+constexpr int kMsWide = 96, kMsPoints = kMsLanes * (kMsLanes + 2);
+template <bool WIDE>
+__global__ void __launch_bounds__(WIDE ? kMsWide : 32) bisect_df_kernel(int n, const dfl* __restrict__ d,
+                                                                       const dfl* __restrict__ e2,
+                                                                       const double* __restrict__ scal,
+                                                                       double rel_tol, double* __restrict__ ev) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = t / kMsLanes;                 // eigenvalue of this group
-  const int m = t % kMsLanes;                 // point m + 1 of the group
+  const int i = WIDE ? (int)blockIdx.x : t / kMsLanes;                 // eigenvalue of this group
+  const int m = (WIDE ? (int)threadIdx.x : t) % kMsLanes;             // point m + 1 of the group
+  const int sub = WIDE ? (int)threadIdx.x / kMsLanes - 1 : -1;        // interval of the round before (-1: none)
   const int gbase = (threadIdx.x & 31) & ~(kMsLanes - 1);
   const bool live = i < n;                    // whole groups are live or not (n * kMsLanes threads)
   const double glo = scal[0], ghi = scal[1], pivmin = scal[3];
@@ -239,20 +256,35 @@ __global__ void bisect_df_kernel(int n, const dfl* __restrict__ d, const dfl* __
   const double tol = fmax(2.0 * kEps * fmax(fabs(glo), fabs(ghi)), rel_tol * fmax(1.0, scal[2])) + pivmin;
   int rounds = 0;
   for (double w = ghi - glo; w > tol && rounds < 64; w /= (double)(kMsLanes + 1)) ++rounds;
-  for (int r = 0; r < rounds; ++r) {
-    const double h = (hi - lo) / (double)(kMsLanes + 1);
-    const double x = lo + (double)(m + 1) * h;
-    const bool above = live && sturm_count_df(n, d, e2, df_from_double(x)) > i;
+  __shared__ unsigned s_above[2][kMsWide / 32];
+  constexpr unsigned kMask = (1u << kMsLanes) - 1u;
+  // counts grow with x: the first point with count > i is the new upper end
+  auto first = [](unsigned g) { return g ? (__ffs(g) - 1) : kMsLanes; };   // 0-based point index, kMsLanes: none
+  for (int r = 0; r < rounds; r += WIDE ? 2 : 1) {
+    double l = lo, u = hi, h = (hi - lo) / (double)(kMsLanes + 1);
+    if (sub >= 0) {
+      ms_interval(l, u, h, sub);
+      h = (u - l) / (double)(kMsLanes + 1);
+    }
+    const double x = l + (double)(m + 1) * h;
+    const bool idle = WIDE && ((int)threadIdx.x >= kMsPoints || (sub >= 0 && r + 1 >= rounds));
+    const bool above = live && !idle && sturm_count_df(n, d, e2, df_from_double(x)) > i;
     const unsigned bal = __ballot_sync(0xffffffffu, above);
-    const unsigned g = (bal >> gbase) & ((1u << kMsLanes) - 1u);
-    // counts grow with x: the first point with count > i is the new upper end
-    const int f = g ? (__ffs(g) - 1) : kMsLanes;      // 0-based point index, kMsLanes: none
-    const double nlo = (f == 0) ? lo : lo + (double)f * h;
-    const double nhi = (f == kMsLanes) ? hi : lo + (double)(f + 1) * h;
-    lo = nlo;
-    hi = nhi;
+    if constexpr (WIDE) {
+      unsigned* w = s_above[(r >> 1) & 1];                             // (the other one was read before the barrier)
+      if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = bal;
+      __syncthreads();
+      const int f0 = first(w[0] & kMask);
+      ms_interval(lo, hi, (hi - lo) / (double)(kMsLanes + 1), f0);
+      if (r + 1 < rounds) {
+        const int at = kMsLanes * (f0 + 1);
+        ms_interval(lo, hi, (hi - lo) / (double)(kMsLanes + 1), first(w[at >> 5] >> (at & 31) & kMask));
+      }
+    } else {
+      ms_interval(lo, hi, h, first((bal >> gbase) & kMask));
+    }
   }
-  if (live && m == 0) ev[i] = 0.5 * (lo + hi);
+  if (live && (WIDE ? threadIdx.x == 0 : m == 0)) ev[i] = 0.5 * (lo + hi);
 }
 
 __global__ void cluster_kernel(int n, const double* __restrict__ ev, const double* __restrict__ scal,
@@ -668,7 +700,7 @@ size_t eig_work_bytes(int n) { return eig_layout(n, nullptr, nullptr); }
 // base must be 256-byte aligned (arena allocations are)
 void eig_work_bind(EigWork& w, void* base, int n) { eig_layout(n, base, &w); }
 
-void eig_bisect(cudaStream_t s, int n, double* eps, EigWork& w, double rel_tol, bool df_path) {
+void eig_bisect(cudaStream_t s, int n, double* eps, EigWork& w, double rel_tol, bool df_path, bool shared) {
   if (n <= 0) return;
   // 2. eigenvalues
   // pbuf (4n doubles, free after the tridiagonalisation) holds the FP32 and double-float copies
@@ -680,16 +712,19 @@ void eig_bisect(cudaStream_t s, int n, double* eps, EigWork& w, double rel_tol, 
   gersh_kernel<<<1, 1024, 0, s>>>(n, w.d, w.e, w.e2, w.scal, df, e2f, d_dfl, e2_dfl, e_dfl);
   count_launch();
   if (df_path) {
-    const long long thr = (long long)n * kMsLanes;
     // one warp (4 eigenvalues) per block, so the n / 4 blocks spread over all SMs
-    bisect_df_kernel<<<(unsigned)((thr + 31) / 32), 32, 0, s>>>(n, d_dfl, e2_dfl, w.scal, rel_tol, eps);
+    if (n <= kMsWideMax && !shared)
+      bisect_df_kernel<true><<<n, kMsWide, 0, s>>>(n, d_dfl, e2_dfl, w.scal, rel_tol, eps);
+    else
+      bisect_df_kernel<false><<<(unsigned)(((long long)n * kMsLanes + 31) / 32), 32, 0, s>>>(n, d_dfl, e2_dfl, w.scal,
+                                                                                           rel_tol, eps);
   } else {
     auto run = [&](auto kernel, int m) {
       kernel<<<(unsigned)(((long long)n * m + 31) / 32), 32, 0, s>>>(n, w.d, w.e2, w.scal, df, e2f, rel_tol, eps);
     };
-    if (n <= kFp64Pipes)
+    if (n <= kFp64Pipes && !shared)
       run(bisect_kernel<32>, 32);
-    else if (n <= 2 * kFp64Pipes)
+    else if (n <= 2 * kFp64Pipes && !shared)
       run(bisect_kernel<16>, 16);
     else if (n <= 8 * kFp64Pipes)
       run(bisect_kernel<8>, 8);
@@ -699,7 +734,7 @@ void eig_bisect(cudaStream_t s, int n, double* eps, EigWork& w, double rel_tol, 
   count_launch();
 }
 
-void eig_vectors(cudaStream_t s, int n, const double* eps, double* Q, EigWork& w, bool df_path) {
+void eig_vectors(cudaStream_t s, int n, const double* eps, double* Q, EigWork& w, bool df_path, bool shared) {
   if (n <= 0) return;
   // 3. eigenvectors of the tridiagonal matrix
   cluster_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, eps, w.scal, w.clus);
@@ -711,7 +746,7 @@ void eig_vectors(cudaStream_t s, int n, const double* eps, double* Q, EigWork& w
                                                                   (dfl*)w.lu, Q);
   } else {
     // (not more warps than there are FP64 pipes, which a partly filled warp holds as long as a full one)
-    int lanes = kIvLanes;
+    int lanes = shared ? 2 * kIvLanes : kIvLanes;
     while (lanes < 32 && n > lanes * kFp64Pipes) lanes *= 2;
     invit_kernel<double><<<(n + lanes - 1) / lanes, 32, 0, s>>>(n, lanes, w.d, w.e, eps, w.scal, w.clus, w.lu, Q);
   }
@@ -998,8 +1033,8 @@ int symmetric_eig(cudaStream_t s, int n, const double* F, double* eps, double* Q
                   int* status, int sm_count) {
   int rc = eig_tridiagonalize(s, n, F, w, status, sm_count, false, false);
   if (rc) return rc;
-  eig_bisect(s, n, eps, w, 1e-12, false);
-  eig_vectors(s, n, eps, Q, w, false);
+  eig_bisect(s, n, eps, w, 1e-12, false, false);
+  eig_vectors(s, n, eps, Q, w, false, false);
   eig_backtransform(s, n, Q, w, nullptr, nullptr);
   return 0;
 }

@@ -85,11 +85,11 @@ int eig_tridiagonalize(cudaStream_t s, int n, const double* F, EigWork& w, int* 
 int eig_tridiag_weight(int n, int sm_count, bool df, bool shared);
 // wall-time limit of the eigensolver's grid barriers on the current device (default 2 s)
 int eig_set_barrier_limit(unsigned long long ns);
-// rel_tol: eigenvalues to rel_tol x max(1, ||T||) (1e-12 FP64 path, 1e-9 mixed path)
-// eigenvalues to rel_tol x ||T||; df_path: double-float multisection (mixed path), else FP64 bisection
-void eig_bisect(cudaStream_t s, int n, double* eps, EigWork& w, double rel_tol, bool df_path);
+// eigenvalues to rel_tol x max(1, ||T||) by multisection; df_path: in double-float (mixed path),
+// else FP64; shared: beside other handles, where work counts more than latency
+void eig_bisect(cudaStream_t s, int n, double* eps, EigWork& w, double rel_tol, bool df_path, bool shared);
 // tridiagonal eigenvectors by inverse iteration; df_path: double-float arithmetic (mixed path)
-void eig_vectors(cudaStream_t s, int n, const double* eps, double* Q, EigWork& w, bool df_path);
+void eig_vectors(cudaStream_t s, int n, const double* eps, double* Q, EigWork& w, bool df_path, bool shared);
 struct TcWork;
 struct Tc64Work;
 // tw != nullptr: the large products run on the tensor cores (mixed path)
