@@ -150,72 +150,88 @@ __host__ __device__ constexpr int pair_nu(int p, int i) {
 }
 __host__ __device__ constexpr double pair_mult(int p) { return (double)pair_cnt(p); }
 
-// one thread per pair (A < B): exchange blocks F_AB, F_BA = F_AB^T (plus h) and
+// per pair (A < B): exchange blocks F_AB, F_BA = F_AB^T (plus h) and
 // the Coulomb contributions cw[A][B][P] = sum_q m_q Pd_B[q] W[P][q],
 // cw[B][A][q] = sum_P m_P Pd_A[P] W[P][q] (m = product multiplicity)
-__global__ void __launch_bounds__(128) fock_pair_kernel(MolDev m, PairDev pd, ElemTable tab,
-                                                       const double* __restrict__ P,
-                                                       const double* __restrict__ Pd, const double* __restrict__ h,
-                                                       double* __restrict__ out, const int* gate) {
-  if (gate && *gate == 0) return;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m.npair) return;
+// Part PART = 0 .. 3 of a pair: row PART of the exchange block and the Coulomb sums over
+// a share of the products.  Every sum is over the same terms in the same order as if one
+// thread did the pair.
+template <int PART>
+__device__ __forceinline__ void fock_pair_part(const MolDev& m, const PairDev& pd, const ElemTable& tab, int t,
+                                               const double* __restrict__ P, const double* __restrict__ Pd,
+                                               const double* __restrict__ h, double* __restrict__ out) {
+  constexpr int k0 = PART < 2 ? 3 * PART : 2 + 2 * PART, k1 = PART < 2 ? k0 + 3 : k0 + 2;   // products 0-2, 3-5, 6-7, 8-9
   const int A = m.pA[t], B = m.pB[t];
   const int na = tab.e[m.elem[A]].norb, nb = tab.e[m.elem[B]].norb;
   const int oa = m.off[A], ob = m.off[B];
   const size_t np = (size_t)m.npair;
   const size_t n = (size_t)m.n;
-  double pab[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) pab[a][b] = (a < na && b < nb) ? P[(oa + a) * n + ob + b] : 0.0;
-  double da[10], db[10];
-#pragma unroll
-  for (int k = 0; k < 10; ++k) {
-    da[k] = pair_mult(k) * Pd[(size_t)A * 10 + k];
-    db[k] = pair_mult(k) * Pd[(size_t)B * 10 + k];
-  }
-  double g[4][4], ca[10], cb[10];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) g[a][b] = 0.0;
-#pragma unroll
-  for (int k = 0; k < 10; ++k) { ca[k] = 0.0; cb[k] = 0.0; }
   const int qa = (na == 4) ? 10 : 1, qb = (nb == 4) ? 10 : 1;
+  const double* W = pd.W + t;
+  if (PART < na) {
+    double pab[4][4], g[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-  for (int pp = 0; pp < 10; ++pp) {
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int qq = 0; qq < 10; ++qq) {
-      if (pp < qa && qq < qb) {
-        const double w = pd.W[(size_t)(pp * 10 + qq) * np + t];
-        ca[pp] += db[qq] * w;
-        cb[qq] += da[pp] * w;
-        // exchange: g[mu][la] -= P[nu][si] (mu nu | la si) over the orbital pairs of pp, qq
+      for (int b = 0; b < 4; ++b) pab[a][b] = (a < na && b < nb) ? P[(oa + a) * n + ob + b] : 0.0;
+    // g[mu][la] -= P[nu][si] (mu nu | la si) over the orbital pairs of pp, qq, mu = PART
 #pragma unroll
-        for (int i = 0; i < pair_cnt(pp); ++i)
+    for (int pp = 0; pp < 10; ++pp)
 #pragma unroll
-          for (int j = 0; j < pair_cnt(qq); ++j)
-            g[pair_mu(pp, i)][pair_mu(qq, j)] -= pab[pair_nu(pp, i)][pair_nu(qq, j)] * w;
+      for (int i = 0; i < pair_cnt(pp); ++i) {
+        if (pair_mu(pp, i) != PART) continue;
+#pragma unroll
+        for (int qq = 0; qq < 10; ++qq) {
+          if (pp < qa && qq < qb) {
+            const double w = W[(size_t)(pp * 10 + qq) * np];
+#pragma unroll
+            for (int j = 0; j < pair_cnt(qq); ++j) g[pair_mu(qq, j)] -= pab[pair_nu(pp, i)][pair_nu(qq, j)] * w;
+          }
+        }
       }
-    }
-  }
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu)
 #pragma unroll
     for (int la = 0; la < 4; ++la) {
-      if (mu < na && la < nb) {
-        const size_t ix = (oa + mu) * n + ob + la, jx = (ob + la) * n + oa + mu;
-        const double v = (h ? h[ix] : 0.0) + g[mu][la];
+      if (la < nb) {
+        const size_t ix = (oa + PART) * n + ob + la, jx = (ob + la) * n + oa + PART;
+        const double v = (h ? h[ix] : 0.0) + g[la];
         out[ix] = v;
         out[jx] = v;
       }
     }
+  }
   double* cA = pd.cw + ((size_t)A * m.N + B) * 10;
   double* cB = pd.cw + ((size_t)B * m.N + A) * 10;
+  const double* PA = Pd + (size_t)A * 10;
+  const double* PB = Pd + (size_t)B * 10;
+  double ca[k1 - k0] = {}, cb[k1 - k0] = {};
 #pragma unroll
-  for (int k = 0; k < 10; ++k) { cA[k] = ca[k]; cB[k] = cb[k]; }
+  for (int q = 0; q < 10; ++q) {
+    const double da = pair_mult(q) * PA[q], db = pair_mult(q) * PB[q];
+#pragma unroll
+    for (int k = k0; k < k1; ++k) {
+      if (k < qa && q < qb) ca[k - k0] += db * W[(size_t)(k * 10 + q) * np];
+      if (q < qa && k < qb) cb[k - k0] += da * W[(size_t)(q * 10 + k) * np];
+    }
+  }
+#pragma unroll
+  for (int k = k0; k < k1; ++k) { cA[k] = ca[k - k0]; cB[k] = cb[k - k0]; }
+}
+
+// a block does 32 pairs, a warp one part of each: one thread a pair was a chain of 460
+// FP64 operations.  @FP@
+__global__ void __launch_bounds__(128) fock_pair_kernel(MolDev m, PairDev pd, ElemTable tab,
+                                                       const double* __restrict__ P,
+                                                       const double* __restrict__ Pd, const double* __restrict__ h,
+                                                       double* __restrict__ out, const int* gate) {
+  if (gate && *gate == 0) return;
+  const int t = blockIdx.x * 32 + (threadIdx.x & 31);
+  if (t >= m.npair) return;
+  switch (threadIdx.x >> 5) {
+    case 0: fock_pair_part<0>(m, pd, tab, t, P, Pd, h, out); break;
+    case 1: fock_pair_part<1>(m, pd, tab, t, P, Pd, h, out); break;
+    case 2: fock_pair_part<2>(m, pd, tab, t, P, Pd, h, out); break;
+    default: fock_pair_part<3>(m, pd, tab, t, P, Pd, h, out); break;
+  }
 }
 
 // g plus the one-centre part of G_mu,nu on one atom, from the packed density block
@@ -397,7 +413,7 @@ void launch_build_h(cudaStream_t s, const MolDev& m, const PairDev& pd, const El
 void launch_build_fock(cudaStream_t s, const MolDev& m, const PairDev& pd, const ElemTable& tab,
                        const double* P, const double* Pd, const double* h, double* out, const int* gate) {
   if (m.npair > 0) {
-    fock_pair_kernel<<<blocks_for(m.npair, 128), 128, 0, s>>>(m, pd, tab, P, Pd, h, out, gate);
+    fock_pair_kernel<<<blocks_for(m.npair, 32), 128, 0, s>>>(m, pd, tab, P, Pd, h, out, gate);
     count_launch();
   }
   fock_atom_kernel<<<blocks_for((long long)m.N * 32, 256), 256, 0, s>>>(m, pd, tab, Pd, h, out, gate);
