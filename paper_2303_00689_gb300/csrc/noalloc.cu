@@ -11,7 +11,7 @@
 // Limits and sharing: n <= kNoAllocMaxN.  Every call on a device uses the
 // same scratch array, which keeps the previous call's contents; the error
 // flag is cleared at the start of each call and the slices are rewritten
-// in full.  Calls whose work overlaps on the GPU (other streams, other
+// in full, both by one launch.  Calls whose work overlaps on the GPU (other streams, other
 // threads) race on the scratch and must be serialised by the caller.  The
 // first call on a device resolves the array's device address with
 // cudaGetSymbolAddress (with that device current); it should come before
@@ -89,9 +89,7 @@ extern "C" int sim_tc_gemm_noalloc(int n, const double* A, const double* B, int 
     if (!tc_encode_map(&mA[a], sa + a * stride, n, ld) || !tc_encode_map(&mB[a], sb + a * stride, n, ld))
       return SIM_EINTERNAL;
   }
-  if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return SIM_EINTERNAL;
-  tc_split_strided(s, n, ld, A, slices, 0, exA, sa, stride);
-  tc_split_strided(s, n, ld, B, slices, 0, exB, sb, stride);
+  tc_split_pair(s, n, ld, A, B, slices, exA, exB, sa, sb, stride, err);
   tc_gemm_on_maps(s, n, mA, mB, terms, 1.0, C, sym ? 1 : 0, err);
   int flag = 0;
   if (cudaMemcpyAsync(&flag, err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SIM_EINTERNAL;

@@ -77,10 +77,47 @@ __device__ __forceinline__ void twosum_acc(float& hi, float& lo, float b) {
 // alpha (hi + lo) in FP64 with one instruction on the FP64 pipe, two unless alpha = +-1:
 // GB300 takes 62 cycles for each, and the conversions, the sum and the product of a
 // 128 x 128 tile were 17 us of it (n = 240, 3 and 4 slices: 31 and 37 us -> 26 and 32).
-// Not in tc_gemm_kernel, which writes straight from registers and was slower with it.
 __device__ __forceinline__ double scaled_sum(double alpha, float hi, float lo) {
   const double v = df_to_double_fast(dfl{hi, lo});
   return alpha == 1.0 ? v : (alpha == -1.0 ? -v : alpha * v);
+}
+
+// The epilogue warps' tile through shared memory (the stages are idle by then: every
+// product has been folded): each thread's 32 values at constant offsets, then
+// row-contiguous stores of the tile and, for a symmetric result, of its transpose.
+// Every epilogue warp reaches the named barrier; the global stores run only when no
+// wait of any CTA expired.
+__device__ __forceinline__ void write_tile(double* tile, const float (&hi)[32], const float (&lo)[32], bool ok,
+                                           int quarter, int cg, int lane, int m0, int n0, int M, int N, double alpha,
+                                           double* __restrict__ C, int ldc, int sym, int beta, int* err) {
+  constexpr int kLdT = kBN + 1;                      // padded row: conflict-free transposed reads
+  if (ok) {
+    const int rl = quarter * 32 + lane;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) tile[rl * kLdT + cg * 32 + j] = scaled_sum(alpha, hi[j], lo[j]);
+  }
+  asm volatile("bar.sync 1, %0;" ::"r"(kEpiWarps * 32) : "memory");
+  if (!ok || *(volatile int*)err != 0) return;
+  const int t = threadIdx.x - 64;
+  for (int idx = t; idx < kBM * kBN; idx += kEpiWarps * 32) {
+    const int rr = idx / kBN, cc = idx - rr * kBN;
+    const int row = m0 + rr, col = n0 + cc;
+    if (row < M && col < N && !(sym && row > col)) {
+      const size_t at = (size_t)row * ldc + col;
+      C[at] = beta ? C[at] + tile[rr * kLdT + cc] : tile[rr * kLdT + cc];
+    }
+  }
+  if (sym) {
+    // C[col][row] for row < col: rows of the output are columns of the tile
+    for (int idx = t; idx < kBM * kBN; idx += kEpiWarps * 32) {
+      const int cr = idx / kBM, rc = idx - cr * kBM;   // output row n0 + cr, column m0 + rc
+      const int row = m0 + rc, col = n0 + cr;
+      if (row < M && col < N && row < col) {
+        const size_t at = (size_t)col * ldc + row;
+        C[at] = beta ? C[at] + tile[rc * kLdT + cr] : tile[rc * kLdT + cr];
+      }
+    }
+  }
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -217,21 +254,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[b]);
     }
-    if (ok && total > 0) {
-      const int row = m0 + quarter * 32 + lane;
-      if (row < M) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          int col = n0 + cg * 32 + j;
-          if (col >= N) break;
-          if (sym && row > col) continue;
-          double v = alpha * ((double)hi[j] + (double)lo[j]);
-          if (beta) v += C[(size_t)row * ldc + col];
-          C[(size_t)row * ldc + col] = v;
-          if (sym && row != col) C[(size_t)col * ldc + row] = v;
-        }
-      }
-    }
+    write_tile((double*)base, hi, lo, ok && total > 0, quarter, cg, lane, m0, n0, M, N, alpha, C, ldc, sym, beta, err);
   }
   tc_fence_before();
   __syncthreads();
@@ -426,40 +449,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[b]);
     }
-    // the tile through shared memory: the thread's 32 values at constant
-    // offsets, then row-contiguous stores of the tile and, for a symmetric
-    // result, of its transpose.  Every epilogue warp reaches the named
-    // barrier; the global stores run only when no wait of any CTA expired.
-    constexpr int kLdT = kBN + 1;                      // padded row: conflict-free transposed reads
-    double* tile = (double*)base;
-    if (ok) {
-      const int rl = quarter * 32 + lane;
-#pragma unroll
-      for (int j = 0; j < 32; ++j) tile[rl * kLdT + cg * 32 + j] = scaled_sum(alpha, hi[j], lo[j]);
-    }
-    asm volatile("bar.sync 1, %0;" ::"r"(kEpiWarps * 32) : "memory");
-    if (ktiles > 0 && *(volatile int*)err == 0) {
-      const int t = threadIdx.x - 64;
-      for (int idx = t; idx < kBM * kBN; idx += kEpiWarps * 32) {
-        const int rr = idx / kBN, cc = idx - rr * kBN;
-        const int row = m0 + rr, col = n0 + cc;
-        if (row < M && col < N && !(sym && row > col)) {
-          const size_t at = (size_t)row * ldc + col;
-          C[at] = beta ? C[at] + tile[rr * kLdT + cc] : tile[rr * kLdT + cc];
-        }
-      }
-      if (sym) {
-        // C[col][row] for row < col: rows of the output are columns of the tile
-        for (int idx = t; idx < kBM * kBN; idx += kEpiWarps * 32) {
-          const int cr = idx / kBM, rc = idx - cr * kBM;   // output row n0 + cr, column m0 + rc
-          const int row = m0 + rc, col = n0 + cr;
-          if (row < M && col < N && row < col) {
-            const size_t at = (size_t)col * ldc + row;
-            C[at] = beta ? C[at] + tile[rc * kLdT + cr] : tile[rc * kLdT + cr];
-          }
-        }
-      }
-    }
+    write_tile((double*)base, hi, lo, ok && ktiles > 0, quarter, cg, lane, m0, n0, M, N, alpha, C, ldc, sym, beta, err);
   }
   tc_fence_before();
   __syncthreads();
@@ -578,19 +568,6 @@ __global__ void split_bf16_kernel(int n, const double* __restrict__ X, int ld, i
     if (a < slices) P[a][t] = v[a];
 }
 
-// same slicing as split_bf16_kernel, slices at base + a * stride (no pointer table)
-__global__ void split_bf16_strided_kernel(int n, const double* __restrict__ X, int ld, int slices, int transpose,
-                                          const int* __restrict__ ex, __nv_bfloat16* __restrict__ base,
-                                          size_t stride) {
-  size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  size_t tot = (size_t)n * ld;
-  if (t >= tot) return;
-  int i = (int)(t / ld), j = (int)(t % ld);
-  double x = 0.0;
-  if (j < n) x = transpose ? X[(size_t)j * n + i] : X[(size_t)i * n + j];
-  slice_value(x, ex[i], slices, base, stride, t);
-}
-
 // per-row exponent of op(X), op(X) = X (rows x cols, ldx) or X^T (X stored cols x rows)
 __global__ void row_exponent_general_kernel(int rows, int cols, const double* __restrict__ X, int ldx,
                                             int transpose, int* __restrict__ ex) {
@@ -684,11 +661,8 @@ __device__ __forceinline__ void split_row_warp(const RowSplit& q, int r, int sli
 // 64, so every group is aligned); columns n..ld-1 are zeros.  The second sweep
 // re-reads the row from L1/L2, so X leaves HBM once.
 constexpr int kSqThreads = 128;
-__global__ void __launch_bounds__(kSqThreads) split_rows_sq_kernel(int n, const double* __restrict__ X, int ld,
-                                                                 int slices, int* __restrict__ ex,
-                                                                 __nv_bfloat16* __restrict__ base, size_t stride,
-                                                                 const int* gate) {
-  if (gate && *gate == 0) return;
+__device__ __forceinline__ void split_row_sq(int n, const double* __restrict__ X, int ld, int slices,
+                                             int* __restrict__ ex, __nv_bfloat16* __restrict__ base, size_t stride) {
   __shared__ unsigned long long s_max[kSqThreads / 32];
   const int r = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -725,6 +699,25 @@ __global__ void __launch_bounds__(kSqThreads) split_rows_sq_kernel(int n, const 
       }
     }
   }
+}
+
+__global__ void __launch_bounds__(kSqThreads) split_rows_sq_kernel(int n, const double* __restrict__ X, int ld,
+                                                                 int slices, int* __restrict__ ex,
+                                                                 __nv_bfloat16* __restrict__ base, size_t stride,
+                                                                 const int* gate) {
+  if (gate && *gate == 0) return;
+  split_row_sq(n, X, ld, slices, ex, base, stride);
+}
+
+// both operands of a small product (blockIdx.y), and the error word cleared for it
+__global__ void __launch_bounds__(kSqThreads) split_pair_kernel(int n, const double* __restrict__ A,
+                                                              const double* __restrict__ B, int ld, int slices,
+                                                              int* __restrict__ exA, int* __restrict__ exB,
+                                                              __nv_bfloat16* __restrict__ a,
+                                                              __nv_bfloat16* __restrict__ b, size_t stride, int* err) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *err = 0;
+  const bool second = blockIdx.y == 1;
+  split_row_sq(n, second ? B : A, ld, slices, second ? exB : exA, second ? b : a, stride);
 }
 
 __global__ void split_rows_kernel(RowSplit q, int slices) {
@@ -1161,13 +1154,9 @@ void tc_mbar_expiry(cudaStream_t s, int* err, long long limit) {
 
 bool tc_encode_map(CUtensorMap* m, void* ptr, int n, int ld) { return make_map(m, ptr, n, ld); }
 
-void tc_split_strided(cudaStream_t s, int n, int ld, const double* X, int slices, int transpose, int* ex,
-                      __nv_bfloat16* base, size_t stride) {
-  row_exponent_kernel<<<(n * 32 + 255) / 256, 256, 0, s>>>(n, X, transpose, ex, nullptr);
-  count_launch();
-  size_t tot = (size_t)n * ld;
-  split_bf16_strided_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(n, X, ld, slices, transpose, ex, base,
-                                                                           stride);
+void tc_split_pair(cudaStream_t s, int n, int ld, const double* A, const double* B, int slices, int* exA, int* exB,
+                   __nv_bfloat16* a, __nv_bfloat16* b, size_t stride, int* err) {
+  split_pair_kernel<<<dim3(n, 2), kSqThreads, 0, s>>>(n, A, B, ld, slices, exA, exB, a, b, stride, err);
   count_launch();
 }
 

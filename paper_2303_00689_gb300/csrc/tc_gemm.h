@@ -50,8 +50,9 @@ int tc_gemm_grouped_rc_splitk(cudaStream_t s, int M, int N, int K, const __nv_bf
 // Building blocks on caller-provided buffers (used by the allocation-free entry point)
 int tc_ld(int n);                                                   // padded slice row length
 bool tc_encode_map(CUtensorMap* m, void* ptr, int n, int ld);       // BF16 slice tensor map
-void tc_split_strided(cudaStream_t s, int n, int ld, const double* X, int slices, int transpose, int* ex,
-                      __nv_bfloat16* base, size_t stride);
+// the slices of both operands in one launch, which clears *err
+void tc_split_pair(cudaStream_t s, int n, int ld, const double* A, const double* B, int slices, int* exA, int* exB,
+                   __nv_bfloat16* a, __nv_bfloat16* b, size_t stride, int* err);
 void tc_gemm_on_maps(cudaStream_t s, int n, const CUtensorMap* mapsA, const CUtensorMap* mapsB, int terms,
                      double alpha, double* C, int sym, int* err);
 
