@@ -229,7 +229,7 @@ __device__ __forceinline__ void f64_reflector(double x1, double sigma, double& b
 // stay in shared memory.  Barriers 0: group 0 and the scalar warp; 1: the scalars;
 // 2 + g: group g.
 template <int NTG, int RG, int CPL, bool SOLO>
-__global__ void __launch_bounds__(NTG * RG + 32, NTG * RG <= 256 ? 2 : 1) tridiag_f64_kernel(TriArgs g) {
+__global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ? 2 : 1) tridiag_f64_kernel(TriArgs g) {
   constexpr int NT = NTG * RG, GW = NTG / 32;                      // workers; warps of a group
   static_assert(GW <= 16 && (RG & (RG - 1)) == 0, "layout");
   extern __shared__ __align__(16) unsigned char smem[];
@@ -835,9 +835,11 @@ struct TriShape {
 #define TRI_SHAPE(NMAX, NTG, RG, CPL, SOLO) \
   {NMAX, NTG, RG, CPL, SOLO, (const void*)tridiag_f64_kernel<NTG, RG, CPL, SOLO>}
 static const TriShape kTriF64[] = {
-    TRI_SHAPE(64, 64, 4, 1, true),    TRI_SHAPE(128, 128, 2, 1, false),  TRI_SHAPE(256, 256, 1, 1, false),
-    TRI_SHAPE(512, 256, 1, 2, false), TRI_SHAPE(1024, 256, 1, 4, false), TRI_SHAPE(1920, 480, 1, 4, false),
-    TRI_SHAPE(3360, 480, 1, 7, false), TRI_SHAPE(4800, 480, 1, 10, false), TRI_SHAPE(10080, 480, 1, 21, false)};
+    TRI_SHAPE(64, 64, 4, 1, true),     TRI_SHAPE(128, 128, 2, 1, false),   TRI_SHAPE(256, 128, 1, 2, false),
+    TRI_SHAPE(384, 128, 1, 3, false),  TRI_SHAPE(480, 160, 1, 3, false),   TRI_SHAPE(576, 192, 1, 3, false),
+    TRI_SHAPE(768, 192, 1, 4, false),  TRI_SHAPE(1120, 224, 1, 5, false),  TRI_SHAPE(1728, 192, 1, 9, false),
+    TRI_SHAPE(2560, 256, 1, 10, false), TRI_SHAPE(3360, 480, 1, 7, false), TRI_SHAPE(4800, 480, 1, 10, false),
+    TRI_SHAPE(10080, 480, 1, 21, false)};
 constexpr size_t kTriSmemMax = 227 * 1024 - 512;       // of dynamic shared memory; the kernels have some of their own
 
 struct TriLaunch {
