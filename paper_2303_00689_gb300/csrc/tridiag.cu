@@ -3,11 +3,12 @@
 // update (v, w of column k - 1), the reflector v_k, tau_k of x, and p = tau A v_k;
 // the rank-2 update of column k is applied one column later, fused with the
 // matrix-vector product, so an element of the trailing matrix is read and written
-// once per column.  One persistent kernel for the FP64 path, one in double-float
-// (df.cuh: FP32 pairs, about 48 bits, on the FP32 pipe) for the mixed path.  What
-// bounds both up to ~1500 columns is the dependent chain of a column (exchange of p
-// between the blocks, reductions, product), n times, so the more blocks share the
-// product the better, until the exchange between them costs more.
+// once per column.  A persistent kernel for the FP64 path, and two in double-float
+// (df.cuh: FP32 pairs, about 48 bits, on the FP32 pipe) for the mixed path: small
+// matrices in one thread-block cluster, others on a grid.  What bounds them up to
+// ~1500 columns is the dependent chain of a column (exchange of p between the blocks,
+// reductions, product), n times, so the more blocks share the product the better, until
+// the exchange between them costs more; above, the FP32 (FP64) operations.
 //
 // A grid that takes much of the device cannot always run beside another one (two
 // handles stepped by two threads).  So a launch on its own starts with a check-in:
@@ -592,23 +593,26 @@ __device__ __forceinline__ float4 pack4(dfl a, dfl b) { return make_float4(a.hi,
 // (v_{k-1}, w_{k-1}) of rows/cols >= k+1, stored back, and sum_j a_ij x_j of
 // each (row, SEG-column segment) item into part[r * S + sg] (a_{i,k+1} of the
 // block's rows into ak1s).  Warp w starts at item w - 1, warp 0 at NW - 1.
-template <int SEG>
-__device__ __forceinline__ void df_items(dfl* __restrict__ A, int n, int k, int G, int R, int wid, int lane,
-                                         bool prev, const float4* PW, const dfl* VC, dfl* part, dfl* ak1s) {
+// The block's rows are i = first + r G, r < R; row r at rows + r ld when they are resident
+// in shared memory (RES), at rows + i ld otherwise.
+template <int SEG, bool RES>
+__device__ __forceinline__ void df_items(float2* __restrict__ rows, int ld, int first_row, int n, int k, int G, int R,
+                                         int wid, int lane, bool prev, const float4* PW, const dfl* VC, dfl* part,
+                                         dfl* ak1s) {
   constexpr int PER = SEG / 32, NW = kTriThreadsDf / 32;
   const int S = (n - (k + 1) + SEG - 1) / SEG;
   const int Q = R * S;
   for (int q = (wid == 0) ? NW - 1 : wid - 1; q < Q; q += NW) {
     const int r = q / S, sg = q - r * S;
-    const int i = k + 1 + (int)blockIdx.x + r * G;
-    float2* row = (float2*)(A + (size_t)i * n);
+    const int i = first_row + r * G;
+    float2* row = rows + (size_t)(RES ? r : i) * ld;
     const int jb = k + 1 + sg * SEG + lane;
     const bool full = (k + 1 + (sg + 1) * SEG) <= n;
     dfl a0 = {0.0f, 0.0f}, a1 = {0.0f, 0.0f}, first = {0.0f, 0.0f};
     if (full) {
       float2 xr[PER];
 #pragma unroll
-      for (int u = 0; u < PER; ++u) xr[u] = __ldcg(row + jb + 32 * u);
+      for (int u = 0; u < PER; ++u) xr[u] = RES ? row[jb + 32 * u] : __ldcg(row + jb + 32 * u);
       if (prev) {
         const float4 pwi = PW[i];
         const dfl vi = lo2(pwi), wi = hi2(pwi);
@@ -635,7 +639,7 @@ __device__ __forceinline__ void df_items(dfl* __restrict__ A, int n, int k, int 
 #pragma unroll
       for (int u = 0; u < PER; ++u) {
         const int j = jb + 32 * u;
-        xr[u] = (j < n) ? __ldcg(row + j) : make_float2(0.0f, 0.0f);
+        xr[u] = (j < n) ? (RES ? row[j] : __ldcg(row + j)) : make_float2(0.0f, 0.0f);
       }
       const float4 pwi = prev ? PW[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       const dfl vi = lo2(pwi), wi = hi2(pwi);
@@ -662,6 +666,8 @@ __device__ __forceinline__ void df_items(dfl* __restrict__ A, int n, int k, int 
   }
 }
 
+// (The compiler gives it more than 64 registers a thread, so one block an SM: with two of
+// them an SM a batch of 16 cages took 20.7 instead of 19.3 ms.)
 template <bool GATED>
 __global__ void __launch_bounds__(kTriThreadsDf) tridiag_df_kernel(int n, dfl* __restrict__ A,
                                                                  double* __restrict__ Vst,
@@ -778,9 +784,15 @@ __global__ void __launch_bounds__(kTriThreadsDf) tridiag_df_kernel(int n, dfl* _
     const int m1 = n - (k + 1);
     const int segw = (m1 > kDfNarrow1) ? kDfSeg : ((m1 > kDfNarrow2) ? 256 : 128);
     const int S = (m1 + segw - 1) / segw;
-    if (segw == kDfSeg) df_items<kDfSeg>(A, n, k, G, R, wid, lane, prev, PW, VC, part, ak1s);
-    else if (segw == 256) df_items<256>(A, n, k, G, R, wid, lane, prev, PW, VC, part, ak1s);
-    else df_items<128>(A, n, k, G, R, wid, lane, prev, PW, VC, part, ak1s);
+    if (segw == kDfSeg)
+      df_items<kDfSeg, false>((float2*)A, n, k + 1 + (int)blockIdx.x, n, k, G, R, wid, lane, prev, PW, VC, part,
+                            ak1s);
+    else if (segw == 256)
+      df_items<256, false>((float2*)A, n, k + 1 + (int)blockIdx.x, n, k, G, R, wid, lane, prev, PW, VC, part,
+                            ak1s);
+    else
+      df_items<128, false>((float2*)A, n, k + 1 + (int)blockIdx.x, n, k, G, R, wid, lane, prev, PW, VC, part,
+                            ak1s);
     __syncthreads();
     const dfl beta_df = s_df[0], ts_df = s_df[1], scale_df = s_df[3];
     tau_prev = s_df[2];
@@ -818,6 +830,188 @@ __global__ void __launch_bounds__(kTriThreadsDf) tridiag_df_kernel(int n, dfl* _
   }
 }
 
+// The same in one thread-block cluster, for matrices that fit its shared memory: block b
+// keeps rows i = b (mod G), pushes row k + 1 and its p_i into every block's shared memory
+// (double-buffered by the column's parity: a buffer is rewritten two cluster barriers
+// after it was filled and one after its last reader), and the cluster barrier takes the
+// place of the grid's counter and polls in L2.  The blocks of a cluster are resident
+// together, so there is nothing to check in or to wait for with a limit.  Same bits as
+// tridiag_df_kernel.
+__device__ __forceinline__ void st_cluster(void* local, int dst, float2 v) {
+  unsigned a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(local)), "r"(dst));
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+
+__global__ void __launch_bounds__(kTriThreadsDf, 1) tridiag_cluster_kernel(int n, const double* __restrict__ F,
+                                                                         double* __restrict__ Vst,
+                                                                         double* __restrict__ d,
+                                                                         double* __restrict__ e,
+                                                                         double* __restrict__ tau, int* status) {
+  extern __shared__ float4 sm4[];
+  __shared__ dfl s_df[4];                    // beta, tau * scale, tau, scale
+  const int G = (int)gridDim.x, rank = (int)blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  constexpr int T = kTriThreadsDf, NW = kTriThreadsDf / 32;
+  const int rmax = (n - 1 + G - 1) / G;
+  float4* PW = sm4;                          // n pairs
+  dfl* VC = (dfl*)(sm4 + n);                 // n
+  dfl* rowb = VC + n;                        // row k, 2 x n
+  dfl* pbuf = rowb + 2 * n;                  // p, 2 x n
+  dfl* redA = pbuf + 2 * n;                  // partials of p.v
+  dfl* redB = redA + kDfRed;                 // partials of sigma
+  dfl* ak1s = redB + kDfRed;                 // a_{i,k+1} of the block's rows (rmax)
+  dfl* part = ak1s + rmax;                   // (row, segment) partial sums (rmax x 2)
+  float2* S = (float2*)(part + 2 * rmax);    // the block's rows > 0 (rmax x n)
+  if (g_barrier_ns == 0) {                   // as a wait that has no time (all blocks alike)
+    if (tid == 0) atomicOr(status, (int)kStatusTimeout);
+    return;
+  }
+  const int f0 = (rank == 0) ? G : rank;     // first row > 0 of this block
+  const int R0 = (f0 < n) ? (n - 1 - f0) / G + 1 : 0;
+  for (int x = tid; x < R0 * n; x += T) {
+    const int r = x / n, j = x - r * n;
+    const dfl a = df_from_double_bits(F[(size_t)(f0 + r * G) * n + j]);
+    S[x] = make_float2(a.hi, a.lo);
+  }
+  for (int j = tid; j < n; j += T) rowb[j] = df_from_double_bits(F[j]);
+  dfl tau_prev = {0.0f, 0.0f};               // tau_{k-1}
+  // (before the first remote stores: every block of the cluster has started)
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  for (int k = 0;; ++k) {
+    const bool prev = k > 0;
+    const bool last = (k == n - 2);
+    const dfl* pbp = pbuf + (size_t)((k + 1) & 1) * n;   // p_{k-1}
+    const dfl* rowk = rowb + (size_t)(k & 1) * n;
+    // pass 1: row k and p_{k-1} in one sweep of loads (kept in PW); partial p.v
+    dfl loc = {0.0f, 0.0f};
+#pragma unroll 4
+    for (int j = k + tid; j < n; j += T) {
+      const dfl a = rowk[j];
+      dfl p = {0.0f, 0.0f};
+      if (prev) {
+        p = pbp[j];
+        df_acc_mul(loc, p, VC[j]);           // VC = v_{k-1}
+      }
+      PW[j] = pack4(a, p);
+    }
+    dfl wk = {0.0f, 0.0f}, vk = {0.0f, 0.0f}, coef = {0.0f, 0.0f};
+    if (prev) {
+      loc = df_warp_sum(df_norm(loc));
+      if (lane == 0) redA[wid] = loc;
+      __syncthreads();
+      const dfl pv = df_sum_partials(redA);
+      coef = df_mul(df_mul(dfl{0.5f, 0.0f}, tau_prev), pv);
+      vk = VC[k];
+      wk = df_sub(hi2(PW[k]), df_mul(coef, vk));   // PW[k] is not overwritten below
+    }
+    // pass 2: w_{k-1} and the updated row k; sigma = sum_{j >= k+2} x_j^2
+    dfl sig = {0.0f, 0.0f};
+    dfl dk = {0.0f, 0.0f};
+    for (int j = k + tid; j < n; j += T) {
+      const float4 ap = PW[j];
+      dfl x = lo2(ap);
+      if (prev) {
+        const dfl vj = VC[j];
+        const dfl wj = (j == k) ? wk : df_sub(hi2(ap), df_mul(coef, vj));
+        x = df_rank2(x, vk, wj, wk, vj);
+        if (j > k) PW[j] = pack4(vj, wj);
+      }
+      if (j == k) {
+        dk = x;
+      } else {
+        VC[j] = x;
+        if (j >= k + 2) df_acc_mul(sig, x, x);
+      }
+    }
+    if (last) {
+      __syncthreads();
+      if ((n - 1) % G == rank && tid == 0) {             // the owner of the last row
+        const int b = n - 1;
+        const float2 ab = S[(size_t)(R0 - 1) * n + b];
+        dfl abb = dfl{ab.x, ab.y};
+        if (prev) abb = df_rank2(abb, lo2(PW[b]), hi2(PW[b]), hi2(PW[b]), lo2(PW[b]));
+        d[n - 2] = df_to_double(dk);
+        e[n - 2] = df_to_double(VC[b]);
+        d[b] = df_to_double(abb);
+      }
+      return;
+    }
+    sig = df_warp_sum(df_norm(sig));
+    if (lane == 0) redB[wid] = sig;
+    __syncthreads();
+    // thread 0: reflector scalars (double-float: GB300's FP64 divide and square
+    // root are long dependent chains) while the other warps start the product
+    if (tid == 0) {
+      const dfl sigma = df_sum_partials(redB);
+      const dfl x1 = VC[k + 1];
+      dfl beta, t, scale;
+      if (sigma.hi == 0.0f) {
+        beta = x1; t = dfl{0.0f, 0.0f}; scale = dfl{0.0f, 0.0f};
+      } else {
+        const dfl nrm = df_sqrt(df_add(df_mul(x1, x1), sigma));
+        beta = (x1.hi >= 0.0f) ? df_neg(nrm) : nrm;
+        t = df_mul(df_sub(beta, x1), df_recip(beta));
+        scale = df_recip(df_sub(x1, beta));
+      }
+      s_df[0] = beta;
+      s_df[1] = df_mul(t, scale);
+      s_df[2] = t;
+      s_df[3] = scale;
+      if (rank == 0) { d[k] = df_to_double(dk); e[k] = df_to_double(beta); tau[k] = df_to_double(t); }
+    }
+    // fused: pending rank-2 update (v_{k-1}, w_{k-1}) of rows/cols >= k+1 and
+    // sum_j a_ij x_j over (row, segment) items
+    const int gone = (k + 1 > f0) ? (k + 1 - f0 + G - 1) / G : 0;   // rows of the list that are <= k
+    const int R = max(R0 - gone, 0), first = f0 + gone * G;
+    float2* Sr = S + (size_t)gone * n;
+    const int m1 = n - (k + 1);
+    const int segw = (m1 > kDfNarrow1) ? kDfSeg : ((m1 > kDfNarrow2) ? 256 : 128);
+    const int nseg = (m1 + segw - 1) / segw;
+    if (segw == kDfSeg) df_items<kDfSeg, true>(Sr, n, first, n, k, G, R, wid, lane, prev, PW, VC, part, ak1s);
+    else if (segw == 256) df_items<256, true>(Sr, n, first, n, k, G, R, wid, lane, prev, PW, VC, part, ak1s);
+    else df_items<128, true>(Sr, n, first, n, k, G, R, wid, lane, prev, PW, VC, part, ak1s);
+    __syncthreads();
+    const dfl beta_df = s_df[0], ts_df = s_df[1], scale_df = s_df[3];
+    tau_prev = s_df[2];
+    // row k + 1 from its owner to every block
+    if (R > 0 && first == k + 1)
+      for (int e = tid; e < m1 * G; e += T) {
+        const int dst = e / m1, j = k + 1 + (e - dst * m1);
+        st_cluster(rowb + (size_t)((k + 1) & 1) * n + j, dst, Sr[j]);
+      }
+    // p_i = tau scale (sum_j a_ij x_j - beta a_{i,k+1}), segments summed as a
+    // fixed tree (one warp per row while a row has at most 32 segments)
+    dfl* pb = pbuf + (size_t)(k & 1) * n;
+    int lpr = 1;                                    // lanes per row: power of two >= S
+    while (lpr < nseg) lpr <<= 1;
+    const int rpw = 32 / lpr;                       // rows per warp
+    const int sub = lane / lpr, sl = lane - sub * lpr;
+    for (int r0 = wid * rpw; r0 < R; r0 += NW * rpw) {
+      const int r = r0 + sub;
+      dfl v = (r < R && sl < nseg) ? part[r * nseg + sl] : dfl{0.0f, 0.0f};
+      for (int o = lpr >> 1; o > 0; o >>= 1) v = df_add(v, df_shfl_xor(v, o));
+      if (r < R) {
+        const dfl p = df_mul(ts_df, df_sub(v, df_mul(beta_df, ak1s[r])));
+        for (int dst = sl; dst < G; dst += lpr) st_cluster(pb + first + r * G, dst, make_float2(p.hi, p.lo));
+      }
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    // while the other blocks finish: v_k = scale x (v_{k+1} = 1) and the
+    // reflector store row k, spread over blocks
+    for (int j = k + 1 + tid; j < n; j += T) {
+      const dfl v = (j == k + 1) ? dfl{1.0f, 0.0f} : df_mul(VC[j], scale_df);
+      VC[j] = v;
+      if (j % G == rank) Vst[(size_t)k * n + j] = df_to_double_fast(v);
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+}
+
 __global__ void to_df_kernel(size_t len, const double* __restrict__ x, dfl* __restrict__ y, const unsigned* gate) {
   if (gate && *gate != 2) return;                       // for the stand-in only
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (size_t)gridDim.x * blockDim.x)
@@ -826,7 +1020,11 @@ __global__ void to_df_kernel(size_t len, const double* __restrict__ x, dfl* __re
 
 // ---- launch plan ----------------------------------------------------------------------
 // FP64: (threads of a group, groups, columns a thread) by matrix size.  Up to 64
-// columns one block does it all; up to 1024 columns 256 workers, two blocks an SM.
+// columns one block does it all.  Few threads with several columns each: less to
+// reduce, and the FP64 pipe is as busy (256 x 2, 3, 4 and 480 x 4 threads and columns at n =
+// 343, 574, 720, 1680: 2.19, 3.95, 4.96, 24.1 ms; 128 x 3, 192 x 3, 192 x 4, 192 x 9: 1.93, 3.33,
+// 4.62, 22.2), except where the rows in L2 set the time (n = 3360: 118 ms with 480 x 7, 121
+// with 256 x 14).
 struct TriShape {
   int n_max, ntg, rg, cpl;
   bool solo;
@@ -864,6 +1062,47 @@ static int tri_blocks(int n, int sm_count, bool df, bool few) {
   return (int)std::min<long long>(std::max<long long>(work, df ? 1 : 2), most);
 }
 
+// Blocks of the cluster that does a double-float matrix, 0: none.  A column is a chain of
+// 3.3 us in a cluster of up to 8 or 16 blocks and of about 5 us on a grid, until the
+// rows of so few blocks take longer: n = 26, 131, 240, 300, 343: 87, 451 (8 blocks), 964, 1361,
+// 1695 us (16); on a grid 139, 659, 1227, 1500, 1740 us.  16 blocks from 160 columns on:
+// n = 131, 180, 240: 458, 675, 964 us, with 8 451, 702, 1049 us.
+static size_t tri_cluster_smem(int n, int G) {
+  const size_t rmax = (size_t)(n - 1 + G - 1) / G;
+  return (7 * (size_t)n + 2 * kDfRed + 3 * rmax + rmax * n) * sizeof(dfl);
+}
+constexpr int kTriClusterMax = 320;
+static bool tri_cluster_ready() {
+  static PerDeviceOnce once;
+  return once_per_device(once, [] {
+    const void* fn = (const void*)tridiag_cluster_kernel;
+    bool ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTriSmemMax) == cudaSuccess &&
+              cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    if (!ok) cudaGetLastError();
+    return ok;
+  });
+}
+static int tri_cluster(int n, bool df, bool shared) {
+  if (!df || shared || n < 2 || n > kTriClusterMax || !tri_cluster_ready()) return 0;
+  return n <= 160 ? 8 : 16;
+}
+static int tri_cluster_launch(cudaStream_t s, int n, int G, const double* F, EigWork& w, int* status) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(G);
+  cfg.blockDim = dim3(kTriThreadsDf);
+  cfg.dynamicSmemBytes = tri_cluster_smem(n, G);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = G;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, tridiag_cluster_kernel, n, F, w.Vst, w.d, w.e, w.tau, status) != cudaSuccess) return -2;
+  count_launch();
+  return 0;
+}
+
 // the FP64 launch that starts at column k0 (few: shared memory for two blocks an SM)
 static TriLaunch tri_launch(int n, int k0, int sm_count, bool few) {
   TriLaunch l;
@@ -892,9 +1131,7 @@ static TriLaunch tri_launch(int n, int k0, int sm_count, bool few) {
 }
 
 // The opt-in dynamic shared memory, once per device: of the FP64 shapes, and of the
-// double-float kernel when it needs it (a kernel that may ask for so much is given
-// room for it beside the small ones of other handles: 16 cages of a batch 20.7
-// instead of 19.3 ms).
+// double-float kernel where it needs it.
 static bool tri_attributes(bool df, size_t smem) {
   static PerDeviceOnce once[2];
   if (df && smem <= 48 * 1024) return true;
@@ -923,6 +1160,7 @@ int eig_tridiag_weight(int n, int sm_count, bool df, bool shared) {
     }
     return (int)((1000LL * blocks + p - 1) / p);
   };
+  if (const int G = tri_cluster(n, df, shared)) return 1000 * G;
   if (df) {
     const int G = tri_blocks(n, sm_count, true, shared);
     return share((const void*)tridiag_df_kernel<false>, G, kTriThreadsDf, tridiag_smem_df(n, G));
@@ -949,6 +1187,7 @@ int eig_tridiagonalize(cudaStream_t s, int n, const double* F, EigWork& w, int* 
     count_launch();
     return 0;
   }
+  if (const int G = tri_cluster(n, df, shared)) return tri_cluster_launch(s, n, G, F, w, status);
   if (df) {
     const size_t nn2 = (size_t)n * n;
     const int few = tri_blocks(n, sm_count, true, true), G = shared ? few : tri_blocks(n, sm_count, true, false);

@@ -24,7 +24,8 @@ def _handle(n, precision, seed=1):
 
 
 @pytest.mark.parametrize("precision", [kx.SIM_PREC_FP64, kx.SIM_PREC_MIXED])
-@pytest.mark.parametrize("n", [1, 2, 3, 5, 33, 63, 64, 65, 100, 127, 128, 129, 255, 256, 257, 511, 513, 1023, 1025])
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 33, 63, 64, 65, 100, 127, 128, 129, 160, 161, 255, 256, 257, 320, 321, 384, 385, 481,
+                               511, 513, 577, 769, 1023, 1025, 1121, 1730])
 def test_eigenpairs_at_the_edges_of_the_launch_shapes(n, precision):
     h = _handle(n, precision)
     try:
@@ -65,3 +66,19 @@ def test_grids_that_do_not_fit_together_give_the_results_of_running_alone(precis
     for seed in (1, 2, 3):
         for a, b in zip(alone[seed], together[seed]):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [2, 3, 9, 63, 65, 131, 160, 161, 320, 321, 500])
+def test_alone_and_beside_others_the_mixed_results_are_the_same(n):
+    """Alone: a cluster or a large grid, more lanes an eigenvalue, more threads a pair;
+    beside others the small grid.  Same sums in the same order."""
+    hs = [_handle(n, kx.SIM_PREC_MIXED, 5) for _ in range(3)]
+    try:
+        kx.sim_step(hs[0], 3)
+        kx.sim_batch_step(hs[1:], 3)
+        a, b, c = (kx.sim_get_state(h, n) for h in hs)
+    finally:
+        for h in hs:
+            kx.sim_destroy(h)
+    for x, y, z in zip(a, b, c):
+        assert np.array_equal(x, y) and np.array_equal(x, z)
