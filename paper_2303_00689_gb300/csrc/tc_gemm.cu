@@ -48,6 +48,7 @@ namespace kx {
 
 constexpr int kBM = 128, kBN = 128, kBK = 64, kStages = 5;
 constexpr int kChunk = 8;                    // k-tiles (512 K) per exact FP32 accumulation chunk
+constexpr int kSmallTiles = 152;             // tiles of 64 columns up to one per SM
 constexpr int kEpiWarps = 16;                // 4 lane quarters x 4 column groups of 32
 constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr int kTileBytesA = kBM * kBK * 2;   // 16 KB
@@ -87,20 +88,21 @@ __device__ __forceinline__ double scaled_sum(double alpha, float hi, float lo) {
 // row-contiguous stores of the tile and, for a symmetric result, of its transpose.
 // Every epilogue warp reaches the named barrier; the global stores run only when no
 // wait of any CTA expired.
-__device__ __forceinline__ void write_tile(double* tile, const float (&hi)[32], const float (&lo)[32], bool ok,
+template <int BN>
+__device__ __forceinline__ void write_tile(double* tile, const float (&hi)[BN / 4], const float (&lo)[BN / 4], bool ok,
                                            int quarter, int cg, int lane, int m0, int n0, int M, int N, double alpha,
                                            double* __restrict__ C, int ldc, int sym, int beta, int* err) {
-  constexpr int kLdT = kBN + 1;                      // padded row: conflict-free transposed reads
+  constexpr int kLdT = BN + 1;                      // padded row: conflict-free transposed reads
   if (ok) {
     const int rl = quarter * 32 + lane;
 #pragma unroll
-    for (int j = 0; j < 32; ++j) tile[rl * kLdT + cg * 32 + j] = scaled_sum(alpha, hi[j], lo[j]);
+    for (int j = 0; j < BN / 4; ++j) tile[rl * kLdT + cg * (BN / 4) + j] = scaled_sum(alpha, hi[j], lo[j]);
   }
   asm volatile("bar.sync 1, %0;" ::"r"(kEpiWarps * 32) : "memory");
   if (!ok || *(volatile int*)err != 0) return;
   const int t = threadIdx.x - 64;
-  for (int idx = t; idx < kBM * kBN; idx += kEpiWarps * 32) {
-    const int rr = idx / kBN, cc = idx - rr * kBN;
+  for (int idx = t; idx < kBM * BN; idx += kEpiWarps * 32) {
+    const int rr = idx / BN, cc = idx - rr * BN;
     const int row = m0 + rr, col = n0 + cc;
     if (row < M && col < N && !(sym && row > col)) {
       const size_t at = (size_t)row * ldc + col;
@@ -109,7 +111,7 @@ __device__ __forceinline__ void write_tile(double* tile, const float (&hi)[32], 
   }
   if (sym) {
     // C[col][row] for row < col: rows of the output are columns of the tile
-    for (int idx = t; idx < kBM * kBN; idx += kEpiWarps * 32) {
+    for (int idx = t; idx < kBM * BN; idx += kEpiWarps * 32) {
       const int cr = idx / kBM, rc = idx - cr * kBM;   // output row n0 + cr, column m0 + rc
       const int row = m0 + rc, col = n0 + cr;
       if (row < M && col < N && row < col) {
@@ -254,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[b]);
     }
-    write_tile((double*)base, hi, lo, ok && total > 0, quarter, cg, lane, m0, n0, M, N, alpha, C, ldc, sym, beta, err);
+    write_tile<kBN>((double*)base, hi, lo, ok && total > 0, quarter, cg, lane, m0, n0, M, N, alpha, C, ldc, sym, beta, err);
   }
   tc_fence_before();
   __syncthreads();
@@ -305,7 +307,7 @@ __device__ __forceinline__ uint64_t grouped_desc(uint32_t addr) {
     return smem_desc_sw64(addr);
 }
 
-template <int S, int BK>
+template <int S, int BK, int BN>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_gemm_grouped_kernel(const __grid_constant__ TcMaps maps, int M, int N, int K, double alpha,
                            double* __restrict__ C, int ldc, int sym, int beta, int* err, const int* gate,
@@ -313,8 +315,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   using Cfg = GroupedCfg<S, BK>;
   constexpr int T = Cfg::kTile, kStages = Cfg::kStages, kStageBytes = Cfg::kStageBytes;
   if (gate && *gate == 0) return;      // whole CTA, before any barrier or TMEM use
-  const int bi = blockIdx.y, bj = blockIdx.x;
-  if (sym && bi > bj) return;
+  const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * BN;
+  if (sym && m0 >= n0 + BN) return;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(base + kStages * kStageBytes);
@@ -324,7 +326,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = bi * kBM, n0 = bj * kBN;
   const int ktiles_all = (K + BK - 1) / BK;
   const int kt0 = (kt_split > 0) ? (int)blockIdx.z * kt_split : 0;
   int ktiles = (kt_split > 0) ? min(kt_split, ktiles_all - kt0) : ktiles_all;
@@ -345,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(4 * kBN)
+                 "r"(4 * BN)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -383,14 +384,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      const uint32_t idesc = make_idesc(kBM, kBN);
+      const uint32_t idesc = make_idesc(kBM, BN);
       bool ok = true;
       for (int c = 0; c < nchunks && ok; ++c) {
         const int b = c & 1;
         if (!mbar_wait(&acc_empty[b], ((uint32_t)(c >> 1) & 1u) ^ 1u, err)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d0 = tmem + (uint32_t)(b * kBN);
-        const uint32_t d1 = tmem + (uint32_t)((2 + b) * kBN);
+        const uint32_t d0 = tmem + (uint32_t)(b * BN);
+        const uint32_t d1 = tmem + (uint32_t)((2 + b) * BN);
         const int it0 = c * Cfg::kChunkTiles;
         const int it1 = (it0 + Cfg::kChunkTiles < ktiles) ? it0 + Cfg::kChunkTiles : ktiles;
         for (int it = it0; it < it1; ++it) {
@@ -424,9 +425,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // epilogue warps: fold both accumulators of each chunk into double-float registers
     const int quarter = warp & 3;
     const int cg = (warp - 2) >> 2;
-    float hi[32], lo[32];
+    constexpr int kCols = BN / 4;
+    float hi[kCols], lo[kCols];
 #pragma unroll
-    for (int j = 0; j < 32; ++j) { hi[j] = 0.0f; lo[j] = 0.0f; }
+    for (int j = 0; j < kCols; ++j) { hi[j] = 0.0f; lo[j] = 0.0f; }
     bool ok = true;
     for (int c = 0; c < nchunks; ++c) {
       const int b = c & 1;
@@ -436,12 +438,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_after();
       const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
+      for (int h = 0; h < kCols / 8; ++h) {
         uint32_t r[8];
-        tmem_ld8(tmem + lane_base + (uint32_t)(b * kBN + cg * 32 + h * 8), r);
+        tmem_ld8(tmem + lane_base + (uint32_t)(b * BN + cg * kCols + h * 8), r);
 #pragma unroll
         for (int j = 0; j < 8; ++j) twosum_acc(hi[h * 8 + j], lo[h * 8 + j], __uint_as_float(r[j]));
-        tmem_ld8(tmem + lane_base + (uint32_t)((2 + b) * kBN + cg * 32 + h * 8), r);
+        tmem_ld8(tmem + lane_base + (uint32_t)((2 + b) * BN + cg * kCols + h * 8), r);
 #pragma unroll
         for (int j = 0; j < 8; ++j) twosum_acc(hi[h * 8 + j], lo[h * 8 + j], __uint_as_float(r[j]));
       }
@@ -449,12 +451,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[b]);
     }
-    write_tile((double*)base, hi, lo, ok && ktiles > 0, quarter, cg, lane, m0, n0, M, N, alpha, C, ldc, sym, beta, err);
+    write_tile<BN>((double*)base, hi, lo, ok && ktiles > 0, quarter, cg, lane, m0, n0, M, N, alpha, C, ldc, sym, beta, err);
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(4 * kBN) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(4 * BN) : "memory");
   }
 }
 
@@ -963,23 +965,30 @@ void tc_gemm(cudaStream_t s, const TcWork& w, int slotA, int slotB, int terms, d
   count_launch();
 }
 
-template <int S, int BK>
-static void grouped_attribute() {
+template <int S, int BK, int BN>
+static void grouped_run(cudaStream_t s, const TcMaps& maps, int M, int N, int K, double alpha, double* C, int ldc,
+                        int sym, int beta, int* err, const int* gate, int kt_split, int z, long long zstride) {
   static PerDeviceOnce flag;
   once_per_device(flag, [] {
-    return cudaFuncSetAttribute(tc_gemm_grouped_kernel<S, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(tc_gemm_grouped_kernel<S, BK, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 GroupedCfg<S, BK>::kSmem) == cudaSuccess;
   });
+  dim3 grid((N + BN - 1) / BN, (M + kBM - 1) / kBM, z);
+  tc_gemm_grouped_kernel<S, BK, BN><<<grid, kThreads, GroupedCfg<S, BK>::kSmem, s>>>(
+      maps, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, zstride);
+  count_launch();
 }
 
+// Tiles of 64 columns while twice as many fit the SMs: a small product's time is mostly
+// the epilogue of a tile (the same boxes are loaded, their second half unused).  n = 240
+// and 720: DMPT 589 -> 464 and 794 -> 663 us a step, back-transformation 454 -> 414, 895 -> 771.
 template <int S, int BK>
 static void grouped_launch(cudaStream_t s, const TcMaps& maps, int M, int N, int K, double alpha, double* C, int ldc,
                            int sym, int beta, int* err, const int* gate, int kt_split, int z, long long zstride) {
-  grouped_attribute<S, BK>();
-  dim3 grid((N + kBN - 1) / kBN, (M + kBM - 1) / kBM, z);
-  tc_gemm_grouped_kernel<S, BK><<<grid, kThreads, GroupedCfg<S, BK>::kSmem, s>>>(
-      maps, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, zstride);
-  count_launch();
+  if ((long long)((M + kBM - 1) / kBM) * ((N + 63) / 64) * z <= kSmallTiles)
+    grouped_run<S, BK, 64>(s, maps, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
+  else
+    grouped_run<S, BK, kBN>(s, maps, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
 }
 
 void tc_gemm_grouped(cudaStream_t s, const TcWork& w, int slotA, int slotB, double alpha, double* C, int sym,
