@@ -48,7 +48,7 @@ namespace kx {
 
 constexpr int kBM = 128, kBN = 128, kBK = 64, kStages = 5;
 constexpr int kChunk = 8;                    // k-tiles (512 K) per exact FP32 accumulation chunk
-constexpr int kSmallTiles = 152;             // tiles of 64 columns up to one per SM
+constexpr int kSmallTiles = 152;             // narrow tiles up to one per SM
 constexpr int kEpiWarps = 16;                // 4 lane quarters x 4 column groups of 32
 constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr int kTileBytesA = kBM * kBK * 2;   // 16 KB
@@ -122,13 +122,14 @@ __device__ __forceinline__ void write_tile(double* tile, const float (&hi)[BN / 
   }
 }
 
+template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_gemm_kernel(const __grid_constant__ TcMaps maps, SegTable seg, int M, int N, int K, double alpha,
                    double* __restrict__ C, int ldc, int sym, int beta, int* err, const int* gate, int kt_split,
                    long long c_zstride) {
   if (gate && *gate == 0) return;      // whole CTA, before any barrier or TMEM use
-  const int bi = blockIdx.y, bj = blockIdx.x;
-  if (sym && bi > bj) return;
+  const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * BN;
+  if (sym && m0 >= n0 + BN) return;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = base;
@@ -140,7 +141,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = bi * kBM, n0 = bj * kBN;
   // split-K (kt_split > 0): CTA z takes k-tiles [z kt_split, (z + 1) kt_split) and
   // writes its partial product to C + z c_zstride
   const int ktiles_all = (K + kBK - 1) / kBK;
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(2 * kBN)
+                 "r"(2 * BN)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -202,13 +202,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 1) {
     if (lane == 0) {
       // MMA issuer: chunk c accumulates into TMEM buffer c & 1
-      const uint32_t idesc = make_idesc(kBM, kBN);
+      const uint32_t idesc = make_idesc(kBM, BN);
       bool ok = true;
       for (int c = 0; c < nchunks && ok; ++c) {
         const int b = c & 1;
         if (!mbar_wait(&acc_empty[b], ((uint32_t)(c >> 1) & 1u) ^ 1u, err)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t dst = tmem + (uint32_t)(b * kBN);
+        const uint32_t dst = tmem + (uint32_t)(b * BN);
         const int sg = c / cps, cc = c % cps;
         const int it0 = sg * ktiles + cc * kChunk;
         const int seg_end = (sg + 1) * ktiles;
@@ -235,9 +235,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // epilogue warps: fold each chunk into double-float accumulators
     const int quarter = warp & 3;              // TMEM lanes 32 * quarter ...
     const int cg = (warp - 2) >> 2;            // columns 32 * cg ...
-    float hi[32], lo[32];
+    constexpr int kCols = BN / 4;
+    float hi[kCols], lo[kCols];
 #pragma unroll
-    for (int j = 0; j < 32; ++j) { hi[j] = 0.0f; lo[j] = 0.0f; }
+    for (int j = 0; j < kCols; ++j) { hi[j] = 0.0f; lo[j] = 0.0f; }
     bool ok = true;
     for (int c = 0; c < nchunks; ++c) {
       const int b = c & 1;
@@ -246,22 +247,22 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!got) { ok = false; break; }
       tc_fence_after();
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t r[16];
-        tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * kBN + cg * 32 + h * 16), r);
+      for (int h = 0; h < kCols / 8; ++h) {
+        uint32_t r[8];
+        tmem_ld8(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN + cg * kCols + h * 8), r);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) twosum_acc(hi[h * 16 + j], lo[h * 16 + j], __uint_as_float(r[j]));
+        for (int j = 0; j < 8; ++j) twosum_acc(hi[h * 8 + j], lo[h * 8 + j], __uint_as_float(r[j]));
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[b]);
     }
-    write_tile<kBN>((double*)base, hi, lo, ok && total > 0, quarter, cg, lane, m0, n0, M, N, alpha, C, ldc, sym, beta, err);
+    write_tile<BN>((double*)base, hi, lo, ok && total > 0, quarter, cg, lane, m0, n0, M, N, alpha, C, ldc, sym, beta, err);
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kBN) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
   }
 }
 
@@ -912,13 +913,35 @@ bool tc_ready(const TcWork& w) { return w.base && ((TcBuffers*)w.base)->maps_ok;
 
 int* tc_error_flag(const TcWork& w) { return w.base ? ((TcBuffers*)w.base)->err : nullptr; }
 
-// the opt-in shared-memory size is a per-device attribute of the kernel
-static void set_smem_attribute() {
+// Tiles of 32 or 64 columns while as many fit the SMs: a small product's time is mostly the
+// epilogue of a tile (the same boxes are loaded, the rest of them unused).  n = 240 and
+// 720: DMPT 589 -> 464 and 794 -> 663 us a step, back-transformation 454 -> 414, 895 -> 771.
+static int tile_columns(int M, int N, int z) {
+  auto fits = [&](int bn) { return (long long)((M + kBM - 1) / kBM) * ((N + bn - 1) / bn) * z <= kSmallTiles; };
+  return fits(32) ? 32 : (fits(64) ? 64 : kBN);
+}
+template <int BN>
+static void exact_run(cudaStream_t s, const TcMaps& maps, const SegTable& seg, int M, int N, int K, double alpha,
+                      double* C, int ldc, int sym, int beta, int* err, const int* gate, int kt_split, int z,
+                      long long zstride) {
   static PerDeviceOnce flag;
   once_per_device(flag, [] {
-    return cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) ==
+    return cudaFuncSetAttribute(tc_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) ==
            cudaSuccess;
   });
+  dim3 grid((N + BN - 1) / BN, (M + kBM - 1) / kBM, z);
+  tc_gemm_kernel<BN><<<grid, kThreads, kSmemBytes, s>>>(maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate,
+                                                       kt_split, zstride);
+  count_launch();
+}
+static void exact_launch(cudaStream_t s, const TcMaps& maps, const SegTable& seg, int M, int N, int K, double alpha,
+                         double* C, int ldc, int sym, int beta, int* err, const int* gate, int kt_split, int z,
+                         long long zstride) {
+  switch (tile_columns(M, N, z)) {
+    case 32: return exact_run<32>(s, maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
+    case 64: return exact_run<64>(s, maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
+    default: return exact_run<kBN>(s, maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
+  }
 }
 
 void tc_split(cudaStream_t s, const TcWork& w, int slot, const double* X, int slices, int transpose,
@@ -943,7 +966,6 @@ void tc_split(cudaStream_t s, const TcWork& w, int slot, const double* X, int sl
 void tc_gemm(cudaStream_t s, const TcWork& w, int slotA, int slotB, int terms, double alpha, double* C, int sym,
              const int* gate) {
   TcBuffers* tb = (TcBuffers*)w.base;
-  set_smem_attribute();
   TcMaps maps;
   for (int k = 0; k < kTcMaxSlices; ++k) {
     maps.a[k] = tb->map[slotA][k];
@@ -960,9 +982,7 @@ void tc_gemm(cudaStream_t s, const TcWork& w, int slotA, int slotB, int terms, d
       ++seg.nseg;
     }
   int n = tb->n;
-  dim3 grid((n + kBN - 1) / kBN, (n + kBM - 1) / kBM);
-  tc_gemm_kernel<<<grid, kThreads, kSmemBytes, s>>>(maps, seg, n, n, n, alpha, C, n, sym, 0, tb->err, gate, 0, 0);
-  count_launch();
+  exact_launch(s, maps, seg, n, n, n, alpha, C, n, sym, 0, tb->err, gate, 0, 1, 0);
 }
 
 template <int S, int BK, int BN>
@@ -979,16 +999,17 @@ static void grouped_run(cudaStream_t s, const TcMaps& maps, int M, int N, int K,
   count_launch();
 }
 
-// Tiles of 64 columns while twice as many fit the SMs: a small product's time is mostly
-// the epilogue of a tile (the same boxes are loaded, their second half unused).  n = 240
-// and 720: DMPT 589 -> 464 and 794 -> 663 us a step, back-transformation 454 -> 414, 895 -> 771.
 template <int S, int BK>
 static void grouped_launch(cudaStream_t s, const TcMaps& maps, int M, int N, int K, double alpha, double* C, int ldc,
                            int sym, int beta, int* err, const int* gate, int kt_split, int z, long long zstride) {
-  if ((long long)((M + kBM - 1) / kBM) * ((N + 63) / 64) * z <= kSmallTiles)
-    grouped_run<S, BK, 64>(s, maps, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
-  else
-    grouped_run<S, BK, kBN>(s, maps, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
+  switch (tile_columns(M, N, z)) {
+    case 32:
+      return grouped_run<S, BK, 32>(s, maps, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
+    case 64:
+      return grouped_run<S, BK, 64>(s, maps, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
+    default:
+      return grouped_run<S, BK, kBN>(s, maps, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
+  }
 }
 
 void tc_gemm_grouped(cudaStream_t s, const TcWork& w, int slotA, int slotB, double alpha, double* C, int sym,
@@ -1075,7 +1096,6 @@ void tc_split_rc(cudaStream_t s, int rows, int cols, const double* X, int ldx, i
 int tc_gemm_rc(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda, size_t astride,
                const __nv_bfloat16* Bbase, int ldb, size_t bstride, int terms, double alpha, double* C, int ldc,
                int beta, int* err) {
-  set_smem_attribute();
   int slices = (terms == 10) ? 4 : (terms == 6) ? 3 : (terms == 3) ? 2 : 1;
   TcMaps maps;
   for (int a = 0; a < kTcMaxSlices; ++a) {
@@ -1091,10 +1111,7 @@ int tc_gemm_rc(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, 
       seg.b[seg.nseg] = d - a;
       ++seg.nseg;
     }
-  dim3 grid((N + kBN - 1) / kBN, (M + kBM - 1) / kBM);
-  tc_gemm_kernel<<<grid, kThreads, kSmemBytes, s>>>(maps, seg, M, N, K, alpha, C, ldc, 0, beta, err, nullptr,
-                                                     0, 0);
-  count_launch();
+  exact_launch(s, maps, seg, M, N, K, alpha, C, ldc, 0, beta, err, nullptr, 0, 1, 0);
   return 0;
 }
 
@@ -1104,7 +1121,6 @@ int tc_gemm_rc(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, 
 int tc_gemm_rc_splitk(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda, size_t astride,
                       const __nv_bfloat16* Bbase, int ldb, size_t bstride, int terms, double alpha, double* P,
                       int ldp, int splits, int* err) {
-  set_smem_attribute();
   int slices = (terms == 10) ? 4 : (terms == 6) ? 3 : (terms == 3) ? 2 : 1;
   TcMaps maps;
   for (int a = 0; a < kTcMaxSlices; ++a) {
@@ -1124,10 +1140,7 @@ int tc_gemm_rc_splitk(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* 
   int per = (ktiles + splits - 1) / splits;
   per = ((per + kChunk - 1) / kChunk) * kChunk;          // whole exact-sum chunks
   const int z = (ktiles + per - 1) / per;
-  dim3 grid((N + kBN - 1) / kBN, (M + kBM - 1) / kBM, z);
-  tc_gemm_kernel<<<grid, kThreads, kSmemBytes, s>>>(maps, seg, M, N, K, alpha, P, ldp, 0, 0, err, nullptr, per,
-                                                     (long long)M * ldp);
-  count_launch();
+  exact_launch(s, maps, seg, M, N, K, alpha, P, ldp, 0, 0, err, nullptr, per, z, (long long)M * ldp);
   return z;
 }
 
@@ -1171,7 +1184,6 @@ void tc_split_pair(cudaStream_t s, int n, int ld, const double* A, const double*
 
 void tc_gemm_on_maps(cudaStream_t s, int n, const CUtensorMap* mapsA, const CUtensorMap* mapsB, int terms,
                      double alpha, double* C, int sym, int* err) {
-  set_smem_attribute();
   TcMaps maps;
   for (int k = 0; k < kTcMaxSlices; ++k) {
     maps.a[k] = mapsA[k];
@@ -1186,9 +1198,7 @@ void tc_gemm_on_maps(cudaStream_t s, int n, const CUtensorMap* mapsA, const CUte
       seg.b[seg.nseg] = d - a;
       ++seg.nseg;
     }
-  dim3 grid((n + kBN - 1) / kBN, (n + kBM - 1) / kBM);
-  tc_gemm_kernel<<<grid, kThreads, kSmemBytes, s>>>(maps, seg, n, n, n, alpha, C, n, sym, 0, err, nullptr, 0, 0);
-  count_launch();
+  exact_launch(s, maps, seg, n, n, n, alpha, C, n, sym, 0, err, nullptr, 0, 1, 0);
 }
 
 }  // namespace kx
