@@ -340,6 +340,7 @@ static bool concurrent(const sim_handle* h) { return h->side && !h->prof; }
 // mu (eq. 8; they need the eigenvalues only) run on the side stream while the
 // eigenvectors are formed, and the caller joins before the density
 static int eig(sim_handle* h, bool fermi_side = false) {
+  h->tw.wide = h->shared;
   phase_begin(h, PH_TRIDIAG);
   int st = eig_tridiagonalize(h->stream, h->n, h->Fock, h->ew, &h->sc->status, h->sms, mixed(h), h->shared);
   phase_end(h);

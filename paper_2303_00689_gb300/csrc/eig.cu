@@ -943,12 +943,13 @@ static int eig_backtransform_tc(cudaStream_t s, int n, double* Q, EigWork& w, co
     double* Zs = Zt + c0;                                // n x m, ld n
     tc_split_rows(s, n, m, Zs, n, 4, sZ, ldm, stride);
     const int parts = tc_gemm_grouped_rc_splitk(s, n, kb, m, sZ, ldm, stride, sc.vs + (size_t)b * sc.vs_blk, ldm,
-                                                sc.vs_slice, 1.0, sc.part, kBtBlockTc, kBtSplitK, err);   // U parts
+                                                sc.vs_slice, 1.0, sc.part, kBtBlockTc, kBtSplitK, err,
+                                                tw.wide);   // U parts
     if (parts <= 0) return -1;
     const int ldk = tc_ld(kb);                           // U slices fit the slot: kb <= n
     tc_reduce_split_rows(s, n, kb, sc.part, parts, kBtBlockTc, 4, sU, ldk, stride);
     if (tc_gemm_grouped_rc(s, n, m, kb, sU, ldk, stride, sc.ys + (size_t)b * sc.ys_blk, kBtBlockTc, sc.ys_slice,
-                           -1.0, Zs, n, 1, err) != 0)                                        // Zs -= U Y_b
+                           -1.0, Zs, n, 1, err, tw.wide) != 0)                                        // Zs -= U Y_b
       return -1;
   }
   transpose_sq(s, n, Zt, Q);

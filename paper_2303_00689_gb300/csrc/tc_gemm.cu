@@ -14,7 +14,7 @@
 // exact in the FP32 tensor-core accumulator.  The product keeps the slice
 // pairs with a + b < slices (1, 3, 6 or 10 terms for 1-4 slices).
 //
-// One CTA computes a 128 x 128 tile with 18 warps:
+// One CTA computes a 128 x 128 tile (128 x 64 or 128 x 32 while SMs are free) with 18 warps:
 //   warp 0 / lane 0 : TMA producer (128B-swizzled boxes of 128 rows x 64 K)
 //   warp 1          : allocates / frees TMEM; lane 0 issues tcgen05.mma
 //                     (M = 128, N = 128, K = 16 slices)
@@ -915,8 +915,11 @@ int* tc_error_flag(const TcWork& w) { return w.base ? ((TcBuffers*)w.base)->err 
 
 // Tiles of 32 or 64 columns while as many fit the SMs: a small product's time is mostly the
 // epilogue of a tile (the same boxes are loaded, the rest of them unused).  n = 240 and
-// 720: DMPT 589 -> 464 and 794 -> 663 us a step, back-transformation 454 -> 414, 895 -> 771.
-static int tile_columns(int M, int N, int z) {
+// 720: DMPT 589 -> 382 and 794 -> 582 us a step, back-transformation 454 -> 393, 895 -> 704;
+// n = 250, exact product: 65 -> 49 us.  Not beside other handles (wide), where the loads of
+// more tiles cost a batch of 16 cages 3 %.
+static int tile_columns(int M, int N, int z, bool wide) {
+  if (wide) return kBN;
   auto fits = [&](int bn) { return (long long)((M + kBM - 1) / kBM) * ((N + bn - 1) / bn) * z <= kSmallTiles; };
   return fits(32) ? 32 : (fits(64) ? 64 : kBN);
 }
@@ -937,7 +940,7 @@ static void exact_run(cudaStream_t s, const TcMaps& maps, const SegTable& seg, i
 static void exact_launch(cudaStream_t s, const TcMaps& maps, const SegTable& seg, int M, int N, int K, double alpha,
                          double* C, int ldc, int sym, int beta, int* err, const int* gate, int kt_split, int z,
                          long long zstride) {
-  switch (tile_columns(M, N, z)) {
+  switch (tile_columns(M, N, z, false)) {
     case 32: return exact_run<32>(s, maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
     case 64: return exact_run<64>(s, maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
     default: return exact_run<kBN>(s, maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
@@ -1001,8 +1004,8 @@ static void grouped_run(cudaStream_t s, const TcMaps& maps, int M, int N, int K,
 
 template <int S, int BK>
 static void grouped_launch(cudaStream_t s, const TcMaps& maps, int M, int N, int K, double alpha, double* C, int ldc,
-                           int sym, int beta, int* err, const int* gate, int kt_split, int z, long long zstride) {
-  switch (tile_columns(M, N, z)) {
+                           int sym, int beta, int* err, const int* gate, int kt_split, int z, long long zstride, bool wide) {
+  switch (tile_columns(M, N, z, wide)) {
     case 32:
       return grouped_run<S, BK, 32>(s, maps, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
     case 64:
@@ -1021,7 +1024,7 @@ void tc_gemm_grouped(cudaStream_t s, const TcWork& w, int slotA, int slotB, doub
     maps.b[k] = tb->map[slotB][k];
   }
   const int n = tb->n;
-  grouped_launch<3, 64>(s, maps, n, n, n, alpha, C, n, sym, 0, tb->err, gate, 0, 1, 0);
+  grouped_launch<3, 64>(s, maps, n, n, n, alpha, C, n, sym, 0, tb->err, gate, 0, 1, 0, w.wide);
 }
 
 void tc_gemm_grouped4(cudaStream_t s, const TcWork& w, int slotA, int slotB, double alpha, double* C, int sym,
@@ -1033,7 +1036,7 @@ void tc_gemm_grouped4(cudaStream_t s, const TcWork& w, int slotA, int slotB, dou
     maps.b[k] = tb->map64[slotB][k];
   }
   const int n = tb->n;
-  grouped_launch<4, 32>(s, maps, n, n, n, alpha, C, n, sym, 0, tb->err, gate, 0, 1, 0);
+  grouped_launch<4, 32>(s, maps, n, n, n, alpha, C, n, sym, 0, tb->err, gate, 0, 1, 0, w.wide);
 }
 
 static bool grouped_rc_maps(TcMaps* maps, int M, int N, int K, const __nv_bfloat16* Abase, int lda, size_t astride,
@@ -1047,16 +1050,16 @@ static bool grouped_rc_maps(TcMaps* maps, int M, int N, int K, const __nv_bfloat
 
 int tc_gemm_grouped_rc(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda, size_t astride,
                        const __nv_bfloat16* Bbase, int ldb, size_t bstride, double alpha, double* C, int ldc,
-                       int beta, int* err) {
+                       int beta, int* err, bool wide) {
   TcMaps maps;
   if (!grouped_rc_maps(&maps, M, N, K, Abase, lda, astride, Bbase, ldb, bstride)) return -1;
-  grouped_launch<4, 32>(s, maps, M, N, K, alpha, C, ldc, 0, beta, err, nullptr, 0, 1, 0);
+  grouped_launch<4, 32>(s, maps, M, N, K, alpha, C, ldc, 0, beta, err, nullptr, 0, 1, 0, wide);
   return 0;
 }
 
 int tc_gemm_grouped_rc_splitk(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda,
                               size_t astride, const __nv_bfloat16* Bbase, int ldb, size_t bstride, double alpha,
-                              double* P, int ldp, int splits, int* err) {
+                              double* P, int ldp, int splits, int* err, bool wide) {
   TcMaps maps;
   if (!grouped_rc_maps(&maps, M, N, K, Abase, lda, astride, Bbase, ldb, bstride)) return -1;
   constexpr int kCh = GroupedCfg<4, 32>::kChunkTiles;
@@ -1064,7 +1067,7 @@ int tc_gemm_grouped_rc_splitk(cudaStream_t s, int M, int N, int K, const __nv_bf
   int per = (ktiles + splits - 1) / splits;
   per = ((per + kCh - 1) / kCh) * kCh;                   // whole exact-sum chunks
   const int z = (ktiles + per - 1) / per;
-  grouped_launch<4, 32>(s, maps, M, N, K, alpha, P, ldp, 0, 0, err, nullptr, per, z, (long long)M * ldp);
+  grouped_launch<4, 32>(s, maps, M, N, K, alpha, P, ldp, 0, 0, err, nullptr, per, z, (long long)M * ldp, wide);
   return z;
 }
 

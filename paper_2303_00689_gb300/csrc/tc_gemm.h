@@ -13,6 +13,7 @@ enum TcSlot { kSlotQs = 0, kSlotQ = 1, kSlotQt = 2, kSlotT0 = 3, kSlotT1 = 4, kS
 
 struct TcWork {
   void* base = nullptr;   // host-side bookkeeping (tensor maps, piece pointers)
+  bool wide = false;      // beside other handles: wide tiles, the least work
   size_t bytes = 0;
 };
 size_t tc_work_bytes(int n);
@@ -42,10 +43,10 @@ void tc_gemm_grouped4(cudaStream_t s, const TcWork& w, int slotA, int slotB, dou
 // partial-product layout as tc_gemm_rc / tc_gemm_rc_splitk; < 0 on a tensor-map error
 int tc_gemm_grouped_rc(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda, size_t astride,
                        const __nv_bfloat16* Bbase, int ldb, size_t bstride, double alpha, double* C, int ldc,
-                       int beta, int* err);
+                       int beta, int* err, bool wide);
 int tc_gemm_grouped_rc_splitk(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda,
                               size_t astride, const __nv_bfloat16* Bbase, int ldb, size_t bstride, double alpha,
-                              double* P, int ldp, int splits, int* err);
+                              double* P, int ldp, int splits, int* err, bool wide);
 
 // Building blocks on caller-provided buffers (used by the allocation-free entry point)
 int tc_ld(int n);                                                   // padded slice row length
