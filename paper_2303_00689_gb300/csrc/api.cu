@@ -73,7 +73,7 @@ struct sim_handle {
   // and energy, forces and dipole (during the Krylov kernel); forked from and
   // joined to `stream` by events, so graph capture records both branches
   cudaStream_t side = nullptr;
-  cudaEvent_t fork_ev[2] = {}, join_ev[2] = {};
+  cudaEvent_t fork_ev[3] = {}, join_ev[3] = {};
   sim_config cfg;
   ElemTable tab;
   int N = 0, n = 0, npair = 0, nocc = 0, mmax = 0;
@@ -341,10 +341,21 @@ static bool concurrent(const sim_handle* h) { return h->side && !h->prof; }
 // eigenvectors are formed, and the caller joins before the density
 static int eig(sim_handle* h, bool fermi_side = false) {
   h->tw.wide = h->shared;
+  const TcWork* tw = mixed(h) ? &h->tw : nullptr;
+  const Tc64Work* t64 = h->t64.base && h->n > kBt64Above ? &h->t64 : nullptr;
   phase_begin(h, PH_TRIDIAG);
   int st = eig_tridiagonalize(h->stream, h->n, h->Fock, h->ew, &h->sc->status, h->sms, mixed(h), h->shared);
   phase_end(h);
   if (st != 0) return fail(SIM_EINTERNAL, "tridiagonalisation launch failed (code " + std::to_string(st) + ")");
+  // the back-transformation's half that needs the reflectors only, beside the eigenpairs
+  // of T (not beside other handles, which have the idle SMs)
+  const bool split = concurrent(h) && !h->shared && eig_backtransform_splits(h->n);
+  int bt = 0;
+  if (split) {
+    fork_side(h, 2);
+    bt = eig_backtransform_prepare(h->side, h->n, h->ew, tw, t64);
+    cudaEventRecord(h->join_ev[2], h->side);
+  }
   phase_begin(h, PH_BISECT);
   eig_bisect(h->stream, h->n, h->eps, h->ew, 1e-12, mixed(h), h->shared);
   phase_end(h);
@@ -356,8 +367,8 @@ static int eig(sim_handle* h, bool fermi_side = false) {
   eig_vectors(h->stream, h->n, h->eps, h->Q, h->ew, mixed(h), h->shared);
   phase_end(h);
   phase_begin(h, PH_BACKTR);
-  const int bt = eig_backtransform(h->stream, h->n, h->Q, h->ew, mixed(h) ? &h->tw : nullptr,
-                                   h->t64.base && h->n > kBt64Above ? &h->t64 : nullptr);
+  if (split) cudaStreamWaitEvent(h->stream, h->join_ev[2], 0);
+  if (bt == 0) bt = eig_backtransform(h->stream, h->n, h->Q, h->ew, tw, t64, split);
   phase_end(h);
   if (bt != 0) return fail(SIM_EINTERNAL, "back-transformation: tensor map encoding failed");
   return SIM_OK;
@@ -909,7 +920,7 @@ static int create_handle(const sim_config* cfg, const sim_param_table* table, in
     cudaGetLastError();
     h->side = nullptr;
   }
-  for (int k = 0; k < 2 && h->side; ++k)
+  for (int k = 0; k < 3 && h->side; ++k)
     if (cudaEventCreateWithFlags(&h->fork_ev[k], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->join_ev[k], cudaEventDisableTiming) != cudaSuccess) {
       cudaGetLastError();
@@ -1567,7 +1578,7 @@ void sim_destroy(sim_handle* h) {
     cudaStreamSynchronize(h->side);
     cudaStreamDestroy(h->side);
   }
-  for (int k = 0; k < 2; ++k) {
+  for (int k = 0; k < 3; ++k) {
     if (h->fork_ev[k]) cudaEventDestroy(h->fork_ev[k]);
     if (h->join_ev[k]) cudaEventDestroy(h->join_ev[k]);
   }

@@ -652,11 +652,19 @@ struct BtScratch;
 static size_t bt_scratch_layout(int n, void* base, BtScratch* out);
 struct Bt64Scratch;
 static size_t bt64_scratch(int n, void* base, Bt64Scratch* out);
+static size_t bt_doubles(int n) {
+  return std::max((bt_scratch_layout(n, nullptr, nullptr) + 7) / 8, bt64_scratch(n, nullptr, nullptr) / 8);
+}
+// Up to this size the half of the back-transformation that needs no eigenvectors (Gram
+// matrices, T factors, T^T V, slices) runs on the side stream during multisection and
+// inverse iteration, which leave most SMs idle there.  Above, the kernels slow one
+// another by as much as is gained (3360).  C60 step 2.90 -> 2.64 ms, C120 4.84 -> 4.57, 574 basis
+// functions in FP64 9.82 -> 9.58.
+constexpr int kBtSideMax = 640;
 // the inverse-iteration workspace (5 n^2) also serves as back-transformation scratch
 static size_t lu_doubles(int n) {
   const size_t a = 5 * (size_t)n * n;
-  const size_t b = (bt_scratch_layout(n, nullptr, nullptr) + 7) / 8;
-  return std::max({a, b, bt64_scratch(n, nullptr, nullptr) / 8});
+  return std::max(a, bt_doubles(n));
 }
 
 // One layout for sizing and binding.  Every buffer starts on a 256-byte
@@ -679,6 +687,8 @@ static size_t eig_layout(int n, void* base, EigWork* w) {
   double* tau = take(n);
   double* pbuf = take(4 * (size_t)n);
   double* lu = take(lu_doubles(n));
+  // back-transformation scratch: of its own where its preparation runs beside the inverse iteration
+  double* bt = (n <= kBtSideMax) ? take(bt_doubles(n)) : lu;
   double* Tm = take((size_t)tc_blocks(n) * kBtBlockTc * kBtBlockTc);   // T and Gram of every reflector block
   double* Gm = take((size_t)tc_blocks(n) * kBtBlockTc * kBtBlockTc);
   double* Wt = take((size_t)kBtBlockTc * n);
@@ -687,7 +697,7 @@ static size_t eig_layout(int n, void* base, EigWork* w) {
   double* bar = take(8);
   double* clus = take(((size_t)n * sizeof(int) + 7) / 8);
   if (w) {
-    w->A = A; w->Vst = Vst; w->d = d; w->e = e; w->e2 = e2; w->tau = tau; w->pbuf = pbuf; w->lu = lu;
+    w->A = A; w->Vst = Vst; w->d = d; w->e = e; w->e2 = e2; w->tau = tau; w->pbuf = pbuf; w->lu = lu; w->bt = bt;
     w->Tm = Tm; w->Gm = Gm; w->Wt = Wt; w->Wt2 = Wt2; w->scal = scal;
     w->bar = (unsigned*)bar;
     w->clus = (int*)clus;
@@ -912,16 +922,11 @@ static void bt_attributes() {
   });
 }
 
-static int eig_backtransform_tc(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork& tw) {
+static void bt_prepare_tc(cudaStream_t s, int n, EigWork& w) {
   bt_attributes();
-  const int nref = n - 2;
-  const int nblk = bt_blocks(n);
-  const size_t stride = tc_slot_stride(tw);
-  int* err = tc_error_flag(tw);
+  const int nref = n - 2, nblk = bt_blocks(n);
   BtScratch sc;
-  bt_scratch_layout(n, w.lu, &sc);
-  double* Zt = w.A;                      // tridiagonalisation workspace is free now
-  transpose_sq(s, n, Q, Zt);
+  bt_scratch_layout(n, w.bt, &sc);
   // Gram matrices and T factors of all blocks, then Y_b^T = V_b^T T_b, then slices
   gram_df_kernel<<<dim3((kBtBlockTc / 32) * (kBtBlockTc / 32), nblk), 256, 0, s>>>(n, nref, w.Vst, w.Gm);
   count_launch();
@@ -934,6 +939,17 @@ static int eig_backtransform_tc(cudaStream_t s, int n, double* Q, EigWork& w, co
   count_launch();
   tc_split_blocks(s, 0, n, nref, kBtBlockTc, w.Vst, sc.vs, sc.vs_blk, sc.vs_slice, 4);
   tc_split_blocks(s, 1, n, nref, kBtBlockTc, sc.yt, sc.ys, sc.ys_blk, sc.ys_slice, 4);
+}
+
+static int eig_backtransform_tc(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork& tw) {
+  const int nref = n - 2;
+  const int nblk = bt_blocks(n);
+  const size_t stride = tc_slot_stride(tw);
+  int* err = tc_error_flag(tw);
+  BtScratch sc;
+  bt_scratch_layout(n, w.bt, &sc);
+  double* Zt = w.A;                      // tridiagonalisation workspace is free now
+  transpose_sq(s, n, Q, Zt);
   __nv_bfloat16* sZ = tc_slot_base(tw, kSlotT0);
   __nv_bfloat16* sU = tc_slot_base(tw, kSlotT1);
   for (int b = nblk - 1; b >= 0; --b) {
@@ -979,15 +995,13 @@ static size_t bt64_scratch(int n, void* base, Bt64Scratch* out) {
   return 2 * u + uo + tc64_op_bytes(rt, kBtBlockTc);
 }
 
-static int eig_backtransform_tc64(cudaStream_t s, int n, double* Q, EigWork& w, const Tc64Work& tw) {
+static int bt_prepare_tc64(cudaStream_t s, int n, EigWork& w, const Tc64Work& tw) {
   constexpr int KB = kBtBlockTc;
   bt_attributes();
   const int nref = n - 2, nblk = bt_blocks(n);
   Bt64Scratch sc;
-  bt64_scratch(n, w.lu, &sc);
-  const Tc64Op V = tc64_slot(tw, 0, nref, n), Vt = tc64_slot(tw, 1, n, nref), Z = tc64_slot(tw, 2, n, n);
-  double* Zt = w.A;
-  transpose_sq(s, n, Q, Zt);
+  bt64_scratch(n, w.bt, &sc);
+  const Tc64Op V = tc64_slot(tw, 0, nref, n), Vt = tc64_slot(tw, 1, n, nref);
   tc64_cut_rows(s, V, 0, n, w.Vst, n);
   tc64_cut_cols(s, Vt, nref, w.Vst, n);
   if (tc64_gemm(s, nref, nref, 0, n, V, 0, V, 0, 0, 1.0, 0, w.Gm, KB, 1, KB, tw.err)) return -1;
@@ -995,6 +1009,17 @@ static int eig_backtransform_tc64(cudaStream_t s, int n, double* Q, EigWork& w, 
   tfactor_all_kernel<<<dim3(KB / kTfRows, nblk), 4 * kTfRows, kTfSmem, s>>>(nref, w.tau, w.Gm, w.Tm);
   count_launch();
   tc64_cut_rows(s, sc.t, 0, KB, w.Tm, KB);
+  return 0;
+}
+
+static int eig_backtransform_tc64(cudaStream_t s, int n, double* Q, EigWork& w, const Tc64Work& tw) {
+  constexpr int KB = kBtBlockTc;
+  const int nref = n - 2, nblk = bt_blocks(n);
+  Bt64Scratch sc;
+  bt64_scratch(n, w.bt, &sc);
+  const Tc64Op V = tc64_slot(tw, 0, nref, n), Vt = tc64_slot(tw, 1, n, nref), Z = tc64_slot(tw, 2, n, n);
+  double* Zt = w.A;
+  transpose_sq(s, n, Q, Zt);
   for (int b = nblk - 1; b >= 0; --b) {
     const int k0 = b * KB, kb = std::min(KB, nref - k0), c0 = k0 + 1, first = c0 & ~31;
     tc64_cut_rows(s, Z, first, n, Zt, n);
@@ -1008,7 +1033,20 @@ static int eig_backtransform_tc64(cudaStream_t s, int n, double* Q, EigWork& w, 
   return 0;
 }
 
-int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork* tw, const Tc64Work* t64) {
+bool eig_backtransform_splits(int n) { return n > 2 && n <= kBtSideMax; }
+
+int eig_backtransform_prepare(cudaStream_t s, int n, EigWork& w, const TcWork* tw, const Tc64Work* t64) {
+  if (n <= 2) return 0;
+  if (tw) {
+    bt_prepare_tc(s, n, w);
+    return 0;
+  }
+  return t64 ? bt_prepare_tc64(s, n, w, *t64) : 0;
+}
+
+int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork* tw, const Tc64Work* t64,
+                      bool prepared) {
+  if (!prepared && eig_backtransform_prepare(s, n, w, tw, t64) != 0) return -1;
   if (tw && n > 2) return eig_backtransform_tc(s, n, Q, w, *tw);
   if (t64 && n > 2) return eig_backtransform_tc64(s, n, Q, w, *t64);
   // 4. back-transformation, last block of reflectors first
@@ -1036,7 +1074,7 @@ int symmetric_eig(cudaStream_t s, int n, const double* F, double* eps, double* Q
   if (rc) return rc;
   eig_bisect(s, n, eps, w, 1e-12, false, false);
   eig_vectors(s, n, eps, Q, w, false, false);
-  eig_backtransform(s, n, Q, w, nullptr, nullptr);
+  eig_backtransform(s, n, Q, w, nullptr, nullptr, false);
   return 0;
 }
 

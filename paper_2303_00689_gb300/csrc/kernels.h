@@ -66,8 +66,9 @@ struct EigWork {
   double *d, *e, *e2, *tau;
   double *pbuf;         // 4 x n
   double *lu;           // 5 x n x n inverse-iteration workspace
+  double *bt;           // back-transformation scratch (lu in large systems)
   double *Tm, *Gm, *Wt, *Wt2;  // back-transform panels
-  unsigned* bar;        // 2 words grid barrier
+  unsigned* bar;        // 2 words grid barrier, 2 words check-in
   int* clus;            // cluster starts
   double* scal;         // scalars (Gershgorin bounds, norm)
 };
@@ -94,7 +95,12 @@ struct TcWork;
 struct Tc64Work;
 // tw != nullptr: the large products run on the tensor cores (mixed path)
 // returns nonzero when the tensor-core path could not encode its tensor maps
-int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork* tw, const Tc64Work* t64);
+int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork* tw, const Tc64Work* t64,
+                      bool prepared);
+// its half that needs no eigenvectors, which may run on another stream after the
+// tridiagonalisation (eig_backtransform_splits: its scratch is its own)
+bool eig_backtransform_splits(int n);
+int eig_backtransform_prepare(cudaStream_t s, int n, EigWork& w, const TcWork* tw, const Tc64Work* t64);
 int symmetric_eig(cudaStream_t s, int n, const double* F, double* eps, double* Q, EigWork& w,
                   int* status, int sm_count);
 
