@@ -658,7 +658,7 @@ static size_t bt_doubles(int n) {
 // Up to this size the half of the back-transformation that needs no eigenvectors (Gram
 // matrices, T factors, T^T V, slices) runs on the side stream during multisection and
 // inverse iteration, which leave most SMs idle there.  Above, the kernels slow one
-// another by as much as is gained (3360).  C60 step 2.90 -> 2.64 ms, C120 4.84 -> 4.57, 574 basis
+// another by more than is gained (1680: 22.95 -> 23.14 ms, FP64 45.4 -> 46.5).  C60 step 2.90 -> 2.64 ms, C120 4.84 -> 4.57, 574 basis
 // functions in FP64 9.82 -> 9.58.
 constexpr int kBtSideMax = 640;
 // the inverse-iteration workspace (5 n^2) also serves as back-transformation scratch
