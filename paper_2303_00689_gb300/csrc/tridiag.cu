@@ -242,8 +242,8 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
   // shared memory: own rows' (v, w), packets (SOLO), resident rows, own rows' x (two columns'),
   // sigma partials (two columns'), p.v partials per group, row partials
   RowVecs* PWr = (RowVecs*)smem;                                           // by row r
-  Packet* spk = (Packet*)(PWr + Rtot);                             // by column (SOLO)
-  double* rows = (double*)(spk + (SOLO ? n : 0));
+  Packet* spk = (Packet*)(PWr + Rtot);                             // by the column's parity, then row (SOLO)
+  double* rows = (double*)(spk + (SOLO ? 2 * n : 0));
   const int ms = n - g.k0 - 1;                                     // a row: columns k0 + 1 ..
   double* Xr = rows + (size_t)g.rs * ms;
   double* redB = Xr + 2 * Rtot;
@@ -332,7 +332,9 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
   for (int k = g.k0; k < g.k1; ++k) {
     if (b + rf * G <= k) ++rf;
     const int par = k & 1;
-    if (SOLO) bar_sync(1, NT + 32);                                // orders the packets before their readers
+    // orders the packets before their readers, and the readers of column k - 2's, which a group
+    // that is ahead overwrites at the end of this column
+    if (SOLO) bar_sync(1, NT + 32);
     // packets of column k - 1, of the columns j >= k (row k of the matrix: by symmetry a_{j,k})
     Packet q[CPL];
     if (rf < Rtot) {
@@ -352,7 +354,7 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
 #pragma unroll
           for (int c = 0; c < CPL; ++c) {
             const int j = t + NTG * c;
-            if (j >= k && j < n) q[c] = SOLO ? spk[j] : packet_load(in + j);
+            if (j >= k && j < n) q[c] = SOLO ? spk[(par ^ 1) * n + j] : packet_load(in + j);
           }
           if (SOLO) break;
           bool old = false;
@@ -474,7 +476,7 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
         const int i = b + r * G;
         const Packet o{((unsigned long long)__double_as_longlong(s) & ~kTag) | tag,
                        (unsigned long long)__double_as_longlong(entry(r, k + 1))};
-        if (SOLO) spk[i] = o;
+        if (SOLO) spk[par * n + i] = o;
         else packet_store(g.pk + ((size_t)l * 2 + par) * n + i, o);
       }
     }
@@ -1116,7 +1118,7 @@ static TriLaunch tri_launch(int n, int k0, int sm_count, bool few) {
   l.fn = s->fn;
   l.threads = s->ntg * s->rg + 32;
   l.packets = s->solo ? 0 : 2;
-  const size_t fixed = R * 16 + (s->solo ? (size_t)n * 16 : 0) + 2 * R * 8 + 2 * (size_t)s->ntg * 8 +
+  const size_t fixed = R * 16 + (s->solo ? 2 * (size_t)n * 16 : 0) + 2 * R * 8 + 2 * (size_t)s->ntg * 8 +
                        (size_t)s->rg * (s->ntg + 4) * 8 + R * (s->ntg / 32) * 8;
   const size_t most = (few && !s->solo) ? kTriSmemMax / 2 - 1024 : kTriSmemMax;
   const int live = tri_rows(n, k0, l.G);

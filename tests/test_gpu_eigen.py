@@ -1,0 +1,42 @@
+"""Eigenpairs of the Fock matrix where the kernels of the eigensolver exchange data: the same
+matrix gives the same bits every time, at the sizes where the exchange can go wrong."""
+import numpy as np
+import pytest
+
+import paper_2303_00689_gb300 as kx
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def lattice(n, precision, seed=1, **cfg):
+    """A lattice of n H atoms (one orbital each)."""
+    side = int(np.ceil(n ** (1.0 / 3.0)))
+    rng = np.random.default_rng(seed)
+    R = 1.9 * np.array([[i % side, i // side % side, i // side ** 2] for i in range(n)], dtype=float)
+    R += 0.1 * rng.normal(size=R.shape)
+    cfg = kx.sim_config_default(Te=5000.0, precision=precision, **{"kernel": kx.SIM_KERNEL_XL, **cfg})
+    table = kx.param_table(synth.table_to_array(synth.synthetic_table(1)))
+    Z = np.ones(n, dtype=np.int32)
+    V = synth.maxwell_boltzmann(Z, 300.0, seed=seed)
+    return kx.sim_create(cfg, table, Z, R, V=V, charge=n % 2, P0=0.5 * (1.0 - (n % 2) / n) * np.eye(n))
+
+
+def eigenpairs(h):
+    return kx.sim_get_vector(h, 0), kx.sim_get_matrix(h, kx.SIM_MAT_Q)
+
+
+@pytest.mark.parametrize("n", [2, 3, 17, 26, 33, 48, 63, 64])
+def test_one_block_gives_the_same_bits_every_time(n):
+    """Four groups of threads hand each other a column's products through shared memory."""
+    h = lattice(n, kx.SIM_PREC_FP64)
+    try:
+        eps, Q = eigenpairs(h)
+        ref = np.linalg.eigvalsh(kx.sim_get_matrix(h, kx.SIM_MAT_FOCK))
+        assert np.abs(eps - ref).max() <= max(1.0, np.abs(ref).max()) * (4e-12 + n * 2.0 ** -50)
+        for _ in range(40):
+            kx.sim_set_state(h)
+            e, q = eigenpairs(h)
+            assert np.array_equal(e, eps) and np.array_equal(q, Q)
+    finally:
+        kx.sim_destroy(h)
