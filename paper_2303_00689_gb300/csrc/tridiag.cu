@@ -252,7 +252,9 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
   __shared__ double s_par[2][4];                                   // beta, tau * scale, tau, scale
   __shared__ double s_x[2][2];                                     // x_k (the diagonal), x_{k+1}
   __shared__ double s_pk[RG];
-  __shared__ int s_fail;
+  // by the column's parity: the scalar warp reads column k's word after barrier 0, when polls of
+  // column k + 1 may already write theirs (k + 2's follow its arrival at barrier 1)
+  __shared__ int s_fail[2];
   double* A = (double*)g.A;
   const int rres = max(Rtot - g.rs, 0);                            // rows r >= rres are resident
   double* rows0 = rows - (ptrdiff_t)rres * ms - (g.k0 + 1);        // column j of resident row r: [r ms + j]
@@ -262,9 +264,9 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
     return;
   }
   if (g.role != 0) {
-    if (tid == 0) s_fail = check_in(g.gate, g.role, G) ? 0 : 1;
+    if (tid == 0) s_fail[0] = check_in(g.gate, g.role, G) ? 0 : 1;
     __syncthreads();
-    if (s_fail) return;
+    if (s_fail[0]) return;
   }
   for (int r = g.F ? 0 : rres; r < Rtot; ++r) {
     const int i = b + r * G;
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
     for (int j = g.k0 + 1 + tid; j < n; j += NT + 32) dst[j] = src[j];
   }
   __syncthreads();                                                 // s_fail has been read
-  if (tid == 0) s_fail = 0;
+  if (tid < 2) s_fail[tid] = 0;
   if (tid < 4) s_par[(g.k0 + 1) & 1][tid] = (g.k0 > 0) ? g.carry[n + tid] : 0.0;
   __syncthreads();
   const bool owns_last = (n - 1) % G == b;                         // alive in every column
@@ -290,8 +292,8 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
       if (b + rf * G <= k) ++rf;
       if (rf >= Rtot) return;
       bar_sync(0, NTG + 32);                                       // x of column k is there
-      if (s_fail || k == n - 2) return;
       const int par = k & 1;
+      if (s_fail[par] || k == n - 2) return;
       const double* red = redB + par * NTG;
       double s0 = red[lane], s1 = 0.0;
 #pragma unroll
@@ -366,7 +368,7 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
           if (!old) break;
           if (poll_expired(it, t0, limit, g.status)) {
             atomicOr(g.status, (int)kStatusTimeout);
-            s_fail = 1;
+            s_fail[par] = 1;
             break;
           }
         }
@@ -374,7 +376,7 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
     }
     if (!SOLO) bar_sync(1, NT + 32);                               // scalars of column k - 1; every group's polls are over
     if (rf >= Rtot) return;                                        // nothing left to do for this block
-    if (s_fail) {
+    if (s_fail[par]) {
       if (rg == 0) bar_sync(0, NTG + 32);                          // lets the scalar warp go
       return;
     }

@@ -40,3 +40,25 @@ def test_one_block_gives_the_same_bits_every_time(n):
             assert np.array_equal(e, eps) and np.array_equal(q, Q)
     finally:
         kx.sim_destroy(h)
+
+
+@pytest.mark.parametrize("n", [70, 128, 131, 300])
+def test_a_limit_that_may_expire_in_any_column_leaves_the_handle_usable(n):
+    """With a limit of 1 ns a poll gives up as soon as it looks at the clock, so a step may end in
+    any column: every warp of every block leaves, and the same state then gives the same bits."""
+    h = lattice(n, kx.SIM_PREC_FP64)
+    try:
+        ref = eigenpairs(h)
+        for _ in range(10):
+            kx.sim_debug_barrier_limit(1)
+            try:
+                kx.sim_set_state(h)
+            except kx.SimError as e:
+                assert e.code == kx.SIM_ETIMEOUT
+            finally:
+                kx.sim_debug_barrier_limit(2_000_000_000)
+        kx.sim_set_state(h)
+        for a, b in zip(ref, eigenpairs(h)):
+            assert np.array_equal(a, b)
+    finally:
+        kx.sim_destroy(h)
