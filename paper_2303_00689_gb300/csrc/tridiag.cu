@@ -1134,11 +1134,10 @@ static TriLaunch tri_launch(int n, int k0, int sm_count, bool few) {
   return l;
 }
 
-// The opt-in dynamic shared memory, once per device: of the FP64 shapes, and of the
-// double-float kernel where it needs it.
-static bool tri_attributes(bool df, size_t smem) {
+// The opt-in dynamic shared memory, once per device, of the kernels of one precision (whatever
+// the size: the limit without it, 48 KB, counts a kernel's static shared memory too).
+static bool tri_attributes(bool df) {
   static PerDeviceOnce once[2];
-  if (df && smem <= 48 * 1024) return true;
   return once_per_device(once[df], [df] {
     auto raise = [](const void* fn) {
       return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTriSmemMax) == cudaSuccess;
@@ -1158,7 +1157,7 @@ int eig_tridiag_weight(int n, int sm_count, bool df, bool shared) {
   if (n <= 1) return n > 0 ? 1 : 0;
   auto share = [&](const void* fn, int blocks, int threads, size_t smem) {
     int p = 0;
-    if (!tri_attributes(df, smem) || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, fn, threads, smem) != cudaSuccess || p < 1) {
+    if (!tri_attributes(df) || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, fn, threads, smem) != cudaSuccess || p < 1) {
       cudaGetLastError();
       p = 1;
     }
@@ -1199,7 +1198,7 @@ int eig_tridiagonalize(cudaStream_t s, int n, const double* F, EigWork& w, int* 
     for (int role = (G > few) ? 1 : 0;;) {
       const int blocks = (role == 2) ? few : G;
       const size_t smem = tridiag_smem_df(n, blocks);
-      if (smem > kTriSmemMax || !tri_attributes(true, smem)) return -1;
+      if (smem > kTriSmemMax || !tri_attributes(true)) return -1;
       to_df_kernel<<<(unsigned)std::min<size_t>((nn2 + 255) / 256, 8 * (size_t)sm_count), 256, 0, s>>>(
           nn2, F, (dfl*)w.A, role == 2 ? w.bar + 3 : nullptr);
       count_launch();
@@ -1218,7 +1217,7 @@ int eig_tridiagonalize(cudaStream_t s, int n, const double* F, EigWork& w, int* 
     }
     return 0;
   }
-  if (!tri_attributes(false, 0)) return -1;
+  if (!tri_attributes(false)) return -1;
   // The packets are in the inverse-iteration workspace (at least 5 n^2 doubles, free
   // until then; n > 64 here, a single block has none).  0xFF: of the parity that is
   // not the first use's.
