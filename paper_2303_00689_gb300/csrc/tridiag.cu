@@ -1043,6 +1043,7 @@ static const TriShape kTriF64[] = {
     TRI_SHAPE(2560, 256, 1, 10, false), TRI_SHAPE(3360, 480, 1, 7, false), TRI_SHAPE(4800, 480, 1, 10, false),
     TRI_SHAPE(10080, 480, 1, 21, false)};
 constexpr size_t kTriSmemMax = 227 * 1024 - 512;       // of dynamic shared memory; the kernels have some of their own
+constexpr size_t kTriSmemDf = 227 * 1024 - 48;         // the same of the double-float grid (40 bytes of its own)
 
 struct TriLaunch {
   const void* fn = nullptr;
@@ -1139,8 +1140,9 @@ static TriLaunch tri_launch(int n, int k0, int sm_count, bool few) {
 static bool tri_attributes(bool df) {
   static PerDeviceOnce once[2];
   return once_per_device(once[df], [df] {
-    auto raise = [](const void* fn) {
-      return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTriSmemMax) == cudaSuccess;
+    auto raise = [df](const void* fn) {
+      return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)(df ? kTriSmemDf : kTriSmemMax)) == cudaSuccess;
     };
     bool ok = true;
     if (df) {
@@ -1198,7 +1200,7 @@ int eig_tridiagonalize(cudaStream_t s, int n, const double* F, EigWork& w, int* 
     for (int role = (G > few) ? 1 : 0;;) {
       const int blocks = (role == 2) ? few : G;
       const size_t smem = tridiag_smem_df(n, blocks);
-      if (smem > kTriSmemMax || !tri_attributes(true)) return -1;
+      if (smem > kTriSmemDf || !tri_attributes(true)) return -1;
       to_df_kernel<<<(unsigned)std::min<size_t>((nn2 + 255) / 256, 8 * (size_t)sm_count), 256, 0, s>>>(
           nn2, F, (dfl*)w.A, role == 2 ? w.bar + 3 : nullptr);
       count_launch();

@@ -92,3 +92,22 @@ def test_grids_at_the_shared_memory_limit_of_a_plain_launch(n):
     # 4-slice products of the back-transformation: 2^-24 of sum |a||b|
     orthogonality, residual = map(float, out.stdout.split())
     assert orthogonality <= 1e-6 and residual <= 1e-5
+
+
+def test_the_largest_mixed_size_that_fits_shared_memory():
+    """n = 9255 (2313 C, 3 H): three vectors of the double-float grid fill an SM's shared memory."""
+    Z = np.array([6] * 2313 + [1] * 3, dtype=np.int32)
+    n, side = 9255, 14
+    R = 2.6 * np.array([[i % side, i // side % side, i // side ** 2] for i in range(len(Z))], dtype=float)
+    R += 0.1 * np.random.default_rng(1).normal(size=R.shape)
+    cfg = kx.sim_config_default(Te=5000.0, precision=kx.SIM_PREC_MIXED, kernel=kx.SIM_KERNEL_XL, m_max=1, m_min=1)
+    table = kx.param_table(synth.table_to_array(synth.synthetic_table(1)))
+    h = kx.sim_create(cfg, table, Z, R, charge=1, P0=4627.0 / n * np.eye(n))
+    try:
+        eps, Q = eigenpairs(h)
+        F = kx.sim_get_matrix(h, kx.SIM_MAT_FOCK)
+    finally:
+        kx.sim_destroy(h)
+    some = np.linspace(0, n - 1, 40).astype(int)
+    assert np.abs(F @ Q[:, some] - Q[:, some] * eps[some]).max() <= 1e-5 * max(1.0, np.abs(eps).max())
+    assert np.abs(Q.T @ Q[:, some] - np.eye(n)[:, some]).max() <= 1e-6
