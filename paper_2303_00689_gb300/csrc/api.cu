@@ -723,7 +723,7 @@ static void layout(sim_handle* h, Arena& a) {
   } else if (tc_available()) {
     // (without tensor maps the products run on the FP64 pipe, gemm64.cu)
     void* t64 = a.take<char>(tc64_work_bytes(h->n));
-    if (a.base && !tc64_work_bind(h->t64, t64, h->n)) h->t64 = Tc64Work{};
+    if (a.base && !tc64_work_bind(h->t64, t64, h->n, h->stream)) h->t64 = Tc64Work{};
   }
 }
 

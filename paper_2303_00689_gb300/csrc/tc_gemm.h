@@ -99,7 +99,8 @@ struct Tc64Work {
   int n = 0;
 };
 size_t tc64_work_bytes(int n);
-bool tc64_work_bind(Tc64Work& w, void* base, int n);   // false: no tensor map of this size
+// clears the error word on the stream of the handle; false: no tensor map of this size
+bool tc64_work_bind(Tc64Work& w, void* base, int n, cudaStream_t s);
 Tc64Op tc64_slot(const Tc64Work& w, int slot, int rows, int cols);
 // columns [c0, cols) of the rows of X (c0 a multiple of 32); the rows of X^T, X of `cols` rows
 void tc64_cut_rows(cudaStream_t s, const Tc64Op& op, int c0, int cols, const double* X, size_t ldx,

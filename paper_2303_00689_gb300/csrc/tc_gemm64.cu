@@ -378,13 +378,13 @@ Tc64Op tc64_op(void* base, int rows, int cols) {
 
 size_t tc64_work_bytes(int n) { return 256 + 3 * tc64_op_bytes(n, n); }
 
-bool tc64_work_bind(Tc64Work& w, void* base, int n) {
+bool tc64_work_bind(Tc64Work& w, void* base, int n, cudaStream_t s) {
   w.base = (char*)base;
   w.err = (int*)base;
   w.n = n;
   const Tc64Op op = tc64_slot(w, 0, n, n);
   CUtensorMap m;
-  return cudaMemset(w.err, 0, sizeof(int)) == cudaSuccess &&
+  return cudaMemsetAsync(w.err, 0, sizeof(int), s) == cudaSuccess &&
          tc_encode_map_box(&m, op.p, k64S * op.rows, op.ld, op.ld, k64BK, k64BM);
 }
 
