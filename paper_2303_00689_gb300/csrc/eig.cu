@@ -126,12 +126,18 @@ __device__ __forceinline__ int sturm_count_f32(int n, const float* __restrict__ 
 
 // FP64 path: eigenvalue i of T by multisection, M lanes a group: FP32 counts down to
 // ~2^-22 of the Gershgorin interval, a round of FP64 counts that takes both ends in
-// (and widens the bracket where the FP32 counts erred), then FP64 rounds to the
-// tolerance.  A count is a chain of n FP64 steps on a pipe that takes ~62 cycles a warp
+// (and widens the bracket where the FP32 counts erred), then FP64 rounds.  A count is a
+// chain of n FP64 steps on a pipe that takes ~62 cycles a warp
 // instruction however many lanes are live, so lanes that count at other points of
 // the same interval are free until there are more warps than FP64 pipes (kFp64Pipes);
-// M = 32, 16, 8 up to 1, 1 and 2 warps a pipe, 8 beside other handles.  n = 26, 240, 574,
-// 1680: 53, 290, 670, 3020 us; 165, 1370, 3160, 9220 with one lane an eigenvalue.
+// M = 32, 16, 8 up to 1, 1 and 2 warps a pipe, 8 beside other handles.  n = 240, 574,
+// 1680: 334, 783, 3450 us; 1370, 3160, 9220 with one lane an eigenvalue.
+// The FP64 counts are taken at points glo + k h of one grid, k an integer, and the
+// eigenvalue is the middle of the cell whose ends have counts <= i and > i.  The cells (a
+// 32nd of the tolerance, 3e-14 of the range) are ten times wider than the rounding of a count
+// shifts an eigenvalue, so there is one such cell and every M, and every bracket to start from,
+// ends in it: the same bits alone and beside other handles.  (Points that depended on M, down to
+// the tolerance itself: 289, 669, 3030 us, and three times the error, 3e-14 of the range.)
 constexpr int kFp64Pipes = 4 * 152;
 template <int M>
 __global__ void __launch_bounds__(32) bisect_kernel(int n, const double* __restrict__ d, const double* __restrict__ e2,
@@ -150,51 +156,49 @@ __global__ void __launch_bounds__(32) bisect_kernel(int n, const double* __restr
   float lo32 = (float)glo, hi32 = (float)ghi;
   const float piv32 = fmaxf((float)(1e-30 * fmax(1.0, width)), 1e-30f);
   for (float left = 0x1p22f; left > 1.0f; left /= (float)(M + 1)) {
-    const float h = (hi32 - lo32) / (float)(M + 1);
-    const unsigned g = above(live && sturm_count_f32(n, df, e2f, lo32 + (float)(m + 1) * h, piv32) > i);
+    const float h32 = (hi32 - lo32) / (float)(M + 1);
+    const unsigned g = above(live && sturm_count_f32(n, df, e2f, lo32 + (float)(m + 1) * h32, piv32) > i);
     const int f = g ? __ffs(g) - 1 : M;       // first point above, M: none
-    const float nlo = (f == 0) ? lo32 : lo32 + (float)f * h;
-    hi32 = (f == M) ? hi32 : lo32 + (float)(f + 1) * h;
+    const float nlo = (f == 0) ? lo32 : lo32 + (float)f * h32;
+    hi32 = (f == M) ? hi32 : lo32 + (float)(f + 1) * h32;
     lo32 = nlo;
   }
-  double w = fmax((double)hi32 - (double)lo32, 1e-12 * width);
-  double lo = (double)lo32 - w, hi = (double)hi32 + w;
   // rel_tol (1e-12) of the spectral range is far below what the occupations and
   // the DMPT weights resolve, and inverse iteration converges from such a shift
   // in two steps.  A looser shift costs orthogonality: after two steps the
   // component along a neighbour at distance g is ~(shift error / g)^2, which at
   // 1e-9 of the range left Q^T Q - I at 5e-7 for n = 3360.
   const double tol = fmax(2.0 * kEps * fmax(fabs(glo), fabs(ghi)), rel_tol * fmax(1.0, scal[2])) + pivmin;
+  const double h = 0x1p-5 * tol;
+  // cells of the grid (2^46 at most with rel_tol = 1e-12)
+  const long long cells = max(1ll, (long long)fmin(ceil(width / h), 0x1p52));
+  auto point = [&](long long k) { return fma((double)k, h, glo); };
+  long long w = max(1ll, (long long)fmin(((double)hi32 - (double)lo32) / h, 0x1p52));
+  long long lo = min(max((long long)(((double)lo32 - glo) / h) - w, 0ll), cells - 1);
+  long long hi = min(max((long long)(((double)hi32 - glo) / h) + w + 1, lo + 1), cells);
   bool done = !live, ends = true;             // ends: the points of the round are 0 .. M - 1, both ends among them
-  for (int it = 0, widened = 0; it < 260 && __any_sync(0xffffffffu, !done); ++it) {
-    const double h = (hi - lo) / (double)(ends ? M - 1 : M + 1);
-    const double x = (ends && m == M - 1) ? hi : lo + (double)(ends ? m : m + 1) * h;
-    const unsigned g = above(!done && sturm_count(n, d, e2, x, pivmin) > i);
+  for (int it = 0; it < 260 && __any_sync(0xffffffffu, !done); ++it) {
+    auto at = [&](int p) { return ends ? lo + (hi - lo) * p / (M - 1) : lo + (hi - lo) * (p + 1) / (M + 1); };
+    const unsigned g = above(!done && sturm_count(n, d, e2, point(at(m)), pivmin) > i);
     if (done) continue;
-    int f = g ? __ffs(g) - 1 : M;             // first point above, M: none
+    const int f = g ? __ffs(g) - 1 : M;       // first point above, M: none
     if (ends) {
-      const bool low = f == 0 && lo > glo, high = f == M && hi < ghi;
-      if ((low || high) && widened < 60) {
-        w *= 4.0;
-        ++widened;
-        if (low) lo = fmax(glo, lo - w);
-        if (high) hi = fmin(ghi, hi + w);
+      const bool low = f == 0 && lo > 0, high = f == M && hi < cells;
+      if (low || high) {
+        w *= 4;
+        if (low) lo = max(0ll, lo - w);
+        if (high) hi = min(cells, hi + w);
         continue;
       }
-      f = min(max(f, 1), M - 1) - 1;          // as a point 1 .. M - 2 between the ends
-      const double nlo = lo + (double)f * h;
-      hi = (f == M - 2) ? hi : lo + (double)(f + 1) * h;
-      lo = nlo;
-      ends = false;
-    } else {
-      const double nlo = (f == 0) ? lo : lo + (double)f * h;
-      hi = (f == M) ? hi : lo + (double)(f + 1) * h;
-      lo = nlo;
     }
-    const double mid = 0.5 * (lo + hi);
-    done = hi - lo <= tol || mid <= lo || mid >= hi;
+    // (the ends of the Gershgorin interval count as below and above whatever the arithmetic says)
+    const long long nlo = (f == 0) ? lo : at(f - 1);
+    hi = (f == M) ? hi : max(at(f), lo + 1);
+    lo = min(nlo, hi - 1);
+    ends = false;
+    done = hi - lo <= 1;
   }
-  if (live && m == 0) ev[i] = 0.5 * (lo + hi);
+  if (live && m == 0) ev[i] = fma((double)lo + 0.5, h, glo);
 }
 
 // Mixed path: eigenvalue i by multisection in double-float arithmetic.  A

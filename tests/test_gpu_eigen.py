@@ -111,3 +111,29 @@ def test_the_largest_mixed_size_that_fits_shared_memory():
     some = np.linspace(0, n - 1, 40).astype(int)
     assert np.abs(F @ Q[:, some] - Q[:, some] * eps[some]).max() <= 1e-5 * max(1.0, np.abs(eps).max())
     assert np.abs(Q.T @ Q[:, some] - np.eye(n)[:, some]).max() <= 1e-6
+
+
+@pytest.mark.parametrize("precision", [kx.SIM_PREC_FP64, kx.SIM_PREC_MIXED])
+@pytest.mark.parametrize("n", [1, 2, 9, 64, 65, 131, 300, 608, 609, 900, 1217])
+def test_alone_and_beside_others_the_results_are_the_same(n, precision):
+    """Grids, lanes per eigenvalue and threads per pair differ beside other handles, results do not:
+    stepped alone, by sim_batch_step (launches, and the handles' graphs), in one graph of a batch."""
+    hs = [lattice(n, precision, 5, kernel=kx.SIM_KERNEL_KRYLOV, m_max=2, m_min=2) for _ in range(7)]
+    batch = None
+    try:
+        for h in hs[3:5]:
+            kx.sim_enable_graphs(h)
+        kx.sim_step(hs[0], 2)
+        kx.sim_batch_step(hs[1:3], 2)
+        kx.sim_batch_step(hs[3:5], 2)
+        batch = kx.sim_batch_create(hs[5:])
+        kx.sim_batch_run(batch, 2)
+        ref = [*kx.sim_get_state(hs[0], n), *eigenpairs(hs[0])]
+        for h in hs[1:]:
+            for a, b in zip(ref, [*kx.sim_get_state(h, n), *eigenpairs(h)]):
+                assert np.array_equal(a, b)
+    finally:
+        if batch:
+            kx.sim_batch_destroy(batch)
+        for h in hs:
+            kx.sim_destroy(h)
