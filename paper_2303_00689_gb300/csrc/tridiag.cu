@@ -27,6 +27,7 @@
 #include "common.cuh"
 #include "df.cuh"
 #include "kernels.h"
+#include "tri_packet.h"
 
 namespace kx {
 
@@ -145,13 +146,13 @@ __host__ __device__ __forceinline__ int tri_rows(int n, int k0, int G) { return 
 // holds matrix rows and the (v, w) of the block's own rows, which every thread
 // needs.  One packet per row carries s_i and, by symmetry, the next pivot row's
 // a_{i,k+1}; the reader forms p_i, so the scalars are off the path from the product
-// to the packets.  The lowest bit of s_i carries the parity of the packet's use
-// (2^-52 of s_i, below the rounding of the sum it is).  Small matrices have more warps
+// to the packets.  The highest exponent bit of s_i carries the parity of the packet's
+// use, all other bits are those of s_i (tri_packet.h).  Small matrices have more warps
 // than columns: RG groups of NTG threads hold the same columns and share the rows
 // out.  A launch covers the columns [k0, k1): with a part of the rows outside
 // shared memory the next launch starts with shorter rows, so more of them fit (all
 // of them from a trailing width of ~1800 with 152 blocks on).
-constexpr unsigned long long kTag = 1ull;
+constexpr unsigned long long kTag = kPacketTag;
 struct __align__(16) RowVecs {
   double v, w;
 };
@@ -389,7 +390,8 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
       for (int c = 0; c < CPL; ++c) {
         const int j = t + NTG * c;
         if (j < k || j >= n) continue;
-        w[c] = ts * (__longlong_as_double((long long)q[c].x) - beta * __longlong_as_double((long long)q[c].y));
+        w[c] = ts * (__longlong_as_double((long long)packet_decode(q[c].x)) -
+                     beta * __longlong_as_double((long long)q[c].y));
         v[c] = (j == k) ? 1.0 : x[c] * scale;
         if (j == k) s_pk[rg] = w[c];
         loc = fma(w[c], v[c], loc);
@@ -476,7 +478,7 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
       for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       if (l < (SOLO ? 1 : g.reps) && r < Rtot) {
         const int i = b + r * G;
-        const Packet o{((unsigned long long)__double_as_longlong(s) & ~kTag) | tag,
+        const Packet o{packet_encode((unsigned long long)__double_as_longlong(s), tag),
                        (unsigned long long)__double_as_longlong(entry(r, k + 1))};
         if (SOLO) spk[par * n + i] = o;
         else packet_store(g.pk + ((size_t)l * 2 + par) * n + i, o);
