@@ -233,7 +233,9 @@ int sim_enable_graphs(sim_handle* h, int enable);
  * each (molecule batches: one trajectory per molecule).  The steps are
  * issued round-robin, each handle on its own stream, so the device runs the
  * small, latency-bound steps of different molecules concurrently (with
- * graphs enabled each step is one graph launch).  Handles are taken in
+ * graphs enabled each step is one graph launch; where the handles' grids do
+ * not fit together this is a second set with smaller grids, each captured
+ * when a batch first steps the handle in that phase of the ring).  Handles are taken in
  * groups whose persistent eigensolver grids fit on the device at the same
  * time; groups run one after the other.  Synchronous; returns the first
  * error.  Records of the steps are read with sim_records. */

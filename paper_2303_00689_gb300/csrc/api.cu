@@ -119,10 +119,11 @@ struct sim_handle {
   int cur_phase = -1;
   cudaEvent_t cur_start = nullptr;
   bool shared = false;   // its eigensolver grid runs beside those of other handles (batches, serving)
-  // CUDA graphs of one step, one per phase of the 8-slot X ring
+  // CUDA graphs of one step, one per phase of the 8-slot X ring: alone, and beside other handles
+  // (`shared`, other grids; captured when a batch first steps the handle in that phase)
   bool graphs = false;
-  cudaGraphExec_t gexec[8] = {};
-  long long gnodes[8] = {};
+  cudaGraphExec_t gexec[2][8] = {};
+  long long gnodes[2][8] = {};
 };
 static const int kRecCap = 4096;
 
@@ -576,48 +577,54 @@ static int one_step(sim_handle* h) {
   return SIM_OK;
 }
 
-// Capture one step per ring phase into CUDA graphs (kernels and copies only:
-// the step has no host synchronisation and no allocation).
-static int capture_graphs(sim_handle* h) {
+static void release_graphs(sim_handle* h) {
+  for (auto& set : h->gexec)
+    for (auto& g : set)
+      if (g) {
+        cudaGraphExecDestroy(g);
+        g = nullptr;
+      }
+}
+
+// Capture the step of ring phase p into a CUDA graph of the set in use (kernels and copies
+// only: the step has no host synchronisation and no allocation).
+static int capture_phase(sim_handle* h, int p) {
+  cudaGraphExec_t& exec = h->gexec[h->shared][p];
   const bool prof = h->prof;
-  h->prof = false;
   const int head = h->xhead;
-  const long long rc0 = h->rec_count;
-  int rc = SIM_OK;
-  for (int p = 0; p < 8 && rc == SIM_OK; ++p) {
-    h->xhead = p;
-    long long c0 = g_launches.load();
-    cudaGraph_t g = nullptr;
-    if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-      rc = fail(SIM_EINTERNAL, "cudaStreamBeginCapture failed");
-      break;
-    }
-    int st = one_step(h);
-    cudaError_t ee = cudaStreamEndCapture(h->stream, &g);
-    if (st != SIM_OK || ee != cudaSuccess || !g) {
-      if (g) cudaGraphDestroy(g);
-      cudaGetLastError();
-      rc = fail(SIM_EINTERNAL, std::string("graph capture of a step failed: ") + cudaGetErrorString(ee));
-      break;
-    }
-    cudaError_t ie = cudaGraphInstantiate(&h->gexec[p], g, 0);
-    cudaGraphDestroy(g);
-    if (ie != cudaSuccess) {
-      cudaGetLastError();
-      h->gexec[p] = nullptr;
-      rc = fail(SIM_EINTERNAL, std::string("graph instantiation failed: ") + cudaGetErrorString(ie));
-      break;
-    }
-    long long nodes = g_launches.load() - c0;
-    g_launches.fetch_sub(nodes);   // captured, not launched
-    h->gnodes[p] = nodes;
-  }
+  const long long rc0 = h->rec_count, c0 = g_launches.load();
+  cudaGraph_t g = nullptr;
+  if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
+    return fail(SIM_EINTERNAL, "cudaStreamBeginCapture failed");
+  h->prof = false;
+  h->xhead = p;
+  const int st = one_step(h);
   h->xhead = head;
   h->rec_count = rc0;
   h->prof = prof;
-  if (rc != SIM_OK)
-    for (int p = 0; p < 8; ++p)
-      if (h->gexec[p]) { cudaGraphExecDestroy(h->gexec[p]); h->gexec[p] = nullptr; }
+  cudaError_t ee = cudaStreamEndCapture(h->stream, &g);
+  if (st != SIM_OK || ee != cudaSuccess || !g) {
+    if (g) cudaGraphDestroy(g);
+    cudaGetLastError();
+    return fail(SIM_EINTERNAL, std::string("graph capture of a step failed: ") + cudaGetErrorString(ee));
+  }
+  const cudaError_t ie = cudaGraphInstantiate(&exec, g, 0);
+  cudaGraphDestroy(g);
+  if (ie != cudaSuccess) {
+    cudaGetLastError();
+    exec = nullptr;
+    return fail(SIM_EINTERNAL, std::string("graph instantiation failed: ") + cudaGetErrorString(ie));
+  }
+  const long long nodes = g_launches.load() - c0;
+  g_launches.fetch_sub(nodes);   // captured, not launched
+  h->gnodes[h->shared][p] = nodes;
+  return SIM_OK;
+}
+
+static int capture_graphs(sim_handle* h) {
+  int rc = SIM_OK;
+  for (int p = 0; p < 8 && rc == SIM_OK; ++p) rc = capture_phase(h, p);
+  if (rc != SIM_OK) release_graphs(h);
   return rc;
 }
 
@@ -625,8 +632,12 @@ static int capture_graphs(sim_handle* h) {
 static int launch_step(sim_handle* h) {
   if (h->graphs && !h->prof) {
     const int p = h->xhead;
-    CUDA_TRY(cudaGraphLaunch(h->gexec[p], h->stream));
-    g_launches.fetch_add(h->gnodes[p]);
+    if (!h->gexec[h->shared][p]) {
+      const int rc = capture_phase(h, p);
+      if (rc) return rc;
+    }
+    CUDA_TRY(cudaGraphLaunch(h->gexec[h->shared][p], h->stream));
+    g_launches.fetch_add(h->gnodes[h->shared][p]);
     h->xhead = (p + 7) % 8;
     h->rec_count += 1;
     return SIM_OK;
@@ -1116,8 +1127,7 @@ int sim_enable_graphs(sim_handle* h, int enable) {
     h->graphs = true;
   } else if (!enable && h->graphs) {
     CUDA_TRY(cudaStreamSynchronize(h->stream));
-    for (int p = 0; p < 8; ++p)
-      if (h->gexec[p]) { cudaGraphExecDestroy(h->gexec[p]); h->gexec[p] = nullptr; }
+    release_graphs(h);
     h->graphs = false;
   }
   return SIM_OK;
@@ -1285,8 +1295,14 @@ int sim_batch_step(sim_handle* const* hs, int count, int nsteps) {
   int first = SIM_OK;
   // groups of consecutive handles whose persistent eigensolver grids fit on
   // the device at the same time (their grid barriers need every block resident)
-  // several handles: small grids, except in step graphs, which are captured already
-  auto few = [count](const sim_handle* h) { return h->shared || (count > 1 && !(h->graphs && !h->prof)); };
+  // several handles: small grids.  Graphs keep those of a handle alone while all of them fit
+  // together (16 of n = 240 in FP64: 10.7 ms a step, 14.2 with the small ones); where they do not,
+  // a second set with the small grids is captured (64 of n = 240, 16 of 480, mixed: 28.7 and 40.8 ms
+  // in groups, 12.8 and 13.3 together).
+  long long all = 0;
+  for (int i = 0; i < count; ++i) all += eig_tridiag_weight(hs[i]->n, hs[i]->sms, mixed(hs[i]), hs[i]->shared);
+  const bool fit = count > 0 && all <= 1000LL * hs[0]->sms;
+  auto few = [=](const sim_handle* h) { return h->shared || (count > 1 && !(fit && h->graphs && !h->prof)); };
   for (int g0 = 0; g0 < count;) {
     const long long cap = 1000LL * hs[g0]->sms;
     long long load = 0;
@@ -1565,8 +1581,7 @@ void sim_destroy(sim_handle* h) {
   if (!h) return;
   DeviceGuard dg(h->dev);
   if (h->stream) cudaStreamSynchronize(h->stream);
-  for (int p = 0; p < 8; ++p)
-    if (h->gexec[p]) cudaGraphExecDestroy(h->gexec[p]);
+  release_graphs(h);
   for (auto& p : h->ev_pending) { cudaEventDestroy(p.second.first); cudaEventDestroy(p.second.second); }
   for (auto e : h->ev_pool) cudaEventDestroy(e);
   if (h->tw.base) tc_work_release(h->tw);
