@@ -119,6 +119,9 @@ struct sim_handle {
   int cur_phase = -1;
   cudaEvent_t cur_start = nullptr;
   bool shared = false;   // its eigensolver grid runs beside those of other handles (batches, serving)
+  int* demand = nullptr; // the device's demand word (tridiag.cu)
+  bool in_step = false;  // the word holds this handle's weight while the step being issued runs
+  int weight[2] = {-1, -1};   // eig_tridiag_weight alone and shared (-1: not asked for yet)
   // CUDA graphs of one step, one per phase of the 8-slot X ring: alone, and beside other handles
   // (`shared`, other grids; captured when a batch first steps the handle in that phase)
   bool graphs = false;
@@ -340,12 +343,19 @@ static bool concurrent(const sim_handle* h) { return h->side && !h->prof; }
 // eigenpairs of the Fock matrix; with fermi_side, the Fermi occupations and
 // mu (eq. 8; they need the eigenvalues only) run on the side stream while the
 // eigenvectors are formed, and the caller joins before the density
+static int grid_weight(sim_handle* h, bool shared) {
+  int& w = h->weight[shared];
+  if (w < 0) w = eig_tridiag_weight(h->n, h->sms, mixed(h), shared);
+  return w;
+}
+
 static int eig(sim_handle* h, bool fermi_side = false) {
   h->tw.wide = h->shared;
   const TcWork* tw = mixed(h) ? &h->tw : nullptr;
   const Tc64Work* t64 = h->t64.base && h->n > kBt64Above ? &h->t64 : nullptr;
   phase_begin(h, PH_TRIDIAG);
-  int st = eig_tridiagonalize(h->stream, h->n, h->Fock, h->ew, &h->sc->status, h->sms, mixed(h), h->shared);
+  int st = eig_tridiagonalize(h->stream, h->n, h->Fock, h->ew, &h->sc->status, h->sms, mixed(h), h->shared,
+                              h->in_step ? 0 : grid_weight(h, h->shared));
   phase_end(h);
   if (st != 0) return fail(SIM_EINTERNAL, "tridiagonalisation launch failed (code " + std::to_string(st) + ")");
   // the back-transformation's half that needs the reflectors only, beside the eigenpairs
@@ -557,7 +567,7 @@ static int one_step(sim_handle* h) {
   double dt = h->cfg.dt;
   phase_begin(h, PH_UPDATE);
   thermostat_half(h, 0);
-  launch_half_kick(s, h->N, h->V, h->F, h->mass, dt);     // eq. 27
+  launch_half_kick(s, h->N, h->V, h->F, h->mass, dt, h->demand, h->sc, grid_weight(h, h->shared));   // eq. 27
   launch_drift(s, h->N, h->R, h->V, dt);                  // eq. 28
   double* Xh[7];
   for (int k = 0; k < 7; ++k) Xh[k] = xslot(h, k);
@@ -565,10 +575,12 @@ static int one_step(sim_handle* h) {
   launch_x_update(s, nn, Xh, h->K, kKappa, kAlphaDamp, Xnew);   // eq. 35
   h->xhead = (h->xhead + 7) % 8;
   phase_end(h);
+  h->in_step = h->demand != nullptr;
   int rc = evaluate(h);
+  h->in_step = false;
   if (rc) return rc;
   phase_begin(h, PH_UPDATE);
-  launch_half_kick(s, h->N, h->V, h->F, h->mass, dt);     // eq. 30
+  launch_half_kick(s, h->N, h->V, h->F, h->mass, dt, h->demand, h->sc);     // eq. 30
   thermostat_half(h, 1);
   if (langevin(h)) launch_step_advance(s, h->sc);
   launch_kinetic(s, h->N, h->V, h->mass, h->sc);
@@ -971,6 +983,7 @@ static int create_handle(const sim_config* cfg, const sim_param_table* table, in
   int rc = SIM_OK;
   do {
     if (cudaMemsetAsync(h->sc, 0, sizeof(Scalars), s) != cudaSuccess) { rc = fail(SIM_EINTERNAL, "memset"); break; }
+    h->demand = eig_demand_word();
     cudaMemcpyAsync(h->elem, h->elem_h.data(), natoms * sizeof(int), cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(h->off, h->off_h.data(), (natoms + 1) * sizeof(int), cudaMemcpyHostToDevice, s);
     if (h->npair) {
@@ -1227,7 +1240,7 @@ int sim_batch_create(sim_handle* const* hs, int count, sim_batch** out) {
   const long long cap = 1000LL * hs[0]->sms;
   long long load = 0;
   for (int i = 0; i < count; ++i) {
-    long long w = eig_tridiag_weight(hs[i]->n, hs[i]->sms, mixed(hs[i]), true);
+    long long w = grid_weight(hs[i], true);
     if (i > 0 && load + w > cap) {
       b->group_end.push_back(i);
       load = 0;
@@ -1300,7 +1313,7 @@ int sim_batch_step(sim_handle* const* hs, int count, int nsteps) {
   // a second set with the small grids is captured (64 of n = 240, 16 of 480, mixed: 28.7 and 40.8 ms
   // in groups, 12.8 and 13.3 together).
   long long all = 0;
-  for (int i = 0; i < count; ++i) all += eig_tridiag_weight(hs[i]->n, hs[i]->sms, mixed(hs[i]), hs[i]->shared);
+  for (int i = 0; i < count; ++i) all += grid_weight(hs[i], hs[i]->shared);
   const bool fit = count > 0 && all <= 1000LL * hs[0]->sms;
   auto few = [=](const sim_handle* h) { return h->shared || (count > 1 && !(fit && h->graphs && !h->prof)); };
   for (int g0 = 0; g0 < count;) {
@@ -1308,7 +1321,7 @@ int sim_batch_step(sim_handle* const* hs, int count, int nsteps) {
     long long load = 0;
     int g1 = g0;
     while (g1 < count) {
-      long long w = eig_tridiag_weight(hs[g1]->n, hs[g1]->sms, mixed(hs[g1]), few(hs[g1]));
+      long long w = grid_weight(hs[g1], few(hs[g1]));
       if (g1 > g0 && load + w > cap) break;
       load += w;
       ++g1;
@@ -1585,6 +1598,7 @@ void sim_destroy(sim_handle* h) {
   for (auto& p : h->ev_pending) { cudaEventDestroy(p.second.first); cudaEventDestroy(p.second.second); }
   for (auto e : h->ev_pool) cudaEventDestroy(e);
   if (h->tw.base) tc_work_release(h->tw);
+  if (h->demand) launch_demand_release(h->stream, h->demand, h->sc);
   if (h->arena) {
     cudaFreeAsync(h->arena, h->stream);
     cudaStreamSynchronize(h->stream);

@@ -1074,7 +1074,7 @@ int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork
 
 int symmetric_eig(cudaStream_t s, int n, const double* F, double* eps, double* Q, EigWork& w,
                   int* status, int sm_count) {
-  int rc = eig_tridiagonalize(s, n, F, w, status, sm_count, false, false);
+  int rc = eig_tridiagonalize(s, n, F, w, status, sm_count, false, false, 0);
   if (rc) return rc;
   eig_bisect(s, n, eps, w, 1e-12, false, false);
   eig_vectors(s, n, eps, Q, w, false, false);

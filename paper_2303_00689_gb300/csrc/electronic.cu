@@ -860,9 +860,14 @@ void launch_step_advance(cudaStream_t s, Scalars* sc) {
 }
 
 // ---- nuclei (eqs. 27, 28, 30) ---------------------------------------------------------------
+__device__ __forceinline__ void set_demand(int* demand, Scalars* sc, int weight) {
+  atomicAdd(demand, weight - sc->demand);      // (what a step that failed left there is replaced)
+  sc->demand = weight;
+}
 __global__ void half_kick_kernel(int N, double* __restrict__ V, const double* __restrict__ F,
-                                 const double* __restrict__ mass, double dt) {
+                                 const double* __restrict__ mass, double dt, int* demand, Scalars* sc, int weight) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t == 0 && demand) set_demand(demand, sc, weight);
   if (t >= 3 * N) return;
   V[t] += 0.5 * dt * kAccel * F[t] / mass[t / 3];
 }
@@ -879,8 +884,14 @@ __global__ void kinetic_kernel(int N, const double* __restrict__ V, const double
   if (threadIdx.x == 0) sc->e_kin = s;
 }
 
-void launch_half_kick(cudaStream_t s, int N, double* V, const double* F, const double* mass, double dt) {
-  half_kick_kernel<<<(3 * N + 255) / 256, 256, 0, s>>>(N, V, F, mass, dt);
+void launch_half_kick(cudaStream_t s, int N, double* V, const double* F, const double* mass, double dt, int* demand,
+                      Scalars* sc, int weight) {
+  half_kick_kernel<<<(3 * N + 255) / 256, 256, 0, s>>>(N, V, F, mass, dt, demand, sc, weight);
+  count_launch();
+}
+__global__ void demand_release_kernel(int* demand, Scalars* sc) { set_demand(demand, sc, 0); }
+void launch_demand_release(cudaStream_t s, int* demand, Scalars* sc) {
+  demand_release_kernel<<<1, 1, 0, s>>>(demand, sc);
   count_launch();
 }
 void launch_drift(cudaStream_t s, int N, double* R, const double* V, double dt) {

@@ -78,8 +78,11 @@ void eig_work_bind(EigWork& w, void* base, int n);
 // in three stages (tridiagonalise; tridiagonal eigenpairs into Q; back-transform Q)
 // df: double-float arithmetic on the FP32 pipe (mixed path), else FP64
 // shared: the grid runs beside those of other handles, whose total is kept within the device
+// own: the weight of this grid if the demand word does not hold it (a call outside a step)
 int eig_tridiagonalize(cudaStream_t s, int n, const double* F, EigWork& w, int* status, int sm_count,
-                       bool df, bool shared);
+                       bool df, bool shared, int own);
+// device word of the current device: the weights of the steps in flight
+int* eig_demand_word();
 // Share of the device, in thousandths of an SM, that the cooperative
 // tridiagonalisation grid of size n occupies while resident (blocks divided by
 // blocks per SM).  Grids that run concurrently must sum to <= 1000 x SMs.
@@ -112,7 +115,7 @@ struct Scalars {         // device-resident per-evaluation scalars
   int rank, active, status, pad;
   unsigned long long step;   // MD steps taken (counter of the thermostat's random numbers)
   unsigned red_count;        // blocks done in the current fused reduction (reset by its last block)
-  unsigned red_pad;
+  int demand;                // this handle's share of the device's demand word
   double dipole[3];          // dipole moment of the cores and D0, e Angstrom
 };
 void launch_fermi(cudaStream_t s, int n, const double* eps, double nocc, double beta, double* f,
@@ -158,8 +161,11 @@ void launch_scaled_residual(cudaStream_t s, size_t len, const double* D, const d
 void launch_x_update(cudaStream_t s, size_t len, double* const* Xh /*7 ptrs, k = 0..6*/,
                      const double* K, double kappa, double alpha, double* Xnew);
 // nuclei
-void launch_half_kick(cudaStream_t s, int N, double* V, const double* F, const double* mass,
-                      double dt);
+// also sets the handle's share of the device's demand word to `weight` (demand: nullable)
+void launch_half_kick(cudaStream_t s, int N, double* V, const double* F, const double* mass, double dt,
+                      int* demand = nullptr, Scalars* sc = nullptr, int weight = 0);
+// takes back what a step that did not end left in the demand word
+void launch_demand_release(cudaStream_t s, int* demand, Scalars* sc);
 void launch_drift(cudaStream_t s, int N, double* R, const double* V, double dt);
 void launch_kinetic(cudaStream_t s, int N, const double* V, const double* mass, Scalars* sc);
 // Langevin (OBABO) Ornstein-Uhlenbeck half step V <- c V + sqrt((1 - c^2) k_B T / M) xi with

@@ -14,13 +14,17 @@
 // handles stepped by two threads).  So a launch on its own starts with a check-in:
 // either every block is there within kCheckInNs and all go on, or all leave, and a
 // second launch behind it, which otherwise returns at once, does the same work with
-// few blocks.  Batches and the server run such small grids from the start and keep
-// their total within what the device holds (eig_tridiag_weight).  The results do
-// not depend on the number of blocks.
+// few blocks.  Double-float grids leave at once while the steps in flight on the device
+// would fill it half as often again (g_demand; handles stepped by several threads): small
+// grids then leave SMs to the other handles' kernels.  Batches and the server run small
+// grids from the start and keep their total within what the device holds
+// (eig_tridiag_weight).  The results do not depend on the number of blocks.
 //
 // Every wait is bounded in wall time (g_barrier_ns): a block that gives up, or
 // that finds another block's timeout flag set, records kStatusTimeout and
 // returns.
+#include <limits.h>
+
 #include <algorithm>
 #include <iterator>
 
@@ -42,6 +46,19 @@ constexpr unsigned long long kCheckInNs = 1000000ull;      // 1 ms
 // eig_set_barrier_limit; 0 makes every launch give up at once, even one whose
 // waits would be satisfied, so a test can force the expiry path of a real step)
 __device__ unsigned long long g_barrier_ns = kBarrierNs;
+
+// what the large grids of the steps in flight on this device take, in thousandths of an SM
+// (eig_tridiag_weight); every step adds its own at its start and takes it back at its end
+__device__ int g_demand = 0;
+
+int* eig_demand_word() {
+  void* p = nullptr;
+  if (cudaGetSymbolAddress(&p, g_demand) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return (int*)p;
+}
 
 int eig_set_barrier_limit(unsigned long long ns) {
   return cudaMemcpyToSymbol(g_barrier_ns, &ns, sizeof(ns)) == cudaSuccess ? 0 : -1;
@@ -80,11 +97,12 @@ struct TriArgs {
 };
 
 // Thread 0: whether this launch is to run.  gate: arrivals, then 0 undecided / 1 go /
-// 2 leave.  Role 1: all blocks are here before one gives up waiting; role 2: the
-// launch before this one was given up.
-__device__ bool check_in(unsigned* gate, int role, int G) {
+// 2 leave.  Role 1: all blocks are here before one gives up waiting, and none has seen a
+// demand above `crowd`; role 2: the launch before this one was given up.
+__device__ bool check_in(unsigned* gate, int role, int G, int crowd) {
   volatile unsigned* state = gate + 1;
   if (role == 1) {
+    if (*(volatile int*)&g_demand > crowd) atomicCAS(gate + 1, 0u, 2u);
     if (atomicAdd(gate, 1u) == (unsigned)G - 1) atomicCAS(gate + 1, 0u, 1u);
     const unsigned long long t0 = global_ns();
     while (*state == 0)
@@ -265,7 +283,7 @@ __global__ void __launch_bounds__(NTG * RG + 32, (NTG * RG <= 256 && CPL <= 4) ?
     return;
   }
   if (g.role != 0) {
-    if (tid == 0) s_fail[0] = check_in(g.gate, g.role, G) ? 0 : 1;
+    if (tid == 0) s_fail[0] = check_in(g.gate, g.role, G, INT_MAX) ? 0 : 1;
     __syncthreads();
     if (s_fail[0]) return;
   }
@@ -681,7 +699,8 @@ __global__ void __launch_bounds__(kTriThreadsDf) tridiag_df_kernel(int n, dfl* _
                                                                  double* __restrict__ e,
                                                                  double* __restrict__ tau,
                                                                  dfl* __restrict__ pbuf,
-                                                                 unsigned* bar, int* status, int rmax, int role) {
+                                                                 unsigned* bar, int* status, int rmax, int role,
+                                                                 int crowd) {
   extern __shared__ float4 sm4[];
   float4* PW = sm4;                          // n pairs
   dfl* VC = (dfl*)(sm4 + n);                 // n
@@ -692,7 +711,7 @@ __global__ void __launch_bounds__(kTriThreadsDf) tridiag_df_kernel(int n, dfl* _
   __shared__ dfl s_df[4];                    // beta, tau * scale, tau, scale
   if constexpr (GATED) {
     __shared__ int s_go;
-    if (threadIdx.x == 0) s_go = check_in(bar + 2, role, (int)gridDim.x) ? 1 : 0;
+    if (threadIdx.x == 0) s_go = check_in(bar + 2, role, (int)gridDim.x, crowd) ? 1 : 0;
     __syncthreads();
     if (!s_go) return;
   }
@@ -1185,7 +1204,11 @@ int eig_tridiag_weight(int n, int sm_count, bool df, bool shared) {
 __global__ void tri_one_kernel(const double* F, double* d) { d[0] = F[0]; }
 
 int eig_tridiagonalize(cudaStream_t s, int n, const double* F, EigWork& w, int* status, int sm_count, bool df,
-                       bool shared) {
+                       bool shared, int own) {
+  // (two steps of n = 1680 together, mixed: 42.5 ms with the large grids, 33.4 with the small ones, eight
+  // of 480 14.3 and 10.7; two and four of 480, a demand of 0.75 and 1.5: 5.1 and 7.7, 7.0 and 8.0.  In
+  // FP64 the small grids are no gain: two of 1680 79 and 75, of 2160 141 and 164)
+  int crowd = 1500 * sm_count - own;
   if (n <= 0) return 0;
   cudaMemsetAsync(w.e, 0, (size_t)n * sizeof(double), s);
   cudaMemsetAsync(w.Vst, 0, (size_t)n * n * sizeof(double), s);               // entries left of the reflectors
@@ -1211,7 +1234,7 @@ int eig_tridiagonalize(cudaStream_t s, int n, const double* F, EigWork& w, int* 
       dfl *A = (dfl*)w.A, *pb = (dfl*)w.pbuf;
       double *V = w.Vst, *d = w.d, *e = w.e, *t = w.tau;
       unsigned* bar = w.bar;
-      void* args[] = {&nn, &A, &V, &d, &e, &t, &pb, &bar, &status, &rmax, &role};
+      void* args[] = {&nn, &A, &V, &d, &e, &t, &pb, &bar, &status, &rmax, &role, &crowd};
       const void* fn = role ? (const void*)tridiag_df_kernel<true> : (const void*)tridiag_df_kernel<false>;
       if (cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kTriThreadsDf), args, smem, s) != cudaSuccess)
         return -2;
