@@ -243,7 +243,7 @@ static bool mixed(const sim_handle* h) { return h->cfg.precision == SIM_PREC_MIX
 // The back-transformation: on the FP64 pipe while one block of reflectors is all there
 // is (n = 26, 59, 131, 240: 59, 169, 410, 756 us and 128, 181, 397, 460 us).
 constexpr int kTc64Above = 256, kBt64Above = 66;
-static bool dmpt64(const sim_handle* h) { return h->t64.base && h->n > kTc64Above; }
+static bool dmpt64(const sim_handle* h) { return h->t64.err && h->n > kTc64Above; }
 
 // C = A B^T of cut n x n operands (the size's tensor map was encoded at creation)
 static void tc64_mul(sim_handle* h, const Tc64Op& A, const Tc64Op& B, double* C, int sym, const int* gate = nullptr) {
@@ -262,7 +262,7 @@ static void density(sim_handle* h) {
     // all slices of a k-tile staged together (tc_gemm_grouped4)
     tc_split(s, h->tw, kSlotQs, h->Qs, 4, 0);
     tc_gemm_grouped4(s, h->tw, kSlotQs, kSlotQs, 1.0, h->D, 1);
-  } else if (h->t64.base) {
+  } else if (h->t64.err) {
     const Tc64Op q = tc64_slot(h->t64, 2, n, n);
     tc64_cut_rows(s, q, 0, n, h->Qs, n);
     tc64_mul(h, q, q, h->D, 1);
@@ -352,7 +352,7 @@ static int grid_weight(sim_handle* h, bool shared) {
 static int eig(sim_handle* h, bool fermi_side = false) {
   h->tw.wide = h->shared;
   const TcWork* tw = mixed(h) ? &h->tw : nullptr;
-  const Tc64Work* t64 = h->t64.base && h->n > kBt64Above ? &h->t64 : nullptr;
+  const Tc64Work* t64 = h->t64.err && h->n > kBt64Above ? &h->t64 : nullptr;
   phase_begin(h, PH_TRIDIAG);
   int st = eig_tridiagonalize(h->stream, h->n, h->Fock, h->ew, &h->sc->status, h->sms, mixed(h), h->shared,
                               h->in_step ? 0 : grid_weight(h, h->shared));
@@ -360,7 +360,7 @@ static int eig(sim_handle* h, bool fermi_side = false) {
   if (st != 0) return fail(SIM_EINTERNAL, "tridiagonalisation launch failed (code " + std::to_string(st) + ")");
   // the back-transformation's half that needs the reflectors only, beside the eigenpairs
   // of T (not beside other handles, which have the idle SMs)
-  const bool split = concurrent(h) && !h->shared && eig_backtransform_splits(h->n);
+  const bool split = concurrent(h) && !h->shared && h->ew.side;
   int bt = 0;
   if (split) {
     fork_side(h, 2);
@@ -738,15 +738,17 @@ static void layout(sim_handle* h, Arena& a) {
   h->sc = a.take<Scalars>(1);
   h->rec = a.take<sim_step_result>(kRecCap);
   h->rec_idx = a.take<int>(4);
-  void* ewb = a.take<char>(eig_work_bytes(h->n));
-  if (a.base) eig_work_bind(h->ew, ewb, h->n);
-  if (h->cfg.precision == SIM_PREC_MIXED) {
+  // (without tensor maps FP64 products run on the FP64 pipe, gemm64.cu)
+  const EigProducts kind =
+      (h->cfg.precision == SIM_PREC_MIXED) ? kEigSlices : (tc_available() ? kEigDigits : kEigPlain);
+  void* ewb = a.take<char>(eig_work_bytes(h->n, kind, !h->shared));
+  if (a.base) eig_work_bind(h->ew, ewb, h->n, kind, !h->shared);
+  if (kind == kEigSlices) {
     void* twb = a.take<char>(tc_work_bytes(h->n));
     if (a.base) tc_work_bind(h->tw, twb, h->n);
-  } else if (tc_available()) {
-    // (without tensor maps the products run on the FP64 pipe, gemm64.cu)
-    void* t64 = a.take<char>(tc64_work_bytes(h->n));
-    if (a.base && !tc64_work_bind(h->t64, t64, h->n, h->stream)) h->t64 = Tc64Work{};
+  } else if (kind == kEigDigits) {
+    int* err = a.take<int>(1);
+    if (a.base && !tc64_work_bind(h->t64, h->ew.op64, err, h->n, h->stream)) h->t64 = Tc64Work{};
   }
 }
 
@@ -1113,7 +1115,7 @@ int sim_wait(sim_handle* h) {
   return check_status(h);
 }
 
-size_t sim_estimate_bytes(const sim_config* cfg, int natoms, const int* Z) {
+static size_t estimate(const sim_config* cfg, int natoms, const int* Z, bool shared) {
   if (!cfg || !Z || natoms < 1 || cfg->m_max < 1 || cfg->m_max > 16) return 0;
   sim_handle tmp;
   tmp.cfg = *cfg;
@@ -1123,9 +1125,13 @@ size_t sim_estimate_bytes(const sim_config* cfg, int natoms, const int* Z) {
   tmp.n = n;
   tmp.npair = natoms * (natoms - 1) / 2;
   tmp.mmax = cfg->m_max;
+  tmp.shared = shared;
   Arena sizing{nullptr, 0, 0};
   layout(&tmp, sizing);
   return sizing.off + 256;
+}
+size_t sim_estimate_bytes(const sim_config* cfg, int natoms, const int* Z) {
+  return estimate(cfg, natoms, Z, false);
 }
 
 int sim_enable_graphs(sim_handle* h, int enable) {
@@ -1616,6 +1622,8 @@ void sim_destroy(sim_handle* h) {
 }
 
 }  // extern "C"
+
+size_t kx::estimate_shared(const sim_config* cfg, int natoms, const int* Z) { return estimate(cfg, natoms, Z, true); }
 
 int kx::create_shared(const sim_config* cfg, const sim_param_table* table, int natoms, const int* Z, const double* R,
                       const double* V, int charge, sim_handle** out) {

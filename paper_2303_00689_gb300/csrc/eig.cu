@@ -652,31 +652,35 @@ __global__ void __launch_bounds__(4 * kTfRows) tfactor_all_kernel(int nref, cons
 // number of blocks of kBtBlockTc reflectors (n - 2 reflectors)
 static int tc_blocks(int n) { return n > 2 ? (n - 2 + kBtBlockTc - 1) / kBtBlockTc : 1; }
 
-struct BtScratch;
-static size_t bt_scratch_layout(int n, void* base, BtScratch* out);
-struct Bt64Scratch;
-static size_t bt64_scratch(int n, void* base, Bt64Scratch* out);
-static size_t bt_doubles(int n) {
-  return std::max((bt_scratch_layout(n, nullptr, nullptr) + 7) / 8, bt64_scratch(n, nullptr, nullptr) / 8);
-}
+// Back-transformation scratch in two parts: `early` is filled by the preparation, which may run
+// beside the inverse iteration, `late` is used after it
+struct BtBytes {
+  size_t early, late;
+};
+static BtBytes bt_bytes(int n);      // slices (mixed path)
+static BtBytes bt64_bytes(int n);    // digits (FP64)
 // Up to this size the half of the back-transformation that needs no eigenvectors (Gram
 // matrices, T factors, T^T V, slices) runs on the side stream during multisection and
 // inverse iteration, which leave most SMs idle there.  Above, the kernels slow one
 // another by more than is gained (1680: 22.95 -> 23.14 ms, FP64 45.4 -> 46.5).  C60 step 2.90 -> 2.64 ms, C120 4.84 -> 4.57, 574 basis
 // functions in FP64 9.82 -> 9.58.
 constexpr int kBtSideMax = 640;
-// the inverse-iteration workspace (5 n^2) also serves as back-transformation scratch
-static size_t lu_doubles(int n) {
-  const size_t a = 5 * (size_t)n * n;
-  return std::max(a, bt_doubles(n));
-}
+static bool bt_splits(int n) { return n > 2 && n <= kBtSideMax; }
 
 // One layout for sizing and binding.  Every buffer starts on a 256-byte
 // boundary: the back-transformation cuts BF16 slices into the lu region and
 // hands them to TMA, whose tensor maps need 16-byte aligned bases (with odd n
 // an unpadded layout would leave the region 8 bytes off).
-static size_t eig_layout(int n, void* base, EigWork* w) {
+// The inverse-iteration workspace (5 n^2) also holds what the later stages need: `late`, the third
+// FP64 operand (tc_gemm64.cu) and, unless the preparation runs beside the inverse iteration
+// (side), `early` and the first two.  FP64 at n = 1680: 137 MB less than with buffers of their own.
+static size_t eig_layout(int n, EigProducts kind, bool side, void* base, EigWork* w) {
   const size_t nn = (size_t)n * n;
+  side = side && bt_splits(n) && kind != kEigPlain;
+  const BtBytes bt = (kind == kEigSlices) ? bt_bytes(n) : (kind == kEigDigits) ? bt64_bytes(n) : BtBytes{0, 0};
+  const size_t op = (kind == kEigDigits) ? tc64_op_bytes(n, n) : 0;
+  const size_t early = bt.early + 2 * op, late = bt.late + op;
+  const size_t lu_bytes = std::max(5 * nn * sizeof(double), late + (side ? 0 : early));
   size_t off = 0;
   auto take = [&](size_t doubles) {
     double* q = base ? (double*)base + off : nullptr;
@@ -690,9 +694,8 @@ static size_t eig_layout(int n, void* base, EigWork* w) {
   double* e2 = take(n);
   double* tau = take(n);
   double* pbuf = take(4 * (size_t)n);
-  double* lu = take(lu_doubles(n));
-  // back-transformation scratch: of its own where its preparation runs beside the inverse iteration
-  double* bt = (n <= kBtSideMax) ? take(bt_doubles(n)) : lu;
+  double* lu = take((lu_bytes + 7) / 8);
+  char* pre = side ? (char*)take((early + 7) / 8) : (char*)lu + (base ? late : 0);
   double* Tm = take((size_t)tc_blocks(n) * kBtBlockTc * kBtBlockTc);   // T and Gram of every reflector block
   double* Gm = take((size_t)tc_blocks(n) * kBtBlockTc * kBtBlockTc);
   double* Wt = take((size_t)kBtBlockTc * n);
@@ -701,7 +704,13 @@ static size_t eig_layout(int n, void* base, EigWork* w) {
   double* bar = take(8);
   double* clus = take(((size_t)n * sizeof(int) + 7) / 8);
   if (w) {
-    w->A = A; w->Vst = Vst; w->d = d; w->e = e; w->e2 = e2; w->tau = tau; w->pbuf = pbuf; w->lu = lu; w->bt = bt;
+    w->A = A; w->Vst = Vst; w->d = d; w->e = e; w->e2 = e2; w->tau = tau; w->pbuf = pbuf; w->lu = lu;
+    w->side = side;
+    w->early = pre + 2 * op;
+    w->late = (char*)lu + op;
+    w->op64[0] = pre;
+    w->op64[1] = pre + op;
+    w->op64[2] = (char*)lu;
     w->Tm = Tm; w->Gm = Gm; w->Wt = Wt; w->Wt2 = Wt2; w->scal = scal;
     w->bar = (unsigned*)bar;
     w->clus = (int*)clus;
@@ -709,10 +718,10 @@ static size_t eig_layout(int n, void* base, EigWork* w) {
   return off * sizeof(double) + 256;
 }
 
-size_t eig_work_bytes(int n) { return eig_layout(n, nullptr, nullptr); }
+size_t eig_work_bytes(int n, EigProducts kind, bool side) { return eig_layout(n, kind, side, nullptr, nullptr); }
 
 // base must be 256-byte aligned (arena allocations are)
-void eig_work_bind(EigWork& w, void* base, int n) { eig_layout(n, base, &w); }
+void eig_work_bind(EigWork& w, void* base, int n, EigProducts kind, bool side) { eig_layout(n, kind, side, base, &w); }
 
 void eig_bisect(cudaStream_t s, int n, double* eps, EigWork& w, double rel_tol, bool df_path, bool shared) {
   if (n <= 0) return;
@@ -882,7 +891,6 @@ __global__ void __launch_bounds__(256) y_df_kernel(int n, int nref, const double
   }
 }
 
-// back-transformation scratch (in the inverse-iteration workspace, free by then)
 static int bt_blocks(int n) { return n > 2 ? (n - 2 + kBtBlockTc - 1) / kBtBlockTc : 0; }
 constexpr int kBtSplitK = 6;
 struct BtScratch {
@@ -891,7 +899,7 @@ struct BtScratch {
   __nv_bfloat16* ys;   size_t ys_blk, ys_slice;   // Y_b^T slices
   double* part;                                   // split-K partial products of U
 };
-static size_t bt_scratch_layout(int n, void* base, BtScratch* out) {
+static BtBytes bt_scratch_layout(int n, const EigWork* w, BtScratch* out) {
   const size_t nblk = (size_t)bt_blocks(n), KB = kBtBlockTc;
   const size_t ldn = (size_t)tc_ld(n > 1 ? n : 1);
   size_t off = 0;
@@ -901,16 +909,16 @@ static size_t bt_scratch_layout(int n, void* base, BtScratch* out) {
   const size_t o_yt = take(nblk * (size_t)n * KB * 8);
   const size_t ys_slice = (size_t)n * KB, ys_blk = (size_t)kTcMaxSlices * ys_slice;
   const size_t o_ys = take(nblk * ys_blk * 2);
-  const size_t o_part = take((size_t)(kBtSplitK + 1) * n * KB * 8);
   if (out) {
-    char* c = (char*)base;
+    char* c = w->early;
     out->vs = (__nv_bfloat16*)(c + o_vs); out->vs_blk = vs_blk; out->vs_slice = vs_slice;
     out->yt = (double*)(c + o_yt);
     out->ys = (__nv_bfloat16*)(c + o_ys); out->ys_blk = ys_blk; out->ys_slice = ys_slice;
-    out->part = (double*)(c + o_part);
+    out->part = (double*)w->late;
   }
-  return off;
+  return BtBytes{off, (size_t)(kBtSplitK + 1) * n * KB * 8};
 }
+static BtBytes bt_bytes(int n) { return bt_scratch_layout(n, nullptr, nullptr); }
 
 static void bt_attributes() {
   static PerDeviceOnce attr;
@@ -930,7 +938,7 @@ static void bt_prepare_tc(cudaStream_t s, int n, EigWork& w) {
   bt_attributes();
   const int nref = n - 2, nblk = bt_blocks(n);
   BtScratch sc;
-  bt_scratch_layout(n, w.bt, &sc);
+  bt_scratch_layout(n, &w, &sc);
   // Gram matrices and T factors of all blocks, then Y_b^T = V_b^T T_b, then slices
   gram_df_kernel<<<dim3((kBtBlockTc / 32) * (kBtBlockTc / 32), nblk), 256, 0, s>>>(n, nref, w.Vst, w.Gm);
   count_launch();
@@ -951,7 +959,7 @@ static int eig_backtransform_tc(cudaStream_t s, int n, double* Q, EigWork& w, co
   const size_t stride = tc_slot_stride(tw);
   int* err = tc_error_flag(tw);
   BtScratch sc;
-  bt_scratch_layout(n, w.bt, &sc);
+  bt_scratch_layout(n, &w, &sc);
   double* Zt = w.A;                      // tridiagonalisation workspace is free now
   transpose_sq(s, n, Q, Zt);
   __nv_bfloat16* sZ = tc_slot_base(tw, kSlotT0);
@@ -985,26 +993,25 @@ struct Bt64Scratch {
   double *U, *W;       // n x kBtBlockTc
   Tc64Op u, t;         // cut U or W, and T of all blocks
 };
-static size_t bt64_scratch(int n, void* base, Bt64Scratch* out) {
+static BtBytes bt64_scratch(int n, const EigWork* w, Bt64Scratch* out) {
   const size_t u = (size_t)n * kBtBlockTc * sizeof(double);        // a multiple of 256
   const int rt = tc_blocks(n) * kBtBlockTc;
-  const size_t uo = tc64_op_bytes(n, kBtBlockTc);
   if (out) {
-    char* c = (char*)base;
-    out->U = (double*)c;
-    out->W = (double*)(c + u);
-    out->u = tc64_op(c + 2 * u, n, kBtBlockTc);
-    out->t = tc64_op(c + 2 * u + uo, rt, kBtBlockTc);
+    out->t = tc64_op(w->early, rt, kBtBlockTc);
+    out->U = (double*)w->late;
+    out->W = (double*)(w->late + u);
+    out->u = tc64_op(w->late + 2 * u, n, kBtBlockTc);
   }
-  return 2 * u + uo + tc64_op_bytes(rt, kBtBlockTc);
+  return BtBytes{tc64_op_bytes(rt, kBtBlockTc), 2 * u + tc64_op_bytes(n, kBtBlockTc)};
 }
+static BtBytes bt64_bytes(int n) { return bt64_scratch(n, nullptr, nullptr); }
 
 static int bt_prepare_tc64(cudaStream_t s, int n, EigWork& w, const Tc64Work& tw) {
   constexpr int KB = kBtBlockTc;
   bt_attributes();
   const int nref = n - 2, nblk = bt_blocks(n);
   Bt64Scratch sc;
-  bt64_scratch(n, w.bt, &sc);
+  bt64_scratch(n, &w, &sc);
   const Tc64Op V = tc64_slot(tw, 0, nref, n), Vt = tc64_slot(tw, 1, n, nref);
   tc64_cut_rows(s, V, 0, n, w.Vst, n);
   tc64_cut_cols(s, Vt, nref, w.Vst, n);
@@ -1020,7 +1027,7 @@ static int eig_backtransform_tc64(cudaStream_t s, int n, double* Q, EigWork& w, 
   constexpr int KB = kBtBlockTc;
   const int nref = n - 2, nblk = bt_blocks(n);
   Bt64Scratch sc;
-  bt64_scratch(n, w.bt, &sc);
+  bt64_scratch(n, &w, &sc);
   const Tc64Op V = tc64_slot(tw, 0, nref, n), Vt = tc64_slot(tw, 1, n, nref), Z = tc64_slot(tw, 2, n, n);
   double* Zt = w.A;
   transpose_sq(s, n, Q, Zt);
@@ -1036,8 +1043,6 @@ static int eig_backtransform_tc64(cudaStream_t s, int n, double* Q, EigWork& w, 
   transpose_sq(s, n, Zt, Q);
   return 0;
 }
-
-bool eig_backtransform_splits(int n) { return n > 2 && n <= kBtSideMax; }
 
 int eig_backtransform_prepare(cudaStream_t s, int n, EigWork& w, const TcWork* tw, const Tc64Work* t64) {
   if (n <= 2) return 0;

@@ -9,7 +9,8 @@ struct sim_param_table;
 namespace kx {
 
 // ---- api.cu -----------------------------------------------------------------
-// sim_create for a handle whose eigensolver grids run beside those of others (server)
+// sim_estimate_bytes and sim_create for a handle whose eigensolver grids run beside those of others (server)
+size_t estimate_shared(const sim_config* cfg, int natoms, const int* Z);
 int create_shared(const sim_config* cfg, const sim_param_table* table, int natoms, const int* Z, const double* R,
                   const double* V, int charge, sim_handle** out);
 
@@ -65,15 +66,19 @@ struct EigWork {
   double *Vst;          // n x n Householder vectors (row k = v_k)
   double *d, *e, *e2, *tau;
   double *pbuf;         // 4 x n
-  double *lu;           // 5 x n x n inverse-iteration workspace
-  double *bt;           // back-transformation scratch (lu in large systems)
+  double *lu;           // 5 x n x n inverse-iteration workspace, then scratch of the later stages
+  bool side;            // early and op64[0], [1] outside lu: the preparation may run beside the inverse iteration
+  char *early, *late;   // back-transformation scratch: of the preparation, of the rest
+  char* op64[3];        // FP64 operands of the products on the tensor cores (tc_gemm64.cu)
   double *Tm, *Gm, *Wt, *Wt2;  // back-transform panels
   unsigned* bar;        // 2 words grid barrier, 2 words check-in
   int* clus;            // cluster starts
   double* scal;         // scalars (Gershgorin bounds, norm)
 };
-size_t eig_work_bytes(int n);
-void eig_work_bind(EigWork& w, void* base, int n);
+enum EigProducts { kEigPlain, kEigSlices, kEigDigits };   // products on the FP64 pipe, mixed, FP64 on the tensor cores
+// side: the handle steps alone, with a side stream for the back-transformation's preparation
+size_t eig_work_bytes(int n, EigProducts kind, bool side);
+void eig_work_bind(EigWork& w, void* base, int n, EigProducts kind, bool side);
 // F (n x n symmetric, row-major) -> eps ascending, Q (eigenvectors as columns),
 // in three stages (tridiagonalise; tridiagonal eigenpairs into Q; back-transform Q)
 // df: double-float arithmetic on the FP32 pipe (mixed path), else FP64
@@ -101,8 +106,7 @@ struct Tc64Work;
 int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork* tw, const Tc64Work* t64,
                       bool prepared);
 // its half that needs no eigenvectors, which may run on another stream after the
-// tridiagonalisation (eig_backtransform_splits: its scratch is its own)
-bool eig_backtransform_splits(int n);
+// tridiagonalisation (EigWork::side: its scratch is its own)
 int eig_backtransform_prepare(cudaStream_t s, int n, EigWork& w, const TcWork* tw, const Tc64Work* t64);
 int symmetric_eig(cudaStream_t s, int n, const double* F, double* eps, double* Q, EigWork& w,
                   int* status, int sm_count);

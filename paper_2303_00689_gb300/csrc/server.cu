@@ -318,7 +318,7 @@ int sim_server_create(const sim_server_config* cfg, sim_server** out) {
 int sim_submit(sim_server* s, const sim_request* req, unsigned long long* ticket) {
   if (!s || !req || !ticket || req->natoms < 1 || !req->Z || !req->R || req->nsteps < 0) return SIM_EINVAL;
   if (req->records && req->nsteps > kMaxRecords) return SIM_EINVAL;
-  size_t bytes = sim_estimate_bytes(&req->cfg, req->natoms, req->Z);
+  size_t bytes = kx::estimate_shared(&req->cfg, req->natoms, req->Z);
   if (bytes == 0 || bytes > s->cfg.hbm_budget_bytes) return SIM_EINVAL;
   Job* j = new Job();
   j->req = *req;

@@ -92,15 +92,14 @@ struct Tc64Op {
 };
 size_t tc64_op_bytes(int rows, int cols);              // a multiple of 256
 Tc64Op tc64_op(void* base, int rows, int cols);        // base 256-byte aligned
-// the device buffers of an FP64 handle: three operands of n x n and an error word
+// the device buffers of an FP64 handle: three operands of n x n (in its eigensolver workspace) and an error word
 struct Tc64Work {
-  char* base = nullptr;
+  char* op[3] = {};
   int* err = nullptr;
   int n = 0;
 };
-size_t tc64_work_bytes(int n);
 // clears the error word on the stream of the handle; false: no tensor map of this size
-bool tc64_work_bind(Tc64Work& w, void* base, int n, cudaStream_t s);
+bool tc64_work_bind(Tc64Work& w, char* const (&op)[3], int* err, int n, cudaStream_t s);
 Tc64Op tc64_slot(const Tc64Work& w, int slot, int rows, int cols);
 // columns [c0, cols) of the rows of X (c0 a multiple of 32); the rows of X^T, X of `cols` rows
 void tc64_cut_rows(cudaStream_t s, const Tc64Op& op, int c0, int cols, const double* X, size_t ldx,

@@ -376,21 +376,17 @@ Tc64Op tc64_op(void* base, int rows, int cols) {
   return op;
 }
 
-size_t tc64_work_bytes(int n) { return 256 + 3 * tc64_op_bytes(n, n); }
-
-bool tc64_work_bind(Tc64Work& w, void* base, int n, cudaStream_t s) {
-  w.base = (char*)base;
-  w.err = (int*)base;
+bool tc64_work_bind(Tc64Work& w, char* const (&op)[3], int* err, int n, cudaStream_t s) {
+  for (int k = 0; k < 3; ++k) w.op[k] = op[k];
+  w.err = err;
   w.n = n;
-  const Tc64Op op = tc64_slot(w, 0, n, n);
+  const Tc64Op first = tc64_slot(w, 0, n, n);
   CUtensorMap m;
   return cudaMemsetAsync(w.err, 0, sizeof(int), s) == cudaSuccess &&
-         tc_encode_map_box(&m, op.p, k64S * op.rows, op.ld, op.ld, k64BK, k64BM);
+         tc_encode_map_box(&m, first.p, k64S * first.rows, first.ld, first.ld, k64BK, k64BM);
 }
 
-Tc64Op tc64_slot(const Tc64Work& w, int slot, int rows, int cols) {
-  return tc64_op(w.base + 256 + (size_t)slot * tc64_op_bytes(w.n, w.n), rows, cols);
-}
+Tc64Op tc64_slot(const Tc64Work& w, int slot, int rows, int cols) { return tc64_op(w.op[slot], rows, cols); }
 
 void tc64_cut_rows(cudaStream_t s, const Tc64Op& op, int c0, int cols, const double* X, size_t ldx, const int* gate) {
   cut64_rows_kernel<<<op.rows, kCutThreads, 0, s>>>(op, c0, cols, X, ldx, gate);
