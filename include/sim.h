@@ -55,7 +55,10 @@ enum sim_status {
 
 /* ---- precision modes ---------------------------------------------------- */
 enum sim_precision {
-  /* every step in FP64 (FP64 SIMT GEMMs for density and DMPT)               */
+  /* every step in FP64.  Matrix products on the FP64 pipe or, beyond small
+   * sizes, on the tensor cores as exact products of 8-bit digits, 63 bits
+   * below the row maximum: to one rounding of the result and K 2^-60 of the
+   * product of the two rows' maxima                                          */
   SIM_PREC_FP64 = 0,
   /* FP64 eigensolve, mu and Krylov Gram/solve; density D0 = Q f Q^T and the
    * DMPT contractions of eq. 36 on tcgen05 tensor cores: operands cut into
