@@ -1097,33 +1097,55 @@ static size_t tri_cluster_smem(int n, int G) {
   const size_t rmax = (size_t)(n - 1 + G - 1) / G;
   return (7 * (size_t)n + 2 * kDfRed + 3 * rmax + rmax * n) * sizeof(dfl);
 }
-constexpr int kTriClusterMax = 320;
-static bool tri_cluster_ready() {
-  static PerDeviceOnce once;
-  return once_per_device(once, [] {
-    const void* fn = (const void*)tridiag_cluster_kernel;
-    bool ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTriSmemMax) == cudaSuccess &&
-              cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-    if (!ok) cudaGetLastError();
-    return ok;
-  });
-}
-static int tri_cluster(int n, bool df, bool shared) {
-  if (!df || shared || n < 2 || n > kTriClusterMax || !tri_cluster_ready()) return 0;
-  return n <= 160 ? 8 : 16;
-}
-static int tri_cluster_launch(cudaStream_t s, int n, int G, const double* F, EigWork& w, int* status) {
+static cudaLaunchConfig_t tri_cluster_config(int G, size_t smem, cudaStream_t s, cudaLaunchAttribute (&at)[1]) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(G);
   cfg.blockDim = dim3(kTriThreadsDf);
-  cfg.dynamicSmemBytes = tri_cluster_smem(n, G);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = G;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  return cfg;
+}
+constexpr int kTriClusterMax = 320;
+// Set-up, and whether a cluster of 8 and one of 16 (more than the portable size) with the shared
+// memory of the largest matrix has a place on the current device (bits 0 and 1): a part of a GPU
+// may have no 16 SMs that form a cluster, and a launch there would fail.
+static int tri_cluster_places() {
+  static PerDeviceOnce once;
+  static int places[kMaxDevices];
+  int dev = 0;
+  if (!once_per_device(once, [] {
+        const void* fn = (const void*)tridiag_cluster_kernel;
+        int dev = 0, bits = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTriSmemMax) == cudaSuccess &&
+            cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+          for (int k = 0; k < 2; ++k) {
+            cudaLaunchAttribute at[1];
+            cudaLaunchConfig_t cfg = tri_cluster_config(8 << k, tri_cluster_smem(kTriClusterMax, 8 << k), nullptr, at);
+            int clusters = 0;
+            if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters > 0) bits |= 1 << k;
+          }
+        cudaGetLastError();
+        if (dev >= 0 && dev < kMaxDevices) places[dev] = bits;
+        return true;
+      }) ||
+      cudaGetDevice(&dev) != cudaSuccess)
+    return 0;
+  return places[dev];
+}
+static int tri_cluster(int n, bool df, bool shared) {
+  if (!df || shared || n < 2 || n > kTriClusterMax) return 0;
+  const int places = tri_cluster_places();
+  return (n > 160 && (places & 2)) ? 16 : ((places & 1) ? 8 : 0);
+}
+static int tri_cluster_launch(cudaStream_t s, int n, int G, const double* F, EigWork& w, int* status) {
+  cudaLaunchAttribute at[1];
+  const cudaLaunchConfig_t cfg = tri_cluster_config(G, tri_cluster_smem(n, G), s, at);
   if (cudaLaunchKernelEx(&cfg, tridiag_cluster_kernel, n, F, w.Vst, w.d, w.e, w.tau, status) != cudaSuccess) return -2;
   count_launch();
   return 0;
