@@ -3,6 +3,7 @@ matrix gives the same bits every time, at the sizes where the exchange can go wr
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -135,5 +136,46 @@ def test_alone_and_beside_others_the_results_are_the_same(n, precision):
     finally:
         if batch:
             kx.sim_batch_destroy(batch)
+        for h in hs:
+            kx.sim_destroy(h)
+
+
+@pytest.mark.parametrize("n", [1801, 2050, 2401, 2561, 3361])
+def test_fp64_with_rows_outside_shared_memory(n):
+    """Several launches with a hand-over between them, rows in L2 beside resident ones (n = 2050 and
+    above), and the shapes of the largest systems."""
+    h = lattice(n, kx.SIM_PREC_FP64, m_max=1, m_min=1)
+    try:
+        eps, Q = eigenpairs(h)
+        F = kx.sim_get_matrix(h, kx.SIM_MAT_FOCK)
+    finally:
+        kx.sim_destroy(h)
+    some = np.linspace(0, n - 1, 60).astype(int)
+    width = max(1.0, np.abs(eps).max())
+    assert np.abs(np.linalg.eigvalsh(F) - eps).max() <= width * (4e-12 + n * 2.0 ** -50)
+    assert np.abs(F @ Q[:, some] - Q[:, some] * eps[some]).max() <= 1e-9 * width
+    assert np.abs(Q.T @ Q[:, some] - np.eye(n)[:, some]).max() <= 1e-10
+
+
+@pytest.mark.parametrize("n,count", [(1000, 2), (2050, 3)])
+def test_fp64_small_grids_and_large_grids_that_meet(n, count):
+    """Beside others the small grid, with rows in L2; three threads at n = 2050 (four launches a
+    tridiagonalisation) so that a launch behind others may leave the work to its stand-in."""
+    hs = [lattice(n, kx.SIM_PREC_FP64, 1, m_max=1, m_min=1) for _ in range(count + 1)]
+    try:
+        kx.sim_step(hs[0], 3)
+        ref = [*kx.sim_get_state(hs[0], n), *eigenpairs(hs[0])]
+        if count == 2:
+            kx.sim_batch_step(hs[1:], 3)
+        else:
+            ts = [threading.Thread(target=kx.sim_step, args=(h, 3)) for h in hs[1:]]
+            for t in ts:
+                t.start()
+            for t in ts:
+                t.join()
+        for h in hs[1:]:
+            for a, b in zip(ref, [*kx.sim_get_state(h, n), *eigenpairs(h)]):
+                assert np.array_equal(a, b)
+    finally:
         for h in hs:
             kx.sim_destroy(h)
