@@ -55,10 +55,23 @@ __host__ __device__ __forceinline__ dfl df_from_double(double x) {
 }
 __host__ __device__ __forceinline__ double df_to_double(dfl a) { return (double)a.hi + (double)a.lo; }
 
-// FP32 -> FP64 by integer operations (exact; a subnormal is first scaled into the normal
-// range, an exact FP32 product): keeps the conversion off GB300's narrow FP64 pipe.  No branch
-// holds a conversion instruction, so none can be evaluated speculatively.
+// FP32 -> FP64 by integer operations (exact for normal numbers, infinities and
+// NaN; subnormal FP32 values, below 2^-126, become zero): keeps the conversion
+// off GB300's narrow FP64 pipe.  No branch holds a conversion instruction, so
+// none can be evaluated speculatively.
 __device__ __forceinline__ double f2d_int(float f) {
+  const unsigned u = __float_as_uint(f);
+  const unsigned ex = (u >> 23) & 0xFFu;
+  unsigned long long b = (unsigned long long)(u & 0x80000000u) << 32;
+  if (ex != 0) {
+    const unsigned long long e64 = (ex == 0xFFu) ? 0x7FFull : (unsigned long long)(ex + 896u);
+    b |= (e64 << 52) | ((unsigned long long)(u & 0x7FFFFFu) << 29);
+  }
+  return __longlong_as_double((long long)b);
+}
+// the same, exact for subnormal values too: they are scaled into the normal range first, an
+// exact FP32 product (epilogues of the slice products, whose low halves may be as small)
+__device__ __forceinline__ double f2d_int_exact(float f) {
   const bool small = (__float_as_uint(f) & 0x7F800000u) == 0;
   const unsigned u = __float_as_uint(small ? __fmul_rn(f, 0x1p32f) : f);
   const unsigned ex = (u >> 23) & 0xFFu;

@@ -79,7 +79,7 @@ __device__ __forceinline__ void twosum_acc(float& hi, float& lo, float b) {
 // GB300 takes 62 cycles for each, and the conversions, the sum and the product of a
 // 128 x 128 tile were 17 us of it (n = 240, 3 and 4 slices: 31 and 37 us -> 26 and 32).
 __device__ __forceinline__ double scaled_sum(double alpha, float hi, float lo) {
-  const double v = df_to_double_fast(dfl{hi, lo});
+  const double v = f2d_int_exact(hi) + f2d_int_exact(lo);
   return alpha == 1.0 ? v : (alpha == -1.0 ? -v : alpha * v);
 }
 
