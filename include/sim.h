@@ -60,11 +60,12 @@ enum sim_precision {
    * below the row maximum: to one rounding of the result and K 2^-60 of the
    * product of the two rows' maxima                                          */
   SIM_PREC_FP64 = 0,
-  /* FP64 eigensolve, mu and Krylov Gram/solve; density D0 = Q f Q^T and the
+  /* eigensolve in double-float (FP32 pairs, about 48 bits), mu and Krylov
+   * Gram/solve in FP64; back-transformation, density D0 = Q f Q^T and the
    * DMPT contractions of eq. 36 on tcgen05 tensor cores: operands cut into
-   * fixed-point BF16 slices (4 for the density, 3 for DMPT; 8 bits each
-   * relative to the row maximum), exact FP32 chunk sums, double-float
-   * accumulation across chunks, FP64 output                                 */
+   * fixed-point BF16 slices (4, and 3 for DMPT; 8 bits each
+   * relative to the row maximum), double-float accumulation across chunks,
+   * FP64 output                                                             */
   SIM_PREC_MIXED = 1,
 };
 

@@ -1,18 +1,19 @@
-// FP64 symmetric eigensolver for F = Q diag(eps) Q^T (eq. 19 needs the
-// eigenpairs; eq. 36 needs them again for the DMPT response).
+// Symmetric eigensolver for F = Q diag(eps) Q^T (eq. 19 needs the eigenpairs; eq. 36
+// needs them again for the DMPT response), in FP64 and, for the mixed path, in double-float.
 //
 //  1. Householder tridiagonalisation (tridiag.cu).
-//  2. Eigenvalues of the tridiagonal matrix by bisection on Sturm counts,
-//     one thread per eigenvalue (ascending order by construction): a coarse
-//     FP32 phase, an FP64 bracket check, then FP64 bisection.
-//  3. Eigenvectors by inverse iteration (two steps) with a partially pivoted
-//     tridiagonal LU, one thread per cluster of close eigenvalues; members of
-//     a cluster are re-orthogonalised (modified Gram-Schmidt) in order.
-//  4. Back-transformation Q = H_0 ... H_{n-3} Z with blocks of reflectors in
-//     compact WY form (I - V T V^T): FP64 GEMMs (64 per block) on the FP64
-//     path; on the mixed path (128 per block) the two large products
-//     V^T Z and V (T W) run on the tensor cores with 4 fixed-point BF16
-//     slices, while the T factor and T W stay in FP64.
+//  2. Eigenvalues of the tridiagonal matrix by multisection on Sturm counts, several lanes
+//     per eigenvalue (ascending order by construction).  FP64: FP32 counts first, then FP64
+//     counts on a grid of points; mixed: double-float counts.
+//  3. Eigenvectors by inverse iteration (two steps) with a partially pivoted tridiagonal
+//     LU, a thread per eigenvalue; members of a cluster of close eigenvalues are made
+//     orthogonal afterwards, a block per cluster.
+//  4. Back-transformation Q = H_0 ... H_{n-3} Z with blocks of 128 reflectors in compact
+//     WY form (I - V T V^T), carried out on Z^T.  Mixed: the two large products V^T Z and
+//     Y^T Z (Y = T^T V, double-float) on the tensor cores with 4 fixed-point BF16 slices.  FP64:
+//     all products on the tensor cores as digits (tc_gemm64.cu); up to 66 columns, and
+//     without tensor maps, blocks of 64 and products on the FP64 pipe (gemm64.cu).  The T
+//     factors are FP64 in both.
 #include <algorithm>
 #include <mutex>
 
@@ -23,8 +24,8 @@
 
 namespace kx {
 
-constexpr int kBtBlock = 64;          // reflectors per back-transform block (FP64 path)
-constexpr int kBtBlockTc = 128;       // reflectors per back-transform block (tensor-core path)
+constexpr int kBtBlock = 64;          // reflectors per back-transform block (products on the FP64 pipe)
+constexpr int kBtBlockTc = 128;       // reflectors per back-transform block (products on the tensor cores)
 constexpr double kEps = 2.220446049250313e-16;
 
 // read-only data of this launch (written by an earlier one): cached loads
@@ -297,7 +298,7 @@ __global__ void cluster_kernel(int n, const double* __restrict__ ev, const doubl
   if (i >= n) return;
   double ctol = 1e-7 * fmax(1.0, scal[2]);
   // a NaN gap starts a new cluster: non-finite input must not merge the whole
-  // spectrum into one cluster (one thread would then orthogonalise n vectors)
+  // spectrum into one cluster (one block would then orthogonalise n vectors)
   clus[i] = (i == 0 || !(ev[i] - ev[i - 1] <= ctol)) ? 1 : 0;
 }
 
@@ -1074,16 +1075,6 @@ int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork
       dgemm(s, 1, 0, m, n, kb, -1.0, Vb, n, w.Wt2, n, 1.0, Q + (size_t)c0 * n, n);
     }
   }
-  return 0;
-}
-
-int symmetric_eig(cudaStream_t s, int n, const double* F, double* eps, double* Q, EigWork& w,
-                  int* status, int sm_count) {
-  int rc = eig_tridiagonalize(s, n, F, w, status, sm_count, false, false, 0);
-  if (rc) return rc;
-  eig_bisect(s, n, eps, w, 1e-12, false, false);
-  eig_vectors(s, n, eps, Q, w, false, false);
-  eig_backtransform(s, n, Q, w, nullptr, nullptr, false);
   return 0;
 }
 

@@ -13,11 +13,11 @@
 //
 // h: diagonal blocks are gathered per atom by one block (deterministic order,
 // no atomics); off-diagonal blocks by one thread per pair.
-// F = h + G(P): one thread per pair reads its 100 integrals once, writes both
-// off-diagonal blocks (exchange) and the pair's Coulomb contributions to the
-// diagonal blocks of both atoms into cw[X][Y][10] (X the receiving atom);
-// one warp per atom then sums its row of cw in a fixed order and adds the
-// one-centre terms.  No atomics: the result does not depend on scheduling.
+// F = h + G(P): four threads per pair, in warps of their own, write a row of
+// both off-diagonal blocks (exchange) and a share of the pair's Coulomb
+// contributions to the diagonal blocks of both atoms into cw[X][Y][10] (X the
+// receiving atom); one warp per atom then sums its row of cw in a fixed order
+// and adds the one-centre terms, a lane per element.  No atomics: the result does not depend on scheduling.
 #include "common.cuh"
 #include "kernels.h"
 

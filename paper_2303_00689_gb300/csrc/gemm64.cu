@@ -1,5 +1,6 @@
-// FP64 GEMM on the CUDA cores: the DMPT products of small FP64 systems, and all FP64
-// products where tensor maps are not available (tc_gemm64.cu does the others).  Row-major
+// FP64 GEMM on the CUDA cores: the DMPT products and the back-transformation of small FP64
+// systems (up to 256 and 66 basis functions), and all FP64 products where tensor maps are
+// not available (tc_gemm64.cu does the others).  Row-major
 // C = alpha op(A) op(B) + beta C.  What bounds it is the FP64 pipe (2 FMAs a clock and
 // SM), so a tile is as small as its loads allow, one output per thread of a
 // 16 x 16 block: no padded work beyond 16 and n^2 / 256 blocks to spread over the SMs;

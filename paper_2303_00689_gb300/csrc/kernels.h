@@ -16,8 +16,6 @@ int create_shared(const sim_config* cfg, const sim_param_table* table, int natom
 
 // ---- pairs.cu ---------------------------------------------------------------
 bool upload_overlap_tables();
-void launch_pair_values(cudaStream_t s, int npair, const int* pA, const int* pB, const int* elem,
-                        const double* R, const ElemTable& tab, double* W, double* S, double* E);
 // df_rotation: the molecular-frame rotation of the integral blocks in
 // double-float on the FP32 pipe (mixed path) instead of FP64
 void launch_pair_derivs(cudaStream_t s, int npair, const int* pA, const int* pB, const int* elem,
@@ -108,8 +106,6 @@ int eig_backtransform(cudaStream_t s, int n, double* Q, EigWork& w, const TcWork
 // its half that needs no eigenvectors, which may run on another stream after the
 // tridiagonalisation (EigWork::side: its scratch is its own)
 int eig_backtransform_prepare(cudaStream_t s, int n, EigWork& w, const TcWork* tw, const Tc64Work* t64);
-int symmetric_eig(cudaStream_t s, int n, const double* F, double* eps, double* Q, EigWork& w,
-                  int* status, int sm_count);
 
 // ---- electronic.cu ----------------------------------------------------------
 struct Scalars {         // device-resident per-evaluation scalars

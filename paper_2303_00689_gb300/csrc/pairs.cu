@@ -618,23 +618,6 @@ __device__ void pair_block(const PairPart& part, const double* dvec, const Elem&
   *Eout = Radial<T>::promote(en + zz * g / Rr, uv);
 }
 
-__global__ void pair_values_kernel(int npair, const int* __restrict__ pA, const int* __restrict__ pB,
-                                   const int* __restrict__ elem, const double* __restrict__ R,
-                                   ElemTable tab, double* __restrict__ W, double* __restrict__ S,
-                                   double* __restrict__ E) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= npair) return;
-  int A = pA[t], B = pB[t];
-  double d[3] = {R[3 * B] - R[3 * A], R[3 * B + 1] - R[3 * A + 1], R[3 * B + 2] - R[3 * A + 2]};
-  const Elem& ea = tab.e[elem[A]];
-  const Elem& eb = tab.e[elem[B]];
-  double w[100], s[16], e;
-  pair_block<false, double>(pair_part(-1), d, ea, eb, w, s, &e);
-  for (int k = 0; k < 100; ++k) W[(size_t)k * npair + t] = w[k];
-  for (int k = 0; k < 16; ++k) S[(size_t)k * npair + t] = s[k];
-  E[t] = e;
-}
-
 template <bool DFROT, bool SHARED>
 __global__ void pair_derivs_kernel(int npair, const int* __restrict__ pA, const int* __restrict__ pB,
                                    const int* __restrict__ elem, const double* __restrict__ R,
@@ -746,13 +729,6 @@ static bool upload_overlap_tables_once() {
 bool upload_overlap_tables() {
   static PerDeviceOnce flag;
   return once_per_device(flag, [] { return upload_overlap_tables_once(); });
-}
-
-void launch_pair_values(cudaStream_t s, int npair, const int* pA, const int* pB, const int* elem,
-                        const double* R, const ElemTable& tab, double* W, double* S, double* E) {
-  if (npair <= 0) return;
-  pair_values_kernel<<<(npair + 127) / 128, 128, 0, s>>>(npair, pA, pB, elem, R, tab, W, S, E);
-  count_launch();
 }
 
 // half as many pairs as FP64 pipes (4 an SM, a warp of 32 each): mixed 1770, 7140, 16110

@@ -17,12 +17,12 @@
 // One CTA computes a 128 x 128 tile (128 x 64 or 128 x 32 while SMs are free) with 18 warps:
 //   warp 0 / lane 0 : TMA producer (128B-swizzled boxes of 128 rows x 64 K)
 //   warp 1          : allocates / frees TMEM; lane 0 issues tcgen05.mma
-//                     (M = 128, N = 128, K = 16 slices)
+//                     (M = 128, N = the tile's columns, K = 16)
 //   warps 2-17      : epilogue; warp w reads TMEM lane quarter w % 4 and
-//                     the 32-column group (w - 2) / 4
+//                     quarter (w - 2) / 4 of the columns
 // K is consumed in chunks of kChunk k-tiles that never straddle two
 // segments.  Each chunk accumulates (exactly, see above) in FP32 in one of
-// two TMEM buffers (2 x 128 columns); the epilogue warps fold every finished
+// two TMEM buffers (of the tile's columns); the epilogue warps fold every finished
 // chunk into double-float registers (FP32 hi + lo, TwoSum).  The final tile
 // is written in FP64.
 // A ring of kStages shared-memory stages is guarded by mbarriers (full: TMA
@@ -125,8 +125,7 @@ __device__ __forceinline__ void write_tile(double* tile, const float (&hi)[BN / 
 template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_gemm_kernel(const __grid_constant__ TcMaps maps, SegTable seg, int M, int N, int K, double alpha,
-                   double* __restrict__ C, int ldc, int sym, int beta, int* err, const int* gate, int kt_split,
-                   long long c_zstride) {
+                   double* __restrict__ C, int ldc, int sym, int* err, const int* gate) {
   if (gate && *gate == 0) return;      // whole CTA, before any barrier or TMEM use
   const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * BN;
   if (sym && m0 >= n0 + BN) return;
@@ -141,13 +140,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // split-K (kt_split > 0): CTA z takes k-tiles [z kt_split, (z + 1) kt_split) and
-  // writes its partial product to C + z c_zstride
-  const int ktiles_all = (K + kBK - 1) / kBK;
-  const int kt0 = (kt_split > 0) ? (int)blockIdx.z * kt_split : 0;
-  int ktiles = (kt_split > 0) ? min(kt_split, ktiles_all - kt0) : ktiles_all;
-  if (ktiles < 0) ktiles = 0;
-  C += (long long)blockIdx.z * c_zstride;
+  const int ktiles = (K + kBK - 1) / kBK;
   const int total = seg.nseg * ktiles;
   const int cps = (ktiles + kChunk - 1) / kChunk;   // chunks per segment
   const int nchunks = seg.nseg * cps;
@@ -185,8 +178,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!mbar_wait(&empty[s], ph ^ 1u, err)) { ok = false; break; }
         int sg = it / ktiles, kt = it % ktiles;
         mbar_expect_tx(&full[s], kTileBytesA + kTileBytesB);
-        tma_load_2d(sA + s * kTileBytesA, &maps.a[seg.a[sg]], &full[s], (kt0 + kt) * kBK, m0);
-        tma_load_2d(sB + s * kTileBytesB, &maps.b[seg.b[sg]], &full[s], (kt0 + kt) * kBK, n0);
+        tma_load_2d(sA + s * kTileBytesA, &maps.a[seg.a[sg]], &full[s], kt * kBK, m0);
+        tma_load_2d(sB + s * kTileBytesB, &maps.b[seg.b[sg]], &full[s], kt * kBK, n0);
         issued = it + 1;
       }
       if (!ok) {
@@ -257,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[b]);
     }
-    write_tile<BN>((double*)base, hi, lo, ok && total > 0, quarter, cg, lane, m0, n0, M, N, alpha, C, ldc, sym, beta, err);
+    write_tile<BN>((double*)base, hi, lo, ok && total > 0, quarter, cg, lane, m0, n0, M, N, alpha, C, ldc, sym, 0, err);
   }
   tc_fence_before();
   __syncthreads();
@@ -287,7 +280,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Split-K (kt_split > 0): CTA z takes k-tiles [z kt_split, (z + 1) kt_split)
 // and writes its partial product to C + z c_zstride.  beta != 0 adds to C.
 // The output tile goes through shared memory (the stages are idle by then).
-// TMEM: 4 x 128 columns (acc0 and acc1, double-buffered).
+// TMEM: 4 x the tile's columns (acc0 and acc1, double-buffered).
 template <int S, int BK>
 struct GroupedCfg {
   static constexpr int kTile = kBM * BK * 2;                 // one slice tile of A or B
@@ -571,37 +564,6 @@ __global__ void split_bf16_kernel(int n, const double* __restrict__ X, int ld, i
     if (a < slices) P[a][t] = v[a];
 }
 
-// per-row exponent of op(X), op(X) = X (rows x cols, ldx) or X^T (X stored cols x rows)
-__global__ void row_exponent_general_kernel(int rows, int cols, const double* __restrict__ X, int ldx,
-                                            int transpose, int* __restrict__ ex) {
-  int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
-  if (r >= rows) return;
-  unsigned long long m = 0;
-  for (int k = lane; k < cols; k += 32) {
-    double v = transpose ? X[(size_t)k * ldx + r] : X[(size_t)r * ldx + k];
-    unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFULL;
-    m = (b > m) ? b : m;
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o);
-    m = (t > m) ? t : m;
-  }
-  if (lane == 0) ex[r] = exponent_of_max(m);
-}
-
-__global__ void split_general_kernel(int rows, int cols, const double* __restrict__ X, int ldx, int transpose,
-                                     int slices, const int* __restrict__ ex, __nv_bfloat16* __restrict__ base,
-                                     int ld, size_t stride) {
-  size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  size_t tot = (size_t)rows * ld;
-  if (t >= tot) return;
-  int i = (int)(t / ld), j = (int)(t % ld);
-  double x = 0.0;
-  if (j < cols) x = transpose ? X[(size_t)j * ldx + i] : X[(size_t)i * ldx + j];
-  slice_value(x, ex[i], slices, base, stride, t);
-}
-
 // Row-wise slicing in one pass per row (a warp per row: the row maximum by
 // shuffles, then the slices); columns cols..ld-1 are written as zeros.  Used
 // by the back-transformation, whose operands change shape block by block.
@@ -850,19 +812,6 @@ static bool make_map_rc_box(CUtensorMap* m, void* ptr, int rows, int cols, int l
   return tc_encode_map_box(m, ptr, rows, cols, ld, bk, kBM);
 }
 
-static bool make_map_rc(CUtensorMap* m, void* ptr, int rows, int cols, int ld) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)kBM};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
 static bool make_map(CUtensorMap* m, void* ptr, int n, int ld) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
@@ -925,25 +874,22 @@ static int tile_columns(int M, int N, int z, bool wide) {
 }
 template <int BN>
 static void exact_run(cudaStream_t s, const TcMaps& maps, const SegTable& seg, int M, int N, int K, double alpha,
-                      double* C, int ldc, int sym, int beta, int* err, const int* gate, int kt_split, int z,
-                      long long zstride) {
+                      double* C, int ldc, int sym, int* err, const int* gate) {
   static PerDeviceOnce flag;
   once_per_device(flag, [] {
     return cudaFuncSetAttribute(tc_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) ==
            cudaSuccess;
   });
-  dim3 grid((N + BN - 1) / BN, (M + kBM - 1) / kBM, z);
-  tc_gemm_kernel<BN><<<grid, kThreads, kSmemBytes, s>>>(maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate,
-                                                       kt_split, zstride);
+  dim3 grid((N + BN - 1) / BN, (M + kBM - 1) / kBM);
+  tc_gemm_kernel<BN><<<grid, kThreads, kSmemBytes, s>>>(maps, seg, M, N, K, alpha, C, ldc, sym, err, gate);
   count_launch();
 }
 static void exact_launch(cudaStream_t s, const TcMaps& maps, const SegTable& seg, int M, int N, int K, double alpha,
-                         double* C, int ldc, int sym, int beta, int* err, const int* gate, int kt_split, int z,
-                         long long zstride) {
-  switch (tile_columns(M, N, z, false)) {
-    case 32: return exact_run<32>(s, maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
-    case 64: return exact_run<64>(s, maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
-    default: return exact_run<kBN>(s, maps, seg, M, N, K, alpha, C, ldc, sym, beta, err, gate, kt_split, z, zstride);
+                         double* C, int ldc, int sym, int* err, const int* gate) {
+  switch (tile_columns(M, N, 1, false)) {
+    case 32: return exact_run<32>(s, maps, seg, M, N, K, alpha, C, ldc, sym, err, gate);
+    case 64: return exact_run<64>(s, maps, seg, M, N, K, alpha, C, ldc, sym, err, gate);
+    default: return exact_run<kBN>(s, maps, seg, M, N, K, alpha, C, ldc, sym, err, gate);
   }
 }
 
@@ -985,7 +931,7 @@ void tc_gemm(cudaStream_t s, const TcWork& w, int slotA, int slotB, int terms, d
       ++seg.nseg;
     }
   int n = tb->n;
-  exact_launch(s, maps, seg, n, n, n, alpha, C, n, sym, 0, tb->err, gate, 0, 1, 0);
+  exact_launch(s, maps, seg, n, n, n, alpha, C, n, sym, tb->err, gate);
 }
 
 template <int S, int BK, int BN>
@@ -1078,75 +1024,6 @@ size_t tc_slot_stride(const TcWork& w) {
   TcBuffers* tb = (TcBuffers*)w.base;
   return (size_t)(tb->piece[0][1] - tb->piece[0][0]);
 }
-int* tc_slot_exponents(const TcWork& w, int slot) {
-  TcBuffers* tb = (TcBuffers*)w.base;
-  return tb->ex + (size_t)slot * tb->n;
-}
-
-// Slices of op(X) (rows x cols, K = cols) into `base` with row length ld and
-// slice stride `stride` elements; ex receives the row exponents.
-void tc_split_rc(cudaStream_t s, int rows, int cols, const double* X, int ldx, int transpose, int slices, int* ex,
-                 __nv_bfloat16* base, int ld, size_t stride) {
-  row_exponent_general_kernel<<<(rows * 32 + 255) / 256, 256, 0, s>>>(rows, cols, X, ldx, transpose, ex);
-  count_launch();
-  size_t tot = (size_t)rows * ld;
-  split_general_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(rows, cols, X, ldx, transpose, slices, ex,
-                                                                       base, ld, stride);
-  count_launch();
-}
-
-// C (M x N, ldc) = alpha * sum slice products A_a B_b^T (+ C if beta), A: M x K slices, B: N x K slices
-int tc_gemm_rc(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda, size_t astride,
-               const __nv_bfloat16* Bbase, int ldb, size_t bstride, int terms, double alpha, double* C, int ldc,
-               int beta, int* err) {
-  int slices = (terms == 10) ? 4 : (terms == 6) ? 3 : (terms == 3) ? 2 : 1;
-  TcMaps maps;
-  for (int a = 0; a < kTcMaxSlices; ++a) {
-    int sa = (a < slices) ? a : 0;
-    if (!make_map_rc(&maps.a[a], (void*)(Abase + sa * astride), M, K, lda)) return -1;
-    if (!make_map_rc(&maps.b[a], (void*)(Bbase + sa * bstride), N, K, ldb)) return -1;
-  }
-  SegTable seg;
-  seg.nseg = 0;
-  for (int d = slices - 1; d >= 0; --d)
-    for (int a = 0; a <= d; ++a) {
-      seg.a[seg.nseg] = a;
-      seg.b[seg.nseg] = d - a;
-      ++seg.nseg;
-    }
-  exact_launch(s, maps, seg, M, N, K, alpha, C, ldc, 0, beta, err, nullptr, 0, 1, 0);
-  return 0;
-}
-
-// Split-K variant of tc_gemm_rc: the K range is cut into `splits` parts (each a
-// whole number of exact-sum chunks), part z writes alpha * (its partial sum) to
-// P + z * M * ldp (M x N, ld ldp); the caller adds the parts in order.
-int tc_gemm_rc_splitk(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda, size_t astride,
-                      const __nv_bfloat16* Bbase, int ldb, size_t bstride, int terms, double alpha, double* P,
-                      int ldp, int splits, int* err) {
-  int slices = (terms == 10) ? 4 : (terms == 6) ? 3 : (terms == 3) ? 2 : 1;
-  TcMaps maps;
-  for (int a = 0; a < kTcMaxSlices; ++a) {
-    int sa = (a < slices) ? a : 0;
-    if (!make_map_rc(&maps.a[a], (void*)(Abase + sa * astride), M, K, lda)) return -1;
-    if (!make_map_rc(&maps.b[a], (void*)(Bbase + sa * bstride), N, K, ldb)) return -1;
-  }
-  SegTable seg;
-  seg.nseg = 0;
-  for (int d = slices - 1; d >= 0; --d)
-    for (int a = 0; a <= d; ++a) {
-      seg.a[seg.nseg] = a;
-      seg.b[seg.nseg] = d - a;
-      ++seg.nseg;
-    }
-  const int ktiles = (K + kBK - 1) / kBK;
-  int per = (ktiles + splits - 1) / splits;
-  per = ((per + kChunk - 1) / kChunk) * kChunk;          // whole exact-sum chunks
-  const int z = (ktiles + per - 1) / per;
-  exact_launch(s, maps, seg, M, N, K, alpha, P, ldp, 0, 0, err, nullptr, per, z, (long long)M * ldp);
-  return z;
-}
-
 void tc_split_rows(cudaStream_t s, int rows, int cols, const double* X, long long ldx, int slices,
                    __nv_bfloat16* base, int ld, size_t stride) {
   if (rows <= 0) return;
@@ -1201,7 +1078,7 @@ void tc_gemm_on_maps(cudaStream_t s, int n, const CUtensorMap* mapsA, const CUte
       seg.b[seg.nseg] = d - a;
       ++seg.nseg;
     }
-  exact_launch(s, maps, seg, n, n, n, alpha, C, n, sym, 0, err, nullptr, 0, 1, 0);
+  exact_launch(s, maps, seg, n, n, n, alpha, C, n, sym, err, nullptr);
 }
 
 }  // namespace kx

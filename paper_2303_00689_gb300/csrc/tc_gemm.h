@@ -39,11 +39,12 @@ void tc_gemm_grouped(cudaStream_t s, const TcWork& w, int slotA, int slotB, doub
 // sum |a||b| of the exact 10-term slice product
 void tc_gemm_grouped4(cudaStream_t s, const TcWork& w, int slotA, int slotB, double alpha, double* C, int sym,
                       const int* gate = nullptr);
-// general shapes with 4 slices (back-transformation); the same operands and
-// partial-product layout as tc_gemm_rc / tc_gemm_rc_splitk; < 0 on a tensor-map error
+// general shapes with 4 slices (back-transformation): C (M x N, ldc) = alpha A B^T (+ C if beta),
+// slice a of A's rows at Abase + a astride (row length lda), of B's likewise; < 0 on a tensor-map error
 int tc_gemm_grouped_rc(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda, size_t astride,
                        const __nv_bfloat16* Bbase, int ldb, size_t bstride, double alpha, double* C, int ldc,
                        int beta, int* err, bool wide);
+// split-K, whole exact-sum chunks a part: returns the number of parts z used (partials at P + z M ldp)
 int tc_gemm_grouped_rc_splitk(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda,
                               size_t astride, const __nv_bfloat16* Bbase, int ldb, size_t bstride, double alpha,
                               double* P, int ldp, int splits, int* err, bool wide);
@@ -57,17 +58,6 @@ void tc_split_pair(cudaStream_t s, int n, int ld, const double* A, const double*
 void tc_gemm_on_maps(cudaStream_t s, int n, const CUtensorMap* mapsA, const CUtensorMap* mapsB, int terms,
                      double alpha, double* C, int sym, int* err);
 
-// General shapes (back-transformation): slices of op(X) (rows x cols, K = cols, row
-// length ld, slice stride `stride` elements) and C (M x N, ldc) (+)= alpha sum A_a B_b^T
-void tc_split_rc(cudaStream_t s, int rows, int cols, const double* X, int ldx, int transpose, int slices, int* ex,
-                 __nv_bfloat16* base, int ld, size_t stride);
-int tc_gemm_rc(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda, size_t astride,
-               const __nv_bfloat16* Bbase, int ldb, size_t bstride, int terms, double alpha, double* C, int ldc,
-               int beta, int* err);
-// split-K: returns the number of parts z actually used (partials at P + z M ldp), < 0 on error
-int tc_gemm_rc_splitk(cudaStream_t s, int M, int N, int K, const __nv_bfloat16* Abase, int lda, size_t astride,
-                      const __nv_bfloat16* Bbase, int ldb, size_t bstride, int terms, double alpha, double* P,
-                      int ldp, int splits, int* err);
 // one-pass row slicing (row maximum and slices per warp), columns cols..ld-1 zero
 void tc_split_rows(cudaStream_t s, int rows, int cols, const double* X, long long ldx, int slices,
                    __nv_bfloat16* base, int ld, size_t stride);
@@ -115,6 +105,5 @@ int tc64_gemm(cudaStream_t s, int M, int N, int k0, int k1, const Tc64Op& A, int
 // raw access to a slot's slice buffers (for the back-transformation)
 __nv_bfloat16* tc_slot_base(const TcWork& w, int slot);
 size_t tc_slot_stride(const TcWork& w);
-int* tc_slot_exponents(const TcWork& w, int slot);
 
 }  // namespace kx

@@ -138,7 +138,7 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 __host__ __device__ __forceinline__ int tri_rows(int n, int k0, int G) { return (n - k0 - 1 + G - 1) / G; }
 
 // ---- FP64 -------------------------------------------------------------------------
-// n = 26, 240, 574, 1680: 100, 1320, 3800, 24000 us; with one block per 2^16 elements,
+// n = 26, 240, 574, 1680: 97, 1310, 3400, 21900 us; with one block per 2^16 elements,
 // rows dealt anew in every column and a grid barrier per column: 178, 8544, 17400,
 // 49545 us.
 //  * Rows i = b (mod G) belong to block b for the whole launch and live in its
