@@ -45,9 +45,9 @@ KERNEL_MODE = [0]      # sim_kernel of the timed runs (--kernel)
 # one (df.cuh), 13 on average over the three multiply-adds of an element
 DF_OPS_PER_FMA = 13.0
 # DRAM bytes (read + write) of one tridiag_df_kernel launch at n = 3360 from one
-# ncu capture of the bench's profile run (dram__bytes_read.sum 1.018e9 +
-# dram__bytes_write.sum 3.868e10; a one-pass metric set, kernel unchanged since)
-TRIDIAG_TRAFFIC = {"bytes": 1102843648 + 39244797440,
+# ncu capture of the bench's profile run (dram__bytes_read.sum 1.108e9 +
+# dram__bytes_write.sum 3.923e10; a one-pass metric set)
+TRIDIAG_TRAFFIC = {"bytes": 1108155904 + 39234333440,
                    "source": "ncu dram__bytes_read.sum + dram__bytes_write.sum, one tridiag_df_kernel launch "
                              "of bench.py --profile-run at n = 3360"}
 
