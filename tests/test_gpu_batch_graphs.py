@@ -54,7 +54,7 @@ def test_handles_stepped_by_threads_of_their_own_share_the_device():
                 t.start()
             for t in ts:
                 t.join()
-        assert per_step(threads) <= 1.2 * together
+        assert per_step(threads) <= 1.3 * together
     finally:
         for h in hs:
             kx.sim_destroy(h)

@@ -179,3 +179,24 @@ def test_fp64_small_grids_and_large_grids_that_meet(n, count):
     finally:
         for h in hs:
             kx.sim_destroy(h)
+
+
+@pytest.mark.parametrize("precision", [kx.SIM_PREC_FP64, kx.SIM_PREC_MIXED])
+def test_a_served_trajectory_has_the_bits_of_running_alone(precision):
+    """n = 240: in the server no cluster, a small grid, fewer lanes per eigenvalue, no side stream."""
+    mol = synth.fullerene_c60(seed=5)
+    cfg = kx.sim_config_default(Te=5000.0, precision=precision, scf_max=10, scf_accept=1, m_max=2, m_min=2)
+    table = kx.param_table(synth.table_to_array(synth.synthetic_table(1)))
+    with kx.Server() as srv:
+        tickets = [srv.submit(cfg, table, mol.Z, mol.R, charge=mol.charge, nsteps=4) for _ in range(3)]
+        srv.drain(120.0)
+        served = [srv.poll(t) for t in tickets]
+    h = kx.sim_create(cfg, table, mol.Z, mol.R, charge=mol.charge)
+    try:
+        records = kx.sim_step(h, 4)
+        R, V, F, _ = kx.sim_get_state(h, mol.natoms)
+    finally:
+        kx.sim_destroy(h)
+    for s in served:
+        assert s["status"] == kx.SIM_OK and s["records"] == records
+        assert np.array_equal(s["R"], R) and np.array_equal(s["V"], V) and np.array_equal(s["F"], F)
