@@ -340,15 +340,16 @@ static void join_side(sim_handle* h, int k) {
 // side work only outside phase profiling (whose events time the main stream)
 static bool concurrent(const sim_handle* h) { return h->side && !h->prof; }
 
-// eigenpairs of the Fock matrix; with fermi_side, the Fermi occupations and
-// mu (eq. 8; they need the eigenvalues only) run on the side stream while the
-// eigenvectors are formed, and the caller joins before the density
+// the eigensolver grid's share of the device (eig_tridiag_weight), asked for once
 static int grid_weight(sim_handle* h, bool shared) {
   int& w = h->weight[shared];
   if (w < 0) w = eig_tridiag_weight(h->n, h->sms, mixed(h), shared);
   return w;
 }
 
+// eigenpairs of the Fock matrix; with fermi_side, the Fermi occupations and
+// mu (eq. 8; they need the eigenvalues only) run on the side stream while the
+// eigenvectors are formed, and the caller joins before the density
 static int eig(sim_handle* h, bool fermi_side = false) {
   h->tw.wide = h->shared;
   const TcWork* tw = mixed(h) ? &h->tw : nullptr;
