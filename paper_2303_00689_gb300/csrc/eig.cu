@@ -662,9 +662,10 @@ static BtBytes bt_bytes(int n);      // slices (mixed path)
 static BtBytes bt64_bytes(int n);    // digits (FP64)
 // Up to this size the half of the back-transformation that needs no eigenvectors (Gram
 // matrices, T factors, T^T V, slices) runs on the side stream during multisection and
-// inverse iteration, which leave most SMs idle there.  Above, the kernels slow one
-// another by more than is gained (1680: 22.95 -> 23.14 ms, FP64 45.4 -> 46.5).  C60 step 2.90 -> 2.64 ms, C120 4.84 -> 4.57, 574 basis
-// functions in FP64 9.82 -> 9.58.
+// inverse iteration, which leave most SMs idle there: C60 step 2.90 -> 2.64 ms, C120 4.84 ->
+// 4.57, 574 basis functions in FP64 9.82 -> 9.58.  At 1680 the kernels slow one another by more
+// than is gained in the mixed path (23.32 -> 23.55 ms); between, 720 to 1440, there would be 2 to
+// 4 % (FP64 0.4 to 2.6 %) for the memory of a scratch of its own.
 constexpr int kBtSideMax = 640;
 static bool bt_splits(int n) { return n > 2 && n <= kBtSideMax; }
 
@@ -674,7 +675,7 @@ static bool bt_splits(int n) { return n > 2 && n <= kBtSideMax; }
 // an unpadded layout would leave the region 8 bytes off).
 // The inverse-iteration workspace (5 n^2) also holds what the later stages need: `late`, the third
 // FP64 operand (tc_gemm64.cu) and, unless the preparation runs beside the inverse iteration
-// (side), `early` and the first two.  FP64 at n = 1680: 137 MB less than with buffers of their own.
+// (side), `early` and the first two.  FP64 at n = 1680: 1182 MB a handle, 1284 with buffers of their own.
 static size_t eig_layout(int n, EigProducts kind, bool side, void* base, EigWork* w) {
   const size_t nn = (size_t)n * n;
   side = side && bt_splits(n) && kind != kEigPlain;
